@@ -52,12 +52,13 @@ extern "C" {
 #define GEM_ECUDA (-3)     /* a CUDA runtime call or kernel launch failed                 */
 #define GEM_ESTATE (-4)    /* call order violated (backward before forward, ...)          */
 #define GEM_ECAPACITY (-5) /* returned by gem_status: the pair list overflowed max_pairs  */
-#define GEM_ETIMEOUT (-6)  /* reserved: a device-side wait ran out.  No kernel of this    */
-                           /* library waits on another (work is claimed from counters    */
-                           /* that never block), so no call returns it today.            */
+#define GEM_ETIMEOUT (-6)  /* returned by gem_status: a wait between the warps of a      */
+                           /* kernel ran out of tries (none does in working order; no    */
+                           /* kernel waits on another), the outputs are incomplete       */
 
 /* Device status bits reported by gem_status. */
 #define GEM_STATUS_CAPACITY 1
+#define GEM_STATUS_TIMEOUT 2
 
 typedef struct gem_ctx gem_ctx;
 
@@ -94,8 +95,8 @@ int gem_config_default(gem_config *cfg, int32_t d, float apix, int32_t max_B, in
 /* Create a context.  cuda_stream is a cudaStream_t (NULL: the legacy default
  * stream).  Allocates all scratch on the current device: about
  * 32 B x max_B x max_M (projected records) + 48 B x max_B x max_M (moments)
- * + 16 B x max_pairs (list entries with their block masks, and the
- * binning's hit records) + 20 B x max_B x d^2 (images, spectra) and
+ * + 18 B x max_pairs (list entries with their block masks, the binning's hit
+ * records, and partial images of tiles with long lists) + 20 B x max_B x d^2 (images, spectra) and
  * a few small tables.  Errors: GEM_EINVAL, GEM_ENOMEM, GEM_ECUDA. */
 int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream);
 
@@ -385,13 +386,11 @@ int gem_ctf_loss_static(int32_t d, float apix, int32_t B, const float *proj, con
 /* ---- rasteriser configurations and the autotuner ----------------------- */
 
 /* Both rasterisers come in several kernel configurations that compute the
- * same result (bitwise, for a given configuration; within float rounding
- * across configurations): the forward (step a3) as equal runs of items
- * across blocks or runs aligned to blocks, at 8 or 9 CTAs per SM, on a
- * per-tile grid or a persistent grid (5 to 9 CTAs per SM) that takes tiles
- * longest-first from a counter; the backward (a5) with 1 or 2 lanes per record, on either grid,
- * and with warp windows of 64, 128 or 256 records and 5 to 8 CTAs per SM
- * on the persistent grid.
+ * same result (the forward bitwise, the backward within the rounding of
+ * float64 sums taken in another order): the forward (step a3) with 6 to 12
+ * warps that evaluate and 2 or 4 that stage records, and 1 to 3 CTAs per SM;
+ * the backward (a5) with 1 or 2 lanes per record, on a per-tile or a persistent
+ * grid, with warp windows of 64, 128 or 256 records and 5 to 8 CTAs per SM.
  * Which is
  * fastest depends on the image side, the batch and the Gaussians' sizes.
  * Counts of each kind (kind 0: forward, 1: backward); a configuration's

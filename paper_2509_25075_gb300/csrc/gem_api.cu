@@ -76,8 +76,9 @@ struct gem_ctx {
   // gem_raster.cu); -1: the autotuner's cached choice for the call's shape,
   // else the default
   int fwd_cfg = -1, bwd_cfg = -1;
-  uint32_t *order = nullptr;     // [max_B * T] tile order of the persistent forward
-  unsigned *next_tile = nullptr;  // [2] work counters of the persistent forward, backward
+  uint32_t *order = nullptr;     // [max_B * T] tile order of the persistent backward
+  unsigned *next_tile = nullptr;  // [1] its work counter
+  RasterTasks tasks{};            // segments of the tile lists
   float *tune_grad = nullptr;     // [max_M][11] gradient the autotuner's backward writes
   std::vector<void *> allocs;
   // per-stage timing (events recorded around each stage when enabled)
@@ -108,7 +109,7 @@ struct gem_ctx {
 
 // The configurations used when neither the context nor the autotuner's cache
 // names one (the fastest measured on the benchmark workloads).
-constexpr int kDefaultFwdCfg = 3;  // block-aligned, 256-record windows, persistent longest-first
+constexpr int kDefaultFwdCfg = 0;  // 6 consumer and 2 producer warps, 3 CTAs per SM
 constexpr int kDefaultBwdCfg = 3;  // one lane per record, persistent longest-first
 
 // The autotuner's choices, shared by every context of the process: keyed by
@@ -284,7 +285,12 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
             alloc(c, &c->Z, (size_t)g.max_B * d * d) && alloc(c, &c->tw, (size_t)d) &&
             alloc(c, &c->lossp, (size_t)g.max_B * (ctf_partials(d) + 1)) && alloc(c, &c->status, 1) &&
             alloc(c, &c->kept, 2) &&
-            alloc(c, &c->order, (size_t)g.max_B * c->T) && alloc(c, &c->next_tile, 2);
+            alloc(c, &c->order, (size_t)g.max_B * c->T) && alloc(c, &c->next_tile, 1);
+  // a task per tile, or two per partial image of tiles with several segments
+  const size_t nparts = raster_part_count(c->cfg.max_pairs);
+  ok = ok && alloc(c, &c->tasks.task, 2 * ((size_t)g.max_B * c->T + nparts)) &&
+       alloc(c, &c->tasks.part, nparts * 256) && alloc(c, &c->tasks.done, (size_t)g.max_B * c->T) &&
+       alloc(c, &c->tasks.ctr, kCtrCount);
   // nearest-neighbour grid: at most 2 max_M + 64 cells
   c->knn.cap = 2 * g.max_M + 64;
   ok = ok && alloc(c, &c->knn.part, 608 * 6) && alloc(c, &c->knn.grid, 1) &&
@@ -309,6 +315,8 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
   }
   c->bin.cap = c->cfg.max_pairs;
   c->bin.status = c->status;
+  c->bin.task_ctr = c->tasks.ctr;
+  c->tasks.status = c->status;
   std::vector<float2> tw(d);
   for (int m = 0; m < d; ++m) {
     double a = -2.0 * 3.14159265358979323846 * m / d;
@@ -318,7 +326,9 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
   if ((e = cudaMemcpy(c->tw, tw.data(), d * sizeof(float2), cudaMemcpyHostToDevice)) !=
           cudaSuccess ||
       (e = cudaMemset(c->status, 0, sizeof(int))) != cudaSuccess ||
-      (e = bin_configure(d)) != cudaSuccess || (e = ctf_configure(d)) != cudaSuccess) {
+      (e = cudaMemset(c->tasks.done, 0, (size_t)g.max_B * c->T * sizeof(unsigned))) != cudaSuccess ||
+      (e = bin_configure(d)) != cudaSuccess || (e = ctf_configure(d)) != cudaSuccess ||
+      (e = raster_configure()) != cudaSuccess) {
     snprintf(g_create_err, sizeof(g_create_err), "set-up: %s", cudaGetErrorString(e));
     gem_destroy(c);
     return GEM_ECUDA;
@@ -357,6 +367,7 @@ int gem_status(gem_ctx *c) {
     return cuda_fail(c, e, "status read");
   if ((e = cudaMemset(c->status, 0, sizeof(int))) != cudaSuccess)
     return cuda_fail(c, e, "status clear");
+  if (st & GEM_STATUS_TIMEOUT) return fail(c, GEM_ETIMEOUT, "a wait inside a kernel ran out");
   if (st & GEM_STATUS_CAPACITY)
     return fail(c, GEM_ECAPACITY, "pair list exceeded max_pairs=%lld",
                 (long long)c->cfg.max_pairs);
@@ -428,12 +439,10 @@ int gem_project(gem_ctx *c, const float *params, int64_t M, int32_t B, const flo
   }
   {
     const int fc = active_fwd(c, B, M);
-    StageScope sc(c, GEM_STAGE_RASTER_FWD, fwd_config(fc).persistent ? 2 : 1);
-    if ((e = launch_raster_fwd(fc, c->rec, c->bin.list,
-                               c->bin.tile_start, c->bin.cap, M, B, g.d, c->l2tau, proj, c->order,
-                               c->next_tile, c->stream)) != cudaSuccess)
+    StageScope sc(c, GEM_STAGE_RASTER_FWD, 2);
+    if ((e = launch_raster_fwd(fc, c->rec, c->bin.list, c->bin.tile_start, c->bin.cap, M, B, g.d,
+                               c->l2tau, proj, c->tasks, true, c->stream)) != cudaSuccess)
       return cuda_fail(c, e, "raster_fwd");
-    if (fwd_config(fc).persistent) c->order_gen = c->bins_gen;
   }
   c->have_proj = true;
   return GEM_OK;
@@ -501,7 +510,7 @@ static int backward_common(gem_ctx *c, const float *dproj, float *grad, bool den
     else
       e = launch_raster_bwd(active_bwd(c, c->B, c->M), c->rec, c->bin.list,
                             c->bin.tile_start, c->bin.cap, c->M, c->B, g.d, c->l2tau, dproj, c->mom,
-                            c->order, c->next_tile + 1, c->order_gen == c->bins_gen, c->stream);
+                            c->order, c->next_tile, c->order_gen == c->bins_gen, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "raster_bwd");
   }
   StageScope sc(c, GEM_STAGE_PREP_BWD, 2);
@@ -652,7 +661,7 @@ int gem_pair_stats(gem_ctx *c, int64_t *kept, int64_t *evaluated) {
           cudaSuccess ||
       (e = launch_count_kept(active_fwd(c, c->bins_B, c->bins_M), c->rec, c->bin.list,
                              c->bin.tile_start, c->bin.cap, c->bins_M, c->bins_B, g.d,
-                             c->bins_l2tau, c->kept, c->order, c->next_tile, c->stream)) !=
+                             c->bins_l2tau, c->kept, c->tasks, c->stream)) !=
           cudaSuccess ||
       (e = cudaStreamSynchronize(c->stream)) != cudaSuccess)
     return cuda_fail(c, e, "pair count");
@@ -726,7 +735,7 @@ int gem_query(gem_ctx *c, const float *params, int64_t M, float tau, float *vol)
             cudaSuccess ||
         (e = launch_raster_fwd(active_fwd(c, ns, M), c->rec, c->bin.list,
                                c->bin.tile_start, c->bin.cap, M, ns, g.d, l2tau,
-                               vol + (size_t)k0 * slice, c->order, c->next_tile, c->stream)) !=
+                               vol + (size_t)k0 * slice, c->tasks, true, c->stream)) !=
             cudaSuccess)
       return cuda_fail(c, e, "query");
     c->have_bins = true;
@@ -942,8 +951,7 @@ int gem_autotune(gem_ctx *c, const float *params, int64_t M, int32_t B, const fl
     for (int r = -1; r < reps; ++r) {  // r = -1: warm-up
       cudaEventRecord(e0, c->stream);
       e = launch_raster_fwd(i, c->rec, c->bin.list, c->bin.tile_start, c->bin.cap, M,
-                            B, g.d, c->l2tau, c->proj, c->order, c->next_tile, c->stream);
-      if (e == cudaSuccess && fwd_config(i).persistent) c->order_gen = c->bins_gen;
+                            B, g.d, c->l2tau, c->proj, c->tasks, false, c->stream);
       cudaEventRecord(e1, c->stream);
       if (e != cudaSuccess || (e = cudaEventSynchronize(e1)) != cudaSuccess) {
         rc = cuda_fail(c, e, "autotune forward");

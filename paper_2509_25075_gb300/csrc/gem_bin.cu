@@ -640,7 +640,8 @@ __global__ void __launch_bounds__(32 * kScanWarps) tile_scan_cols_kernel(
 // counts as four consecutive runs of 1024 (one per sub-round q), with one
 // set of barriers; every thread keeps the running carry itself.
 __global__ void __launch_bounds__(1024) scan_tiles_kernel(int64_t *__restrict__ x, int64_t n,
-                                                          int64_t cap, int *__restrict__ status) {
+                                                          int64_t cap, int *__restrict__ status,
+                                                          unsigned *__restrict__ task_ctr) {
   constexpr int kQ = 4;
   __shared__ int64_t wtot[kQ][32];  // per run: exclusive prefix of the warps' sums
   __shared__ int64_t qtot[kQ];      // per run: its total
@@ -684,6 +685,7 @@ __global__ void __launch_bounds__(1024) scan_tiles_kernel(int64_t *__restrict__ 
     }
     __syncthreads();  // wtot and qtot are read before the next round rewrites them
   }
+  if (threadIdx.x < kCtrCount) task_ctr[threadIdx.x] = 0u;
   if (threadIdx.x == 0) {
     x[n] = carry;
     if (carry > cap) atomicOr(status, kStatusCapacity);
@@ -848,7 +850,7 @@ cudaError_t launch_bin(const Rec *rec, const uint16_t *key, int64_t M, int B, in
   int64_t ncols = (int64_t)B * T;
   tile_scan_cols_kernel<<<dim3((unsigned)((T + 31) / 32), (unsigned)B), 32 * kScanWarps, 0, st>>>(
       s.tcnt, nch, T, s.tile_start);
-  scan_tiles_kernel<<<1, 1024, 0, st>>>(s.tile_start, ncols, s.cap, s.status);
+  scan_tiles_kernel<<<1, 1024, 0, st>>>(s.tile_start, ncols, s.cap, s.status, s.task_ctr);
   tile_scatter_kernel<<<g, 256, tile_smem_bytes(d), st>>>(perm, M, d, nch, s.tcnt, s.tile_start, s);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   *perm_out = perm;

@@ -17,6 +17,7 @@ constexpr float kMargin = 1e-3f;
 
 // Device status bits (mirror GEM_STATUS_* in gem.h).
 constexpr int kStatusCapacity = 1;
+constexpr int kStatusTimeout = 2;
 
 // Per-Gaussian quantities independent of the view (64 B): p (3), log2 of
 // the amplitude constant (-inf for a Gaussian that contributes nothing),
@@ -292,6 +293,7 @@ struct BinScratch {
   unsigned long long *hit_ctr;  // [1] hits[] allocation cursor
   int64_t cap;
   int *status;
+  unsigned *task_ctr;  // [kCtrCount] the rasterisers' counters, reset by the scan
 };
 // Stable sort of 16-bit keys [B][M] per row (two 8-bit counting passes,
 // ties in index order): perm[b][r] = index of rank r.  dcnt and packed are
@@ -311,21 +313,32 @@ size_t bin_chunks_tiles(int64_t M);
 cudaError_t bin_configure(int d);
 
 // gem_raster.cu
-// A configuration of the forward rasteriser: form 0 = equal runs across
-// blocks, 1 = block-aligned runs; sub = 128-record sub-windows per window;
-// minb = CTAs per SM the launch bound asks for; persistent = a grid of
-// minb CTAs per SM pulling tiles longest-first from a counter.
+// Tasks of the rasterisers (segments of the tiles' lists, see gem_raster.cu).
+constexpr int kCtrFwd = 0, kCtrBwd = 1;      // next task of the forward, the backward
+constexpr int kCtrTasks = 2, kCtrParts = 3;  // tasks made, partial images handed out
+constexpr int kCtrCount = 4;
+struct RasterTasks {
+  uint4 *task;     // two words per task: (list start, lo and hi; entries; image * T + tile),
+                   // (segment, segments of the tile, the tile's first partial image, 0)
+  float *part;     // [parts][256] partial images of tiles with several segments
+  unsigned *done;  // [B * T] segments finished, zero between calls
+  unsigned *ctr;   // [kCtrCount], reset by the binning
+  int *status;     // kStatusTimeout when a wait ran out
+};
+size_t raster_part_count(int64_t cap);
+cudaError_t raster_configure();
+// A configuration of the forward rasteriser: consumer and producer warps per
+// CTA, CTAs per SM.
 struct FwdCfg {
-  int form, sub, minb, persistent;
-  int ctas;  // persistent grid: CTAs per SM (at most minb, the kernel's bound)
+  int cons, prod, ctas;
   const char *name;
 };
 int fwd_config_count();
 const FwdCfg &fwd_config(int i);
-// order [B*T] and next_tile [1] are scratch of the persistent forms.
+// fresh: the binning has just reset the counters; else they are reset here.
 cudaError_t launch_raster_fwd(int cfg, const Rec *rec, const uint2 *list,
                               const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
-                              float l2tau, float *proj, uint32_t *order, unsigned *next_tile,
+                              float l2tau, float *proj, const RasterTasks &tk, bool fresh,
                               cudaStream_t st);
 // A configuration of the backward rasteriser: lanes sharing one record,
 // records per lane per warp window, persistent grid (tiles longest-first
@@ -346,9 +359,9 @@ cudaError_t launch_raster_bwd(int cfg, const Rec *rec, const uint2 *list,
                               float l2tau, const float *dproj, double *mom, uint32_t *order,
                               unsigned *next_tile, bool order_ready, cudaStream_t st);
 cudaError_t launch_count_kept(int cfg, const Rec *rec, const uint2 *list,
-                              const int64_t *tile_start, int64_t cap,
-                              int64_t M, int B, int d, float l2tau, unsigned long long *kept,
-                              uint32_t *order, unsigned *next_tile, cudaStream_t st);
+                              const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
+                              float l2tau, unsigned long long *kept, const RasterTasks &tk,
+                              cudaStream_t st);
 cudaError_t launch_dense_fwd(const Rec *rec, int64_t M, int B, int d, float l2tau, float *proj,
                              cudaStream_t st);
 cudaError_t launch_dense_bwd(const Rec *rec, int64_t M, int B, int d, float l2tau,

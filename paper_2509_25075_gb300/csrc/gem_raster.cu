@@ -1,29 +1,22 @@
 // Steps a3 (raster forward) and a5 (raster backward) of the GEM hot path,
 // plus the plain dense forms used as the baseline.
 //
-// Both rasterisers run CTAs of 128 threads over (image, 16x16 tile) work
-// items — one per tile on a per-tile grid, or taken from a counter over a
-// longest-first tile order on a persistent grid of a chosen number of CTAs
-// per SM — and walk the tile's list, which is in ascending depth and
-// carries, per entry, the mask of the 4x4 pixel blocks the Gaussian's
-// region above tau meets (computed once by the binning).  A Gaussian
-// therefore costs 16 pixel evaluations per block it touches, instead of 256
-// per tile.  Pixels are evaluated in whitened coordinates (Rec): the
-// exponent is l2A - (u11 dx + u12 dy)^2 - (u22 dy)^2.
+// A tile's list is in ascending depth and carries, per entry, the mask of
+// the 4x4 pixel blocks the Gaussian's region above tau meets (computed once
+// by the binning).  A Gaussian therefore costs 16 pixel evaluations per block
+// it touches, instead of 256 per tile.  Pixels are evaluated in whitened
+// coordinates (Rec): the exponent is l2A - (u11 dx + u12 dy)^2 - (u22 dy)^2.
 //
-// a3: Eq. render restricted by Eq. accu.  Records are staged 256 at a time
-//     (a window; only the 24 bytes the evaluation reads).  One warp bit
-//     transpose of the lanes' packed block masks gives each block's record
-//     set; the window's (block, record) items are laid out block after
-//     block, each block's records in list order, and each block gets a
-//     share of the 128 threads in proportion to its items, so a thread
-//     never leaves its block.  A thread evaluates the 16 pixels of its block
-//     for each of its items (packed float pairs) and writes one partial
-//     image of the block; at the end of the window each pixel sums its
-//     block's partials in thread order and joins its running sum with Kahan
-//     compensation.  (The equal-runs form, raster_fwd_kernel, cuts the
-//     items into 128 equal runs across blocks instead.)  The result is
-//     deterministic and follows the list's depth order run by run.
+// a3: Eq. render restricted by Eq. accu.  The lists are cut into segments of
+//     at most 1024 entries, taken from a counter by persistent CTAs.  Producer
+//     warps stage a segment's records (only the 24 bytes the evaluation reads)
+//     and, by warp bit transposes of the packed block masks, each block's
+//     record set; consumer warps take the window's blocks one after the other
+//     and evaluate 32 of a block's records at a time, one record and 16 pixels
+//     per lane (packed float pairs).  A pixel's sum within a segment runs
+//     over lanes, then by a tree over the 32 lanes; a tile's segments join in
+//     list order with Kahan compensation.  The result is deterministic and
+//     follows the list's depth order segment by segment.
 // a5: the "efficient gradient" of Sec. 1 (iii) / Sec. 3.2: only pairs kept by
 //     Eq. accu.  Each warp takes windows of 64, 128 or 256 records of the
 //     list (the next one not yet taken), sorts the window by block count
@@ -40,8 +33,6 @@
 //     atomics), so the sum over a Gaussian's tiles loses nothing to
 //     rounding.  No barrier couples the warps within a tile.  a6 turns the
 //     moments into parameter gradients.
-#include <type_traits>
-
 #include "gem_internal.cuh"
 
 namespace gem {
@@ -69,206 +60,435 @@ __device__ __forceinline__ unsigned warp_transpose32(unsigned x, int lane) {
   return x;
 }
 
-constexpr int kSub = 2;                // forward: records staged per thread per window
-constexpr int kWin = kThreads * kSub;  // records staged per window
-static_assert(kThreads == 128, "the forward splits items with shifts by 7");
-constexpr int kFwdMinBlocks = 9;      // forward: CTAs per SM (10, with fewer registers, ran slower)
 
+// One record in one 256-bit load: a warp's gather of 32 records then takes
+// one pass over the L1 tags, not one for each half.
+__device__ __forceinline__ Rec load_rec(const Rec *p) {
+  Rec r;
+  asm volatile("ld.global.nc.L1::no_allocate.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=f"(r.a.x), "=f"(r.a.y), "=f"(r.a.z), "=f"(r.a.w), "=f"(r.b.x), "=f"(r.b.y),
+                 "=f"(r.b.z), "=f"(r.b.w)
+               : "l"(p));
+  return r;
+}
+
+// Barrier id over the given number of threads of the CTA.
+__device__ __forceinline__ void named_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// mbarriers in shared memory: arrivals release, waits acquire.
+__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(a) : "memory");
+}
+// Waits for the phase of the given parity, at most kWaitTries tries (each
+// suspends the thread for a hardware time slice; seconds in all); false when
+// it did not complete.
+constexpr int kWaitTries = 1 << 22;
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
+  for (int i = 0; i < kWaitTries; ++i) {
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(a), "r"(parity)
+        : "memory");
+    if (ok) return true;
+  }
+  return false;
+}
+
+constexpr int kFwdWin = 1024;  // forward: records staged per window
+
+// Tasks of the rasterisers.  A tile's list is cut into segments of S entries
+// (the last one shorter); a task is one segment, staged as one window, so
+// that no CTA walks a long list alone (the longest list of a workload holds
+// five to twenty times the mean) and a call with few tiles still fills the
+// SMs.  S is 1024, less (down to 256) where that would leave resident CTAs
+// without a segment.  Tasks follow the tiles' index order up to the order in
+// which the CTAs here claim their ranges, so neighbouring tiles, which share
+// records, are in flight together.  Empty tiles get their zeros here and no
+// task.
+__device__ __forceinline__ int64_t segment_length(int64_t total, int slots) {
+  const int64_t S = total / (2 * (int64_t)slots);
+  return (max((int64_t)256, min((int64_t)kFwdWin, S)) + 63) / 64 * 64;
+}
+
+__global__ void __launch_bounds__(256) raster_tasks_kernel(const int64_t *__restrict__ tile_start,
+                                                           int ntiles, int64_t cap, int d, int slots,
+                                                           RasterTasks tk, float *__restrict__ proj) {
+  __shared__ unsigned wsum[2][8], base_sh[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  const int64_t total = tile_start[ntiles];
+  // lists that overflowed their capacity are incomplete: every list counts
+  // as empty (the status word reports it)
+  const bool over = total > cap;
+  const int64_t S = segment_length(total, slots);
+  int64_t s = 0, len = 0;
+  if (i < ntiles) {
+    s = tile_start[i];
+    len = over ? 0 : tile_start[i + 1] - s;
+  }
+  unsigned nseg = (unsigned)((len + S - 1) / S);
+  // exclusive prefixes of the tasks and of the partial images they need
+  unsigned inc = nseg, incp = nseg > 1 ? nseg : 0;
+  const unsigned mine = incp;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned u = __shfl_up_sync(0xffffffffu, inc, o), v = __shfl_up_sync(0xffffffffu, incp, o);
+    if (lane >= o) {
+      inc += u;
+      incp += v;
+    }
+  }
+  if (lane == 31) {
+    wsum[0][warp] = inc;
+    wsum[1][warp] = incp;
+  }
+  __syncthreads();
+  unsigned at = inc - nseg, part = incp - mine, all = 0, allp = 0;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    if (w < warp) {
+      at += wsum[0][w];
+      part += wsum[1][w];
+    }
+    all += wsum[0][w];
+    allp += wsum[1][w];
+  }
+  if (threadIdx.x == 0) {
+    base_sh[0] = atomicAdd(tk.ctr + kCtrTasks, all);
+    base_sh[1] = atomicAdd(tk.ctr + kCtrParts, allp);
+  }
+  __syncthreads();
+  at += base_sh[0];
+  part += base_sh[1];
+  if (nseg > 0) {
+    for (unsigned k = 0; k < nseg; ++k) {
+      const int64_t a = s + k * S, n = min(S, s + len - a);
+      uint4 *t = tk.task + 2 * (int64_t)(at + k);
+      t[0] = make_uint4((unsigned)a, (unsigned)((uint64_t)a >> 32), (unsigned)n, (unsigned)i);
+      t[1] = make_uint4(k, nseg, part, 0u);
+    }
+  }
+  if (proj) {
+    const int nt = d / kTile, T = nt * nt;
+    for (unsigned e = __ballot_sync(0xffffffffu, i < ntiles && nseg == 0); e; e &= e - 1) {
+      const int bt = blockIdx.x * 256 + warp * 32 + __ffs(e) - 1;
+      const int b = bt / T, t = bt - b * T;
+      float *o = proj + ((int64_t)b * d + (t / nt) * kTile) * d + (t % nt) * kTile;
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+        *reinterpret_cast<float4 *>(o + (int64_t)(8 * q + (lane >> 2)) * d + 4 * (lane & 3)) =
+            make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+}
+
+// Shared memory of one forward CTA: two staged windows, the lists of the
+// consumer warps, and the barriers.
+struct FwdWindow {
+  float4 sa[kFwdWin];        // px, py, u11, u12
+  float2 sb[kFwdWin];        // u22, log2 A
+  unsigned bal[16][33];      // block, 32 records: which touch it
+  float out[16][16];         // block, pixel: the window's sums
+  int n, bt;                 // entries (-1: no more tasks), image * T + tile
+  unsigned seg, nseg, part;  // segment of the tile, how many, first partial image
+  int next_block, done;      // blocks handed out, blocks finished
+};
+template <int kCons>
+struct FwdShared {
+  uint4 desc[2][2];                      // the producers' current and next task
+  FwdWindow win[2];
+  unsigned short slots[kCons][kFwdWin];  // a block's records, in list order
+  uint64_t full[2], empty[2];            // mbarriers
+};
+
+// a3.  One producer warp and kCons consumer warps per CTA, two windows in
+// shared memory.  The producer claims tasks and stages their records; the
+// lanes' packed masks, transposed as bit matrices, give for every block one
+// 32-bit word per 32 records (which of them touch the block).  A consumer
+// warp takes the next block of the window, turns the block's words into the
+// list of the records that touch it (lane l lists those of 32 slots, in
+// order), its 32 lanes evaluate 32 of those records at a time, one record
+// and 16 pixels per lane, and the lanes' partial images are added by a
+// butterfly that halves the pixels a lane holds at each of four steps.  A
+// warp that finds no block left goes on to the other window without waiting
+// for its neighbours; the warp that finishes the last block writes the
+// window's 256 pixels.  Windows of a tile with several segments go to
+// partial images, which the last segment to finish adds in segment order
+// (Kahan).  Nothing depends on which warp or CTA did what, so the result is
+// deterministic.
+//
+// What bounds it: issue (about 60% of the slots) and the L1, through which
+// every entry's 32 scattered bytes come (one 256-bit load per record: two
+// loads of 16 and 8 bytes cost 8% of the launch) and which serves the record
+// reads of the evaluation.  Against CTAs of four warps that staged 256
+// records between barriers and gave each block a share of the threads
+// (us per launch): d 384, M 500000, B 16: 680 -> 467; d 128, M 20000, B 256:
+// 388 -> 367; d 256, M 100000, B 64: 498 -> 418; d 128, M 50000, B 64, scales
+// 0.3-12 px, whose longest lists hold 14000 entries: 745-850 -> 391; d 64,
+// M 2000, B 32: 37 -> 24.  Staging by the consumers between barriers: 553 at
+// the first of these; one producer warp with small copies in flight: 494-518;
+// windows of 512 records: 610.
+//
 // kCount = true: the same walk, counting kept pairs into kept[0] and
 // evaluated pairs into kept[1] instead of writing the projection
 // (inspection only, never on the timed path).
-template <bool kCount>
-__global__ void __launch_bounds__(kThreads, kFwdMinBlocks) raster_fwd_kernel(
-    const Rec *__restrict__ rec, const uint2 *__restrict__ list,
-    const int64_t *__restrict__ tile_start, int64_t cap,
-    int64_t M, int d, float l2tau, float *__restrict__ proj,
-    unsigned long long *__restrict__ kept) {
-  constexpr int kWarps = kThreads / 32;
-  constexpr int kPieces = 16 + kThreads - 1;
-  __shared__ float4 sa[kWin];                         // px, py, u11, u12
-  __shared__ float2 sb[kWin];                         // u22, log2 A
-  __shared__ unsigned char flat[16 * kWin];           // staged slot of each (block, record) item,
-                                                      // blocks in order, records in list order
-  __shared__ unsigned short wcnt[kSub][kWarps][16];  // per sub-window, warp, block: how many
-  __shared__ unsigned wbal[kSub][kWarps][16];        // per sub-window, warp, block: which lanes
-  __shared__ int woff[kWarps][kSub][16];             // where a warp's records go in flat
-  __shared__ int pstart[kWarps][17];                 // block k's items: [pstart[k], pstart[k+1])
-  __shared__ float4 part[kPieces][4];                // piece (block k, thread u) at k + u
+template <int kCons, int kProd, int kMinB, bool kCount>
+__global__ void __launch_bounds__(32 * (kCons + kProd), kMinB) raster_fwd_kernel(
+    const Rec *__restrict__ rec, const uint2 *__restrict__ list, int64_t M, int d, float l2tau,
+    RasterTasks tk, float *__restrict__ proj, unsigned long long *__restrict__ kept) {
+  extern __shared__ __align__(16) unsigned char fwd_smem[];
+  FwdShared<kCons> &S = *reinterpret_cast<FwdShared<kCons> *>(fwd_smem);
   const int nt = d / kTile, T = nt * nt;
-  const int t = blockIdx.x, b = blockIdx.y;
-  const int tx = t % nt, ty = t / nt;
-  const int x0 = tx * kTile, y0 = ty * kTile;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const float nl2tau = -l2tau;  // kept: -e < -log2(tau)
-  int64_t s = tile_start[(int64_t)b * T + t];
-  int64_t e = tile_start[(int64_t)b * T + t + 1];
-  e = min(e, cap);
-  s = min(s, e);
-  // lists that overflowed their capacity are incomplete: every list counts
-  // as empty (the status word reports it)
-  if (tile_start[(int64_t)gridDim.y * T] > cap) e = s;
-  const Rec *rb = rec + (int64_t)b * M;
-  const unsigned lt = (1u << lane) - 1u;
-  // pixels owned across windows: two columns of one row of block ob
-  const int ob = tid >> 3, ow = tid & 7;
-  float2 own0 = make_float2(0.f, 0.f), own1 = make_float2(0.f, 0.f);  // Kahan (sum, comp)
-  unsigned nkept = 0, neval = 0;
-  for (int64_t base = s; base < e; base += kWin) {
-    const int n = (int)min((int64_t)kWin, e - base);
-    __syncthreads();  // previous window fully consumed
-    // record slot u * kThreads + tid of sub-window u
-    unsigned m[kSub];
-#pragma unroll
-    for (int u = 0; u < kSub; ++u) {
-      const int slot = u * kThreads + tid;
-      m[u] = 0;
-      // an entry whose Gaussian index is out of range (a list position left
-      // unwritten when the lists overflowed their capacity) counts as empty
-      const uint2 ent = slot < n ? list[base + slot] : make_uint2(0u, 0u);
-      const uint32_t jj = ent.x;
-      if (slot < n && jj < (uint64_t)M) {
-        const Rec *rp = rb + jj;
-        const float4 ra = rp->a;
-        const float2 rbv = *reinterpret_cast<const float2 *>(&rp->b);
-        m[u] = ent.y & 0xffffu;
-        sa[slot] = ra;
-        sb[slot] = rbv;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&S.full[i], 32 * kProd);
+      mbar_init(&S.empty[i], kCons);
+    }
+  }
+  __syncthreads();
+  if (warp >= kCons) {
+    // ---- producers ----
+    const int pw = warp - kCons;
+    const bool leader = pw == 0 && lane == 0;
+    const int ntasks = (int)tk.ctr[kCtrTasks];
+    // the leader claims a task two windows ahead and reads its descriptor one
+    // window ahead; t1.w marks the end
+    int nq = 0;
+    if (leader) {
+      const int q = blockIdx.x;
+      if (q < ntasks) {
+        S.desc[0][0] = tk.task[2 * (int64_t)q];
+        S.desc[0][1] = tk.task[2 * (int64_t)q + 1];
+      } else {
+        S.desc[0][1].w = 1u;
       }
+      nq = (int)(atomicAdd(tk.ctr + kCtrFwd, 1u) + gridDim.x);
     }
-    // which of this warp's records touch block k, both sub-windows at once:
-    // lane k < 16 gets block k of sub-window 0, lane 16 + k block k of
-    // sub-window 1 (the lanes' packed masks, transposed as a bit matrix)
-    static_assert(kSub == 2, "two 16-bit masks per lane");
-    {
-      const unsigned bal = warp_transpose32(m[0] | (m[1] << 16), lane);
-      wcnt[lane >> 4][warp][lane & 15] = (unsigned short)__popc(bal);
-      wbal[lane >> 4][warp][lane & 15] = bal;
-    }
-    __syncthreads();
-    // every warp: block lengths, their prefix (the items of all blocks laid
-    // out block after block) and where its own records go: after the
-    // records of earlier sub-windows and lower warps touching the block
-    {
-      int len = 0, wo[kSub];
+    for (int it = 0;; ++it) {
+      FwdWindow &W = S.win[it & 1];
+      named_sync(1, 32 * kProd);
+      const uint4 t0 = S.desc[it & 1][0], t1 = S.desc[it & 1][1];
+      // the other parity passes at once on a fresh barrier
+      if (!mbar_wait(&S.empty[it & 1], ((it >> 1) & 1) ^ 1)) {
+        if (lane == 0) atomicOr(tk.status, kStatusTimeout);
+        return;
+      }
+      if (t1.w) {
+        if (leader) W.n = -1;
+        mbar_arrive(&S.full[it & 1]);
+        return;
+      }
+      uint4 n0 = make_uint4(0u, 0u, 0u, 0u), n1 = make_uint4(0u, 0u, 0u, 1u);
+      int nq2 = 0;
+      if (leader) {
+        if (nq < ntasks) {
+          n0 = tk.task[2 * (int64_t)nq];
+          n1 = tk.task[2 * (int64_t)nq + 1];
+        }
+        nq2 = (int)(atomicAdd(tk.ctr + kCtrFwd, 1u) + gridDim.x);
+      }
+      const uint2 *L = list + (int64_t)(((uint64_t)t0.y << 32) | t0.x);
+      const int n = (int)t0.z, bt = (int)t0.w;
+      const Rec *rb = rec + (int64_t)(bt / T) * M;
+      if (leader) {
+        W.n = n;
+        W.bt = bt;
+        W.seg = t1.x;
+        W.nseg = t1.y;
+        W.part = t1.z;
+        W.next_block = 0;
+        W.done = 0;
+      }
+      // this warp's pairs of 32-entry chunks, all their entries in flight together
+      constexpr int kPairs = kFwdWin / 64 / kProd;
+      uint2 ent[2 * kPairs];
 #pragma unroll
-      for (int u = 0; u < kSub; ++u) {
-        wo[u] = 0;
+      for (int u = 0; u < 2 * kPairs; ++u) {
+        const int slot = 64 * ((u >> 1) * kProd + pw) + 32 * (u & 1) + lane;
+        ent[u] = slot < n ? L[slot] : make_uint2(0xffffffffu, 0u);
+      }
+      // records in batches of kB chunks in flight
+      constexpr int kB = kPairs >= 2 ? 4 : 2;
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) {
-          if (w == warp) wo[u] = len;
-          if (lane < 16) len += wcnt[u][w][lane];
+      for (int u0 = 0; u0 < 2 * kPairs; u0 += kB) {
+        if (64 * ((u0 >> 1) * kProd + pw) >= n) break;
+        Rec r[kB];
+#pragma unroll
+        for (int u = 0; u < kB; ++u) {
+          // an entry whose Gaussian index is out of range counts as empty
+          if (ent[u0 + u].x < (uint64_t)M)
+            r[u] = load_rec(rb + ent[u0 + u].x);
+          else
+            ent[u0 + u].y = 0u;
+        }
+        // lane k < 16: block k of the first chunk of a pair, lane 16 + k: of the second
+#pragma unroll
+        for (int u = 0; u < kB; u += 2)
+          W.bal[lane & 15][2 * (((u0 + u) >> 1) * kProd + pw) + (lane >> 4)] =
+              warp_transpose32((ent[u0 + u].y & 0xffffu) | (ent[u0 + u + 1].y << 16), lane);
+#pragma unroll
+        for (int u = 0; u < kB; ++u) {
+          const int slot = 64 * (((u0 + u) >> 1) * kProd + pw) + 32 * (u & 1) + lane;
+          W.sa[slot] = r[u].a;
+          W.sb[slot] = make_float2(r[u].b.x, r[u].b.y);
         }
       }
-      int incl = len;
+      if (leader) {
+        S.desc[(it + 1) & 1][0] = n0;
+        S.desc[(it + 1) & 1][1] = n1;
+        nq = nq2;
+      }
+      __syncwarp();
+      mbar_arrive(&S.full[it & 1]);
+    }
+  }
+  // ---- consumers ----
+  const float nl2tau = -l2tau;  // kept: -e < -log2(tau)
+  unsigned short *slots = S.slots[warp];
+  unsigned nkept = 0, neval = 0;
+  for (int it = 0;; ++it) {
+    FwdWindow &W = S.win[it & 1];
+    if (!mbar_wait(&S.full[it & 1], (it >> 1) & 1)) {
+      if (lane == 0) atomicOr(tk.status, kStatusTimeout);
+      return;
+    }
+    const int n = W.n;
+    if (n < 0) break;
+    const int bt = W.bt;
+    const int b = bt / T, t = bt - b * T;
+    const int tx = t % nt, ty = t / nt;
+    const int x0 = tx * kTile, y0 = ty * kTile;
+    const int nw = ((n + 63) >> 6) << 1;  // words staged
+    for (;;) {
+      int k = 0;
+      if (lane == 0) k = atomicAdd(&W.next_block, 1);
+      k = __shfl_sync(0xffffffffu, k, 0);
+      if (k >= 16) break;
+      unsigned bits = lane < nw ? W.bal[k][lane] : 0u;
+      const int c = __popc(bits);
+      int incl = c;
 #pragma unroll
-      for (int o = 1; o < 16; o <<= 1) {
+      for (int o = 1; o < 32; o <<= 1) {
         const int v = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += v;
       }
-      if (lane < 16) {
-        pstart[warp][lane] = incl - len;
-#pragma unroll
-        for (int u = 0; u < kSub; ++u) woff[warp][u][lane] = incl - len + wo[u];
+      const int nk = __shfl_sync(0xffffffffu, incl, 31);
+      {
+        unsigned short *w = slots + (incl - c);
+        for (; bits; bits &= bits - 1) *w++ = (unsigned short)(32 * lane + __ffs(bits) - 1);
       }
-      if (lane == 15) pstart[warp][16] = incl;
       __syncwarp();
-    }
-#pragma unroll
-    for (int u = 0; u < kSub; ++u) {
-      for (unsigned mm = m[u]; mm; mm &= mm - 1) {
-        const int k = __ffs(mm) - 1;
-        flat[woff[warp][u][k] + __popc(wbal[u][warp][k] & lt)] = (unsigned char)(u * kThreads + tid);
-      }
-    }
-    __syncthreads();
-    // thread tid takes items [lo, hi) of the concatenation: a run of
-    // records of one block or a few consecutive blocks, 16 pixels each;
-    // each block it leaves (a piece) goes to part[k + tid]
-    const int *ps = pstart[0];
-    const int N = ps[16];
-    const int lo = (tid * N) >> 7, hi = ((tid + 1) * N) >> 7;
-    if (lo < hi) {
-      int k = 0;
-      while (ps[k + 1] <= lo) ++k;
+      // acc[4 h + x]: column x, rows 2 h and 2 h + 1
       float2 acc[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) acc[q] = make_float2(0.f, 0.f);
-      float X0 = (float)(x0 + 4 * (k & 3)), Y0 = (float)(y0 + 4 * (k >> 2));
-      int kend = ps[k + 1];  // end of block k's items
-      for (int i = lo; i < hi; ++i) {
-        if (i >= kend) {  // the run enters the next non-empty block
-          if (!kCount) {
+      for (int j = 0; j < 8; ++j) acc[j] = make_float2(0.f, 0.f);
+      const float X0 = (float)(x0 + 4 * (k & 3)), Y0 = (float)(y0 + 4 * (k >> 2));
+      const float2 ys0 = make_float2(Y0, Y0 + 1.f), ys1 = make_float2(Y0 + 2.f, Y0 + 3.f);
+      for (int i = lane; i < nk; i += 32) {
+        const int slot = slots[i];
+        const float4 A = W.sa[slot];
+        const float2 Bv = W.sb[slot];
+        // -e = z1^2 + (z2^2 - l2A), z1 = u11 dx + u12 dy, z2 = u22 dy, two
+        // rows of a column in one packed operation
+        float2 ux[4];
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
-              part[k + tid][r] = make_float4(acc[2 * r].x, acc[2 * r].y, acc[2 * r + 1].x,
-                                             acc[2 * r + 1].y);
-          }
+        for (int x = 0; x < 4; ++x) ux[x] = f2(__fmul_rn(A.z, __fsub_rn(X0 + (float)x, A.x)));
 #pragma unroll
-          for (int q = 0; q < 8; ++q) acc[q] = make_float2(0.f, 0.f);
-          do ++k;
-          while (ps[k + 1] <= i);
-          kend = ps[k + 1];
-          X0 = (float)(x0 + 4 * (k & 3));
-          Y0 = (float)(y0 + 4 * (k >> 2));
-        }
-        const int slot = flat[i];
-        const float4 A = sa[slot];
-        const float2 Bv = sb[slot];
-        const float2 npx = f2(-A.x);
-        const float2 dx01 = add2(make_float2(X0, X0 + 1.f), npx);
-        const float2 dx23 = add2(make_float2(X0 + 2.f, X0 + 3.f), npx);
-        const float2 u11 = f2(A.z);
-        const float2 ux01 = mul2(u11, dx01), ux23 = mul2(u11, dx23);
+        for (int h = 0; h < 2; ++h) {
+          const float2 dy = add2(h ? ys1 : ys0, f2(-A.y));
+          const float2 uy = mul2(f2(A.w), dy);
+          const float2 z2 = mul2(f2(Bv.x), dy);
+          const float2 nc = fma2(z2, z2, f2(-Bv.y));
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          // -e = z1^2 + (z2^2 - l2A), z1 = u11 dx + u12 dy, z2 = u22 dy
-          const float dy = Y0 + (float)r - A.y;
-          const float2 uy = f2(A.w * dy);
-          const float z2 = Bv.x * dy;
-          const float2 nc = f2(fmaf(z2, z2, -Bv.y));
-          const float2 z01 = add2(ux01, uy), z23 = add2(ux23, uy);
-          const float2 f01 = fma2(z01, z01, nc), f23 = fma2(z23, z23, nc);
-          if (kCount) {
-            nkept += (f01.x < nl2tau) + (f01.y < nl2tau) + (f23.x < nl2tau) + (f23.y < nl2tau);
-          } else {
-            // value on kept pairs (value > tau), zero elsewhere
-            acc[2 * r] = fma2(make_float2(ex2_approx(-f01.x), ex2_approx(-f01.y)),
-                              make_float2(set_lt(f01.x, nl2tau), set_lt(f01.y, nl2tau)), acc[2 * r]);
-            acc[2 * r + 1] =
-                fma2(make_float2(ex2_approx(-f23.x), ex2_approx(-f23.y)),
-                     make_float2(set_lt(f23.x, nl2tau), set_lt(f23.y, nl2tau)), acc[2 * r + 1]);
+          for (int x = 0; x < 4; ++x) {
+            const float2 z = add2(ux[x], uy);
+            const float2 f = fma2(z, z, nc);
+            if (kCount)
+              nkept += (f.x < nl2tau) + (f.y < nl2tau);
+            else  // value on kept pairs (value > tau), zero elsewhere
+              acc[4 * h + x] = fma2(make_float2(ex2_approx(-f.x), ex2_approx(-f.y)),
+                                    make_float2(set_lt(f.x, nl2tau), set_lt(f.y, nl2tau)),
+                                    acc[4 * h + x]);
           }
         }
         if (kCount) neval += 16;
       }
-      if (!kCount) {
+      __syncwarp();  // the slots are read before the next block's replace them
+      if (kCount) continue;
+      // 16 pixels x 32 lanes -> the pixel of lane pair (2 p, 2 p + 1)
+      float v8[8], v4[4], v2[2];
+      const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
-          part[k + tid][r] =
-              make_float4(acc[2 * r].x, acc[2 * r].y, acc[2 * r + 1].x, acc[2 * r + 1].y);
+      for (int x = 0; x < 4; ++x) {
+        // lanes with bit 4 clear keep rows 0 and 1, the others rows 2 and 3
+        const float2 keep = b4 ? acc[4 + x] : acc[x], give = b4 ? acc[x] : acc[4 + x];
+        v8[x] = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 16);
+        v8[4 + x] = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 16);
       }
-    }
-    if (kCount) continue;
-    __syncthreads();
-    // each owned pixel sums the pieces of its block in thread order (runs
-    // in list order), then joins its running sum (Kahan)
-    {
-      const int pk = ps[ob], pe = ps[ob + 1];
-      if (pe > pk) {
-        // threads holding items pk and pe - 1
-        const int ulo = (kThreads * (pk + 1) + N - 1) / N - 1;
-        const int uhi = (kThreads * pe + N - 1) / N - 1;
-        float2 w = make_float2(0.f, 0.f);
-        for (int u = ulo; u <= uhi; ++u) {
-          if (((u * N) >> 7) == (((u + 1) * N) >> 7)) continue;  // empty run
-          const float2 v = reinterpret_cast<const float2 *>(&part[ob + u][ow >> 1])[ow & 1];
-          w.x += v.x;
-          w.y += v.y;
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+        v4[x] = (b3 ? v8[4 + x] : v8[x]) + __shfl_xor_sync(0xffffffffu, b3 ? v8[x] : v8[4 + x], 8);
+#pragma unroll
+      for (int x = 0; x < 2; ++x)
+        v2[x] = (b2 ? v4[2 + x] : v4[x]) + __shfl_xor_sync(0xffffffffu, b2 ? v4[x] : v4[2 + x], 4);
+      float v1 = (b1 ? v2[1] : v2[0]) + __shfl_xor_sync(0xffffffffu, b1 ? v2[0] : v2[1], 2);
+      v1 += __shfl_xor_sync(0xffffffffu, v1, 1);
+      if (!(lane & 1)) W.out[k][lane >> 1] = v1;
+      // the warp that finishes the window's last block writes its pixels
+      __threadfence_block();
+      __syncwarp();
+      int dn = 0;
+      if (lane == 0) dn = atomicAdd(&W.done, 1);
+      dn = __shfl_sync(0xffffffffu, dn, 0);
+      if (dn != 15) continue;
+      __threadfence_block();
+      // lane: half a pixel row of the tile, two blocks' rows of four
+      const int row = lane >> 1, k0 = 4 * (row >> 2) + 2 * (lane & 1), p0 = 4 * (row & 3);
+      float4 v[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) v[h] = *reinterpret_cast<const float4 *>(&W.out[k0 + h][p0]);
+      const unsigned nseg = W.nseg;
+      float4 *o = reinterpret_cast<float4 *>(proj + ((int64_t)b * d + y0 + row) * d + x0 + 8 * (lane & 1));
+      if (nseg > 1) {
+        float4 *part = reinterpret_cast<float4 *>(tk.part + (int64_t)W.part * 256) + 2 * lane;
+        __stcg(part + (int64_t)W.seg * 64, v[0]);
+        __stcg(part + (int64_t)W.seg * 64 + 1, v[1]);
+        __threadfence();
+        __syncwarp();
+        unsigned prev = 0;
+        if (lane == 0) prev = atomicAdd(tk.done + bt, 1u);
+        if (__shfl_sync(0xffffffffu, prev, 0) != nseg - 1) continue;
+        __threadfence();
+        float2 s[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) s[j] = make_float2(0.f, 0.f);
+        for (unsigned g = 0; g < nseg; ++g) {
+          const float4 a = __ldcg(part + (int64_t)g * 64), c4 = __ldcg(part + (int64_t)g * 64 + 1);
+          const float x[8] = {a.x, a.y, a.z, a.w, c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+          for (int j = 0; j < 8; ++j) s[j] = kahan_add(s[j], x[j]);
         }
-        own0 = kahan_add(own0, w.x);
-        own1 = kahan_add(own1, w.y);
+        if (lane == 0) tk.done[bt] = 0u;  // as the next call expects it
+        v[0] = make_float4(s[0].x - s[0].y, s[1].x - s[1].y, s[2].x - s[2].y, s[3].x - s[3].y);
+        v[1] = make_float4(s[4].x - s[4].y, s[5].x - s[5].y, s[6].x - s[6].y, s[7].x - s[7].y);
       }
+      o[0] = v[0];
+      o[1] = v[1];
     }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&S.empty[it & 1]);
   }
   if (kCount) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -279,257 +499,102 @@ __global__ void __launch_bounds__(kThreads, kFwdMinBlocks) raster_fwd_kernel(
       atomicAdd(kept, (unsigned long long)nkept);
       atomicAdd(kept + 1, (unsigned long long)neval);
     }
-    return;
   }
-  const int px = x0 + 4 * (ob & 3) + 2 * (ow & 1), py = y0 + 4 * (ob >> 2) + (ow >> 1);
-  *reinterpret_cast<float2 *>(proj + ((int64_t)b * d + py) * d + px) =
-      make_float2(own0.x - own0.y, own1.x - own1.y);
 }
 
-// a3, block-aligned form.  The window's (block, record) items are laid out
-// block after block as above, but the 128 threads are shared among the
-// blocks in proportion to their item counts (every non-empty block gets at
-// least one thread: thread range [T_k, T_k+1) with T_k = (non-empty blocks
-// before k) + floor((128 - non-empty) * start_k / N)), and a block's threads
-// take its items interleaved.  A thread never leaves its block, so each thread ends
-// the window with one partial image of its block (16 pixels), and each pixel
-// sums the partials of its block's thread range in thread order (runs in
-// list order), then joins its running sum with Kahan compensation.  The
-// longest run is within 128 / (128 - 16) of the mean.  kSub sub-windows of
-// 128 records make a window; flat slots are bytes up to 256 records.
-template <int kSubW>
-struct FlatSlot {
-  using T = typename std::conditional<(kSubW * 128 <= 256), unsigned char, unsigned short>::type;
+// The forward's kernel configurations (the autotuner's search space).
+static const FwdCfg kFwdCfgs[] = {
+    {6, 2, 3, "6 consumer and 2 producer warps, 3 CTAs/SM"},
+    {8, 2, 3, "8 consumer and 2 producer warps, 3 CTAs/SM"},
+    {8, 4, 2, "8 consumer and 4 producer warps, 2 CTAs/SM"},
+    {12, 4, 2, "12 consumer and 4 producer warps, 2 CTAs/SM"},
+    {10, 2, 2, "10 consumer and 2 producer warps, 2 CTAs/SM"},
+    {6, 2, 2, "6 consumer and 2 producer warps, 2 CTAs/SM"},
+    {8, 2, 2, "8 consumer and 2 producer warps, 2 CTAs/SM"},
+    {12, 4, 1, "12 consumer and 4 producer warps, 1 CTA/SM"},
 };
+int fwd_config_count() { return (int)(sizeof(kFwdCfgs) / sizeof(kFwdCfgs[0])); }
+const FwdCfg &fwd_config(int i) { return kFwdCfgs[i]; }
 
-template <int kSubW, int kMinB, bool kCount>
-__global__ void __launch_bounds__(kThreads, kMinB) raster_fwd_aligned_kernel(
-    const Rec *__restrict__ rec, const uint2 *__restrict__ list,
-    const int64_t *__restrict__ tile_start, int64_t cap,
-    int64_t M, int d, float l2tau, const uint32_t *__restrict__ order, int ntiles,
-    unsigned *__restrict__ next_tile, float *__restrict__ proj,
-    unsigned long long *__restrict__ kept) {
-  constexpr int kWarps = kThreads / 32;
-  constexpr int kWinW = kThreads * kSubW;
-  using Slot = typename FlatSlot<kSubW>::T;
-  __shared__ float4 sa[kWinW];                        // px, py, u11, u12
-  __shared__ float2 sb[kWinW];                        // u22, log2 A
-  __shared__ Slot flat[16 * kWinW];                   // staged slot of each (block, record) item
-  __shared__ unsigned short wcnt[kSubW][kWarps][16];  // per sub-window, warp, block: how many
-  __shared__ unsigned wbal[kSubW][kWarps][16];        // per sub-window, warp, block: which lanes
-  __shared__ int woff[kWarps][kSubW][16];             // where a warp's records go in flat
-  __shared__ int pstart[kWarps][17];                  // block k's items: [pstart[k], pstart[k+1])
-  __shared__ int tfirst[kWarps][17];                  // block k's threads: [tfirst[k], tfirst[k+1])
-  __shared__ float4 part[kThreads][4];                // each thread's partial image of its block
-  __shared__ int tile_sh;
-  const int nt = d / kTile, T = nt * nt;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const float nl2tau = -l2tau;  // kept: -e < -log2(tau)
-  const unsigned lt = (1u << lane) - 1u;
-  // pixels owned across windows: two columns of one row of block ob
-  const int ob = tid >> 3, ow = tid & 7;
-  unsigned nkept = 0, neval = 0;
-  // tiles come from the grid (order == nullptr) or, in the persistent form,
-  // from a shared counter over a longest-first order
-  for (int it = 0;; ++it) {
-    int bt;
-    if (order == nullptr) {
-      if (it > 0) break;
-      bt = blockIdx.y * T + blockIdx.x;
-    } else {
-      __syncthreads();  // every thread has read the previous tile_sh
-      if (tid == 0) tile_sh = (int)atomicAdd(next_tile, 1u);
-      __syncthreads();
-      const int q = tile_sh;
-      if (q >= ntiles) break;
-      bt = (int)order[q];
-    }
-    const int b = bt / T, t = bt - b * T;
-    const int tx = t % nt, ty = t / nt;
-    const int x0 = tx * kTile, y0 = ty * kTile;
-    int64_t s = tile_start[bt];
-    int64_t e = tile_start[bt + 1];
-    e = min(e, cap);
-    s = min(s, e);
-    // lists that overflowed their capacity are incomplete: every list
-    // counts as empty (the status word reports it)
-    if (tile_start[order == nullptr ? (int64_t)gridDim.y * T : (int64_t)ntiles] > cap) e = s;
-    const Rec *rb = rec + (int64_t)b * M;
-    float2 own0 = make_float2(0.f, 0.f), own1 = make_float2(0.f, 0.f);  // Kahan (sum, comp)
-    for (int64_t base = s; base < e; base += kWinW) {
-      const int n = (int)min((int64_t)kWinW, e - base);
-      __syncthreads();  // previous window fully consumed
-      unsigned m[kSubW];
-#pragma unroll
-      for (int u = 0; u < kSubW; ++u) {
-        const int slot = u * kThreads + tid;
-        m[u] = 0;
-        // an entry whose Gaussian index is out of range (a list position
-        // left unwritten when the lists overflowed their capacity) counts as
-        // empty
-        const uint2 ent = slot < n ? list[base + slot] : make_uint2(0u, 0u);
-        const uint32_t jj = ent.x;
-        if (slot < n && jj < (uint64_t)M) {
-          const Rec *rp = rb + jj;
-          const float4 ra = rp->a;
-          const float2 rbv = *reinterpret_cast<const float2 *>(&rp->b);
-          m[u] = ent.y & 0xffffu;
-          sa[slot] = ra;
-          sb[slot] = rbv;
-        }
-      }
-      // which of this warp's records touch block k, both sub-windows at once:
-      // lane k < 16 gets block k of sub-window 0, lane 16 + k block k of
-      // sub-window 1 (the lanes' packed masks, transposed as a bit matrix)
-      static_assert(kSubW == 2, "two 16-bit masks per lane");
-      {
-        const unsigned bal = warp_transpose32(m[0] | (m[1] << 16), lane);
-        wcnt[lane >> 4][warp][lane & 15] = (unsigned short)__popc(bal);
-        wbal[lane >> 4][warp][lane & 15] = bal;
-      }
-      __syncthreads();
-      // every warp: block lengths, their prefix, where its own records go,
-      // and the thread ranges of the blocks
-      {
-        int len = 0, wo[kSubW];
-#pragma unroll
-        for (int u = 0; u < kSubW; ++u) {
-          wo[u] = 0;
-#pragma unroll
-          for (int w = 0; w < kWarps; ++w) {
-            if (w == warp) wo[u] = len;
-            if (lane < 16) len += wcnt[u][w][lane];
-          }
-        }
-        int incl = len, ne = (lane < 16 && len > 0) ? 1 : 0;
-#pragma unroll
-        for (int o = 1; o < 16; o <<= 1) {
-          const int v = __shfl_up_sync(0xffffffffu, incl, o);
-          const int c = __shfl_up_sync(0xffffffffu, ne, o);
-          if (lane >= o) {
-            incl += v;
-            ne += c;
-          }
-        }
-        const int N = __shfl_sync(0xffffffffu, incl, 15);
-        const int nne = __shfl_sync(0xffffffffu, ne, 15);
-        if (lane < 16) {
-          const int st = incl - len;
-          pstart[warp][lane] = st;
-#pragma unroll
-          for (int u = 0; u < kSubW; ++u) woff[warp][u][lane] = st + wo[u];
-          // non-empty blocks before this one, plus its share of the rest
-          const int neb = ne - ((len > 0) ? 1 : 0);
-          // floor(a / N) for a = (128 - nne) st < 2^19, N <= 16 kWinW: a / N is a
-          // multiple of 1 / N, so (a + 1/2) / N sits at least 1 / (2 N) from
-          // an integer, far more than the few-ulp error of the fast division
-          const float a = (float)((kThreads - nne) * st) + 0.5f;
-          tfirst[warp][lane] = neb + (N > 0 ? (int)__fdividef(a, (float)N) : 0);
-        }
-        if (lane == 15) {
-          pstart[warp][16] = incl;
-          tfirst[warp][16] = kThreads;
-        }
-        __syncwarp();
-      }
-#pragma unroll
-      for (int u = 0; u < kSubW; ++u) {
-        for (unsigned mm = m[u]; mm; mm &= mm - 1) {
-          const int k = __ffs(mm) - 1;
-          flat[woff[warp][u][k] + __popc(wbal[u][warp][k] & lt)] = (Slot)(u * kThreads + tid);
-        }
-      }
-      __syncthreads();
-      // this thread's block and its share of the block's items
-      const int *ps = pstart[warp];
-      const int *tf = tfirst[warp];
-      int k = 0;
-#pragma unroll
-      for (int q = 8; q >= 1; q >>= 1)
-        if (k + q <= 15 && tf[k + q] <= tid) k += q;
-      // tf is non-decreasing and tf[16] = 128 > tid: k is the last block
-      // whose range starts at or before tid; an empty block's range is empty
-      const int t0 = tf[k], tk = tf[k + 1] - t0;
-      float2 acc[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) acc[q] = make_float2(0.f, 0.f);
-      if (tk > 0 && tid < tf[k + 1]) {
-        const int j = tid - t0;
-        // the block's threads take its items interleaved (thread j: items
-        // j, j + tk, ...), each in list order; at every step they read
-        // neighbouring items, whose slots ascend, which spreads the record
-        // gathers over the banks better than contiguous runs did
-        const int L = ps[k + 1] - ps[k];
-        const float X0 = (float)(x0 + 4 * (k & 3)), Y0 = (float)(y0 + 4 * (k >> 2));
-        const float2 xs01 = make_float2(X0, X0 + 1.f), xs23 = make_float2(X0 + 2.f, X0 + 3.f);
-        for (int i = ps[k] + j; i < ps[k] + L; i += tk) {
-          const int slot = flat[i];
-          const float4 A = sa[slot];
-          const float2 Bv = sb[slot];
-          const float2 npx = f2(-A.x);
-          const float2 dx01 = add2(xs01, npx);
-          const float2 dx23 = add2(xs23, npx);
-          const float2 u11 = f2(A.z);
-          const float2 ux01 = mul2(u11, dx01), ux23 = mul2(u11, dx23);
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            // -e = z1^2 + (z2^2 - l2A), z1 = u11 dx + u12 dy, z2 = u22 dy
-            const float dy = Y0 + (float)r - A.y;
-            const float2 uy = f2(A.w * dy);
-            const float z2 = Bv.x * dy;
-            const float2 nc = f2(fmaf(z2, z2, -Bv.y));
-            const float2 z01 = add2(ux01, uy), z23 = add2(ux23, uy);
-            const float2 f01 = fma2(z01, z01, nc), f23 = fma2(z23, z23, nc);
-            if (kCount) {
-              nkept += (f01.x < nl2tau) + (f01.y < nl2tau) + (f23.x < nl2tau) + (f23.y < nl2tau);
-            } else {
-              // value on kept pairs (value > tau), zero elsewhere
-              acc[2 * r] = fma2(make_float2(ex2_approx(-f01.x), ex2_approx(-f01.y)),
-                                make_float2(set_lt(f01.x, nl2tau), set_lt(f01.y, nl2tau)), acc[2 * r]);
-              acc[2 * r + 1] =
-                  fma2(make_float2(ex2_approx(-f23.x), ex2_approx(-f23.y)),
-                       make_float2(set_lt(f23.x, nl2tau), set_lt(f23.y, nl2tau)), acc[2 * r + 1]);
-            }
-          }
-          if (kCount) neval += 16;
-        }
-      }
-      if (!kCount) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-          part[tid][r] = make_float4(acc[2 * r].x, acc[2 * r].y, acc[2 * r + 1].x, acc[2 * r + 1].y);
-        __syncthreads();
-        // each owned pixel sums its block's partials in thread order (runs
-        // in list order), then joins its running sum (Kahan)
-        const int u0 = tf[ob], u1 = tf[ob + 1];
-        float2 w = make_float2(0.f, 0.f);
-        for (int u = u0; u < u1; ++u) {
-          const float2 v = reinterpret_cast<const float2 *>(&part[u][ow >> 1])[ow & 1];
-          w.x += v.x;
-          w.y += v.y;
-        }
-        if (u1 > u0) {
-          own0 = kahan_add(own0, w.x);
-          own1 = kahan_add(own1, w.y);
-        }
-      }
-    }
-    if (!kCount) {
-      const int px = x0 + 4 * (ob & 3) + 2 * (ow & 1), py = y0 + 4 * (ob >> 2) + (ow >> 1);
-      *reinterpret_cast<float2 *>(proj + ((int64_t)b * d + py) * d + px) =
-          make_float2(own0.x - own0.y, own1.x - own1.y);
-    }
+static int sm_count() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms;
+}
+
+// Partial images that any lists of up to cap entries can need: a tile of
+// more than S entries has fewer than 2 len / S segments, and S is at least
+// total / (2 slots) (at most 4 slots of them) or 1024.
+constexpr int kFwdSlots = 3 * 256;  // CTAs that fit up to 256 SMs
+size_t raster_part_count(int64_t cap) {
+  return (size_t)(4 * kFwdSlots + 2 * (cap / kFwdWin + 1));
+}
+
+template <int kCons, int kProd, int kMinB, bool kCount>
+static cudaError_t launch_fwd_one(int grid, const Rec *rec, const uint2 *list, int64_t M, int d,
+                                  float l2tau, const RasterTasks &tk, float *proj,
+                                  unsigned long long *kept, cudaStream_t st) {
+  raster_fwd_kernel<kCons, kProd, kMinB, kCount>
+      <<<grid, 32 * (kCons + kProd), sizeof(FwdShared<kCons>), st>>>(rec, list, M, d, l2tau, tk, proj, kept);
+  return cudaGetLastError();
+}
+
+template <int kCons, int kProd, int kMinB>
+static cudaError_t configure_fwd_one() {
+  const int smem = (int)sizeof(FwdShared<kCons>);
+  const cudaError_t e = cudaFuncSetAttribute(raster_fwd_kernel<kCons, kProd, kMinB, false>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(raster_fwd_kernel<kCons, kProd, kMinB, true>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+}
+
+cudaError_t raster_configure() {
+  cudaError_t e;
+  if ((e = configure_fwd_one<6, 2, 3>()) != cudaSuccess || (e = configure_fwd_one<8, 2, 3>()) != cudaSuccess ||
+      (e = configure_fwd_one<8, 4, 2>()) != cudaSuccess || (e = configure_fwd_one<12, 4, 2>()) != cudaSuccess ||
+      (e = configure_fwd_one<10, 2, 2>()) != cudaSuccess)
+    return e;
+  return cudaSuccess;
+}
+
+template <bool kCount>
+static cudaError_t launch_fwd_any(int cfg, const Rec *rec, const uint2 *list,
+                                  const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
+                                  float l2tau, float *proj, unsigned long long *kept,
+                                  const RasterTasks &tk, bool fresh, cudaStream_t st) {
+  if (cfg < 0 || cfg >= fwd_config_count()) return cudaErrorInvalidValue;
+  const FwdCfg &c = kFwdCfgs[cfg];
+  const int nt = d / kTile, ntiles = nt * nt * B, sms = sm_count();
+  if (!fresh) {
+    const cudaError_t e = cudaMemsetAsync(tk.ctr, 0, kCtrCount * sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
   }
-  if (kCount) {
-    for (int o = 16; o > 0; o >>= 1) {
-      nkept += __shfl_xor_sync(0xffffffffu, nkept, o);
-      neval += __shfl_xor_sync(0xffffffffu, neval, o);
-    }
-    if (lane == 0) {
-      atomicAdd(kept, (unsigned long long)nkept);
-      atomicAdd(kept + 1, (unsigned long long)neval);
-    }
-  }
+  raster_tasks_kernel<<<(ntiles + 255) / 256, 256, 0, st>>>(tile_start, ntiles, cap, d,
+                                                            min(sms * 3, kFwdSlots), tk, proj);
+  const int grid = sms * c.ctas;
+  if (c.cons == 6) return launch_fwd_one<6, 2, 3, kCount>(grid, rec, list, M, d, l2tau, tk, proj, kept, st);
+  if (c.cons == 10) return launch_fwd_one<10, 2, 2, kCount>(grid, rec, list, M, d, l2tau, tk, proj, kept, st);
+  if (c.cons == 12) return launch_fwd_one<12, 4, 2, kCount>(grid, rec, list, M, d, l2tau, tk, proj, kept, st);
+  if (c.prod == 4) return launch_fwd_one<8, 4, 2, kCount>(grid, rec, list, M, d, l2tau, tk, proj, kept, st);
+  return launch_fwd_one<8, 2, 3, kCount>(grid, rec, list, M, d, l2tau, tk, proj, kept, st);
+}
+
+cudaError_t launch_raster_fwd(int cfg, const Rec *rec, const uint2 *list,
+                              const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
+                              float l2tau, float *proj, const RasterTasks &tk, bool fresh,
+                              cudaStream_t st) {
+  return launch_fwd_any<false>(cfg, rec, list, tile_start, cap, M, B, d, l2tau, proj, nullptr, tk,
+                               fresh, st);
+}
+
+cudaError_t launch_count_kept(int cfg, const Rec *rec, const uint2 *list,
+                              const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
+                              float l2tau, unsigned long long *kept, const RasterTasks &tk,
+                              cudaStream_t st) {
+  return launch_fwd_any<true>(cfg, rec, list, tile_start, cap, M, B, d, l2tau, nullptr, kept, tk,
+                              false, st);
 }
 
 // Longest-first order of the B*T tiles for the persistent forms: a counting
@@ -586,82 +651,6 @@ __global__ void __launch_bounds__(1024) tile_order_kernel(const int64_t *__restr
     if (c < 32) order[base + __popc(peers & lt)] = (uint32_t)i;
     __syncthreads();  // rounds in index order
   }
-}
-
-// The forward's kernel configurations (the autotuner's search space).
-static const FwdCfg kFwdCfgs[] = {
-    {0, 2, 9, 0, 0, "runs, 256-record windows, 9 CTAs/SM"},
-    {1, 2, 9, 0, 0, "aligned, 256-record windows, 9 CTAs/SM"},
-    {1, 2, 8, 0, 0, "aligned, 256-record windows, 8 CTAs/SM"},
-    {1, 2, 9, 1, 9, "aligned, 256-record windows, 9 CTAs/SM, persistent longest-first"},
-    {1, 2, 8, 1, 8, "aligned, 256-record windows, 8 CTAs/SM, persistent longest-first"},
-    {1, 2, 8, 1, 7, "aligned, 256-record windows, 7 CTAs/SM, persistent longest-first"},
-    {1, 2, 8, 1, 6, "aligned, 256-record windows, 6 CTAs/SM, persistent longest-first"},
-    {1, 2, 8, 1, 5, "aligned, 256-record windows, 5 CTAs/SM, persistent longest-first"},
-};
-int fwd_config_count() { return (int)(sizeof(kFwdCfgs) / sizeof(kFwdCfgs[0])); }
-const FwdCfg &fwd_config(int i) { return kFwdCfgs[i]; }
-
-template <int kSubW, int kMinB, bool kCount>
-static cudaError_t launch_aligned(const FwdCfg &c, const Rec *rec, const uint2 *list,
-                                  const int64_t *tile_start, int64_t cap,
-                                  int64_t M, int B, int d, float l2tau, float *proj,
-                                  unsigned long long *kept, uint32_t *order, unsigned *next_tile,
-                                  cudaStream_t st) {
-  const int nt = d / kTile, ntiles = nt * nt * B;
-  if (c.persistent) {
-    tile_order_kernel<<<1, 1024, 0, st>>>(tile_start, ntiles, order, next_tile);
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int grid = max(1, min(ntiles, sms * min(c.ctas, kMinB)));
-    raster_fwd_aligned_kernel<kSubW, kMinB, kCount><<<grid, kThreads, 0, st>>>(
-        rec, list, tile_start, cap, M, d, l2tau, order, ntiles, next_tile, proj, kept);
-  } else {
-    dim3 grid(nt * nt, B);
-    raster_fwd_aligned_kernel<kSubW, kMinB, kCount><<<grid, kThreads, 0, st>>>(
-        rec, list, tile_start, cap, M, d, l2tau, nullptr, 0, nullptr, proj, kept);
-  }
-  return cudaGetLastError();
-}
-
-template <bool kCount>
-static cudaError_t launch_fwd_any(int cfg, const Rec *rec, const uint2 *list,
-                                  const int64_t *tile_start, int64_t cap,
-                                  int64_t M, int B, int d, float l2tau, float *proj,
-                                  unsigned long long *kept, uint32_t *order, unsigned *next_tile,
-                                  cudaStream_t st) {
-  if (cfg < 0 || cfg >= fwd_config_count()) return cudaErrorInvalidValue;
-  const FwdCfg &c = kFwdCfgs[cfg];
-  if (c.persistent && (order == nullptr || next_tile == nullptr)) return cudaErrorInvalidValue;
-  if (c.form == 0) {
-    const int nt = d / kTile;
-    dim3 grid(nt * nt, B);
-    raster_fwd_kernel<kCount><<<grid, kThreads, 0, st>>>(rec, list, tile_start, cap, M, d,
-                                                         l2tau, proj, kept);
-    return cudaGetLastError();
-  }
-  if (c.minb == 9)
-    return launch_aligned<2, 9, kCount>(c, rec, list, tile_start, cap, M, B, d, l2tau, proj,
-                                        kept, order, next_tile, st);
-  return launch_aligned<2, 8, kCount>(c, rec, list, tile_start, cap, M, B, d, l2tau, proj,
-                                      kept, order, next_tile, st);
-}
-
-cudaError_t launch_raster_fwd(int cfg, const Rec *rec, const uint2 *list,
-                              const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
-                              float l2tau, float *proj, uint32_t *order, unsigned *next_tile,
-                              cudaStream_t st) {
-  return launch_fwd_any<false>(cfg, rec, list, tile_start, cap, M, B, d, l2tau, proj,
-                               nullptr, order, next_tile, st);
-}
-
-cudaError_t launch_count_kept(int cfg, const Rec *rec, const uint2 *list,
-                              const int64_t *tile_start, int64_t cap,
-                              int64_t M, int B, int d, float l2tau, unsigned long long *kept,
-                              uint32_t *order, unsigned *next_tile, cudaStream_t st) {
-  return launch_fwd_any<true>(cfg, rec, list, tile_start, cap, M, B, d, l2tau, nullptr,
-                              kept, order, next_tile, st);
 }
 
 // The g tile is stored [pixel row in block][block ^ g_swizzle(row)]: rows 2

@@ -1,0 +1,50 @@
+"""Tile lists at the lengths where the rasterisers cut them: one tile (d = 16)
+that holds every Gaussian, so a list's length is the Gaussian count; the
+segments are 256 entries in small calls and 1024 in large ones, chunks of 32
+and 64 entries inside them.  Held to the contract's tolerances (gemtest.py)."""
+import numpy as np
+import pytest
+import torch
+
+import gemtest as gt
+import oracle
+from paper_2509_25075_gb300 import synthetic as syn
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(M, B, seed, tau=None):
+    w = syn.Workload("seg", d=16, M=M, B=B, apix=1.2, n_clusters=1, s_lo=0.8, s_hi=3.0, seed=seed)
+    tau = w.tau if tau is None else tau
+    inp = gt.inputs(w)
+    ctx = gt.context(w, tau=tau)
+    args = [gt.to_dev(inp[k]) for k in ("params", "R", "t")]
+    proj = torch.empty(B, 16, 16, device=gt.DEV)
+    ctx.gem_project(*args, proj)
+    ref = oracle.project(inp["params"], inp["R"], inp["t"], w.d, w.apix, tau)
+    border = None if tau == 0 else gt.borderline_pairs(inp, w, tau) if M * B <= 20000 else np.full(B, 40)
+    gt.assert_proj_close(proj.cpu().numpy(), ref, tau, border)
+    again = torch.empty_like(proj)
+    ctx.gem_project(*args, again)
+    assert torch.equal(proj, again)
+    g = syn.smooth_field(w) * 1e-3
+    grad = torch.empty(M, 11, device=gt.DEV)
+    ctx.gem_project_backward(gt.to_dev(g), grad)
+    assert ctx.gem_status() == 0
+    ref = oracle.grad(inp["params"], inp["R"], inp["t"], w.d, w.apix, tau, g)
+    edge = oracle.grad_border(inp["params"], inp["R"], inp["t"], w.d, w.apix, tau, g, rel=1e-5) if tau else 0 * ref
+    got = grad.cpu().numpy().astype(np.float64)
+    assert np.linalg.norm(got - ref) <= 1e-4 * np.linalg.norm(ref) + np.linalg.norm(edge)
+    ctx.close()
+
+
+@pytest.mark.parametrize("M", [1, 31, 32, 33, 63, 64, 65, 127, 129, 255, 256, 257, 511, 513, 1023, 1025, 2100])
+def test_list_lengths_in_a_small_call(M):
+    _check(M, 2, seed=M)
+
+
+@pytest.mark.parametrize("M", [1023, 1024, 1025, 2049])
+def test_list_lengths_in_a_large_call(M):
+    """About a million entries: segments of 1024.  tau = 0, so that no pair
+    is near the threshold."""
+    _check(M, 1 + 1000000 // M, seed=M, tau=0.0)
