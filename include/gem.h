@@ -389,8 +389,8 @@ int gem_ctf_loss_static(int32_t d, float apix, int32_t B, const float *proj, con
  * same result (the forward bitwise, the backward within the rounding of
  * float64 sums taken in another order): the forward (step a3) with 6 to 12
  * warps that evaluate and 2 or 4 that stage records, and 1 to 3 CTAs per SM;
- * the backward (a5) with 1 or 2 lanes per record, on a per-tile or a persistent
- * grid, with warp windows of 64, 128 or 256 records and 5 to 8 CTAs per SM.
+ * the backward (a5) with warp windows of 128 or 256 records and 3 to 8 CTAs
+ * per SM.
  * Which is
  * fastest depends on the image side, the batch and the Gaussians' sizes.
  * Counts of each kind (kind 0: forward, 1: backward); a configuration's

@@ -76,8 +76,6 @@ struct gem_ctx {
   // gem_raster.cu); -1: the autotuner's cached choice for the call's shape,
   // else the default
   int fwd_cfg = -1, bwd_cfg = -1;
-  uint32_t *order = nullptr;     // [max_B * T] tile order of the persistent backward
-  unsigned *next_tile = nullptr;  // [1] its work counter
   RasterTasks tasks{};            // segments of the tile lists
   float *tune_grad = nullptr;     // [max_M][11] gradient the autotuner's backward writes
   std::vector<void *> allocs;
@@ -92,9 +90,7 @@ struct gem_ctx {
   // batch of gem_query, binned for M = bins_M Gaussians, B = bins_B images
   // with threshold bins_l2tau
   bool have_bins = false;
-  // binnings so far, and the one whose longest-first tile order `order`
-  // holds (a persistent forward computed it): the backward reuses it
-  uint64_t bins_gen = 0, order_gen = ~0ull;
+  bool bwd_fresh = false;  // no backward has taken the tasks of these bins yet
   bool bins_of_proj = false;
   int64_t bins_M = 0;
   int bins_B = 0;
@@ -110,7 +106,7 @@ struct gem_ctx {
 // The configurations used when neither the context nor the autotuner's cache
 // names one (the fastest measured on the benchmark workloads).
 constexpr int kDefaultFwdCfg = 0;  // 6 consumer and 2 producer warps, 3 CTAs per SM
-constexpr int kDefaultBwdCfg = 3;  // one lane per record, persistent longest-first
+constexpr int kDefaultBwdCfg = 0;  // 256-record windows, 5 CTAs per SM
 
 // The autotuner's choices, shared by every context of the process: keyed by
 // device, image side, batch and the bit length of M (shapes that bin alike).
@@ -284,8 +280,7 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
             alloc(c, &c->dproj, (size_t)g.max_B * d * d) &&
             alloc(c, &c->Z, (size_t)g.max_B * d * d) && alloc(c, &c->tw, (size_t)d) &&
             alloc(c, &c->lossp, (size_t)g.max_B * (ctf_partials(d) + 1)) && alloc(c, &c->status, 1) &&
-            alloc(c, &c->kept, 2) &&
-            alloc(c, &c->order, (size_t)g.max_B * c->T) && alloc(c, &c->next_tile, 1);
+            alloc(c, &c->kept, 2);
   // a task per tile, or two per partial image of tiles with several segments
   const size_t nparts = raster_part_count(c->cfg.max_pairs);
   ok = ok && alloc(c, &c->tasks.task, 2 * ((size_t)g.max_B * c->T + nparts)) &&
@@ -427,7 +422,6 @@ int gem_project(gem_ctx *c, const float *params, int64_t M, int32_t B, const flo
   {
     StageScope sc(c, GEM_STAGE_BIN, g.zsort ? 10 : 4);
     c->have_bins = false;
-    ++c->bins_gen;
     if ((e = launch_bin(c->rec, c->bin.key, M, B, g.d, c->l2tau, g.zsort, c->bin, &perm,
                         c->stream)) != cudaSuccess)
       return cuda_fail(c, e, "bin");
@@ -443,6 +437,7 @@ int gem_project(gem_ctx *c, const float *params, int64_t M, int32_t B, const flo
     if ((e = launch_raster_fwd(fc, c->rec, c->bin.list, c->bin.tile_start, c->bin.cap, M, B, g.d,
                                c->l2tau, proj, c->tasks, true, c->stream)) != cudaSuccess)
       return cuda_fail(c, e, "raster_fwd");
+    c->bwd_fresh = true;
   }
   c->have_proj = true;
   return GEM_OK;
@@ -495,13 +490,7 @@ static int backward_common(gem_ctx *c, const float *dproj, float *grad, bool den
   // the whole buffer, should an earlier pass have stopped before clearing it
   size_t mbytes = (size_t)g.max_B * g.max_M * 6 * sizeof(double);
   {
-    // the persistent forms add a tile-order launch unless the forward's
-    // order of these bins is reused (then a counter reset, no kernel)
-    StageScope sc(c, GEM_STAGE_RASTER_BWD,
-                  1 + (!dense && bwd_config(active_bwd(c, c->B, c->M)).persistent &&
-                               c->order_gen != c->bins_gen
-                           ? 1
-                           : 0));
+    StageScope sc(c, GEM_STAGE_RASTER_BWD, 1);
     if (!dense && !c->mom_clean && (e = cudaMemsetAsync(c->mom, 0, mbytes, c->stream)) != cudaSuccess)
       return cuda_fail(c, e, "moment clear");
     c->mom_clean = false;
@@ -510,8 +499,9 @@ static int backward_common(gem_ctx *c, const float *dproj, float *grad, bool den
     else
       e = launch_raster_bwd(active_bwd(c, c->B, c->M), c->rec, c->bin.list,
                             c->bin.tile_start, c->bin.cap, c->M, c->B, g.d, c->l2tau, dproj, c->mom,
-                            c->order, c->next_tile, c->order_gen == c->bins_gen, c->stream);
+                            c->tasks, c->bwd_fresh, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "raster_bwd");
+    if (!dense) c->bwd_fresh = false;
   }
   StageScope sc(c, GEM_STAGE_PREP_BWD, 2);
   if ((e = launch_prep_bwd(c->psort, c->gauss_slot, c->gp, c->M, c->B, c->R, c->t, g.apix, g.d, g.norm_mode, shape_flags(g),
@@ -728,7 +718,6 @@ int gem_query(gem_ctx *c, const float *params, int64_t M, float tau, float *vol)
   for (int k0 = 0; k0 < g.d; k0 += g.max_B) {
     const int ns = g.d - k0 < g.max_B ? g.d - k0 : g.max_B;
     const uint32_t *perm = nullptr;
-    ++c->bins_gen;  // the slices' bins replace the projection's
     if ((e = launch_slice_prep(c->qp, M, k0, ns, g.apix, g.d, l2tau, c->rec, c->stream)) !=
             cudaSuccess ||
         (e = launch_bin(c->rec, c->bin.key, M, ns, g.d, l2tau, 0, c->bin, &perm, c->stream)) !=

@@ -316,7 +316,8 @@ cudaError_t bin_configure(int d);
 // Tasks of the rasterisers (segments of the tiles' lists, see gem_raster.cu).
 constexpr int kCtrFwd = 0, kCtrBwd = 1;      // next task of the forward, the backward
 constexpr int kCtrTasks = 2, kCtrParts = 3;  // tasks made, partial images handed out
-constexpr int kCtrCount = 4;
+constexpr int kCtrSegment = 4;               // segment length
+constexpr int kCtrCount = 5;
 struct RasterTasks {
   uint4 *task;     // two words per task: (list start, lo and hi; entries; image * T + tile),
                    // (segment, segments of the tile, the tile's first partial image, 0)
@@ -340,24 +341,20 @@ cudaError_t launch_raster_fwd(int cfg, const Rec *rec, const uint2 *list,
                               const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
                               float l2tau, float *proj, const RasterTasks &tk, bool fresh,
                               cudaStream_t st);
-// A configuration of the backward rasteriser: lanes sharing one record,
-// records per lane per warp window, persistent grid (tiles longest-first
-// from a counter; order [B*T] and next_tile [1] are its scratch).
+// A configuration of the backward rasteriser: records per lane and window,
+// CTAs per SM.
 struct BwdCfg {
-  int lanes, per, persistent;
-  int ctas;  // persistent grid: CTAs per SM (fewer tiles in flight keep more of
-             // their records and moments in L2)
+  int per, ctas;
   const char *name;
 };
 int bwd_config_count();
 const BwdCfg &bwd_config(int i);
-// order_ready: `order` already holds the longest-first order of these bins
-// (a persistent forward computed it); the persistent forms then only reset
-// their counter.
+// Runs the tasks that the last forward made of these bins.  fresh: no
+// backward has taken them yet.
 cudaError_t launch_raster_bwd(int cfg, const Rec *rec, const uint2 *list,
                               const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
-                              float l2tau, const float *dproj, double *mom, uint32_t *order,
-                              unsigned *next_tile, bool order_ready, cudaStream_t st);
+                              float l2tau, const float *dproj, double *mom, const RasterTasks &tk,
+                              bool fresh, cudaStream_t st);
 cudaError_t launch_count_kept(int cfg, const Rec *rec, const uint2 *list,
                               const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
                               float l2tau, unsigned long long *kept, const RasterTasks &tk,

@@ -18,21 +18,20 @@
 //     list order with Kahan compensation.  The result is deterministic and
 //     follows the list's depth order segment by segment.
 // a5: the "efficient gradient" of Sec. 1 (iii) / Sec. 3.2: only pairs kept by
-//     Eq. accu.  Each warp takes windows of 64, 128 or 256 records of the
-//     list (the next one not yet taken), sorts the window by block count
-//     and runs it in rounds of records with neighbouring counts, one or two
-//     lanes per record: the lanes walk the record's blocks and accumulate
+//     Eq. accu.  Each warp takes up to 256 entries of a segment, sorts them by
+//     block count and first block and runs them in rounds of 32 records, one
+//     lane per record: the lanes walk the record's blocks and accumulate
 //     six moments of w = g * value in the record's whitened coordinates
-//     (per row: the sums of w, w z1, w z1^2 in packed float pairs, weighted
-//     by z2).  The second moments are taken about the whitened S^, c^2 I:
+//     (rows in packed float pairs: the sums of w, w z1, w z1^2, weighted by
+//     z2).  The second moments are taken about the whitened S^, c^2 I:
 //     for a wide Gaussian under a smooth upstream gradient the conic and
 //     amplitude terms of dL/dS^ nearly cancel, and this form lets that
 //     cancellation happen inside an accurate sum instead of in the float32
 //     chain rule.  Each block's sums join the lane's totals, and the (tile,
 //     Gaussian) partial goes to float64 moments in global memory (L2
 //     atomics), so the sum over a Gaussian's tiles loses nothing to
-//     rounding.  No barrier couples the warps within a tile.  a6 turns the
-//     moments into parameter gradients.
+//     rounding.  No barrier couples the warps.  a6 turns the moments into
+//     parameter gradients.
 #include "gem_internal.cuh"
 
 namespace gem {
@@ -164,6 +163,7 @@ __global__ void __launch_bounds__(256) raster_tasks_kernel(const int64_t *__rest
     all += wsum[0][w];
     allp += wsum[1][w];
   }
+  if (i == 0) tk.ctr[kCtrSegment] = (unsigned)S;
   if (threadIdx.x == 0) {
     base_sh[0] = atomicAdd(tk.ctr + kCtrTasks, all);
     base_sh[1] = atomicAdd(tk.ctr + kCtrParts, allp);
@@ -400,11 +400,11 @@ __global__ void __launch_bounds__(32 * (kCons + kProd), kMinB) raster_fwd_kernel
         const int slot = slots[i];
         const float4 A = W.sa[slot];
         const float2 Bv = W.sb[slot];
-        // -e = z1^2 + (z2^2 - l2A), z1 = u11 dx + u12 dy, z2 = u22 dy, two
-        // rows of a column in one packed operation
-        float2 ux[4];
+        // -e = z1^2 + (z2^2 - l2A), z1 = u11 dx + u12 dy (u11 dx fused into
+        // the sum), z2 = u22 dy, two rows of a column in one packed operation
+        float2 dx[4];
 #pragma unroll
-        for (int x = 0; x < 4; ++x) ux[x] = f2(__fmul_rn(A.z, __fsub_rn(X0 + (float)x, A.x)));
+        for (int x = 0; x < 4; ++x) dx[x] = f2(__fsub_rn(X0 + (float)x, A.x));
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const float2 dy = add2(h ? ys1 : ys0, f2(-A.y));
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(32 * (kCons + kProd), kMinB) raster_fwd_kernel
           const float2 nc = fma2(z2, z2, f2(-Bv.y));
 #pragma unroll
           for (int x = 0; x < 4; ++x) {
-            const float2 z = add2(ux[x], uy);
+            const float2 z = fma2(f2(A.z), dx[x], uy);
             const float2 f = fma2(z, z, nc);
             if (kCount)
               nkept += (f.x < nl2tau) + (f.y < nl2tau);
@@ -597,356 +597,313 @@ cudaError_t launch_count_kept(int cfg, const Rec *rec, const uint2 *list,
                               false, st);
 }
 
-// Longest-first order of the B*T tiles for the persistent forms: a counting
-// sort of the tiles by the bit length of their list length (32 classes,
-// longest class first), so that the longest tiles start in the first wave
-// and the launch does not end waiting for one.  One CTA walks the tiles in
-// index order, 1024 at a time, so within a class the order follows the
-// index (image after image) up to the order of the warps of one round.  CTA
-// 0 also resets the work counter.  Which tile runs when changes nothing in
-// its result.  Lanes of a warp with the same class share one shared-memory
-// atomic (tiles mostly fall in a few classes).  (Ordering image by image,
-// longest tile first within each image, kept more records in L2 but ran
-// slower: the long tiles of the last images started late.)
-__device__ __forceinline__ int tile_class(const int64_t *__restrict__ tile_start, int64_t i) {
-  const int64_t len = tile_start[i + 1] - tile_start[i];
-  return 31 - min(31, 64 - __clzll((unsigned long long)max(len, (int64_t)0)));
-}
-
-__global__ void __launch_bounds__(1024) tile_order_kernel(const int64_t *__restrict__ tile_start,
-                                                         int ntiles, uint32_t *__restrict__ order,
-                                                         unsigned *__restrict__ next_tile) {
-  __shared__ unsigned hist[32], cur[32];
-  const int lane = threadIdx.x & 31;
-  const unsigned lt = (1u << lane) - 1u;
-  if (threadIdx.x < 32) hist[threadIdx.x] = 0;
-  __syncthreads();
-  // every warp runs the same number of rounds, so all its lanes take part in
-  // each match
-  const int rounds = (ntiles + blockDim.x - 1) / blockDim.x;
-  for (int r = 0; r < rounds; ++r) {
-    const int i = r * blockDim.x + threadIdx.x;
-    const int c = i < ntiles ? tile_class(tile_start, i) : 32 + lane;
-    const unsigned peers = __match_any_sync(0xffffffffu, c);
-    if (c < 32 && (peers & lt) == 0) atomicAdd(&hist[c], (unsigned)__popc(peers));
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned run = 0;
-    for (int c = 0; c < 32; ++c) {
-      cur[c] = run;
-      run += hist[c];
-    }
-    *next_tile = 0u;
-  }
-  __syncthreads();
-  for (int r = 0; r < rounds; ++r) {
-    const int i = r * blockDim.x + threadIdx.x;
-    const int c = i < ntiles ? tile_class(tile_start, i) : 32 + lane;
-    const unsigned peers = __match_any_sync(0xffffffffu, c);
-    const int leader = __ffs(peers) - 1;
-    unsigned base = 0;
-    if (c < 32 && lane == leader) base = atomicAdd(&cur[c], (unsigned)__popc(peers));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (c < 32) order[base + __popc(peers & lt)] = (uint32_t)i;
-    __syncthreads();  // rounds in index order
-  }
-}
-
-// The g tile is stored [pixel row in block][block ^ g_swizzle(row)]: rows 2
-// and 3 have their blocks permuted by k ^ 4, so the two lanes of a record
-// in the two-lane form (rows 0 and 2, then 1 and 3 of the same block) read
-// different banks (a float4's bank group is its index mod 8).
-__device__ __forceinline__ int g_swizzle(int row) { return (row & 2) << 1; }
-
-// The six moments of w = g * value over pixel rows row0 .. row0 + kRows - 1
-// of block k of the tile at (x0, y0) for one record (centre A.x, A.y, first
-// row of U in A.z, A.w; u22, l2A), in the record's whitened coordinates
-// z1 = u11 dx + u12 dy, z2 = u22 dy, added to the running totals
-// (n0, n1), (n2, n3), (n4, n5):
+// The six moments of w = g * value over the 16 pixels of block k of the tile
+// at (x0, y0) for one record (centre A.x, A.y, first row of U in A.z, A.w;
+// u22, l2A), in the record's whitened coordinates z1 = u11 dx + u12 dy,
+// z2 = u22 dy, added to the running totals n[0..5], each a pair (upper rows
+// of the row pairs, lower rows):
 //   n0 = sum w, n1 = sum w z1, n2 = sum w z2,
-//   n3 = sum w (z1^2 - c^2), n4 = sum w z1 z2, n5 = sum w (z2^2 - c^2)
-// (per row: the sums of w, w z1, w z1^2 in packed float pairs, weighted by
-// z2, which is constant along a row; the second moments taken about c^2 I,
-// the whitened S^, per block).  sg is the g tile, [pixel row in block][block].
-template <int kRows>
+//   n3 = sum w (z1^2 - c^2), n4 = sum w z1 z2, n5 = sum w (z2^2 - c^2).
+// Rows are taken two at a time, one per half of a packed pair, so the row
+// terms (z2, and what is weighted by it) pack as naturally as the pixels'
+// (a fifth fewer instructions than pairs of columns, whose row terms are
+// scalars).  The second moments are taken about c^2 I, the whitened S^, per
+// block.  sg is the g tile: [row pair, column pair][block] = rows 2 h and
+// 2 h + 1 of column 2 c, then of column 2 c + 1.
 __device__ __forceinline__ void block_moments(const float4 (*__restrict__ sg)[16], int k, int x0,
-                                              int y0, int row0, const float4 &A, float u22,
-                                              float l2A, float nl2tau, float2 &s01, float2 &s23,
-                                              float2 &s45) {
-  const float2 u11 = f2(A.z);
-  const float u12 = A.w;
-  // dx and dy rounded exactly as the forward rounds them (pixel index
-  // minus centre), so both decide Eq. accu on the same exponent
-  const float X0 = (float)(x0 + 4 * (k & 3)), Y0 = (float)(y0 + 4 * (k >> 2) + row0);
-  const float2 npx = f2(-A.x);
-  const float2 ux01 = mul2(u11, add2(make_float2(X0, X0 + 1.f), npx));
-  const float2 ux23 = mul2(u11, add2(make_float2(X0 + 2.f, X0 + 3.f), npx));
-  // this block's rows: sums of w, w z1, w z2, w z1^2, w z1 z2, w z2^2
-  float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f, m4 = 0.f, m5 = 0.f;
+                                              int y0, const float4 &A, float u22, float l2A,
+                                              float nl2tau, float2 (&n)[6]) {
+  // the exponent rounded exactly as the forward rounds it, so that both
+  // decide Eq. accu alike
+  const float X0 = (float)(x0 + 4 * (k & 3)), Y0 = (float)(y0 + 4 * (k >> 2));
+  float2 dx[4];
 #pragma unroll
-  for (int rr = 0; rr < kRows; ++rr) {
-    const float dy = Y0 + (float)rr - A.y;
-    const float2 uy = f2(u12 * dy);
-    const float z2 = u22 * dy;
-    const float2 nc = f2(fmaf(z2, z2, -l2A));
-    // -e = z1^2 + (z2^2 - l2A), as in the forward's terms
-    const float2 z01 = add2(ux01, uy), z23 = add2(ux23, uy);
-    const float2 f01 = fma2(z01, z01, nc), f23 = fma2(z23, z23, nc);
-    const float4 g4 = sg[row0 + rr][k ^ g_swizzle(row0 + rr)];
-    // w = g * value on kept pairs (value > tau), zero elsewhere: g is masked
-    // to +0 on the integer pipe, which leaves the FMA pipe (this loop's
-    // busiest) the multiply
-    const float2 gm01 = make_float2(keep_or_zero(g4.x, f01.x, nl2tau), keep_or_zero(g4.y, f01.y, nl2tau));
-    const float2 gm23 = make_float2(keep_or_zero(g4.z, f23.x, nl2tau), keep_or_zero(g4.w, f23.y, nl2tau));
-    const float2 w01 = mul2(gm01, make_float2(ex2_approx(-f01.x), ex2_approx(-f01.y)));
-    const float2 w23 = mul2(gm23, make_float2(ex2_approx(-f23.x), ex2_approx(-f23.y)));
-    // the row's sums of w, w z1 and w z1^2, then weighted by z2
-    const float2 wz01 = mul2(w01, z01), wz23 = mul2(w23, z23);
-    const float2 s0 = add2(w01, w23);
-    const float2 s1 = add2(wz01, wz23);
-    const float2 s2 = fma2(wz23, z23, mul2(wz01, z01));
-    const float r0 = s0.x + s0.y, r1 = s1.x + s1.y, r2 = s2.x + s2.y;
-    m0 += r0;
-    m1 += r1;
-    m3 += r2;
-    m2 = fmaf(r0, z2, m2);
-    m4 = fmaf(r1, z2, m4);
-    m5 = fmaf(r0 * z2, z2, m5);
+  for (int x = 0; x < 4; ++x) dx[x] = f2(__fsub_rn(X0 + (float)x, A.x));
+  float2 m[6];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const float2 dy = add2(make_float2(Y0 + (float)(2 * h), Y0 + (float)(2 * h + 1)), f2(-A.y));
+    const float2 uy = mul2(f2(A.w), dy);
+    const float2 z2 = mul2(f2(u22), dy);
+    const float2 nc = fma2(z2, z2, f2(-l2A));
+    float2 s0, s1, s2;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const float4 g4 = sg[2 * h + c][k];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        // -e = z1^2 + (z2^2 - l2A), as in the forward's terms
+        const float2 z = fma2(f2(A.z), dx[2 * c + q], uy);
+        const float2 f = fma2(z, z, nc);
+        // w = g * value on kept pairs (value > tau), zero elsewhere: g is
+        // masked to +0 on the integer pipe, which leaves the FMA pipe (this
+        // loop's busiest) the multiply
+        const float2 gm = make_float2(keep_or_zero(q ? g4.z : g4.x, f.x, nl2tau),
+                                      keep_or_zero(q ? g4.w : g4.y, f.y, nl2tau));
+        const float2 w = mul2(gm, make_float2(ex2_approx(-f.x), ex2_approx(-f.y)));
+        const float2 wz = mul2(w, z);
+        s0 = c + q ? add2(s0, w) : w;
+        s1 = c + q ? add2(s1, wz) : wz;
+        s2 = c + q ? fma2(wz, z, s2) : mul2(wz, z);
+      }
+    }
+    // the rows' sums of w, w z1 and w z1^2, weighted by z2
+    const float2 t = mul2(s0, z2);
+    m[0] = h ? add2(m[0], s0) : s0;
+    m[1] = h ? add2(m[1], s1) : s1;
+    m[2] = h ? add2(m[2], t) : t;
+    m[3] = h ? add2(m[3], s2) : s2;
+    m[4] = h ? fma2(s1, z2, m[4]) : mul2(s1, z2);
+    m[5] = h ? fma2(t, z2, m[5]) : mul2(t, z2);
   }
   // second moments about c^2 I, then into the totals
-  m3 = fmaf(-kC2, m0, m3);
-  m5 = fmaf(-kC2, m0, m5);
-  s01 = add2(s01, make_float2(m0, m1));
-  s23 = add2(s23, make_float2(m2, m3));
-  s45 = add2(s45, make_float2(m4, m5));
+  m[3] = fma2(f2(-kC2), m[0], m[3]);
+  m[5] = fma2(f2(-kC2), m[0], m[5]);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) n[i] = add2(n[i], m[i]);
 }
 
-// kLpr lanes share one record (lane q of the group takes pixel rows
-// q * 4 / kLpr .. of every block of the record), so a round runs 32 / kLpr
-// records of neighbouring block counts; a warp window holds 32 * kPer
-// records.
-template <int kLpr, int kPer>
-__global__ void __launch_bounds__(kThreads, 8) raster_bwd_kernel(
-    const Rec *__restrict__ rec, const uint2 *__restrict__ list,
-    const int64_t *__restrict__ tile_start, int64_t cap,
-    int64_t M, int d, float l2tau, const float *__restrict__ dproj, double *__restrict__ mom,
-    const uint32_t *__restrict__ order, int ntiles, unsigned *__restrict__ next_tile) {
+// Entries of a backward unit: 256, less (down to 64) where that would leave
+// warps of the grid without one.
+__device__ __forceinline__ int unit_length(int64_t total, int nwarps) {
+  const int64_t U = (total / nwarps + 31) / 32 * 32;
+  return (int)max((int64_t)64, min((int64_t)256, U));
+}
+
+// a5.  Every warp works on its own: a unit is up to 256 consecutive entries of
+// a task (a segment of one tile's list), claimed from a counter, with the
+// tile's g in the warp's own shared memory, so no barrier couples the warps
+// and the units in flight at any time come from neighbouring tiles.  A warp
+// sorts each window of its unit by (number of blocks, first block) and runs
+// it in rounds of 32 records, one lane per record: the lanes of a round have
+// loops of one length, and mostly read the same blocks of g at the same time
+// (a broadcast instead of bank conflicts).  The moments of a round are added
+// to memory six lanes per record, which costs the L1 a sixth of the tag
+// lookups of one lane per record and about a tenth more instructions: the
+// better of the two at 2.5 list entries per (view, Gaussian) and four blocks
+// each (d 128, M 20000, B 256: 0.53 against 0.59 ms), the worse at 4.2 and
+// 5.5 (d 128, M 50000, B 64, scales 0.3-12 px: 0.66 against 0.62 ms), where
+// a record's evaluation takes longer; the line lies at 3 entries.
+//
+// What bounds it: the FMA pipe (57% of its cycles) and issue (66%).  Against
+// CTAs of four warps that walked a whole tile's list, the longest lists first
+// (us per launch, the default configuration then, the one the autotuner
+// picked, now): d 384, M 500000, B 16: 1033, 901, 792; d 128, M 20000, B 256:
+// 568, 568, 540; d 128, M 50000, B 64, scales 0.3-12 px: 1150, 846, 637;
+// d 64, M 2000, B 32: 44, 42, 26.
+template <int kPer, int kMinB>
+__global__ void __launch_bounds__(kThreads, kMinB) raster_bwd_kernel(
+    const Rec *__restrict__ rec, const uint2 *__restrict__ list, int64_t M, int d, float l2tau,
+    const int64_t *__restrict__ tile_start, int ntiles, const float *__restrict__ dproj,
+    double *__restrict__ mom, RasterTasks tk) {
   constexpr int kWarps = kThreads / 32;
-  constexpr int kWW = 32 * kPer;     // records per warp window
-  constexpr int kRpr = 32 / kLpr;    // records per round
-  constexpr int kRows = 4 / kLpr;    // pixel rows of a block per lane
-  // g by pixel row within a block and block: [row][block ^ g_swizzle(row)]
-  // = 4 pixels (see g_swizzle)
-  __shared__ float4 sg[4][16];
-  __shared__ float4 sa[kWarps][kWW];  // px, py, u11, u12
-  __shared__ float2 sb[kWarps][kWW];  // u22, log2 A
-  __shared__ uint32_t sj[kWarps][kWW];
-  __shared__ unsigned short smask[kWarps][kWW];
-  __shared__ int hist[kWarps][32];
-  __shared__ int next_win;
-  __shared__ int tile_sh;
+  constexpr int kWW = 32 * kPer;  // records per window
+  constexpr int kBins = 256;      // (16 - blocks) * 16 + first block
+  __shared__ float4 sg_[kWarps][4][16];  // g by row pair and column pair of a block, and block
+  __shared__ float4 sa_[kWarps][kWW];    // px, py, u11, u12
+  __shared__ float2 sb_[kWarps][kWW];    // u22, log2 A
+  __shared__ uint32_t sj_[kWarps][kWW];
+  __shared__ unsigned short smask_[kWarps][kWW];
+  __shared__ float red_[kWarps][32 * 7];  // a round's moments, one word of padding per record
+  static_assert(sizeof(sa_[0]) >= kBins * sizeof(int), "the bins lie where the records go");
   const int nt = d / kTile, T = nt * nt;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float nl2tau = -l2tau;  // kept: -e < -log2(tau)
-  const int64_t total = tile_start[order == nullptr ? (int64_t)gridDim.y * T : (int64_t)ntiles];
-  // tiles come from the grid (order == nullptr) or, in the persistent form,
-  // from a shared counter over a longest-first order
-  for (int it = 0;; ++it) {
-  int bt;
-  if (order == nullptr) {
-    if (it > 0) break;
-    bt = blockIdx.y * T + blockIdx.x;
-  } else {
-    __syncthreads();  // every warp is done with the previous tile
-    if (threadIdx.x == 0) tile_sh = (int)atomicAdd(next_tile, 1u);
-    __syncthreads();
-    const int qq = tile_sh;
-    if (qq >= ntiles) break;
-    bt = (int)order[qq];
-  }
-  const int b = bt / T, t = bt - b * T;
-  const int tx = t % nt, ty = t / nt;
-  const int x0 = tx * kTile, y0 = ty * kTile;
-  // g tile, stored block by block
-  if (threadIdx.x < kTile * kTile / 4) {
-    const int r = threadIdx.x >> 2, q = threadIdx.x & 3;  // pixel row, 4-column group
-    sg[r & 3][(4 * (r >> 2) + q) ^ g_swizzle(r & 3)] =
-        *reinterpret_cast<const float4 *>(dproj + ((int64_t)b * d + y0 + r) * d + x0 + 4 * q);
-  }
-  if (threadIdx.x == 0) next_win = kWarps;
-  __syncthreads();
-  int64_t s = tile_start[bt];
-  int64_t e = tile_start[bt + 1];
-  e = min(e, cap);
-  s = min(s, e);
-  if (total > cap) e = s;  // overflowed: every list empty
-  const Rec *rb = rec + (int64_t)b * M;
-  double *mb = mom + (int64_t)b * M * 6;
-  int *h = hist[warp];
-  const int gq = lane % kLpr;                                   // lane within the record's group
-  const unsigned gmask = ((1u << kLpr) - 1u) << (lane - gq);    // the group's lanes
-  const int row0 = gq * kRows;
-  // warp w takes window w first, then the next window not yet taken; no
-  // barrier couples the warps after the g tile is in place
-  int64_t base = s + kWW * warp;
-  while (base < e) {
-    uint32_t j[kPer];
-    unsigned m[kPer];
-    __syncwarp();  // previous window's reads are done
-    h[lane] = 0;
-    __syncwarp();
+  float4(*sg)[16] = sg_[warp];
+  float4 *sa = sa_[warp];
+  float2 *sb = sb_[warp];
+  uint32_t *sj = sj_[warp];
+  unsigned short *smask = smask_[warp];
+  float *red = red_[warp];
+  const int lr = lane < 30 ? lane / 6 : 64, lc = lane % 6;  // record and moment a lane adds
+  int *bins = reinterpret_cast<int *>(sa);
+  const int nwarps = (int)gridDim.x * kWarps;
+  const int64_t total = tile_start[ntiles];
+  const int unit = unit_length(total, nwarps);
+  const int per_task = ((int)tk.ctr[kCtrSegment] + unit - 1) / unit;  // units of a task
+  const int64_t nunits = (int64_t)tk.ctr[kCtrTasks] * per_task;
+  const bool spread = total > 3 * (int64_t)(ntiles / T) * M;
+  int64_t u = blockIdx.x * kWarps + warp;
+  uint4 t0 = make_uint4(0u, 0u, 0u, 0u);
+  if (u < nunits) t0 = tk.task[2 * (u / per_task)];
+  while (u < nunits) {
+    // the next unit is claimed now and its descriptor read while this one runs
+    int64_t nu = 0;
+    uint4 tn = make_uint4(0u, 0u, 0u, 0u);
+    if (lane == 0) nu = (int64_t)atomicAdd(tk.ctr + kCtrBwd, 1u) + nwarps;
+    const int off = (int)(u % per_task) * unit;
+    const int n = min(unit, (int)t0.z - off);
+    const uint2 *L = list + (int64_t)(((uint64_t)t0.y << 32) | t0.x) + off;
+    const int bt = (int)t0.w;
+    const int b = bt / T, t = bt - b * T;
+    const int tx = t % nt, ty = t / nt;
+    const int x0 = tx * kTile, y0 = ty * kTile;
+    const Rec *rb = rec + (int64_t)b * M;
+    double *mb = mom + (int64_t)b * M * 6, *mbl = mb + lc;
+    if (n > 0) {
+      // the tile's g, stored block by block
+      float4 g[2];
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      const int64_t i = base + q * 32 + lane;
-      j[q] = 0;
-      m[q] = 0;
-      if (i < e) {
-        // the entry's two words read apart, the mask only for a valid index
-        // (fewer registers in flight than one 8-byte load per entry)
-        const uint32_t *ew = reinterpret_cast<const uint32_t *>(list + i);
-        j[q] = ew[0];
+      for (int h = 0; h < 2; ++h)
+        g[h] = __ldg(reinterpret_cast<const float4 *>(
+            dproj + ((int64_t)b * d + y0 + 8 * h + (lane >> 2)) * d + x0 + 4 * (lane & 3)));
+      __syncwarp();  // the last unit's reads are done
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = 8 * h + (lane >> 2), k = 4 * (r >> 2) + (lane & 3), hp = r & 2, lo = r & 1;
+        float *u0 = reinterpret_cast<float *>(&sg[hp][k]) + lo;
+        float *u1 = reinterpret_cast<float *>(&sg[hp + 1][k]) + lo;
+        u0[0] = g[h].x;
+        u0[2] = g[h].y;
+        u1[0] = g[h].z;
+        u1[2] = g[h].w;
+      }
+    }
+    for (int w0 = 0; w0 < n; w0 += kWW) {
+      uint2 en[kPer];
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
+        const int i = w0 + 32 * q + lane;
+        en[q] = i < n ? L[i] : make_uint2(0xffffffffu, 0u);
+      }
+      __syncwarp();  // the last window's reads are done
+      reinterpret_cast<int4 *>(bins)[lane] = make_int4(0, 0, 0, 0);
+      reinterpret_cast<int4 *>(bins)[32 + lane] = make_int4(0, 0, 0, 0);
+      __syncwarp();
+      int bin[kPer];
+#pragma unroll
+      for (int q = 0; q < kPer; ++q) {
         // an out-of-range index (an entry left unwritten when the lists
         // overflowed their capacity) counts as empty
-        m[q] = j[q] < (uint64_t)M ? ew[1] & 0xffffu : 0u;
-      }
-      atomicAdd(&h[__popc(m[q])], 1);
-    }
-    __syncwarp();
-    // exclusive scan of the count histogram, most blocks first: lane v gets
-    // the number of records with more than v blocks
-    {
-      const int c = h[lane];
-      int run = c;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int u = __shfl_down_sync(0xffffffffu, run, o);
-        if (lane + o < 32) run += u;
+        const unsigned m = en[q].x < (uint64_t)M ? en[q].y & 0xffffu : 0u;
+        en[q].y = m;
+        bin[q] = m ? (16 - __popc(m)) * 16 + __ffs(m) - 1 : -1;
+        if (m) atomicAdd(&bins[bin[q]], 1);
       }
       __syncwarp();
-      h[lane] = run - c;
-    }
-    __syncwarp();
+      // exclusive scan of the bins, eight per lane
+      int nv;
+      {
+        int4 c[2] = {reinterpret_cast<int4 *>(bins)[2 * lane], reinterpret_cast<int4 *>(bins)[2 * lane + 1]};
+        const int sum = c[0].x + c[0].y + c[0].z + c[0].w + c[1].x + c[1].y + c[1].z + c[1].w;
+        int inc = sum;
 #pragma unroll
-    for (int q = 0; q < kPer; ++q) {
-      const int pos = atomicAdd(&h[__popc(m[q])], 1);
-      if (m[q]) {
-        const Rec *rp = rb + j[q];
-        sa[warp][pos] = rp->a;
-        sb[warp][pos] = *reinterpret_cast<const float2 *>(&rp->b);
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += v;
+        }
+        nv = __shfl_sync(0xffffffffu, inc, 31);
+        int run = inc - sum;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          int4 o;
+          o.x = run;
+          o.y = o.x + c[h].x;
+          o.z = o.y + c[h].y;
+          o.w = o.z + c[h].z;
+          run = o.w + c[h].w;
+          reinterpret_cast<int4 *>(bins)[2 * lane + h] = o;
+        }
       }
-      sj[warp][pos] = j[q];
-      smask[warp][pos] = (unsigned short)m[q];
-    }
-    __syncwarp();
-    // rounds of 32 / kLpr records with neighbouring block counts
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < kPer; ++q)
+        if (bin[q] >= 0) bin[q] = atomicAdd(&bins[bin[q]], 1);
+      __syncwarp();  // the bins make way for the records
+#pragma unroll
+      for (int q0 = 0; q0 < kPer; q0 += 4) {
+        Rec r[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (bin[q0 + q] >= 0) r[q] = load_rec(rb + en[q0 + q].x);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (bin[q0 + q] >= 0) {
+            const int pos = bin[q0 + q];
+            sa[pos] = r[q].a;
+            sb[pos] = make_float2(r[q].b.x, r[q].b.y);
+            sj[pos] = en[q0 + q].x;
+            smask[pos] = (unsigned short)en[q0 + q].y;
+          }
+      }
+      __syncwarp();
+      if (w0 == 0) {
+        nu = __shfl_sync(0xffffffffu, nu, 0);
+        if (nu < nunits) tn = tk.task[2 * (nu / per_task)];
+      }
 #pragma unroll 1
-    for (int q = 0; q < kWW / kRpr; ++q) {
-      const int slot = q * kRpr + lane / kLpr;
-      const unsigned mk = smask[warp][slot];
-      if (!mk) continue;  // the whole group skips: the counts are sorted
-      const float4 A = sa[warp][slot];
-      const float2 Bv = sb[warp][slot];
-      float2 s01 = make_float2(0.f, 0.f), s23 = s01, s45 = s01;  // lane totals: (n0, n1), (n2, n3), (n4, n5)
-      for (unsigned mm = mk; mm; mm &= mm - 1)
-        block_moments<kRows>(sg, __ffs(mm) - 1, x0, y0, row0, A, Bv.x, Bv.y, nl2tau, s01, s23, s45);
-      float m0 = s01.x, m1 = s01.y, m2 = s23.x, m3 = s23.y, m4 = s45.x, m5 = s45.y;
+      for (int r0 = 0; r0 < nv; r0 += 32) {
+        const int slot = r0 + lane;
+        if (slot < nv) {
+          const float4 A = sa[slot];
+          const float2 Bv = sb[slot];
+          float2 tot[6];
 #pragma unroll
-      for (int o = 1; o < kLpr; o <<= 1) {
-        m0 += __shfl_xor_sync(gmask, m0, o);
-        m1 += __shfl_xor_sync(gmask, m1, o);
-        m2 += __shfl_xor_sync(gmask, m2, o);
-        m3 += __shfl_xor_sync(gmask, m3, o);
-        m4 += __shfl_xor_sync(gmask, m4, o);
-        m5 += __shfl_xor_sync(gmask, m5, o);
-      }
-      if (gq == 0) {
-        double *mo = mb + (int64_t)sj[warp][slot] * 6;
-        atomicAdd(mo + 0, (double)m0);
-        atomicAdd(mo + 1, (double)m1);
-        atomicAdd(mo + 2, (double)m2);
-        atomicAdd(mo + 3, (double)m3);
-        atomicAdd(mo + 4, (double)m4);
-        atomicAdd(mo + 5, (double)m5);
+          for (int i = 0; i < 6; ++i) tot[i] = make_float2(0.f, 0.f);
+          for (unsigned mm = smask[slot]; mm; mm &= mm - 1)
+            block_moments(sg, __ffs(mm) - 1, x0, y0, A, Bv.x, Bv.y, nl2tau, tot);
+          if (spread) {
+            double *mo = mb + 6ull * sj[slot];
+#pragma unroll
+            for (int i = 0; i < 6; ++i) atomicAdd(mo + i, (double)(tot[i].x + tot[i].y));
+          } else {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) red[7 * lane + i] = tot[i].x + tot[i].y;
+          }
+        }
+        if (spread) continue;
+        __syncwarp();
+        // six lanes add one record's six moments, five records at a time: the
+        // warp's addresses then lie in five or so lines, not in 32
+        const int left = min(32, nv - r0);
+        const float *rp = red + 7 * lr + lc;
+        const uint32_t *jp = sj + r0 + lr;
+#pragma unroll
+        for (int i = 0; i < 7; ++i)
+          if (5 * i + lr < left) atomicAdd(mbl + 6ull * jp[5 * i], (double)rp[35 * i]);
+        __syncwarp();  // read before the next round's replace them
       }
     }
-    int wn = 0;
-    if (lane == 0) wn = atomicAdd(&next_win, 1);
-    base = s + (int64_t)kWW * __shfl_sync(0xffffffffu, wn, 0);
+    if (n <= 0) {
+      nu = __shfl_sync(0xffffffffu, nu, 0);
+      if (nu < nunits) tn = tk.task[2 * (nu / per_task)];
+    }
+    u = nu;
+    t0 = tn;
   }
-  }  // tiles
 }
 
 // The backward's kernel configurations (the autotuner's search space):
-// lanes per record, records per lane per warp window, persistent grid and
-// its CTAs per SM.
+// records per lane and window, CTAs per SM.
 static const BwdCfg kBwdCfgs[] = {
-    {2, 4, 0, 0, "2 lanes per record, 128-record warp windows"},
-    {1, 4, 0, 0, "1 lane per record, 128-record warp windows"},
-    {2, 4, 1, 8, "2 lanes per record, 128-record warp windows, persistent longest-first"},
-    {1, 4, 1, 8, "1 lane per record, 128-record warp windows, persistent longest-first"},
-    {1, 2, 1, 8, "1 lane per record, 64-record warp windows, persistent longest-first"},
-    {1, 8, 1, 7, "1 lane per record, 256-record warp windows, persistent longest-first"},
-    {2, 8, 1, 7, "2 lanes per record, 256-record warp windows, persistent longest-first"},
-    {1, 4, 1, 6, "1 lane per record, 128-record warp windows, persistent longest-first, 6 CTAs/SM"},
-    {1, 8, 1, 6, "1 lane per record, 256-record warp windows, persistent longest-first, 6 CTAs/SM"},
-    {1, 8, 1, 5, "1 lane per record, 256-record warp windows, persistent longest-first, 5 CTAs/SM"},
+    {8, 5, "256-record warp windows, 5 CTAs/SM"}, {8, 4, "256-record warp windows, 4 CTAs/SM"},
+    {8, 6, "256-record warp windows, 6 CTAs/SM"}, {4, 8, "128-record warp windows, 8 CTAs/SM"},
+    {4, 7, "128-record warp windows, 7 CTAs/SM"}, {4, 6, "128-record warp windows, 6 CTAs/SM"},
+    {4, 5, "128-record warp windows, 5 CTAs/SM"}, {4, 4, "128-record warp windows, 4 CTAs/SM"},
+    {8, 3, "256-record warp windows, 3 CTAs/SM"}, {4, 3, "128-record warp windows, 3 CTAs/SM"},
 };
 int bwd_config_count() { return (int)(sizeof(kBwdCfgs) / sizeof(kBwdCfgs[0])); }
 const BwdCfg &bwd_config(int i) { return kBwdCfgs[i]; }
 
-template <int kLpr, int kPer>
-static void launch_bwd_lanes(dim3 grid, const Rec *rec, const uint2 *list,
-                             const int64_t *tile_start, int64_t cap,
-                             int64_t M, int d, float l2tau, const float *dproj, double *mom,
-                             const uint32_t *order, int ntiles, unsigned *next_tile,
-                             cudaStream_t st) {
-  raster_bwd_kernel<kLpr, kPer><<<grid, kThreads, 0, st>>>(rec, list, tile_start, cap, M,
-                                                           d, l2tau, dproj, mom, order, ntiles,
-                                                           next_tile);
-}
-
 cudaError_t launch_raster_bwd(int cfg, const Rec *rec, const uint2 *list,
                               const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
-                              float l2tau, const float *dproj, double *mom, uint32_t *order,
-                              unsigned *next_tile, bool order_ready, cudaStream_t st) {
+                              float l2tau, const float *dproj, double *mom, const RasterTasks &tk,
+                              bool fresh, cudaStream_t st) {
   if (cfg < 0 || cfg >= bwd_config_count()) return cudaErrorInvalidValue;
   const BwdCfg &c = kBwdCfgs[cfg];
-  if (c.persistent && (order == nullptr || next_tile == nullptr)) return cudaErrorInvalidValue;
-  const int nt = d / kTile, ntiles = nt * nt * B;
-  dim3 grid(nt * nt, B);
-  const uint32_t *ord = nullptr;
-  unsigned *ctr = nullptr;
-  if (c.persistent) {
-    if (order_ready) {
-      const cudaError_t e = cudaMemsetAsync(next_tile, 0, sizeof(unsigned), st);
-      if (e != cudaSuccess) return e;
-    } else {
-      tile_order_kernel<<<1, 1024, 0, st>>>(tile_start, ntiles, order, next_tile);
-    }
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    grid = dim3((unsigned)max(1, min(ntiles, sms * c.ctas)), 1);
-    ord = order;
-    ctr = next_tile;
+  if (!fresh) {  // the tasks stand; only the backward's counter starts again
+    const cudaError_t e = cudaMemsetAsync(tk.ctr + kCtrBwd, 0, sizeof(unsigned), st);
+    if (e != cudaSuccess) return e;
   }
-  if (c.lanes == 2 && c.per == 8)
-    launch_bwd_lanes<2, 8>(grid, rec, list, tile_start, cap, M, d, l2tau, dproj, mom, ord,
-                           ntiles, ctr, st);
-  else if (c.lanes == 2)
-    launch_bwd_lanes<2, 4>(grid, rec, list, tile_start, cap, M, d, l2tau, dproj, mom, ord,
-                           ntiles, ctr, st);
-
-  else if (c.per == 2)
-    launch_bwd_lanes<1, 2>(grid, rec, list, tile_start, cap, M, d, l2tau, dproj, mom, ord,
-                           ntiles, ctr, st);
+  const int grid = sm_count() * c.ctas, nt = d / kTile, ntiles = nt * nt * B;
+  if (c.per == 8 && c.ctas == 6)
+    raster_bwd_kernel<8, 6><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tile_start, ntiles, dproj, mom, tk);
   else if (c.per == 8)
-    launch_bwd_lanes<1, 8>(grid, rec, list, tile_start, cap, M, d, l2tau, dproj, mom, ord,
-                           ntiles, ctr, st);
+    raster_bwd_kernel<8, 5><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tile_start, ntiles, dproj, mom, tk);
+  else if (c.ctas >= 7)
+    raster_bwd_kernel<4, 8><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tile_start, ntiles, dproj, mom, tk);
   else
-    launch_bwd_lanes<1, 4>(grid, rec, list, tile_start, cap, M, d, l2tau, dproj, mom, ord,
-                           ntiles, ctr, st);
+    raster_bwd_kernel<4, 6><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tile_start, ntiles, dproj, mom, tk);
   return cudaGetLastError();
 }
 
