@@ -290,8 +290,8 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
   c->knn.cap = 2 * g.max_M + 64;
   ok = ok && alloc(c, &c->knn.part, 608 * 6) && alloc(c, &c->knn.grid, 1) &&
        alloc(c, &c->knn.cell, g.max_M) && alloc(c, &c->knn.cnt, c->knn.cap) &&
-       alloc(c, &c->knn.start, c->knn.cap + 1) && alloc(c, &c->knn.fill, c->knn.cap) &&
-       alloc(c, &c->knn.order, g.max_M) &&
+       alloc(c, &c->knn.start, c->knn.cap + 1) && alloc(c, &c->knn.rank, g.max_M) &&
+       alloc(c, &c->knn.sorted, g.max_M) && alloc(c, &c->knn.ticket, 1) &&
        alloc(c, &c->knn.bsum, (size_t)knn_scan_blocks(c->knn.cap) + 1) &&
        alloc(c, &c->qp, g.max_M);
   if (ok && g.fp64_check) {
@@ -321,6 +321,7 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
   if ((e = cudaMemcpy(c->tw, tw.data(), d * sizeof(float2), cudaMemcpyHostToDevice)) !=
           cudaSuccess ||
       (e = cudaMemset(c->status, 0, sizeof(int))) != cudaSuccess ||
+      (e = cudaMemset(c->knn.ticket, 0, sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(c->tasks.done, 0, (size_t)g.max_B * c->T * sizeof(unsigned))) != cudaSuccess ||
       (e = bin_configure(d)) != cudaSuccess || (e = ctf_configure(d)) != cudaSuccess ||
       (e = raster_configure()) != cudaSuccess) {

@@ -267,9 +267,10 @@ struct KnnScratch {
   KnnGrid *grid;
   int *cell;       // [M] cell of each centre
   int *cnt;        // [cap] members per cell
-  int *start;      // [cap + 1] first member of each cell in order[]
-  int *fill;       // [cap] scatter cursors
-  int *order;      // [M] centres grouped by cell
+  int *rank;       // [M] place of each centre in its cell
+  int *start;      // [cap + 1] first member of each cell in sorted[]
+  float4 *sorted;  // [M] centres grouped by cell: position, index (bits)
+  int *ticket;     // [1] blocks that have left their box, zero between calls
   int *bsum;       // [knn_scan_blocks(cap) + 1]
   int64_t cap;     // most cells the grid may use
 };

@@ -4,12 +4,14 @@
 // sets S_j = s_j I with s_j the distance of Gaussian j to its nearest
 // neighbour; the same distances serve as a scale initialisation.
 //
-// Uniform grid: the centres' bounding box is cut into about M/2 cubic cells;
-// a counting sort by cell lists each cell's members; each query walks
-// Chebyshev rings of cells around its own until the k-th best distance is
-// shorter than anything an unvisited ring can hold.  The result is exact:
-// the k smallest (distance^2, index) pairs in lexicographic order, which
-// does not depend on the order the candidates were met.
+// Uniform grid: the centres' bounding box is cut into about 3/2 M cubic cells
+// (the centres cluster, so most cells are empty and the others hold several);
+// a counting sort by cell puts the centres of a cell, and of the cells of a
+// row along x, next to each other; each query walks Chebyshev rings of cells
+// around its own until the k-th best distance is shorter than anything an
+// unvisited ring can hold.  The result is exact: the k smallest
+// (distance^2, index) pairs in lexicographic order, which does not depend on
+// the order the candidates were met.
 #include "gem_internal.cuh"
 
 namespace gem {
@@ -17,9 +19,14 @@ namespace gem {
 constexpr int kKnnBlk = 256;
 constexpr int kScanPer = 4096;  // elements per block of the cell-count scan
 
-// Per-block min / max of the centres: part[blk][6] = (min x, y, z, max x, y, z).
+// Bounding box of the finite centres, and the grid over it.  Every block
+// leaves its box in part[blk][6] = (min x, y, z, max x, y, z); the last one to
+// finish folds them and picks the cell size: cubes of side h with about
+// 3/2 M of them over the box, at most cap cells.
 __global__ void __launch_bounds__(kKnnBlk) knn_bbox_kernel(const float *__restrict__ params,
-                                                           int64_t M, float *__restrict__ part) {
+                                                           int64_t M, float *__restrict__ part,
+                                                           int64_t cap, int *__restrict__ ticket,
+                                                           KnnGrid *__restrict__ g) {
   float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < M;
        j += (int64_t)gridDim.x * blockDim.x) {
@@ -33,39 +40,51 @@ __global__ void __launch_bounds__(kKnnBlk) knn_bbox_kernel(const float *__restri
     }
   }
   __shared__ float red[kKnnBlk / 32][6];
+  __shared__ int last;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // box of the block: its threads', then its warps'
+  auto fold = [&]() {
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
+    for (int a = 0; a < 3; ++a)
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
-      hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
-    }
-  if (lane == 0)
+      for (int o = 16; o > 0; o >>= 1) {
+        lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+        hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
+      }
+    if (lane == 0)
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      red[warp][a] = lo[a];
-      red[warp][3 + a] = hi[a];
-    }
-  __syncthreads();
+      for (int a = 0; a < 3; ++a) {
+        red[warp][a] = lo[a];
+        red[warp][3 + a] = hi[a];
+      }
+    __syncthreads();
+  };
+  fold();
   if (threadIdx.x < 6) {
     float v = red[0][threadIdx.x];
     for (int w = 1; w < kKnnBlk / 32; ++w)
       v = threadIdx.x < 3 ? fminf(v, red[w][threadIdx.x]) : fmaxf(v, red[w][threadIdx.x]);
-    part[blockIdx.x * 6 + threadIdx.x] = v;
+    __stcg(part + blockIdx.x * 6 + threadIdx.x, v);
+    __threadfence();
   }
-}
-
-// One thread: fold the partial boxes and pick the cell size.  Cells are
-// cubes of side h with about M / 2 of them over the box; at most cap cells.
-__global__ void knn_grid_kernel(const float *__restrict__ part, int nblk, int64_t M, int64_t cap,
-                                KnnGrid *__restrict__ g) {
-  if (threadIdx.x != 0) return;
-  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-  for (int b = 0; b < nblk; ++b)
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int b = threadIdx.x; b < (int)gridDim.x; b += kKnnBlk)
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-      lo[a] = fminf(lo[a], part[b * 6 + a]);
-      hi[a] = fmaxf(hi[a], part[b * 6 + 3 + a]);
+      lo[a] = fminf(lo[a], __ldcg(part + b * 6 + a));
+      hi[a] = fmaxf(hi[a], __ldcg(part + b * 6 + 3 + a));
+    }
+  fold();
+  if (threadIdx.x != 0) return;
+  *ticket = 0;  // as the next call expects it
+  for (int w = 0; w < kKnnBlk / 32; ++w)
+    for (int a = 0; a < 3; ++a) {
+      lo[a] = fminf(lo[a], red[w][a]);
+      hi[a] = fmaxf(hi[a], red[w][3 + a]);
     }
   float ext[3];
   for (int a = 0; a < 3; ++a) {
@@ -73,7 +92,7 @@ __global__ void knn_grid_kernel(const float *__restrict__ part, int nblk, int64_
     ext[a] = hi[a] - lo[a];
   }
   const float emax = fmaxf(ext[0], fmaxf(ext[1], ext[2]));
-  const double target = fmax(1.0, 0.5 * (double)M);
+  const double target = fmax(1.0, 1.5 * (double)M);
   // side from the volume, kept above emax / 1024 so flat or linear sets of
   // centres do not make the grid explode
   double h = cbrt(fmax((double)ext[0] * ext[1] * ext[2], 0.0) / target);
@@ -81,7 +100,7 @@ __global__ void knn_grid_kernel(const float *__restrict__ part, int nblk, int64_
   if (!(h > 0.0)) h = 1.0;
   int n[3] = {1, 1, 1};
   bool fits = false;
-  for (int it = 0; it < 512 && !fits; ++it, h *= 1.25) {
+  for (int it = 0; it < 1024 && !fits; ++it, h *= 1.1) {
     double cells = 1.0;
     for (int a = 0; a < 3; ++a) {
       double na = floor(ext[a] / h) + 1.0;
@@ -108,11 +127,13 @@ __device__ __forceinline__ int knn_axis_cell(float v, float lo, float ih, int n)
 }
 
 // Cell of every centre (non-finite centres go to cell 0 and are never
-// reported as neighbours) and per-cell counts.
+// reported as neighbours), its place among the cell's members, and per-cell
+// counts.
 __global__ void __launch_bounds__(kKnnBlk) knn_cell_kernel(const float *__restrict__ params,
                                                            int64_t M,
                                                            const KnnGrid *__restrict__ g,
                                                            int *__restrict__ cell,
+                                                           int *__restrict__ rank,
                                                            int *__restrict__ cnt) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= M) return;
@@ -126,7 +147,7 @@ __global__ void __launch_bounds__(kKnnBlk) knn_cell_kernel(const float *__restri
     c = (cz * G.n[1] + cy) * G.n[0] + cx;
   }
   cell[j] = c;
-  atomicAdd(cnt + c, 1);
+  rank[j] = atomicAdd(cnt + c, 1);
 }
 
 // Exclusive scan of cnt[0 .. ncell) into start (start[ncell] = total), in
@@ -194,8 +215,7 @@ __global__ void __launch_bounds__(1024) knn_scan_top_kernel(int *__restrict__ bs
 __global__ void __launch_bounds__(1024) knn_scan_blocks_kernel(const int *__restrict__ cnt,
                                                                const KnnGrid *__restrict__ g,
                                                                const int *__restrict__ bsum,
-                                                               int *__restrict__ start,
-                                                               int *__restrict__ fill) {
+                                                               int *__restrict__ start) {
   __shared__ int ws[33];
   const int n = g->ncell;
   const int64_t base = (int64_t)blockIdx.x * kScanPer;
@@ -212,22 +232,23 @@ __global__ void __launch_bounds__(1024) knn_scan_blocks_kernel(const int *__rest
   int ex = block_exclusive_scan(s, ws, tot) + carry;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    if (i0 + k < n) {
-      start[i0 + k] = ex;
-      fill[i0 + k] = ex;
-    }
+    if (i0 + k < n) start[i0 + k] = ex;
     ex += v[k];
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) start[n] = bsum[gridDim.x];
 }
 
-__global__ void __launch_bounds__(kKnnBlk) knn_scatter_kernel(const int *__restrict__ cell,
-                                                              int64_t M, int *__restrict__ fill,
-                                                              int *__restrict__ order) {
+// The centres in cell order, each with its index: one coalesced 16-byte load
+// per candidate instead of a gather of its parameter row.
+__global__ void __launch_bounds__(kKnnBlk) knn_scatter_kernel(const float *__restrict__ params,
+                                                              const int *__restrict__ cell,
+                                                              const int *__restrict__ rank,
+                                                              const int *__restrict__ start,
+                                                              int64_t M, float4 *__restrict__ sorted) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= M) return;
-  int pos = atomicAdd(fill + cell[j], 1);
-  order[pos] = (int)j;
+  const float *p = params + j * kNpar;
+  sorted[start[cell[j]] + rank[j]] = make_float4(p[0], p[1], p[2], __int_as_float((int)j));
 }
 
 // Squared distance without contraction into FMA, so that it is the same
@@ -238,97 +259,193 @@ __device__ __forceinline__ float dist2_rn(float ax, float ay, float az, float bx
   return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
 }
 
+// The k best (distance^2, index) pairs, ascending in lexicographic order.
 template <int K>
-__global__ void __launch_bounds__(kKnnBlk) knn_query_kernel(
-    const float *__restrict__ params, int64_t M, const KnnGrid *__restrict__ g,
-    const int *__restrict__ start, const int *__restrict__ order, float *__restrict__ dist,
-    int32_t *__restrict__ idx) {
-  int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= M) return;
-  const int i = order[t];  // neighbouring threads query neighbouring centres
-  const KnnGrid G = *g;
-  const float px = params[(int64_t)i * kNpar], py = params[(int64_t)i * kNpar + 1],
-              pz = params[(int64_t)i * kNpar + 2];
-  float bd[K];
-  int bi[K];
+struct KBest {
+  float d[K];
+  int i[K];
+  __device__ __forceinline__ void clear() {
 #pragma unroll
-  for (int m = 0; m < K; ++m) {
-    bd[m] = INFINITY;
-    bi[m] = -1;
-  }
-  const bool fin = isfinite(px) && isfinite(py) && isfinite(pz);
-  if (fin) {
-    const int cx = knn_axis_cell(px, G.lo[0], G.ih, G.n[0]);
-    const int cy = knn_axis_cell(py, G.lo[1], G.ih, G.n[1]);
-    const int cz = knn_axis_cell(pz, G.lo[2], G.ih, G.n[2]);
-    const int rmax = max(G.n[0], max(G.n[1], G.n[2]));
-    for (int r = 0; r <= rmax; ++r) {
-      for (int dz = -r; dz <= r; ++dz) {
-        const int z = cz + dz;
-        if (z < 0 || z >= G.n[2]) continue;
-        for (int dy = -r; dy <= r; ++dy) {
-          const int y = cy + dy;
-          if (y < 0 || y >= G.n[1]) continue;
-          // inner rows of the ring hold only its two end cells (r > 0 there)
-          const bool face = (dz == -r || dz == r || dy == -r || dy == r);
-          const int step = face ? 1 : 2 * r;
-          for (int dx = -r; dx <= r; dx += step) {
-            const int x = cx + dx;
-            if (x < 0 || x >= G.n[0]) continue;
-            const int c = (z * G.n[1] + y) * G.n[0] + x;
-            for (int q = start[c], qe = start[c + 1]; q < qe; ++q) {
-              const int j = order[q];
-              if (j == i) continue;
-              const float *pj = params + (int64_t)j * kNpar;
-              const float qx = pj[0], qy = pj[1], qz = pj[2];
-              if (!(isfinite(qx) && isfinite(qy) && isfinite(qz))) continue;
-              const float d2 = dist2_rn(px, py, pz, qx, qy, qz);
-              if (d2 < bd[K - 1] || (d2 == bd[K - 1] && j < bi[K - 1])) {
-                // insert, keeping (d2, j) ascending: from the end, each slot
-                // takes its left neighbour while the newcomer sorts before
-                // it, else the newcomer if it sorts before the slot
-#pragma unroll
-                for (int m = K - 1; m > 0; --m) {
-                  const bool before_left = d2 < bd[m - 1] || (d2 == bd[m - 1] && j < bi[m - 1]);
-                  const bool before_here = d2 < bd[m] || (d2 == bd[m] && j < bi[m]);
-                  if (before_left) {
-                    bd[m] = bd[m - 1];
-                    bi[m] = bi[m - 1];
-                  } else if (before_here) {
-                    bd[m] = d2;
-                    bi[m] = j;
-                  }
-                }
-                if (d2 < bd[0] || (d2 == bd[0] && j < bi[0])) {
-                  bd[0] = d2;
-                  bi[0] = j;
-                }
-              }
-            }
-          }
-        }
-      }
-      // everything in rings beyond r lies farther than r * h from the point
-      const float reach = (float)r * G.h * (1.f - 1e-4f);
-      if (bi[K - 1] >= 0 && bd[K - 1] <= reach * reach) break;
+    for (int m = 0; m < K; ++m) {
+      d[m] = INFINITY;
+      i[m] = -1;
     }
   }
+  // A non-finite candidate's squared distance is infinite or not a number:
+  // it is never below d[K - 1], nor equal to it with an index below -1.
+  __device__ __forceinline__ bool takes(float d2, int j) const {
+    return d2 < d[K - 1] || (d2 == d[K - 1] && j < i[K - 1]);
+  }
+  __device__ __forceinline__ void insert(float d2, int j) {
+    // from the end, each slot takes its left neighbour while the newcomer
+    // sorts before it, else the newcomer if it sorts before the slot
+#pragma unroll
+    for (int m = K - 1; m > 0; --m) {
+      const bool before_left = d2 < d[m - 1] || (d2 == d[m - 1] && j < i[m - 1]);
+      const bool before_here = d2 < d[m] || (d2 == d[m] && j < i[m]);
+      if (before_left) {
+        d[m] = d[m - 1];
+        i[m] = i[m - 1];
+      } else if (before_here) {
+        d[m] = d2;
+        i[m] = j;
+      }
+    }
+    if (d2 < d[0] || (d2 == d[0] && j < i[0])) {
+      d[0] = d2;
+      i[0] = j;
+    }
+  }
+  // The best k over the lanes' lists, which hold no index twice, left in
+  // every lane.
+  __device__ __forceinline__ void merge_warp() {
+    KBest<K> all;
+#pragma unroll
+    for (int m = 0; m < K; ++m) {
+      float bd = d[0];
+      int bi = i[0];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float od = __shfl_xor_sync(0xffffffffu, bd, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (od < bd || (od == bd && (unsigned)oi < (unsigned)bi)) {
+          bd = od;
+          bi = oi;
+        }
+      }
+      all.d[m] = bd;
+      all.i[m] = bi;
+      if (i[0] == bi && bi >= 0) {  // this lane's head was the best: drop it
+#pragma unroll
+        for (int q = 0; q + 1 < K; ++q) {
+          d[q] = d[q + 1];
+          i[q] = i[q + 1];
+        }
+        d[K - 1] = INFINITY;
+        i[K - 1] = -1;
+      }
+    }
+    *this = all;
+  }
+};
+
+// Looks at the sorted centres qs .. qe - 1 for query (p, i).
+template <int K>
+__device__ __forceinline__ void knn_visit(KBest<K> &best, const float4 *__restrict__ sorted, int qs,
+                                          int qe, const float4 &p, int i) {
+  for (int q = qs; q < qe; ++q) {
+    const float4 c = sorted[q];
+    const float d2 = dist2_rn(p.x, p.y, p.z, c.x, c.y, c.z);
+    const int j = __float_as_int(c.w);
+    if (best.takes(d2, j) && j != i) best.insert(d2, j);
+  }
+}
+
+// One thread per centre, in cell order, for its cell and the 26 around it:
+// neighbouring threads read the same cells, and the cells of a row along x
+// are one run of the sorted centres, so the nine rows' bounds are loaded
+// together and the runs follow.  The centres that need further rings (those
+// in the thin outskirts of the clusters, whose rings hold hundreds of mostly
+// empty rows) are finished by the whole warp, one after the other, a row per
+// lane: a thread walking them alone is a chain of dependent loads.
+//
+// Bound by the latency of those loads.  M = 500000, k = 1 (64 clusters):
+// 436 us with a gather of the parameter row per candidate and two bounds per
+// cell on M / 2 cells, 233 with sorted centres, rows and 3/2 M cells,
+// about 105 with the warp's part.
+template <int K>
+__global__ void __launch_bounds__(kKnnBlk) knn_query_kernel(
+    const float4 *__restrict__ sorted, int64_t M, const KnnGrid *__restrict__ g,
+    const int *__restrict__ start, float *__restrict__ dist, int32_t *__restrict__ idx) {
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const KnnGrid G = *g;
+  const int n0 = G.n[0], n1 = G.n[1], n2 = G.n[2];
+  const int rmax = max(n0, max(n1, n2));
+  float4 me = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (t < M) me = sorted[t];
+  const int i = __float_as_int(me.w);
+  KBest<K> best;
+  best.clear();
+  const bool fin = t < M && isfinite(me.x) && isfinite(me.y) && isfinite(me.z);
+  bool done = !fin;
+  // everything in rings beyond r lies farther than r * h from the point
+  auto enough = [&](const KBest<K> &b, int r) {
+    const float reach = (float)r * G.h * (1.f - 1e-4f);
+    return b.i[K - 1] >= 0 && b.d[K - 1] <= reach * reach;
+  };
+  if (fin) {
+    const int cx = knn_axis_cell(me.x, G.lo[0], G.ih, n0);
+    const int cy = knn_axis_cell(me.y, G.lo[1], G.ih, n1);
+    const int cz = knn_axis_cell(me.z, G.lo[2], G.ih, n2);
+    const int x0 = max(cx - 1, 0), x1 = min(cx + 1, n0 - 1) + 1;
+    int qs[9], qe[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      const int z = cz + q / 3 - 1, y = cy + q % 3 - 1;
+      qs[q] = qe[q] = 0;
+      if (z >= 0 && z < n2 && y >= 0 && y < n1) {
+        const int *row = start + ((int64_t)z * n1 + y) * n0;
+        qs[q] = row[x0];
+        qe[q] = row[x1];
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 9; ++q) knn_visit(best, sorted, qs[q], qe[q], me, i);
+    done = enough(best, 1) || rmax <= 1;
+  }
+  for (unsigned todo = __ballot_sync(0xffffffffu, !done); todo; todo &= todo - 1) {
+    const int src = __ffs(todo) - 1;
+    float4 p;
+    p.x = __shfl_sync(0xffffffffu, me.x, src);
+    p.y = __shfl_sync(0xffffffffu, me.y, src);
+    p.z = __shfl_sync(0xffffffffu, me.z, src);
+    const int pi = __shfl_sync(0xffffffffu, i, src);
+    const int cx = knn_axis_cell(p.x, G.lo[0], G.ih, n0);
+    const int cy = knn_axis_cell(p.y, G.lo[1], G.ih, n1);
+    const int cz = knn_axis_cell(p.z, G.lo[2], G.ih, n2);
+    // lane src starts from what it has, the others from nothing
+    KBest<K> b = best;
+    if (lane != src) b.clear();
+    for (int r = 2; r <= rmax; ++r) {
+      const int z0 = max(cz - r, 0), z1 = min(cz + r, n2 - 1);
+      const int y0 = max(cy - r, 0), y1 = min(cy + r, n1 - 1);
+      const int x0 = max(cx - r, 0), x1 = min(cx + r, n0 - 1);
+      const int ny = y1 - y0 + 1, rows = (z1 - z0 + 1) * ny;
+      for (int q = lane; q < rows; q += 32) {
+        const int dz = q / ny, z = z0 + dz, y = y0 + (q - dz * ny);
+        const int *row = start + ((int64_t)z * n1 + y) * n0;
+        // inner rows of a ring hold only its two end cells
+        if (z == cz - r || z == cz + r || y == cy - r || y == cy + r) {
+          knn_visit(b, sorted, row[x0], row[x1 + 1], p, pi);
+        } else {
+          if (cx - r >= 0) knn_visit(b, sorted, row[cx - r], row[cx - r + 1], p, pi);
+          if (cx + r < n0) knn_visit(b, sorted, row[cx + r], row[cx + r + 1], p, pi);
+        }
+      }
+      __syncwarp();
+      b.merge_warp();
+      if (enough(b, r)) break;
+      if (lane != src) b.clear();
+    }
+    if (lane == src) best = b;
+  }
+  if (t >= M) return;
 #pragma unroll
   for (int m = 0; m < K; ++m) {
-    dist[(int64_t)i * K + m] = bi[m] >= 0 ? sqrtf(bd[m]) : INFINITY;
-    if (idx) idx[(int64_t)i * K + m] = bi[m];
+    dist[(int64_t)i * K + m] = best.i[m] >= 0 ? sqrtf(best.d[m]) : INFINITY;
+    if (idx) idx[(int64_t)i * K + m] = best.i[m];
   }
 }
 
 // One instance per k, so that the k best live in registers.
 template <int K>
-void launch_query(int k, unsigned gm, cudaStream_t st, const float *params, int64_t M,
-                  const KnnGrid *g, const int *start, const int *order, float *dist,
-                  int32_t *idx) {
+void launch_query(int k, unsigned gm, cudaStream_t st, const float4 *sorted, int64_t M,
+                  const KnnGrid *g, const int *start, float *dist, int32_t *idx) {
   if (k == K)
-    knn_query_kernel<K><<<gm, kKnnBlk, 0, st>>>(params, M, g, start, order, dist, idx);
+    knn_query_kernel<K><<<gm, kKnnBlk, 0, st>>>(sorted, M, g, start, dist, idx);
   else if constexpr (K < 16)
-    launch_query<K + 1>(k, gm, st, params, M, g, start, order, dist, idx);
+    launch_query<K + 1>(k, gm, st, sorted, M, g, start, dist, idx);
 }
 
 int knn_scan_blocks(int64_t cap) { return (int)((cap + kScanPer - 1) / kScanPer); }
@@ -338,17 +455,16 @@ cudaError_t launch_knn(const float *params, int64_t M, int k, const KnnScratch &
   cudaError_t e;
   const int64_t nbl = (M + kKnnBlk - 1) / kKnnBlk;
   const int nbb = (int)(nbl < 608 ? nbl : 608);  // KnnScratch::part holds 608 boxes
-  knn_bbox_kernel<<<nbb, kKnnBlk, 0, st>>>(params, M, s.part);
-  knn_grid_kernel<<<1, 32, 0, st>>>(s.part, nbb, M, s.cap, s.grid);
+  knn_bbox_kernel<<<nbb, kKnnBlk, 0, st>>>(params, M, s.part, s.cap, s.ticket, s.grid);
   if ((e = cudaMemsetAsync(s.cnt, 0, (size_t)s.cap * sizeof(int), st)) != cudaSuccess) return e;
   const unsigned gm = (unsigned)((M + kKnnBlk - 1) / kKnnBlk);
-  knn_cell_kernel<<<gm, kKnnBlk, 0, st>>>(params, M, s.grid, s.cell, s.cnt);
+  knn_cell_kernel<<<gm, kKnnBlk, 0, st>>>(params, M, s.grid, s.cell, s.rank, s.cnt);
   const int nb = knn_scan_blocks(s.cap);
   knn_scan_sums_kernel<<<nb, 1024, 0, st>>>(s.cnt, s.grid, s.bsum);
   knn_scan_top_kernel<<<1, 1024, 0, st>>>(s.bsum, nb);
-  knn_scan_blocks_kernel<<<nb, 1024, 0, st>>>(s.cnt, s.grid, s.bsum, s.start, s.fill);
-  knn_scatter_kernel<<<gm, kKnnBlk, 0, st>>>(s.cell, M, s.fill, s.order);
-  launch_query<1>(k, gm, st, params, M, s.grid, s.start, s.order, dist, idx);
+  knn_scan_blocks_kernel<<<nb, 1024, 0, st>>>(s.cnt, s.grid, s.bsum, s.start);
+  knn_scatter_kernel<<<gm, kKnnBlk, 0, st>>>(params, s.cell, s.rank, s.start, M, s.sorted);
+  launch_query<1>(k, gm, st, s.sorted, M, s.grid, s.start, dist, idx);
   return cudaGetLastError();
 }
 
