@@ -49,6 +49,7 @@ struct gem_ctx {
   unsigned long long *kept = nullptr;
   KnnScratch knn{};
   QueryPrep *qp = nullptr;
+  uint32_t *slice_range = nullptr, *nsel = nullptr;  // [max_M], [max_B]
   // FSC scratch, allocated by the first gem_fsc: two d^3 complex volumes
   float2 *fscP = nullptr, *fscQ = nullptr;
   double *fsc_part = nullptr;
@@ -293,7 +294,8 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
        alloc(c, &c->knn.start, c->knn.cap + 1) && alloc(c, &c->knn.rank, g.max_M) &&
        alloc(c, &c->knn.sorted, g.max_M) && alloc(c, &c->knn.ticket, 1) &&
        alloc(c, &c->knn.bsum, (size_t)knn_scan_blocks(c->knn.cap) + 1) &&
-       alloc(c, &c->qp, g.max_M);
+       alloc(c, &c->qp, g.max_M) && alloc(c, &c->slice_range, g.max_M) &&
+       alloc(c, &c->nsel, g.max_B) && alloc(c, &c->bin.tile_n, (size_t)g.max_B * c->T);
   if (ok && g.fp64_check) {
     const size_t n = (size_t)g.max_B * d * d;
     ok = f64_scratch(c) == GEM_OK && alloc(c, &c->f64.params_in, (size_t)g.max_M * kNpar) &&
@@ -712,17 +714,16 @@ int gem_query(gem_ctx *c, const float *params, int64_t M, float tau, float *vol)
   c->have_bins = false;
   const float l2tau = tau > 0.f ? log2f(tau) : -INFINITY;
   cudaError_t e;
-  if ((e = launch_query_prep(params, M, g.norm_mode, shape_flags(g), c->qp, c->stream)) !=
-      cudaSuccess)
+  if ((e = launch_query_prep(params, M, g.norm_mode, shape_flags(g), g.apix, g.d, l2tau, c->qp,
+                             c->slice_range, c->stream)) != cudaSuccess)
     return cuda_fail(c, e, "query prep");
   const size_t slice = (size_t)g.d * g.d;
   for (int k0 = 0; k0 < g.d; k0 += g.max_B) {
     const int ns = g.d - k0 < g.max_B ? g.d - k0 : g.max_B;
-    const uint32_t *perm = nullptr;
-    if ((e = launch_slice_prep(c->qp, M, k0, ns, g.apix, g.d, l2tau, c->rec, c->stream)) !=
-            cudaSuccess ||
-        (e = launch_bin(c->rec, c->bin.key, M, ns, g.d, l2tau, 0, c->bin, &perm, c->stream)) !=
-            cudaSuccess ||
+    if ((e = launch_slices(c->qp, c->slice_range, M, k0, ns, g.apix, g.d, l2tau, c->bin.tcnt, c->rec,
+                           c->bin.perm, c->nsel, c->stream)) != cudaSuccess ||
+        (e = launch_bin_selected(c->rec, c->bin.perm, c->nsel, M, ns, g.d, l2tau, c->bin,
+                                 c->stream)) != cudaSuccess ||
         (e = launch_raster_fwd(active_fwd(c, ns, M), c->rec, c->bin.list,
                                c->bin.tile_start, c->bin.cap, M, ns, g.d, l2tau,
                                vol + (size_t)k0 * slice, c->tasks, true, c->stream)) !=

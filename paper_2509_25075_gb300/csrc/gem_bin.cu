@@ -21,7 +21,6 @@ namespace gem {
 
 constexpr int kChunkD = 4096;   // elements per chunk, depth passes
 constexpr int kDThreads = 512;  // 16 warps x 256 elements
-constexpr int kChunkT = 256;    // Gaussians per chunk, tile binning
 
 size_t bin_chunks_depth(int64_t M) { return (size_t)((M + kChunkD - 1) / kChunkD); }
 size_t bin_chunks_tiles(int64_t M) { return (size_t)((M + kChunkT - 1) / kChunkT); }
@@ -331,13 +330,14 @@ struct SmallBox {
 
 __device__ __forceinline__ void stage_chunk(ChunkStage &S, const Rec *__restrict__ rec,
                                             const uint32_t *__restrict__ perm, int64_t M,
-                                            int b, int c, int d, float l2tau, SmallBox &sbx) {
+                                            int64_t nrank, int b, int c, int d, float l2tau,
+                                            SmallBox &sbx) {
   const int i = threadIdx.x, lane = i & 31, warp = i >> 5;
   const int64_t r = (int64_t)c * kChunkT + i;
   int ncand = 0, nrow = 0;
   unsigned packed = 0;
   sbx.w = 0;
-  if (r < M) {
+  if (r < nrank) {
     const uint32_t j = perm ? perm[(int64_t)b * M + r] : (uint32_t)r;
     const Rec rc = rec[(int64_t)b * M + j];
     S.geo[i] = make_row_geo(rc, l2tau);
@@ -456,19 +456,29 @@ __device__ __forceinline__ uint64_t pack_hit(int o, int t, unsigned mask) {
   return (uint64_t)o | ((uint64_t)t << 8) | ((uint64_t)mask << 24);
 }
 
+// kSel: image b holds only the nsel[b] Gaussians perm[b][0 .. nsel[b]), and a
+// CTA takes every gridDim.x-th of their chunks (the host does not know how
+// many there are); else every Gaussian, one chunk per CTA.
+template <bool kSel>
 __global__ void __launch_bounds__(kChunkT, 6) tile_count_kernel(
-    const Rec *__restrict__ rec, const uint32_t *__restrict__ perm, int64_t M, int d,
-    float l2tau, int nch, uint32_t *__restrict__ tcnt, BinScratch bs) {
+    const Rec *__restrict__ rec, const uint32_t *__restrict__ perm, int64_t M,
+    const uint32_t *__restrict__ nsel, int d, float l2tau, int nch, uint32_t *__restrict__ tcnt,
+    BinScratch bs) {
   extern __shared__ uint32_t tc[];
   __shared__ ChunkStage S;
   __shared__ int wh[kChunkT / 32];
   __shared__ int64_t run_base;
-  const int c = blockIdx.x, b = blockIdx.y;
+  int c = blockIdx.x;
+  const int b = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nt = d / kTile, T = nt * nt, nb = d / 4;
+  const int64_t nrank = kSel ? (int64_t)nsel[b] : M;
+  const int nc = kSel ? (int)((nrank + kChunkT - 1) / kChunkT) : nch;
+  if (kSel && c >= nc) return;
+  do {
   for (int i = threadIdx.x; i < T; i += blockDim.x) tc[i] = 0;
   SmallBox sbx;
-  stage_chunk(S, rec, perm, M, b, c, d, l2tau, sbx);
+  stage_chunk(S, rec, perm, M, nrank, b, c, d, l2tau, sbx);
   const int total = S.off[kChunkT], rows = S.roff[kChunkT];
   const bool staged = rows <= kRowCap;
   if (staged && rows > 0) {  // (rows is the chunk's: the barrier is uniform)
@@ -576,25 +586,29 @@ __global__ void __launch_bounds__(kChunkT, 6) tile_count_kernel(
   __syncthreads();
   uint32_t *out = tcnt + ((int64_t)b * nch + c) * T;
   for (int i = threadIdx.x; i < T; i += blockDim.x) out[i] = tc[i];
+  } while (kSel && (c += gridDim.x) < nc);
 }
 
 // Exclusive scan over the chunks of every (image, tile) column of
-// tcnt[b][c][t], in place; the column totals go to tile_n[b * T + t].  A
+// tcnt[b][c][t], in place; the column totals go to tile_n[b * T + t].  With
+// nsel, image b has only the chunks of nsel[b] Gaussians.  A
 // CTA takes 32 tiles of one image (one per lane, so every access reads 32
 // consecutive counts of a chunk row) and its 8 warps take 8 consecutive
 // ranges of chunks: a pass of range sums, their exclusive prefix across the
 // warps, then a pass that writes the prefix.
 constexpr int kScanWarps = 8;
 __global__ void __launch_bounds__(32 * kScanWarps) tile_scan_cols_kernel(
-    uint32_t *__restrict__ tcnt, int nch, int T, int64_t *__restrict__ tile_n) {
+    uint32_t *__restrict__ tcnt, int nch, int T, const uint32_t *__restrict__ nsel,
+    uint32_t *__restrict__ tile_n) {
   __shared__ uint32_t part[kScanWarps][32];
   const int b = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int t = blockIdx.x * 32 + lane;
   const bool act = t < T;
   uint32_t *col = tcnt + (int64_t)b * nch * T + t;
-  const int per = (nch + kScanWarps - 1) / kScanWarps;
-  const int c0 = min(nch, warp * per), c1 = min(nch, c0 + per);
+  const int nc = nsel ? (int)((nsel[b] + kChunkT - 1) / kChunkT) : nch;
+  const int per = (nc + kScanWarps - 1) / kScanWarps;
+  const int c0 = min(nc, warp * per), c1 = min(nc, c0 + per);
   // eight loads in flight per lane in both passes (the chunk walk is
   // otherwise one dependent load per step)
   constexpr int kU = 8;
@@ -635,58 +649,75 @@ __global__ void __launch_bounds__(32 * kScanWarps) tile_scan_cols_kernel(
   }
 }
 
-// In-place exclusive scan of n counts (one block of 1024), total in x[n].
-// Flags the capacity bit when the total exceeds cap.  Each round scans 4096
-// counts as four consecutive runs of 1024 (one per sub-round q), with one
-// set of barriers; every thread keeps the running carry itself.
-__global__ void __launch_bounds__(1024) scan_tiles_kernel(int64_t *__restrict__ x, int64_t n,
-                                                          int64_t cap, int *__restrict__ status,
+// Exclusive scan of n counts into x, the total in x[n]; flags the capacity
+// bit when it exceeds cap and resets the rasterisers' counters.  A block scans
+// `per` counts (a multiple of 1024) and adds up all the counts before its own
+// itself, so no block waits for another: up to 128 blocks of at least 1024
+// counts, whose re-reads stay in L2 (16384 counts: 13 us with one block
+// walking all of them).
+__global__ void __launch_bounds__(1024) scan_tiles_kernel(const uint32_t *__restrict__ cnt,
+                                                          int64_t *__restrict__ x, int64_t n,
+                                                          int64_t per, int64_t cap,
+                                                          int *__restrict__ status,
                                                           unsigned *__restrict__ task_ctr) {
-  constexpr int kQ = 4;
-  __shared__ int64_t wtot[kQ][32];  // per run: exclusive prefix of the warps' sums
-  __shared__ int64_t qtot[kQ];      // per run: its total
+  __shared__ int64_t wtot[32];
+  __shared__ int64_t sum_sh;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int64_t carry = 0;
-  for (int64_t base = 0; base < n; base += kQ * 1024) {
-    int64_t v[kQ], inc[kQ];
+  const int64_t i0 = (int64_t)blockIdx.x * per;
+  // the counts before this block's, four loads in flight per thread
+  int64_t before = 0;
+  {
+    int64_t i = threadIdx.x;
+    for (; i + 3 * 1024 < i0; i += 4 * 1024) {
+      uint32_t v[4];
 #pragma unroll
-    for (int q = 0; q < kQ; ++q) {
-      const int64_t i = base + q * 1024 + threadIdx.x;
-      v[q] = i < n ? x[i] : 0;
+      for (int u = 0; u < 4; ++u) v[u] = cnt[i + u * 1024];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) before += v[u];
     }
+    for (; i < i0; i += 1024) before += cnt[i];
 #pragma unroll
-    for (int q = 0; q < kQ; ++q) {
-      inc[q] = v[q];
+    for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+    if (lane == 0) wtot[warp] = before;
+    __syncthreads();
+    if (warp == 0) {
+      int64_t w = wtot[lane];
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int64_t u = __shfl_up_sync(0xffffffffu, inc[q], o);
-        if (lane >= o) inc[q] += u;
-      }
-      if (lane == 31) wtot[q][warp] = inc[q];
+      for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+      if (lane == 0) sum_sh = w;
     }
     __syncthreads();
-    if (warp < kQ) {
-      const int64_t w = wtot[warp][lane];
+  }
+  int64_t carry = sum_sh;
+  for (int64_t base = i0; base < min(n, i0 + per); base += 1024) {
+    const int64_t i = base + threadIdx.x;
+    const int64_t v = i < n ? (int64_t)cnt[i] : 0;
+    int64_t inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t u = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += u;
+    }
+    __syncthreads();  // wtot and sum_sh of the last round are read
+    if (lane == 31) wtot[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+      const int64_t w = wtot[lane];
       int64_t wi = w;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int64_t u = __shfl_up_sync(0xffffffffu, wi, o);
         if (lane >= o) wi += u;
       }
-      wtot[warp][lane] = wi - w;
-      if (lane == 31) qtot[warp] = wi;
+      wtot[lane] = wi - w;
+      if (lane == 31) sum_sh = wi;
     }
     __syncthreads();
-#pragma unroll
-    for (int q = 0; q < kQ; ++q) {
-      const int64_t i = base + q * 1024 + threadIdx.x;
-      if (i < n) x[i] = carry + wtot[q][warp] + inc[q] - v[q];
-      carry += qtot[q];
-    }
-    __syncthreads();  // wtot and qtot are read before the next round rewrites them
+    if (i < n) x[i] = carry + wtot[warp] + inc - v;
+    carry += sum_sh;
   }
-  if (threadIdx.x < kCtrCount) task_ctr[threadIdx.x] = 0u;
-  if (threadIdx.x == 0) {
+  if (blockIdx.x == 0 && threadIdx.x < kCtrCount) task_ctr[threadIdx.x] = 0u;
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
     x[n] = carry;
     if (carry > cap) atomicOr(status, kStatusCapacity);
   }
@@ -701,17 +732,23 @@ __global__ void __launch_bounds__(1024) scan_tiles_kernel(int64_t *__restrict__ 
 // touched: each hit clears its own tile's bitmap words first (a chunk hits
 // a few hundred of the image's tiles at most, and large images have
 // thousands), and looks up its own tile's list base.
+template <bool kSel>
 __global__ void __launch_bounds__(kChunkT) tile_scatter_kernel(
-    const uint32_t *__restrict__ perm, int64_t M, int d, int nch,
+    const uint32_t *__restrict__ perm, int64_t M, const uint32_t *__restrict__ nsel, int d, int nch,
     const uint32_t *__restrict__ tcnt, const int64_t *__restrict__ tile_start, BinScratch bs) {
   // bitmaps word-major, [8][T]: a warp's hits are mostly one Gaussian's
   // neighbouring tiles, which then fall in neighbouring banks
   extern __shared__ __align__(16) uint32_t bm[];
   __shared__ uint32_t sj[kChunkT];   // Gaussian index of each slot
-  const int c = blockIdx.x, b = blockIdx.y;
+  int c = blockIdx.x;
+  const int b = blockIdx.y;
   const int nt = d / kTile, T = nt * nt;
+  const int64_t nrank = kSel ? (int64_t)nsel[b] : M;
+  const int nc = kSel ? (int)((nrank + kChunkT - 1) / kChunkT) : nch;
+  if (kSel && c >= nc) return;
+  do {
   const int64_t r0 = (int64_t)c * kChunkT;
-  if (r0 + threadIdx.x < M)
+  if (r0 + threadIdx.x < nrank)
     sj[threadIdx.x] = perm ? perm[(int64_t)b * M + r0 + threadIdx.x] : (uint32_t)(r0 + threadIdx.x);
   // up to 1024 tiles (d <= 512) every bitmap word is cleared at once, while
   // the hits are still on their way; above that each hit clears its own
@@ -784,6 +821,8 @@ __global__ void __launch_bounds__(kChunkT) tile_scatter_kernel(
     const uint64_t h = hr[i];
     place(h, list_base(h));
   }
+  if (kSel) __syncthreads();  // the bitmaps and indices make way for the next chunk's
+  } while (kSel && (c += gridDim.x) < nc);
 }
 
 // Bitmaps (8 words per tile, word-major).
@@ -795,13 +834,17 @@ static int tile_smem_bytes(int d) {
 // The dynamic shared memory of both tile kernels (bitmaps, counters) is
 // declared for every image side, so that it never depends on what the
 // static part leaves of the default 48 KB.
-cudaError_t bin_configure(int d) {
-  const int smem = tile_smem_bytes(d);
-  cudaError_t e = cudaFuncSetAttribute(tile_scatter_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+template <bool kSel>
+static cudaError_t bin_configure_one(int d) {
+  const cudaError_t e = cudaFuncSetAttribute(
+      tile_scatter_kernel<kSel>, cudaFuncAttributeMaxDynamicSharedMemorySize, tile_smem_bytes(d));
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(tile_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(tile_count_kernel<kSel>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (d / kTile) * (d / kTile) * (int)sizeof(uint32_t));
+}
+cudaError_t bin_configure(int d) {
+  const cudaError_t e = bin_configure_one<false>(d);
+  return e != cudaSuccess ? e : bin_configure_one<true>(d);
 }
 
 cudaError_t launch_sort16(const uint16_t *key, int64_t M, int B, uint32_t *dcnt,
@@ -832,29 +875,53 @@ cudaError_t launch_map_slots(const uint2 *list, const uint32_t *slot_gauss, int6
   return cudaGetLastError();
 }
 
+cudaError_t launch_scan_cols(uint32_t *tcnt, int nch, int T, int B, const uint32_t *nsel,
+                             uint32_t *tile_n, cudaStream_t st) {
+  tile_scan_cols_kernel<<<dim3((unsigned)((T + 31) / 32), (unsigned)B), 32 * kScanWarps, 0, st>>>(
+      tcnt, nch, T, nsel, tile_n);
+  return cudaGetLastError();
+}
+
+// The tile pass: count, scans, scatter.
+template <bool kSel>
+static cudaError_t launch_tiles(const Rec *rec, const uint32_t *perm, const uint32_t *nsel, int64_t M,
+                                int B, int d, float l2tau, BinScratch &s, cudaStream_t st) {
+  cudaError_t e;
+  const int nt = d / kTile, T = nt * nt;
+  const int nch = (int)bin_chunks_tiles(M);
+  // selected Gaussians: a grid of a few waves whose CTAs walk the chunks (an
+  // image's share of a slice batch is a twentieth of the Gaussians or less)
+  dim3 g(kSel ? min(nch, max(64, 4096 / B)) : nch, B);
+  const int cnt_smem = T * (int)sizeof(uint32_t);
+  if ((e = cudaMemsetAsync(s.hit_ctr, 0, sizeof(unsigned long long), st)) != cudaSuccess) return e;
+  tile_count_kernel<kSel><<<g, 256, cnt_smem, st>>>(rec, perm, M, nsel, d, l2tau, nch, s.tcnt, s);
+  const int64_t n = (int64_t)B * T;
+  if ((e = launch_scan_cols(s.tcnt, nch, T, B, nsel, s.tile_n, st)) != cudaSuccess) return e;
+  const int64_t blocks = min((n + 1023) / 1024, (int64_t)128);
+  const int64_t per = ((n + blocks - 1) / blocks + 1023) / 1024 * 1024;
+  scan_tiles_kernel<<<(unsigned)((n + per - 1) / per), 1024, 0, st>>>(s.tile_n, s.tile_start, n, per,
+                                                                      s.cap, s.status, s.task_ctr);
+  tile_scatter_kernel<kSel><<<g, 256, tile_smem_bytes(d), st>>>(perm, M, nsel, d, nch, s.tcnt,
+                                                                s.tile_start, s);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_bin(const Rec *rec, const uint16_t *key, int64_t M, int B, int d,
                        float l2tau, int zsort, BinScratch &s, const uint32_t **perm_out,
                        cudaStream_t st) {
-  cudaError_t e;
   const uint32_t *perm = nullptr;
   if (zsort) {
-    if ((e = launch_sort16(key, M, B, s.dcnt, s.packed, s.perm, st)) != cudaSuccess) return e;
+    const cudaError_t e = launch_sort16(key, M, B, s.dcnt, s.packed, s.perm, st);
+    if (e != cudaSuccess) return e;
     perm = s.perm;
   }
-  int nt = d / kTile, T = nt * nt;
-  int nch = (int)bin_chunks_tiles(M);
-  dim3 g(nch, B);
-  int cnt_smem = T * (int)sizeof(uint32_t);
-  if ((e = cudaMemsetAsync(s.hit_ctr, 0, sizeof(unsigned long long), st)) != cudaSuccess) return e;
-  tile_count_kernel<<<g, 256, cnt_smem, st>>>(rec, perm, M, d, l2tau, nch, s.tcnt, s);
-  int64_t ncols = (int64_t)B * T;
-  tile_scan_cols_kernel<<<dim3((unsigned)((T + 31) / 32), (unsigned)B), 32 * kScanWarps, 0, st>>>(
-      s.tcnt, nch, T, s.tile_start);
-  scan_tiles_kernel<<<1, 1024, 0, st>>>(s.tile_start, ncols, s.cap, s.status, s.task_ctr);
-  tile_scatter_kernel<<<g, 256, tile_smem_bytes(d), st>>>(perm, M, d, nch, s.tcnt, s.tile_start, s);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
   *perm_out = perm;
-  return cudaSuccess;
+  return launch_tiles<false>(rec, perm, nullptr, M, B, d, l2tau, s, st);
+}
+
+cudaError_t launch_bin_selected(const Rec *rec, const uint32_t *sel, const uint32_t *nsel, int64_t M,
+                                int B, int d, float l2tau, BinScratch &s, cudaStream_t st) {
+  return launch_tiles<true>(rec, sel, nsel, M, B, d, l2tau, s, st);
 }
 
 }  // namespace gem

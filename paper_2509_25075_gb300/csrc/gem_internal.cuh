@@ -217,10 +217,16 @@ struct __align__(16) QueryPrep {
   float valid;
   float pdet;  // det of the xy block of Sigma^-1 (1/Angstrom^4), by Cauchy-Binet
 };
-cudaError_t launch_query_prep(const float *params, int64_t M, int norm_mode, int shape,
-                              QueryPrep *qp, cudaStream_t st);
-cudaError_t launch_slice_prep(const QueryPrep *qp, int64_t M, int k0, int nslice, float apix,
-                              int d, float l2tau, Rec *rec, cudaStream_t st);
+// range [M]: the slices where a Gaussian can exceed tau, first | last << 16
+// (first > last: none).
+cudaError_t launch_query_prep(const float *params, int64_t M, int norm_mode, int shape, float apix,
+                              int d, float l2tau, QueryPrep *qp, uint32_t *range, cudaStream_t st);
+// Records of the slices k0 .. k0 + nslice - 1 for the Gaussians that can
+// exceed tau there: rec[b][j], their indices in ascending order sel[b][..],
+// their number nsel[b].  cnt [chunks][nslice] is scratch.
+cudaError_t launch_slices(const QueryPrep *qp, const uint32_t *range, int64_t M, int k0, int nslice,
+                          float apix, int d, float l2tau, uint32_t *cnt, Rec *rec, uint32_t *sel,
+                          uint32_t *nsel, cudaStream_t st);
 
 // gem_f64.cu (FP64 check mode)
 struct G64 {
@@ -285,6 +291,7 @@ struct BinScratch {
   uint32_t *perm;          // [B][M] Gaussian indices in depth order
   uint32_t *dcnt;          // [B][nchD][256]
   uint32_t *tcnt;          // [B][nchT][T] per chunk: hits per tile, then offsets
+  uint32_t *tile_n;        // [B*T] list lengths
   int64_t *tile_start;     // [B*T + 1]
   uint2 *list;             // [cap] entries: x = Gaussian index, y = 4x4-block mask (16 bits)
   uint64_t *hits;          // [cap] (slot in chunk, tile, 4x4-block mask) of every hit,
@@ -309,6 +316,15 @@ cudaError_t launch_map_slots(const uint2 *list, const uint32_t *slot_gauss, int6
 cudaError_t launch_bin(const Rec *rec, const uint16_t *key, int64_t M, int B, int d,
                        float l2tau, int zsort, BinScratch &s, const uint32_t **perm_out,
                        cudaStream_t st);
+// The same for images that hold only some Gaussians: image b the nsel[b]
+// (device) Gaussians sel[b][0 .. nsel[b]), row stride M, in list order.
+cudaError_t launch_bin_selected(const Rec *rec, const uint32_t *sel, const uint32_t *nsel, int64_t M,
+                                int B, int d, float l2tau, BinScratch &s, cudaStream_t st);
+// Exclusive scan over the nch rows c of each column of tcnt[b][c][t], in
+// place; the column totals go to tile_n[b * T + t].
+cudaError_t launch_scan_cols(uint32_t *tcnt, int nch, int T, int B, const uint32_t *nsel,
+                             uint32_t *tile_n, cudaStream_t st);
+constexpr int kChunkT = 256;  // Gaussians per chunk of the tile pass
 size_t bin_chunks_depth(int64_t M);
 size_t bin_chunks_tiles(int64_t M);
 cudaError_t bin_configure(int d);

@@ -10,13 +10,22 @@
 // so the slice record has conic P_aa, centre m(z_k) and log2 amplitude
 // log2 A3 - (log2 e / 2) (z_k - p_z)^2 / Sigma_zz.  Slices are independent
 // "images" and run in batches of the context's max_B.
+//
+// A Gaussian exceeds tau in a dozen slices, so each slice gets the list of
+// the Gaussians that can matter there (their range of slices is known once
+// the threshold is), and only those get a record and enter the binning.  With
+// a record of every Gaussian in every slice, the records and the count pass
+// over them were 60% of a query (d 256, M 100000, batches of 64 slices:
+// 1.27 ms; 0.49 ms now).
 #include "gem_internal.cuh"
 
 namespace gem {
 
 __global__ void __launch_bounds__(256) query_prep_kernel(const float *__restrict__ params,
                                                          int64_t M, int norm_mode, int shape,
-                                                         QueryPrep *__restrict__ qp) {
+                                                         float apix, int d, float l2tau,
+                                                         QueryPrep *__restrict__ qp,
+                                                         uint32_t *__restrict__ range) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= M) return;
   const float *th = params + j * kNpar;
@@ -64,17 +73,22 @@ __global__ void __launch_bounds__(256) query_prep_kernel(const float *__restrict
                   isfinite(o.p[2]) && a0 > 0.f && a1 > 0.f && a2 > 0.f;
   o.valid = ok ? 1.f : 0.f;
   qp[j] = o;
+  // headroom l2A - (log2 e / 2) dz^2 hz > l2tau, widened by far more than the
+  // rounding of either side; the record's own test stays exact
+  unsigned r = 1u;  // none
+  const float head = o.l2A - l2tau;
+  if (ok && head > 0.f) {
+    const float D = sqrtf(head * (2.f / kLog2e) / o.hz) / apix * (1.f + 1e-4f) + 0.05f;
+    const float c = o.p[2] / apix + 0.5f * d;
+    const float lo = fmaxf(ceilf(c - D), 0.f), hi = fminf(floorf(c + D), (float)(d - 1));
+    if (lo <= hi) r = (unsigned)lo | ((unsigned)hi << 16);
+  }
+  range[j] = r;
 }
 
-// Record of (slice k0 + blockIdx.y, Gaussian j), in the layout of Rec.
-__global__ void __launch_bounds__(256) slice_prep_kernel(const QueryPrep *__restrict__ qp,
-                                                         int64_t M, int k0, float apix, int d,
-                                                         float l2tau, Rec *__restrict__ rec) {
-  int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int b = blockIdx.y;
-  if (j >= M) return;
-  const QueryPrep g = qp[j];
-  const float z = ((float)(k0 + b) - 0.5f * d) * apix;
+// Record of (slice k, Gaussian g), in the layout of Rec.
+__device__ __forceinline__ Rec slice_record(const QueryPrep &g, int k, float apix, int d, float l2tau) {
+  const float z = ((float)k - 0.5f * d) * apix;
   const float dz = z - g.p[2];
   const float inv = 1.f / apix;
   const float px = fmaf(fmaf(g.mx, dz, g.p[0]), inv, 0.5f * d);
@@ -102,19 +116,78 @@ __global__ void __launch_bounds__(256) slice_prep_kernel(const QueryPrep *__rest
     r.a = make_float4(px, py, 0.f, 0.f);
     r.b = make_float4(0.f, -INFINITY, -1.f, -1.f);
   }
-  rec[(int64_t)b * M + j] = r;
+  return r;
 }
 
-cudaError_t launch_query_prep(const float *params, int64_t M, int norm_mode, int shape,
-                              QueryPrep *qp, cudaStream_t st) {
-  query_prep_kernel<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(params, M, norm_mode, shape, qp);
+// Which Gaussians of chunk blockIdx.x (256 of them) meet which slices of the
+// batch: one bit per Gaussian, bm[slice][8].
+__device__ __forceinline__ void slice_bits(uint32_t *bm, const uint32_t *__restrict__ range, int64_t M,
+                                           int k0, int ns, int &lo, int &hi) {
+  const int64_t j = (int64_t)blockIdx.x * kChunkT + threadIdx.x;
+  const unsigned r = j < M ? range[j] : 1u;
+  lo = max((int)(r & 0xffffu) - k0, 0);
+  hi = min((int)(r >> 16) - k0, ns - 1);
+  if ((r & 0xffffu) > (r >> 16)) hi = lo - 1;
+  for (int q = threadIdx.x; q < 8 * ns; q += kChunkT) bm[q] = 0u;
+  __syncthreads();
+  for (int k = lo; k <= hi; ++k) atomicOr(&bm[8 * k + (threadIdx.x >> 5)], 1u << (threadIdx.x & 31));
+  __syncthreads();
+}
+
+// How many Gaussians of each chunk meet each slice: cnt[chunk][ns].
+__global__ void __launch_bounds__(kChunkT) slice_count_kernel(const uint32_t *__restrict__ range,
+                                                              int64_t M, int k0, int ns,
+                                                              uint32_t *__restrict__ cnt) {
+  extern __shared__ uint32_t bm[];
+  int lo, hi;
+  slice_bits(bm, range, M, k0, ns, lo, hi);
+  for (int k = threadIdx.x; k < ns; k += kChunkT) {
+    uint32_t n = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) n += __popc(bm[8 * k + w]);
+    cnt[(int64_t)blockIdx.x * ns + k] = n;
+  }
+}
+
+// The records and the lists, off[chunk][ns] (exclusive prefix over the
+// chunks) saying where each chunk's Gaussians go in a slice's list.
+__global__ void __launch_bounds__(kChunkT) slice_write_kernel(
+    const QueryPrep *__restrict__ qp, const uint32_t *__restrict__ range, int64_t M, int k0, int ns,
+    float apix, int d, float l2tau, const uint32_t *__restrict__ off, Rec *__restrict__ rec,
+    uint32_t *__restrict__ sel) {
+  extern __shared__ uint32_t bm[];
+  int lo, hi;
+  slice_bits(bm, range, M, k0, ns, lo, hi);
+  if (lo > hi) return;
+  const int64_t j = (int64_t)blockIdx.x * kChunkT + threadIdx.x;
+  const QueryPrep g = qp[j];
+  const int word = threadIdx.x >> 5;
+  const uint32_t below = (1u << (threadIdx.x & 31)) - 1u;
+  for (int k = lo; k <= hi; ++k) {
+    uint32_t pos = off[(int64_t)blockIdx.x * ns + k] + __popc(bm[8 * k + word] & below);
+    for (int w = 0; w < word; ++w) pos += __popc(bm[8 * k + w]);
+    sel[(int64_t)k * M + pos] = (uint32_t)j;
+    rec[(int64_t)k * M + j] = slice_record(g, k0 + k, apix, d, l2tau);
+  }
+}
+
+cudaError_t launch_query_prep(const float *params, int64_t M, int norm_mode, int shape, float apix,
+                              int d, float l2tau, QueryPrep *qp, uint32_t *range, cudaStream_t st) {
+  query_prep_kernel<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(params, M, norm_mode, shape, apix, d,
+                                                                 l2tau, qp, range);
   return cudaGetLastError();
 }
 
-cudaError_t launch_slice_prep(const QueryPrep *qp, int64_t M, int k0, int nslice, float apix,
-                              int d, float l2tau, Rec *rec, cudaStream_t st) {
-  dim3 grid((unsigned)((M + 255) / 256), (unsigned)nslice);
-  slice_prep_kernel<<<grid, 256, 0, st>>>(qp, M, k0, apix, d, l2tau, rec);
+cudaError_t launch_slices(const QueryPrep *qp, const uint32_t *range, int64_t M, int k0, int nslice,
+                          float apix, int d, float l2tau, uint32_t *cnt, Rec *rec, uint32_t *sel,
+                          uint32_t *nsel, cudaStream_t st) {
+  const int nch = (int)bin_chunks_tiles(M);
+  const size_t smem = (size_t)nslice * 8 * sizeof(uint32_t);  // at most 24 KB (768 slices)
+  slice_count_kernel<<<nch, kChunkT, smem, st>>>(range, M, k0, nslice, cnt);
+  const cudaError_t e = launch_scan_cols(cnt, nch, nslice, 1, nullptr, nsel, st);
+  if (e != cudaSuccess) return e;
+  slice_write_kernel<<<nch, kChunkT, smem, st>>>(qp, range, M, k0, nslice, apix, d, l2tau, cnt, rec,
+                                                 sel);
   return cudaGetLastError();
 }
 
