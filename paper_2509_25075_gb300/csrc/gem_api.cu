@@ -26,7 +26,6 @@ struct gem_ctx {
   char err[512] = {0};
   int T = 0;
   float l2tau = 0.f;
-  FftPlan plan{};
   // scratch
   GaussPrep *gp = nullptr;       // [max_M] by slot
   Rec *rec = nullptr;            // [max_B][max_M] by view, slot
@@ -260,7 +259,6 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
   const int d = g.d;
   c->T = (d / kTile) * (d / kTile);
   c->l2tau = g.tau > 0.f ? log2f(g.tau) : -INFINITY;
-  fft_plan(d, c->plan);
   const size_t BM = (size_t)g.max_B * (size_t)g.max_M;
   const size_t nchD = bin_chunks_depth(g.max_M), nchT = bin_chunks_tiles(g.max_M);
   c->nbg = g.max_B < 16 ? g.max_B : 16;
@@ -474,7 +472,7 @@ int gem_ctf_loss(gem_ctx *c, int32_t B, const float *proj, const float *ctf,
   if (B < 1 || B > c->cfg.max_B)
     return fail(c, GEM_EINVAL, "B=%d outside 1..max_B=%d", B, c->cfg.max_B);
   StageScope sc(c, GEM_STAGE_CTF, 3 + (loss_img || loss ? 1 : 0) + (loss ? 1 : 0));
-  cudaError_t e = launch_ctf_loss(c->cfg.d, B, c->cfg.apix, c->plan, c->tw, proj, ctf,
+  cudaError_t e = launch_ctf_loss(c->cfg.d, B, c->cfg.apix, c->tw, proj, ctf,
                                   ctf_params, images, c->Z, c->lossp, pred, dproj, loss_img,
                                   loss, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "ctf_loss");
@@ -753,7 +751,7 @@ int gem_fsc(gem_ctx *c, const float *map1, const float *map2, float threshold, d
     cudaError_t e = fsc_configure(d);
     if (e != cudaSuccess) return cuda_fail(c, e, "fsc configure");
   }
-  cudaError_t e = launch_fsc(d, c->cfg.apix, threshold, c->plan, c->tw, map1, map2, c->fscP,
+  cudaError_t e = launch_fsc(d, c->cfg.apix, threshold, c->tw, map1, map2, c->fscP,
                              c->fscQ, c->fsc_part, fsc, sums, resolution, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "fsc");
   return GEM_OK;

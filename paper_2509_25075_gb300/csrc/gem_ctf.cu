@@ -21,7 +21,13 @@
 //           of line 0's pair), CTF, loss, W, inverse FFT along y, written
 //           back in place;
 //   pass 3: inverse FFT along x of kLines rows, split into I_pred and dL/dI^.
-// FFTs are radix-4/2/3 Stockham transforms in shared memory (d = 2^a 3^b).
+// FFTs are radix-4/2/3 Stockham transforms (gem_fft.cuh), instantiated for
+// every side.
+//
+// Bound by latency (two or three barriers per pass and the reads of the
+// spectrum, which stays in L2).  Against a shared-memory round trip per radix
+// stage and separate copies in and out, same arithmetic and bits: d 144, B 50,
+// transfer arrays, every output: the call 51.7 -> 34.8 us.
 #include <math.h>
 
 #include "gem_fft.cuh"
@@ -29,72 +35,35 @@
 
 namespace gem {
 
-bool fft_plan(int n, FftPlan &p) {
-  p.n = n;
-  p.nst = 0;
-  p.code = 0;
-  int m = n;
-  auto push = [&](unsigned c) {
-    p.code |= c << (2 * p.nst);
-    ++p.nst;
-  };
-  while (m % 3 == 0 && p.nst < 16) {
-    push(1);
-    m /= 3;
-  }
-  while (m % 4 == 0 && p.nst < 16) {
-    push(2);
-    m /= 4;
-  }
-  if (m % 2 == 0 && p.nst < 16) {
-    push(0);
-    m /= 2;
-  }
-  return m == 1;
-}
-
-// Lines per CTA in every pass (kLines, a template parameter): 16 where two
-// line buffers of 16 lines leave room for four CTAs per SM, else 8 (large
-// images: more, smaller CTAs, so the last wave is short).
+// Lines per CTA in every pass: 16 where two line buffers of 16 lines would
+// leave room for four CTAs per SM (sides up to 208), else 8 (large images:
+// more, smaller CTAs, so the last wave is short).
 constexpr int kCtfThreads = 256;
+__host__ __device__ constexpr int ctf_lines(int d) { return d <= 208 ? 16 : 8; }
 
-// line stride in shared memory: one element of padding per line
-__host__ __device__ constexpr int ctf_ls(int d) { return d + 1; }
-static size_t ctf_smem(int lines, int d) {
-  return (size_t)(2 * lines * ctf_ls(d) + d) * sizeof(float2);
-}
-static int ctf_lines(int d) { return ctf_smem(16, d) <= 56 * 1024 ? 16 : 8; }
+template <int N>
+struct CtfSmem {
+  float2 lines[ctf_lines(N) * fft_stride(N)];
+  float2 tw[N];
+};
 
-__device__ __forceinline__ void load_twiddles(float2 *tw_s, const float2 *__restrict__ tw,
-                                              int n) {
-  for (int i = threadIdx.x; i < n; i += blockDim.x) tw_s[i] = tw[i];
-}
-
-// pass 1: rows y0 .. y0 + kLines - 1 of z = proj + i images -> FFT along x -> Z[b][kx][y]
-template <int kLines>
+// pass 1: rows y0 .. y0 + L - 1 of z = proj + i images -> FFT along x -> Z[b][kx][y]
+template <int N>
 __global__ void __launch_bounds__(kCtfThreads) ctf_pass1_kernel(
-    const float *__restrict__ proj, const float *__restrict__ images, FftPlan pl,
+    const float *__restrict__ proj, const float *__restrict__ images,
     const float2 *__restrict__ tw, float2 *__restrict__ Z) {
-  extern __shared__ float2 sm[];
-  const int d = pl.n;
-  const int ls = ctf_ls(d);
-  float2 *a = sm, *bb = sm + kLines * ls, *tws = sm + 2 * kLines * ls;
-  const int y0 = blockIdx.x * kLines, b = blockIdx.y;
-  load_twiddles(tws, tw, d);
-  const float *pr = proj + ((int64_t)b * d + y0) * d;
-  const float *im = images + ((int64_t)b * d + y0) * d;
-  const float rd = 1.f / (float)d;
-  for (int i = threadIdx.x; i < kLines * d; i += blockDim.x) {
-    const int l = fdiv_small(i, rd), x = i - l * d;
-    a[l * ls + x] = make_float2(pr[i], im[i]);
-  }
+  constexpr int L = ctf_lines(N);
+  extern __shared__ __align__(16) unsigned char ctf_sm[];
+  CtfSmem<N> &S = *reinterpret_cast<CtfSmem<N> *>(ctf_sm);
+  const int y0 = blockIdx.x * L, b = blockIdx.y;
+  load_twiddles<N, kCtfThreads>(S.tw, tw);
   __syncthreads();
-  float2 *res = fft_lines(a, bb, kLines, pl, tws, ls);
-  float2 *zb = Z + (int64_t)b * d * d;
-  for (int i = threadIdx.x; i < kLines * d; i += blockDim.x) {
-    int l = i % kLines, kx = i / kLines;
-    zb[(int64_t)kx * d + y0 + l] = res[l * ls + kx];
-  }
+  const float *pr = proj + ((int64_t)b * N + y0) * N;
+  const float *im = images + ((int64_t)b * N + y0) * N;
+  float2 *zb = Z + (int64_t)b * N * N + y0;
+  fft_lines<N, L, kCtfThreads, false, false, false, true>(
+      [&](int l, int x) { return make_float2(pr[l * N + x], im[l * N + x]); },
+      [&](int l, int kx, float2 v) { zb[kx * N + l] = v; }, S.lines, S.tw);
 }
 
 // A float-float number hi + lo (|lo| <= ulp(hi) / 2).
@@ -203,44 +172,39 @@ __device__ __forceinline__ int pass2_line(int blk, int i, int d) {
 // pass 2: slots i < kHalf hold the lines kx1 = kHalf c + i (kx1 < d/2),
 // slots kHalf + i their partners d - kx1; line 0 is its own partner, so its
 // slot kHalf holds the other self-paired line, d/2.  d is a multiple of
-// kLines, so the d / kLines CTAs of an image hold every line once.
-template <int kLines>
+// the line count, so the d / L CTAs of an image hold every line once.
+template <int N>
 __global__ void __launch_bounds__(kCtfThreads) ctf_pass2_kernel(
-    FftPlan pl, const float2 *__restrict__ tw, const float *__restrict__ ctf,
+    const float2 *__restrict__ tw, const float *__restrict__ ctf,
     const float *__restrict__ ctf_params, float apix, float2 *__restrict__ Z,
     double *__restrict__ lossp, int nblk) {
-  constexpr int kHalf = kLines / 2;  // line pairs per CTA
-  extern __shared__ float2 sm[];
+  constexpr int kLines = ctf_lines(N), kHalf = kLines / 2;  // line pairs per CTA
+  constexpr int d = N, hd = N / 2, ls = fft_stride(N);
+  extern __shared__ __align__(16) unsigned char ctf_sm[];
+  CtfSmem<N> &S = *reinterpret_cast<CtfSmem<N> *>(ctf_sm);
   __shared__ CtfConst cc;
   __shared__ double red[kCtfThreads / 32];
-  const int d = pl.n, hd = d / 2;
-  const int ls = ctf_ls(d);
-  float2 *a = sm, *bb = sm + kLines * ls, *tws = sm + 2 * kLines * ls;
   const int blk = blockIdx.x, b = blockIdx.y;
-  load_twiddles(tws, tw, d);
+  load_twiddles<N, kCtfThreads>(S.tw, tw);
   if (ctf_params && threadIdx.x == 0) cc = ctf_const(ctf_params + 8 * b, d, apix);
   float2 *zb = Z + (int64_t)b * d * d;
-  const float rd = 1.f / (float)d;
-  // load the kLines lines
-  for (int idx = threadIdx.x; idx < kLines * d; idx += blockDim.x) {
-    const int i = fdiv_small(idx, rd), y = idx - i * d;
-    a[i * ls + y] = zb[(int64_t)pass2_line<kHalf>(blk, i, d) * d + y];
-  }
   __syncthreads();
-  float2 *L = fft_lines(a, bb, kLines, pl, tws, ls);
+  float2 *L = S.lines;
+  fft_lines<N, kLines, kCtfThreads, false, true, false, false>(
+      [&](int i, int y) { return zb[pass2_line<kHalf>(blk, i, d) * d + y]; }, FftNone{}, L, S.tw);
   // combine: thread per (pair i, ky); the first CTA has one more "pair",
   // the self-paired line d/2 in slot kHalf
   float lsum = 0.f;
   const int npair = blk == 0 ? kHalf + 1 : kHalf;
   for (int idx = threadIdx.x; idx < npair * d; idx += blockDim.x) {
-    int i = fdiv_small(idx, rd), ky = idx - i * d;
+    int i = idx / d, ky = idx - i * d;
     int kx = i < kHalf ? kHalf * blk + i : hd;
     bool self = (kx == 0 || kx == hd);
     if (self && ky > hd) continue;
     int mky = ky == 0 ? 0 : d - ky;
     float2 *l1 = L + i * ls;
     float2 *l2 = self ? l1 : L + (kHalf + i) * ls;
-    float2 z1 = l1[ky], z2 = l2[mky];
+    float2 z1 = l1[fft_at(ky)], z2 = l2[fft_at(mky)];
     // X = (z1 + conj z2) / 2,  Y = (z1 - conj z2) / (2 i)
     float2 X = make_float2(0.5f * (z1.x + z2.x), 0.5f * (z1.y - z2.y));
     float2 Yv = make_float2(0.5f * (z1.y + z2.y), -0.5f * (z1.x - z2.x));
@@ -267,8 +231,8 @@ __global__ void __launch_bounds__(kCtfThreads) ctf_pass2_kernel(
     // inverse transform runs as conj(FFT(conj .)).
     float2 W = make_float2(P.x - G.y, P.y + G.x);
     float2 Wm = make_float2(P.x + G.y, -P.y + G.x);
-    l1[ky] = make_float2(W.x, -W.y);
-    l2[mky] = make_float2(Wm.x, -Wm.y);
+    l1[fft_at(ky)] = make_float2(W.x, -W.y);
+    l2[fft_at(mky)] = make_float2(Wm.x, -Wm.y);
   }
   // block reduction of the loss partial in float64
   double lw = (double)lsum;
@@ -281,43 +245,38 @@ __global__ void __launch_bounds__(kCtfThreads) ctf_pass2_kernel(
     lossp[(int64_t)b * nblk + blk] = s;
   }
   // inverse along y (conjugated forward transform)
-  float2 *other = (L == a) ? bb : a;
-  float2 *R2 = fft_lines(L, other, kLines, pl, tws, ls);
-  for (int idx = threadIdx.x; idx < kLines * d; idx += blockDim.x) {
-    const int i = fdiv_small(idx, rd), y = idx - i * d;
-    const float2 v = R2[i * ls + y];
-    zb[(int64_t)pass2_line<kHalf>(blk, i, d) * d + y] = make_float2(v.x, -v.y);
-  }
+  fft_lines<N, kLines, kCtfThreads, true, false, false, false>(
+      FftNone{},
+      [&](int i, int y, float2 v) {
+        zb[pass2_line<kHalf>(blk, i, d) * d + y] = make_float2(v.x, -v.y);
+      },
+      L, S.tw);
 }
 
-// pass 3: rows y0 .. y0 + kLines - 1 of W (read transposed) -> inverse FFT along x ->
+// pass 3: rows y0 .. y0 + L - 1 of W (read transposed) -> inverse FFT along x ->
 // I_pred = Re / d^2, dL/dI^ = Im (2 / (B d^2)) / d^2.
-template <int kLines>
+template <int N>
 __global__ void __launch_bounds__(kCtfThreads) ctf_pass3_kernel(
-    FftPlan pl, const float2 *__restrict__ tw, const float2 *__restrict__ Z, float inv_n2,
+    const float2 *__restrict__ tw, const float2 *__restrict__ Z, float inv_n2,
     float gscale, float *__restrict__ pred, float *__restrict__ dproj) {
-  extern __shared__ float2 sm[];
-  const int d = pl.n;
-  const int ls = ctf_ls(d);
-  float2 *a = sm, *bb = sm + kLines * ls, *tws = sm + 2 * kLines * ls;
-  const int y0 = blockIdx.x * kLines, b = blockIdx.y;
-  load_twiddles(tws, tw, d);
-  const float2 *zb = Z + (int64_t)b * d * d;
-  for (int i = threadIdx.x; i < kLines * d; i += blockDim.x) {
-    int l = i % kLines, kx = i / kLines;
-    float2 v = zb[(int64_t)kx * d + y0 + l];
-    a[l * ls + kx] = make_float2(v.x, -v.y);
-  }
+  constexpr int L = ctf_lines(N);
+  extern __shared__ __align__(16) unsigned char ctf_sm[];
+  CtfSmem<N> &S = *reinterpret_cast<CtfSmem<N> *>(ctf_sm);
+  const int y0 = blockIdx.x * L, b = blockIdx.y;
+  load_twiddles<N, kCtfThreads>(S.tw, tw);
   __syncthreads();
-  float2 *res = fft_lines(a, bb, kLines, pl, tws, ls);
-  int64_t off = ((int64_t)b * d + y0) * d;
-  const float rd = 1.f / (float)d;
-  for (int i = threadIdx.x; i < kLines * d; i += blockDim.x) {
-    const int l = fdiv_small(i, rd), x = i - l * d;
-    float2 v = res[l * ls + x];
-    if (pred) pred[off + i] = v.x * inv_n2;
-    if (dproj) dproj[off + i] = -v.y * gscale;
-  }
+  const float2 *zb = Z + (int64_t)b * N * N + y0;
+  const int64_t off = ((int64_t)b * N + y0) * N;
+  fft_lines<N, L, kCtfThreads, false, false, true, false>(
+      [&](int l, int kx) {
+        const float2 v = zb[kx * N + l];
+        return make_float2(v.x, -v.y);
+      },
+      [&](int l, int x, float2 v) {
+        if (pred) pred[off + l * N + x] = v.x * inv_n2;
+        if (dproj) dproj[off + l * N + x] = -v.y * gscale;
+      },
+      S.lines, S.tw);
 }
 
 // loss_img[b] = sum of image b's partials / d^4 (one warp per image, fixed
@@ -350,52 +309,58 @@ __global__ void __launch_bounds__(256) loss_mean_kernel(const double *__restrict
 
 size_t ctf_partials(int d) { return (size_t)(d / ctf_lines(d)); }
 
-template <int kLines>
-static cudaError_t ctf_configure_lines(int d) {
-  int smem = (int)ctf_smem(kLines, d);
+template <int N>
+static cudaError_t ctf_configure_side() {
+  const int smem = (int)sizeof(CtfSmem<N>);
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(ctf_pass1_kernel<kLines>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+  if ((e = cudaFuncSetAttribute(ctf_pass1_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                smem)) != cudaSuccess)
     return e;
-  if ((e = cudaFuncSetAttribute(ctf_pass2_kernel<kLines>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
+  if ((e = cudaFuncSetAttribute(ctf_pass2_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                smem)) != cudaSuccess)
     return e;
-  return cudaFuncSetAttribute(ctf_pass3_kernel<kLines>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  return cudaFuncSetAttribute(ctf_pass3_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 cudaError_t ctf_configure(int d) {
-  return ctf_lines(d) == 16 ? ctf_configure_lines<16>(d) : ctf_configure_lines<8>(d);
+  switch (d) {
+#define X(N) \
+  case N:    \
+    return ctf_configure_side<N>();
+    GEM_FFT_SIDES(X)
+#undef X
+  }
+  return cudaErrorInvalidValue;
 }
 
-template <int kLines>
-static void launch_ctf_passes(int d, int B, float apix, const FftPlan &plan, const float2 *tw,
-                              const float *proj, const float *ctf, const float *ctf_params,
-                              const float *images, float2 *Z, double *lossp, float *pred,
-                              float *dproj, cudaStream_t st) {
-  const size_t smem = ctf_smem(kLines, d);
-  const int nblk = d / kLines;
-  const float cscale = (float)(2.0 / ((double)B * d * d));
-  ctf_pass1_kernel<kLines><<<dim3(d / kLines, B), kCtfThreads, smem, st>>>(proj, images, plan, tw,
-                                                                           Z);
-  ctf_pass2_kernel<kLines><<<dim3(nblk, B), kCtfThreads, smem, st>>>(plan, tw, ctf, ctf_params,
-                                                                     apix, Z, lossp, nblk);
-  ctf_pass3_kernel<kLines><<<dim3(d / kLines, B), kCtfThreads, smem, st>>>(
-      plan, tw, Z, (float)(1.0 / ((double)d * d)), (float)(cscale / ((double)d * d)), pred,
-      dproj);
+template <int N>
+static void launch_ctf_passes(int B, float apix, const float2 *tw, const float *proj,
+                              const float *ctf, const float *ctf_params, const float *images,
+                              float2 *Z, double *lossp, float *pred, float *dproj, cudaStream_t st) {
+  const size_t smem = sizeof(CtfSmem<N>);
+  const dim3 grid(N / ctf_lines(N), B);
+  const float cscale = (float)(2.0 / ((double)B * N * N));
+  ctf_pass1_kernel<N><<<grid, kCtfThreads, smem, st>>>(proj, images, tw, Z);
+  ctf_pass2_kernel<N><<<grid, kCtfThreads, smem, st>>>(tw, ctf, ctf_params, apix, Z, lossp, grid.x);
+  ctf_pass3_kernel<N><<<grid, kCtfThreads, smem, st>>>(tw, Z, (float)(1.0 / ((double)N * N)),
+                                                       (float)(cscale / ((double)N * N)), pred, dproj);
 }
 
-cudaError_t launch_ctf_loss(int d, int B, float apix, const FftPlan &plan, const float2 *tw,
+cudaError_t launch_ctf_loss(int d, int B, float apix, const float2 *tw,
                             const float *proj, const float *ctf, const float *ctf_params,
                             const float *images, float2 *Z, double *lossp, float *pred,
                             float *dproj, double *loss_img, double *loss, cudaStream_t st) {
   const int nblk = (int)ctf_partials(d);
-  if (ctf_lines(d) == 16)
-    launch_ctf_passes<16>(d, B, apix, plan, tw, proj, ctf, ctf_params, images, Z, lossp, pred,
-                          dproj, st);
-  else
-    launch_ctf_passes<8>(d, B, apix, plan, tw, proj, ctf, ctf_params, images, Z, lossp, pred,
-                         dproj, st);
+  switch (d) {
+#define X(N)                                                                                        \
+  case N:                                                                                           \
+    launch_ctf_passes<N>(B, apix, tw, proj, ctf, ctf_params, images, Z, lossp, pred, dproj, st);    \
+    break;
+    GEM_FFT_SIDES(X)
+#undef X
+    default:
+      return cudaErrorInvalidValue;
+  }
   if (loss_img || loss) {
     // per-image losses land in loss_img, or after the partials when the
     // caller does not want them (lossp holds max_B * nblk + max_B doubles)

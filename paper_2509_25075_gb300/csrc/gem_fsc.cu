@@ -11,6 +11,9 @@
 // in shared memory, each along the contiguous axis, each writing its output
 // with the axes rotated so the next axis becomes contiguous:
 //   [z][y][x] -> [kx][z][y] -> [ky][kx][z] -> [kz][ky][kx].
+// Each pass reads and writes the volume once; its stages meet shared memory
+// once or twice (gem_fft.cuh).  Same bits as a round trip per stage: two
+// 256^3 maps 664 -> 292 us.
 #include <math.h>
 
 #include "gem_fft.cuh"
@@ -18,60 +21,56 @@
 
 namespace gem {
 
-constexpr int kFL = 16;  // lines per CTA
 constexpr int kFThreads = 256;
 constexpr int kShellBlocks = 608;  // 4 per SM on 152 SMs
+// Lines per CTA of the transform passes: 16 (their transposed stores then
+// fill 128-byte lines) up to sides whose 16 lines leave room for four CTAs
+// per SM, else 8.
+__host__ __device__ constexpr int fsc_lines(int d) { return d <= 384 ? 16 : 8; }
 
-// shared-memory lines padded by one element (conflict-free column access)
-static size_t fsc_smem(int d) { return (size_t)(2 * kFL * (d + 1) + d) * sizeof(float2); }
+template <int N>
+struct FscSmem {
+  float2 lines[fsc_lines(N) * fft_stride(N)];
+  float2 tw[N];
+};
 
-// x pass: rows y0 .. y0+15 of slab z of z = X1 + i X2, FFT along x, written
-// as A[kx][z][y].
+// x pass: rows y0 .. y0 + L - 1 of slab z of z = X1 + i X2, FFT along x,
+// written as A[kx][z][y].
+template <int N>
 __global__ void __launch_bounds__(kFThreads) fsc_pass_real_kernel(
-    const float *__restrict__ X1, const float *__restrict__ X2, FftPlan pl,
-    const float2 *__restrict__ tw, float2 *__restrict__ A) {
-  extern __shared__ float2 sm[];
-  const int d = pl.n;
-  const int ls = d + 1;
-  float2 *a = sm, *bb = sm + kFL * ls, *tws = sm + 2 * kFL * ls;
-  const int y0 = blockIdx.x * kFL, z = blockIdx.y;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) tws[i] = tw[i];
-  const int64_t base = ((int64_t)z * d + y0) * d;
-  for (int i = threadIdx.x; i < kFL * d; i += blockDim.x) {
-    const int l = fdiv_small(i, 1.f / (float)d), x = i - l * d;
-    a[l * ls + x] = make_float2(X1[base + i], X2[base + i]);
-  }
+    const float *__restrict__ X1, const float *__restrict__ X2, const float2 *__restrict__ tw,
+    float2 *__restrict__ A) {
+  constexpr int L = fsc_lines(N);
+  extern __shared__ __align__(16) unsigned char fsc_sm[];
+  FscSmem<N> &S = *reinterpret_cast<FscSmem<N> *>(fsc_sm);
+  const int y0 = blockIdx.x * L, z = blockIdx.y;
+  load_twiddles<N, kFThreads>(S.tw, tw);
   __syncthreads();
-  const float2 *res = fft_lines(a, bb, kFL, pl, tws, ls);
-  for (int i = threadIdx.x; i < kFL * d; i += blockDim.x) {
-    const int l = i % kFL, k = i / kFL;
-    A[((int64_t)k * d + z) * d + y0 + l] = res[l * ls + k];
-  }
+  const int64_t base = ((int64_t)z * N + y0) * N;
+  const float *x1 = X1 + base, *x2 = X2 + base;
+  float2 *out = A + (int64_t)z * N + y0;
+  fft_lines<N, L, kFThreads, false, false, false, true>(
+      [&](int l, int x) { return make_float2(x1[l * N + x], x2[l * N + x]); },
+      [&](int l, int k, float2 v) { out[k * (N * N) + l] = v; }, S.lines, S.tw);
 }
 
 // Complex pass: B[k][i0][i1] = FFT along i2 of A[i0][i1][:], lines
-// i1 = i1_0 .. i1_0 + 15 of slab i0.
+// i1 = i1_0 .. i1_0 + L - 1 of slab i0.
+template <int N>
 __global__ void __launch_bounds__(kFThreads) fsc_pass_cplx_kernel(const float2 *__restrict__ A,
-                                                                  FftPlan pl,
                                                                   const float2 *__restrict__ tw,
                                                                   float2 *__restrict__ Bo) {
-  extern __shared__ float2 sm[];
-  const int d = pl.n;
-  const int ls = d + 1;
-  float2 *a = sm, *bb = sm + kFL * ls, *tws = sm + 2 * kFL * ls;
-  const int i10 = blockIdx.x * kFL, i0 = blockIdx.y;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) tws[i] = tw[i];
-  const int64_t base = ((int64_t)i0 * d + i10) * d;
-  for (int i = threadIdx.x; i < kFL * d; i += blockDim.x) {
-    const int l = fdiv_small(i, 1.f / (float)d), x = i - l * d;
-    a[l * ls + x] = A[base + i];
-  }
+  constexpr int L = fsc_lines(N);
+  extern __shared__ __align__(16) unsigned char fsc_sm[];
+  FscSmem<N> &S = *reinterpret_cast<FscSmem<N> *>(fsc_sm);
+  const int i10 = blockIdx.x * L, i0 = blockIdx.y;
+  load_twiddles<N, kFThreads>(S.tw, tw);
   __syncthreads();
-  const float2 *res = fft_lines(a, bb, kFL, pl, tws, ls);
-  for (int i = threadIdx.x; i < kFL * d; i += blockDim.x) {
-    const int l = i % kFL, k = i / kFL;
-    Bo[((int64_t)k * d + i0) * d + i10 + l] = res[l * ls + k];
-  }
+  const float2 *in = A + ((int64_t)i0 * N + i10) * N;
+  float2 *out = Bo + (int64_t)i0 * N + i10;
+  fft_lines<N, L, kFThreads, false, false, false, true>(
+      [&](int l, int x) { return in[l * N + x]; },
+      [&](int l, int k, float2 v) { out[k * (N * N) + l] = v; }, S.lines, S.tw);
 }
 
 // Shell of a frequency with squared norm k2: the integer s with
@@ -212,26 +211,53 @@ __global__ void __launch_bounds__(512) fsc_final_kernel(const double *__restrict
   }
 }
 
-cudaError_t fsc_configure(int d) {
-  const size_t smem = fsc_smem(d);
-  cudaError_t e = cudaFuncSetAttribute(fsc_pass_real_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int N>
+static cudaError_t fsc_configure_side() {
+  const int smem = (int)sizeof(FscSmem<N>);
+  const cudaError_t e = cudaFuncSetAttribute(fsc_pass_real_kernel<N>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(fsc_pass_cplx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)smem);
+  return cudaFuncSetAttribute(fsc_pass_cplx_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              smem);
+}
+
+cudaError_t fsc_configure(int d) {
+  switch (d) {
+#define X(N) \
+  case N:    \
+    return fsc_configure_side<N>();
+    GEM_FFT_SIDES(X)
+#undef X
+  }
+  return cudaErrorInvalidValue;
+}
+
+template <int N>
+static void launch_fsc_passes(const float2 *tw, const float *X1, const float *X2, float2 *P, float2 *Q,
+                              cudaStream_t st) {
+  const size_t smem = sizeof(FscSmem<N>);
+  const dim3 g(N / fsc_lines(N), N);
+  fsc_pass_real_kernel<N><<<g, kFThreads, smem, st>>>(X1, X2, tw, P);
+  fsc_pass_cplx_kernel<N><<<g, kFThreads, smem, st>>>(P, tw, Q);
+  fsc_pass_cplx_kernel<N><<<g, kFThreads, smem, st>>>(Q, tw, P);
 }
 
 // block partials, then the folded sums
 int fsc_partial_count(int d) { return (kShellBlocks + 1) * 3 * (d / 2 + 1); }
 
-cudaError_t launch_fsc(int d, float apix, float thr, const FftPlan &plan, const float2 *tw,
-                       const float *X1, const float *X2, float2 *P, float2 *Q, double *part,
-                       double *fsc, double *sums, double *resolution, cudaStream_t st) {
-  const size_t smem = fsc_smem(d);
-  const dim3 g(d / kFL, d);
-  fsc_pass_real_kernel<<<g, kFThreads, smem, st>>>(X1, X2, plan, tw, P);
-  fsc_pass_cplx_kernel<<<g, kFThreads, smem, st>>>(P, plan, tw, Q);
-  fsc_pass_cplx_kernel<<<g, kFThreads, smem, st>>>(Q, plan, tw, P);
+cudaError_t launch_fsc(int d, float apix, float thr, const float2 *tw, const float *X1,
+                       const float *X2, float2 *P, float2 *Q, double *part, double *fsc,
+                       double *sums, double *resolution, cudaStream_t st) {
+  switch (d) {
+#define X(N)                                     \
+  case N:                                        \
+    launch_fsc_passes<N>(tw, X1, X2, P, Q, st);  \
+    break;
+    GEM_FFT_SIDES(X)
+#undef X
+    default:
+      return cudaErrorInvalidValue;
+  }
   const int nsh = d / 2 + 1;
   fsc_shell_kernel<<<kShellBlocks, kFThreads, 3 * nsh * sizeof(double), st>>>(P, d, nsh, part);
   double *tot = part + (size_t)kShellBlocks * 3 * nsh;

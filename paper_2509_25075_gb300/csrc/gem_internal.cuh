@@ -382,24 +382,16 @@ cudaError_t launch_dense_bwd(const Rec *rec, int64_t M, int B, int d, float l2ta
                              const float *dproj, double *mom, cudaStream_t st);
 
 // gem_ctf.cu
-// Radix sequence of an n-point FFT, 2 bits per stage (0: radix 2,
-// 1: radix 3, 2: radix 4), first stage in the low bits.
-struct FftPlan {
-  int n;
-  int nst;
-  unsigned code;
-};
-bool fft_plan(int n, FftPlan &p);
 cudaError_t ctf_configure(int d);
 size_t ctf_partials(int d);
 // gem_fsc.cu
 cudaError_t fsc_configure(int d);
 int fsc_partial_count(int d);  // doubles of block partial sums
-cudaError_t launch_fsc(int d, float apix, float thr, const FftPlan &plan, const float2 *tw,
-                       const float *X1, const float *X2, float2 *P, float2 *Q, double *part,
-                       double *fsc, double *sums, double *resolution, cudaStream_t st);
+cudaError_t launch_fsc(int d, float apix, float thr, const float2 *tw, const float *X1,
+                       const float *X2, float2 *P, float2 *Q, double *part, double *fsc,
+                       double *sums, double *resolution, cudaStream_t st);
 
-cudaError_t launch_ctf_loss(int d, int B, float apix, const FftPlan &plan, const float2 *tw,
+cudaError_t launch_ctf_loss(int d, int B, float apix, const float2 *tw,
                             const float *proj, const float *ctf, const float *ctf_params,
                             const float *images, float2 *Z, double *lossp, float *pred,
                             float *dproj, double *loss_img, double *loss, cudaStream_t st);

@@ -103,13 +103,11 @@ extern "C" int gem_ctf_loss_static(int32_t d, float apix, int32_t B, const float
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return GEM_ECUDA;
   StaticScratch s;
   if (static_scratch(dev, s) != cudaSuccess) return GEM_ECUDA;
-  FftPlan plan;
-  if (!fft_plan(d, plan)) return GEM_EINVAL;
   if (ctf_configure(d) != cudaSuccess) return GEM_ECUDA;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   static_twiddle_kernel<<<(d + 255) / 256, 256, 0, st>>>(s.twiddle, d);
   if (cudaGetLastError() != cudaSuccess) return GEM_ECUDA;
-  if (launch_ctf_loss(d, B, apix, plan, s.twiddle, proj, ctf, ctf_params, images, s.spectrum,
+  if (launch_ctf_loss(d, B, apix, s.twiddle, proj, ctf, ctf_params, images, s.spectrum,
                       s.lossp, pred, dproj, loss_img, loss, st) != cudaSuccess)
     return GEM_ECUDA;
   return GEM_OK;
