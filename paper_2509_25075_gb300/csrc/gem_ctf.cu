@@ -229,8 +229,9 @@ __global__ void __launch_bounds__(kCtfThreads) ctf_pass2_kernel(
     lsum += lone ? r2 : 2.f * r2;
     // W(k) = P + i G;  W(-k) = conj P + i conj G.  Stored conjugated: the
     // inverse transform runs as conj(FFT(conj .)).
-    float2 W = make_float2(P.x - G.y, P.y + G.x);
-    float2 Wm = make_float2(P.x + G.y, -P.y + G.x);
+    // (products and sums rounded on their own, whatever the side's instance)
+    float2 W = make_float2(__fsub_rn(P.x, G.y), __fadd_rn(P.y, G.x));
+    float2 Wm = make_float2(__fadd_rn(P.x, G.y), __fsub_rn(G.x, P.y));
     l1[fft_at(ky)] = make_float2(W.x, -W.y);
     l2[fft_at(mky)] = make_float2(Wm.x, -Wm.y);
   }
