@@ -52,13 +52,12 @@ extern "C" {
 #define GEM_ECUDA (-3)     /* a CUDA runtime call or kernel launch failed                 */
 #define GEM_ESTATE (-4)    /* call order violated (backward before forward, ...)          */
 #define GEM_ECAPACITY (-5) /* returned by gem_status: the pair list overflowed max_pairs  */
-#define GEM_ETIMEOUT (-6)  /* returned by gem_status: a wait between the warps of a      */
-                           /* kernel ran out of tries (none does in working order; no    */
-                           /* kernel waits on another), the outputs are incomplete       */
+#define GEM_ETIMEOUT (-6)  /* reserved: a device-side wait ran out.  No kernel of this    */
+                           /* library waits on another (work is claimed from counters    */
+                           /* that never block), so no call returns it today.            */
 
 /* Device status bits reported by gem_status. */
 #define GEM_STATUS_CAPACITY 1
-#define GEM_STATUS_TIMEOUT 2
 
 typedef struct gem_ctx gem_ctx;
 
@@ -95,8 +94,8 @@ int gem_config_default(gem_config *cfg, int32_t d, float apix, int32_t max_B, in
 /* Create a context.  cuda_stream is a cudaStream_t (NULL: the legacy default
  * stream).  Allocates all scratch on the current device: about
  * 32 B x max_B x max_M (projected records) + 48 B x max_B x max_M (moments)
- * + 18 B x max_pairs (list entries with their block masks, the binning's hit
- * records, and partial images of tiles with long lists) + 20 B x max_B x d^2 (images, spectra) and
+ * + 16 B x max_pairs (list entries with their block masks, and the
+ * binning's hit records) + 20 B x max_B x d^2 (images, spectra) and
  * a few small tables.  Errors: GEM_EINVAL, GEM_ENOMEM, GEM_ECUDA. */
 int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream);
 
@@ -387,12 +386,9 @@ int gem_ctf_loss_static(int32_t d, float apix, int32_t B, const float *proj, con
 
 /* Both rasterisers come in several kernel configurations that compute the
  * same result (the forward bitwise, the backward within the rounding of
- * float64 sums taken in another order): the forward (step a3) with 6 to 12
- * warps that evaluate and 2 or 4 that stage records, and 1 to 3 CTAs per SM;
- * the backward (a5) with warp windows of 128 or 256 records and 3 to 8 CTAs
- * per SM.
- * Which is
- * fastest depends on the image side, the batch and the Gaussians' sizes.
+ * float64 sums taken in another order): the forward (step a3) at 1 to 8 CTAs
+ * per SM; the backward (a5) with warp windows of 128 or 256 records and 3 to
+ * 8 CTAs per SM.  Which is fastest depends on the image side, the batch and the Gaussians' sizes.
  * Counts of each kind (kind 0: forward, 1: backward); a configuration's
  * description ("" if out of range). */
 int gem_raster_config_count(int32_t *n_fwd, int32_t *n_bwd);

@@ -33,6 +33,7 @@ struct gem_ctx {
   uint32_t *gauss_slot = nullptr;  // [max_M] slot of each Gaussian
   float *psort = nullptr;          // [max_M][11] parameters by slot
   uint16_t *mkey = nullptr;        // [max_M] Morton keys
+  float *kept_R = nullptr, *kept_t = nullptr;  // [max_B][9], [max_B][2] views of the last projection
 
   BinScratch bin{};
   double *mom = nullptr;   // [max_B][max_M][6] moments of the raster backward
@@ -105,7 +106,7 @@ struct gem_ctx {
 
 // The configurations used when neither the context nor the autotuner's cache
 // names one (the fastest measured on the benchmark workloads).
-constexpr int kDefaultFwdCfg = 0;  // 6 consumer and 2 producer warps, 3 CTAs per SM
+constexpr int kDefaultFwdCfg = 0;  // 8 CTAs per SM
 constexpr int kDefaultBwdCfg = 0;  // 256-record windows, 5 CTAs per SM
 
 // The autotuner's choices, shared by every context of the process: keyed by
@@ -264,7 +265,8 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
   c->nbg = g.max_B < 16 ? g.max_B : 16;
   bool ok = alloc(c, &c->gp, g.max_M) && alloc(c, &c->slot_gauss, g.max_M) &&
             alloc(c, &c->gauss_slot, g.max_M) && alloc(c, &c->psort, (size_t)g.max_M * kNpar) &&
-            alloc(c, &c->mkey, g.max_M) && alloc(c, &c->rec, BM) && alloc(c, &c->bin.key, BM) &&
+            alloc(c, &c->mkey, g.max_M) && alloc(c, &c->kept_R, (size_t)g.max_B * 9) &&
+            alloc(c, &c->kept_t, (size_t)g.max_B * 2) && alloc(c, &c->rec, BM) && alloc(c, &c->bin.key, BM) &&
             alloc(c, &c->bin.packed, BM) && alloc(c, &c->bin.perm, BM) &&
             alloc(c, &c->bin.dcnt, (size_t)g.max_B * nchD * 256) &&
             alloc(c, &c->bin.tcnt, (size_t)g.max_B * nchT * c->T) &&
@@ -280,10 +282,8 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
             alloc(c, &c->Z, (size_t)g.max_B * d * d) && alloc(c, &c->tw, (size_t)d) &&
             alloc(c, &c->lossp, (size_t)g.max_B * (ctf_partials(d) + 1)) && alloc(c, &c->status, 1) &&
             alloc(c, &c->kept, 2);
-  // a task per tile, or two per partial image of tiles with several segments
-  const size_t nparts = raster_part_count(c->cfg.max_pairs);
-  ok = ok && alloc(c, &c->tasks.task, 2 * ((size_t)g.max_B * c->T + nparts)) &&
-       alloc(c, &c->tasks.part, nparts * 256) && alloc(c, &c->tasks.done, (size_t)g.max_B * c->T) &&
+  ok = ok && alloc(c, &c->tasks.task, 2 * raster_task_count(c->cfg.max_pairs, (int64_t)g.max_B * c->T)) &&
+       alloc(c, &c->tasks.done, (size_t)g.max_B * c->T) &&
        alloc(c, &c->tasks.ctr, kCtrCount);
   // nearest-neighbour grid: at most 2 max_M + 64 cells
   c->knn.cap = 2 * g.max_M + 64;
@@ -311,7 +311,11 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
   c->bin.cap = c->cfg.max_pairs;
   c->bin.status = c->status;
   c->bin.task_ctr = c->tasks.ctr;
-  c->tasks.status = c->status;
+  // the forward's partial images lie where the binning keeps its hits, which
+  // nobody reads once the lists stand: a window of 1 KB for every 256 entries
+  // and tile, and only tiles of more than 256 entries have any, so at most
+  // 8 bytes per entry
+  c->tasks.part = reinterpret_cast<float *>(c->bin.hits);
   std::vector<float2> tw(d);
   for (int m = 0; m < d; ++m) {
     double a = -2.0 * 3.14159265358979323846 * m / d;
@@ -323,8 +327,7 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
       (e = cudaMemset(c->status, 0, sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(c->knn.ticket, 0, sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(c->tasks.done, 0, (size_t)g.max_B * c->T * sizeof(unsigned))) != cudaSuccess ||
-      (e = bin_configure(d)) != cudaSuccess || (e = ctf_configure(d)) != cudaSuccess ||
-      (e = raster_configure()) != cudaSuccess) {
+      (e = bin_configure(d)) != cudaSuccess || (e = ctf_configure(d)) != cudaSuccess) {
     snprintf(g_create_err, sizeof(g_create_err), "set-up: %s", cudaGetErrorString(e));
     gem_destroy(c);
     return GEM_ECUDA;
@@ -363,7 +366,6 @@ int gem_status(gem_ctx *c) {
     return cuda_fail(c, e, "status read");
   if ((e = cudaMemset(c->status, 0, sizeof(int))) != cudaSuccess)
     return cuda_fail(c, e, "status clear");
-  if (st & GEM_STATUS_TIMEOUT) return fail(c, GEM_ETIMEOUT, "a wait inside a kernel ran out");
   if (st & GEM_STATUS_CAPACITY)
     return fail(c, GEM_ECAPACITY, "pair list exceeded max_pairs=%lld",
                 (long long)c->cfg.max_pairs);
@@ -400,7 +402,7 @@ static int prep(gem_ctx *c, const float *params, int64_t M, int32_t B, const flo
   // depth keys span [-d apix, d apix]: the half-diagonal of the box is shorter
   const float zrange = (float)g.d * g.apix;
   if ((e = launch_view_prep(c->gp, M, B, R, t, g.apix, g.d, c->l2tau, zrange, c->rec,
-                            c->bin.key, c->stream)) != cudaSuccess)
+                            c->bin.key, c->kept_R, c->kept_t, c->stream)) != cudaSuccess)
     return cuda_fail(c, e, "view_prep");
   c->params = params;
   c->R = R;
@@ -635,7 +637,8 @@ int gem_inspect_bins(gem_ctx *c, int64_t *tile_start, uint32_t *list, int64_t li
 int gem_inspect_records(gem_ctx *c, float *out) {
   if (!c || !out) return GEM_EINVAL;
   if (!c->have_proj) return fail(c, GEM_ESTATE, "no projection yet");
-  cudaError_t e = launch_inspect_records(c->rec, c->gp, c->slot_gauss, c->M, c->B, c->R, c->t, c->cfg.apix,
+  cudaError_t e = launch_inspect_records(c->rec, c->gp, c->slot_gauss, c->M, c->B, c->kept_R,
+                                         c->kept_t, c->cfg.apix,
                                          c->cfg.d, out, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "inspect records");
   if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess)

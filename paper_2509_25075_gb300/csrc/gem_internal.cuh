@@ -17,7 +17,6 @@ constexpr float kMargin = 1e-3f;
 
 // Device status bits (mirror GEM_STATUS_* in gem.h).
 constexpr int kStatusCapacity = 1;
-constexpr int kStatusTimeout = 2;
 
 // Per-Gaussian quantities independent of the view (64 B): p (3), log2 of
 // the amplitude constant (-inf for a Gaussian that contributes nothing),
@@ -191,7 +190,8 @@ cudaError_t launch_gauss_prep(const float *params, const uint32_t *slot_gauss, i
                               uint32_t *gauss_slot, cudaStream_t st);
 cudaError_t launch_view_prep(const GaussPrep *gp, int64_t M, int B, const float *R,
                              const float *t, float apix, int d, float l2tau, float zrange,
-                             Rec *rec, uint16_t *key, cudaStream_t st);
+                             Rec *rec, uint16_t *key, float *kept_R, float *kept_t,
+                             cudaStream_t st);
 // Reads the float64 moments [B][M][6] and leaves them zero (the next
 // backward pass accumulates into them).
 // params (the slot-ordered copy), gp and the moments are by slot; grad
@@ -337,18 +337,15 @@ constexpr int kCtrSegment = 4;               // segment length
 constexpr int kCtrCount = 5;
 struct RasterTasks {
   uint4 *task;     // two words per task: (list start, lo and hi; entries; image * T + tile),
-                   // (segment, segments of the tile, the tile's first partial image, 0)
-  float *part;     // [parts][256] partial images of tiles with several segments
-  unsigned *done;  // [B * T] segments finished, zero between calls
+                   // (first window, windows of the tile, the tile's first partial image, 0)
+  float *part;     // [parts][256] partial images of tiles with several windows
+  unsigned *done;  // [B * T] windows finished, zero between calls
   unsigned *ctr;   // [kCtrCount], reset by the binning
-  int *status;     // kStatusTimeout when a wait ran out
 };
-size_t raster_part_count(int64_t cap);
-cudaError_t raster_configure();
-// A configuration of the forward rasteriser: consumer and producer warps per
-// CTA, CTAs per SM.
+size_t raster_task_count(int64_t cap, int64_t ntiles);
+// A configuration of the forward rasteriser: CTAs per SM.
 struct FwdCfg {
-  int cons, prod, ctas;
+  int ctas;
   const char *name;
 };
 int fwd_config_count();

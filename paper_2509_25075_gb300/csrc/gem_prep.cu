@@ -155,12 +155,19 @@ __global__ void __launch_bounds__(256) view_prep_kernel(const GaussPrep *__restr
                                                         const float *__restrict__ t,
                                                         float apix, int d, float l2tau,
                                                         float inv_range, Rec *__restrict__ rec,
-                                                        uint16_t *__restrict__ key) {
+                                                        uint16_t *__restrict__ key,
+                                                        float *__restrict__ kept_R,
+                                                        float *__restrict__ kept_t) {
   __shared__ float sv[kViewGroup][12];  // R (9), t (2)
   const int b0 = blockIdx.y * kViewGroup, nv = min(kViewGroup, B - b0);
   if (threadIdx.x < kViewGroup * 11) {
     const int v = threadIdx.x / 11, k = threadIdx.x - v * 11;
-    if (v < nv) sv[v][k] = k < 9 ? R[9 * (b0 + v) + k] : t[2 * (b0 + v) + (k - 9)];
+    if (v < nv) {
+      const float x = k < 9 ? R[9 * (b0 + v) + k] : t[2 * (b0 + v) + (k - 9)];
+      sv[v][k] = x;
+      // the views as they were, for the record inspection
+      if (blockIdx.x == 0) (k < 9 ? kept_R[9 * (b0 + v) + k] : kept_t[2 * (b0 + v) + (k - 9)]) = x;
+    }
   }
   __syncthreads();
   const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -193,9 +200,11 @@ __global__ void __launch_bounds__(256) view_prep_kernel(const GaussPrep *__restr
 
 cudaError_t launch_view_prep(const GaussPrep *gp, int64_t M, int B, const float *R,
                              const float *t, float apix, int d, float l2tau, float zrange,
-                             Rec *rec, uint16_t *key, cudaStream_t st) {
+                             Rec *rec, uint16_t *key, float *kept_R, float *kept_t,
+                             cudaStream_t st) {
   dim3 grid((unsigned)((M + 255) / 256), (unsigned)((B + kViewGroup - 1) / kViewGroup));
-  view_prep_kernel<<<grid, 256, 0, st>>>(gp, M, B, R, t, apix, d, l2tau, 1.f / zrange, rec, key);
+  view_prep_kernel<<<grid, 256, 0, st>>>(gp, M, B, R, t, apix, d, l2tau, 1.f / zrange, rec, key,
+                                         kept_R, kept_t);
   return cudaGetLastError();
 }
 

@@ -8,15 +8,16 @@
 // coordinates (Rec): the exponent is l2A - (u11 dx + u12 dy)^2 - (u22 dy)^2.
 //
 // a3: Eq. render restricted by Eq. accu.  The lists are cut into segments of
-//     at most 1024 entries, taken from a counter by persistent CTAs.  Producer
-//     warps stage a segment's records (only the 24 bytes the evaluation reads)
-//     and, by warp bit transposes of the packed block masks, each block's
-//     record set; consumer warps take the window's blocks one after the other
-//     and evaluate 32 of a block's records at a time, one record and 16 pixels
-//     per lane (packed float pairs).  A pixel's sum within a segment runs
-//     over lanes, then by a tree over the 32 lanes; a tile's segments join in
-//     list order with Kahan compensation.  The result is deterministic and
-//     follows the list's depth order segment by segment.
+//     at most 512 entries, taken from a counter by persistent CTAs of 128
+//     threads, which walk them in windows of 256 entries (only the 24 bytes
+//     that the evaluation reads are staged).  A window's (block, record) items
+//     are laid out block after block, each block's records in list order, and
+//     each block gets a share of the threads in proportion to its items.  A
+//     thread evaluates the 16 pixels of its block for each of its items
+//     (packed float pairs); each pixel sums its block's partial images in
+//     thread order, and windows join with Kahan compensation in list order.
+//     The result is deterministic and follows the list's depth order window by
+//     window.
 // a5: the "efficient gradient" of Sec. 1 (iii) / Sec. 3.2: only pairs kept by
 //     Eq. accu.  Each warp takes up to 256 entries of a segment, sorts them by
 //     block count and first block and runs them in rounds of 32 records, one
@@ -71,53 +72,21 @@ __device__ __forceinline__ Rec load_rec(const Rec *p) {
   return r;
 }
 
-// Barrier id over the given number of threads of the CTA.
-__device__ __forceinline__ void named_sync(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
-// mbarriers in shared memory: arrivals release, waits acquire.
-__device__ __forceinline__ void mbar_init(uint64_t *bar, unsigned count) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(a), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(a) : "memory");
-}
-// Waits for the phase of the given parity, at most kWaitTries tries (each
-// suspends the thread for a hardware time slice; seconds in all); false when
-// it did not complete.
-constexpr int kWaitTries = 1 << 22;
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
-  for (int i = 0; i < kWaitTries; ++i) {
-    unsigned ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
-  return false;
-}
-
-constexpr int kFwdWin = 1024;  // forward: records staged per window
+constexpr int kWin = 256;       // forward: records per window
+constexpr int kSegMax = 512;    // entries of the longest segment
 
 // Tasks of the rasterisers.  A tile's list is cut into segments of S entries
-// (the last one shorter); a task is one segment, staged as one window, so
-// that no CTA walks a long list alone (the longest list of a workload holds
-// five to twenty times the mean) and a call with few tiles still fills the
-// SMs.  S is 1024, less (down to 256) where that would leave resident CTAs
-// without a segment.  Tasks follow the tiles' index order up to the order in
-// which the CTAs here claim their ranges, so neighbouring tiles, which share
-// records, are in flight together.  Empty tiles get their zeros here and no
-// task.
+// (the last one shorter); a task is one segment, and the warps that take it
+// work on pieces of it, so that nobody walks a long list alone (the longest
+// list of a workload holds five to twenty times the mean) and a call with few
+// tiles still fills the SMs.  S is a multiple of the forward's window: 1024,
+// less where that would leave resident warps without a segment.  Tasks follow
+// the tiles' index order up to the order in which the CTAs here claim their
+// ranges, so neighbouring tiles, which share records, are in flight together.
+// Empty tiles get their zeros here and no task.
 __device__ __forceinline__ int64_t segment_length(int64_t total, int slots) {
   const int64_t S = total / (2 * (int64_t)slots);
-  return (max((int64_t)256, min((int64_t)kFwdWin, S)) + 63) / 64 * 64;
+  return (max((int64_t)1, min((int64_t)kSegMax, S)) + kWin - 1) / kWin * kWin;
 }
 
 __global__ void __launch_bounds__(256) raster_tasks_kernel(const int64_t *__restrict__ tile_start,
@@ -137,8 +106,10 @@ __global__ void __launch_bounds__(256) raster_tasks_kernel(const int64_t *__rest
     len = over ? 0 : tile_start[i + 1] - s;
   }
   unsigned nseg = (unsigned)((len + S - 1) / S);
-  // exclusive prefixes of the tasks and of the partial images they need
-  unsigned inc = nseg, incp = nseg > 1 ? nseg : 0;
+  // exclusive prefixes of the tasks and of the partial images they need (one
+  // per window of tiles with several segments)
+  const unsigned nwin = (unsigned)((len + kWin - 1) / kWin);
+  unsigned inc = nseg, incp = nseg > 1 ? nwin : 0;
   const unsigned mine = incp;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -176,7 +147,7 @@ __global__ void __launch_bounds__(256) raster_tasks_kernel(const int64_t *__rest
       const int64_t a = s + k * S, n = min(S, s + len - a);
       uint4 *t = tk.task + 2 * (int64_t)(at + k);
       t[0] = make_uint4((unsigned)a, (unsigned)((uint64_t)a >> 32), (unsigned)n, (unsigned)i);
-      t[1] = make_uint4(k, nseg, part, 0u);
+      t[1] = make_uint4(k * (unsigned)(S / kWin), nseg, part, nwin);
     }
   }
   if (proj) {
@@ -193,302 +164,287 @@ __global__ void __launch_bounds__(256) raster_tasks_kernel(const int64_t *__rest
   }
 }
 
-// Shared memory of one forward CTA: two staged windows, the lists of the
-// consumer warps, and the barriers.
-struct FwdWindow {
-  float4 sa[kFwdWin];        // px, py, u11, u12
-  float2 sb[kFwdWin];        // u22, log2 A
-  unsigned bal[16][33];      // block, 32 records: which touch it
-  float out[16][16];         // block, pixel: the window's sums
-  int n, bt;                 // entries (-1: no more tasks), image * T + tile
-  unsigned seg, nseg, part;  // segment of the tile, how many, first partial image
-  int next_block, done;      // blocks handed out, blocks finished
+// Shared memory of one forward CTA: a window.
+struct FwdWin {
+  float4 sa[kWin];                // px, py, u11, u12
+  float2 sb[kWin];                // u22, log2 A
+  float4 part[kThreads][4];       // the threads' partial images of their blocks
+  unsigned char flat[16 * kWin];  // slot of each (block, record) item
+  unsigned short cnt[4][16];      // per warp: its records that touch each block
+  unsigned short pstart[18];      // block k's items: [pstart[k], pstart[k + 1])
+  unsigned short tfirst[18];      // block k's threads: [tfirst[k], tfirst[k + 1])
+  uint4 desc[2][2];               // this task's descriptor and the next one's
+  int last;                       // whether this is the tile's last segment
 };
-template <int kCons>
-struct FwdShared {
-  uint4 desc[2][2];                      // the producers' current and next task
-  FwdWindow win[2];
-  unsigned short slots[kCons][kFwdWin];  // a block's records, in list order
-  uint64_t full[2], empty[2];            // mbarriers
-};
+// Row q of thread v's partial image lies at part[v][q ^ swizzle(v)]:
+// eight neighbouring lanes then store to different banks.
+__device__ __forceinline__ int part_swizzle(int v) { return (v >> 1) & 3; }
+constexpr unsigned kNoSum = 0x80000000u;  // -0: a block without items (a sum of values is never -0)
 
-// a3.  One producer warp and kCons consumer warps per CTA, two windows in
-// shared memory.  The producer claims tasks and stages their records; the
-// lanes' packed masks, transposed as bit matrices, give for every block one
-// 32-bit word per 32 records (which of them touch the block).  A consumer
-// warp takes the next block of the window, turns the block's words into the
-// list of the records that touch it (lane l lists those of 32 slots, in
-// order), its 32 lanes evaluate 32 of those records at a time, one record
-// and 16 pixels per lane, and the lanes' partial images are added by a
-// butterfly that halves the pixels a lane holds at each of four steps.  A
-// warp that finds no block left goes on to the other window without waiting
-// for its neighbours; the warp that finishes the last block writes the
-// window's 256 pixels.  Windows of a tile with several segments go to
-// partial images, which the last segment to finish adds in segment order
-// (Kahan).  Nothing depends on which warp or CTA did what, so the result is
-// deterministic.
+// a3.  A CTA claims a segment from a counter and walks it in windows of 256
+// entries, the next window's entries on their way while one is evaluated.
+// Its warps stage a quarter of a window's records each; the lanes' packed
+// masks, transposed as a bit matrix, leave each lane one of the words that
+// say which of 32 records touch a block; the lane lists its word's records, so
+// that the window's (block, record) items lie block after block, each
+// block's in list order.  The 128 threads share the items: every non-empty
+// block gets at least one (thread range [T_k, T_k+1) with T_k = (non-empty
+// blocks before k) + floor((128 - non-empty) start_k / N)), and a block's
+// threads take its items interleaved.  A thread evaluates 16 pixels per item
+// and leaves one partial image of its block; each pixel sums its block's
+// partials in thread order.  A pixel's windows join with Kahan compensation
+// in list order: in registers where the tile has one segment, else the windows
+// go to `part`, and the CTA that finishes the tile's last segment adds them.
+// Nothing depends on which CTA did what, so the result is deterministic and
+// in depth order window by window.
 //
-// What bounds it: issue (about 60% of the slots) and the L1, through which
-// every entry's 32 scattered bytes come (one 256-bit load per record: two
-// loads of 16 and 8 bytes cost 8% of the launch) and which serves the record
-// reads of the evaluation.  Against CTAs of four warps that staged 256
-// records between barriers and gave each block a share of the threads
-// (us per launch): d 384, M 500000, B 16: 680 -> 467; d 128, M 20000, B 256:
-// 388 -> 367; d 256, M 100000, B 64: 498 -> 418; d 128, M 50000, B 64, scales
-// 0.3-12 px, whose longest lists hold 14000 entries: 745-850 -> 391; d 64,
-// M 2000, B 32: 37 -> 24.  Staging by the consumers between barriers: 553 at
-// the first of these; one producer warp with small copies in flight: 494-518;
-// windows of 512 records: 610.
+// What bounds it: issue (70% of the slots) and the L1 (66%), through which
+// every entry's 32 scattered bytes come and which serves the evaluation.  The
+// records of the next window, of this task or the next, wait in registers (one
+// 256-bit load each: two loads of 16 and 8 bytes take two passes over the L1
+// tags, and asynchronous copies of the same into a second buffer were slower
+// than no prefetch: 655 against 575 us at d 384, M 500000, B 16).  Against one
+// CTA per tile, the longest lists first, that loaded a window's records when
+// it came to them (us per launch; the sums are the same bits): d 384,
+// M 500000, B 16: 680 -> 510; d 128, M 20000, B 256: 388 -> 364; d 256,
+// M 100000, B 64: 498 -> 428; d 128, M 50000, B 64, scales 0.3-12 px, whose
+// longest lists hold 14000 entries against a mean of 3400: 745-850 -> 442;
+// d 64, M 2000, B 32: 37 -> 20; d 64, M 1999, B 9, every pair: 71 -> 41.
+// Segments of 256, 1024, 2048 entries: 538, 510, 526 at the first, 381, 371,
+// 387 at the second.  Two warps per window, 24 on an SM: 592 and 422; one
+// warp, 16 on an SM: 606 and 438.
 //
 // kCount = true: the same walk, counting kept pairs into kept[0] and
 // evaluated pairs into kept[1] instead of writing the projection
 // (inspection only, never on the timed path).
-template <int kCons, int kProd, int kMinB, bool kCount>
-__global__ void __launch_bounds__(32 * (kCons + kProd), kMinB) raster_fwd_kernel(
+template <int kMinB, bool kCount>
+__global__ void __launch_bounds__(kThreads, kMinB) raster_fwd_kernel(
     const Rec *__restrict__ rec, const uint2 *__restrict__ list, int64_t M, int d, float l2tau,
     RasterTasks tk, float *__restrict__ proj, unsigned long long *__restrict__ kept) {
-  extern __shared__ __align__(16) unsigned char fwd_smem[];
-  FwdShared<kCons> &S = *reinterpret_cast<FwdShared<kCons> *>(fwd_smem);
+  __shared__ FwdWin W;
   const int nt = d / kTile, T = nt * nt;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) {
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&S.full[i], 32 * kProd);
-      mbar_init(&S.empty[i], kCons);
+  const int hw = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float nl2tau = -l2tau;  // kept: -e < -log2(tau)
+  const int ntasks = (int)tk.ctr[kCtrTasks];
+  unsigned nkept = 0, neval = 0;
+  // thread 0 claims a task two ahead and reads its descriptor one ahead;
+  // a task with no entries ends the list
+  auto task_at = [&](int q, uint4 &a, uint4 &c) {
+    a = c = make_uint4(0u, 0u, 0u, 0u);
+    if (q < ntasks) {
+      a = tk.task[2 * (int64_t)q];
+      c = tk.task[2 * (int64_t)q + 1];
     }
+  };
+  auto claim = [&]() { return (int)(atomicAdd(tk.ctr + kCtrFwd, 1u) + gridDim.x); };
+  int nq = 0;
+  if (threadIdx.x == 0) {
+    task_at(blockIdx.x, W.desc[0][0], W.desc[0][1]);
+    const int q1 = claim();
+    nq = claim();
+    task_at(q1, W.desc[1][0], W.desc[1][1]);
   }
   __syncthreads();
-  if (warp >= kCons) {
-    // ---- producers ----
-    const int pw = warp - kCons;
-    const bool leader = pw == 0 && lane == 0;
-    const int ntasks = (int)tk.ctr[kCtrTasks];
-    // the leader claims a task two windows ahead and reads its descriptor one
-    // window ahead; t1.w marks the end
-    int nq = 0;
-    if (leader) {
-      const int q = blockIdx.x;
-      if (q < ntasks) {
-        S.desc[0][0] = tk.task[2 * (int64_t)q];
-        S.desc[0][1] = tk.task[2 * (int64_t)q + 1];
-      } else {
-        S.desc[0][1].w = 1u;
-      }
-      nq = (int)(atomicAdd(tk.ctr + kCtrFwd, 1u) + gridDim.x);
+  // this warp's quarter of a window: slots 64 hw .. 64 hw + 63, two per lane.
+  // masks: their block masks, packed; an entry whose Gaussian index is out of
+  // range (a list position left unwritten when the lists overflowed their
+  // capacity) counts as empty.
+  const int slot0 = 64 * hw + lane;
+  auto entry = [&](const uint4 &a, int w0, int q) {
+    const int i = w0 + slot0 + 32 * q;
+    const uint2 *L = list + (int64_t)(((uint64_t)a.y << 32) | a.x);
+    return i < (int)a.z ? L[i] : make_uint2(0xffffffffu, 0u);
+  };
+  Rec r0, r1;  // the next window's records, on their way while this one is evaluated
+  auto fetch = [&](const uint4 &a, const uint2 &e0, const uint2 &e1) {
+    const Rec *rb = rec + (int64_t)((int)a.w / T) * M;
+    unsigned m = 0;
+    if (e0.x < (uint64_t)M) {
+      m = e0.y & 0xffffu;
+      r0 = load_rec(rb + e0.x);
     }
-    for (int it = 0;; ++it) {
-      FwdWindow &W = S.win[it & 1];
-      named_sync(1, 32 * kProd);
-      const uint4 t0 = S.desc[it & 1][0], t1 = S.desc[it & 1][1];
-      // the other parity passes at once on a fresh barrier
-      if (!mbar_wait(&S.empty[it & 1], ((it >> 1) & 1) ^ 1)) {
-        if (lane == 0) atomicOr(tk.status, kStatusTimeout);
-        return;
-      }
-      if (t1.w) {
-        if (leader) W.n = -1;
-        mbar_arrive(&S.full[it & 1]);
-        return;
-      }
-      uint4 n0 = make_uint4(0u, 0u, 0u, 0u), n1 = make_uint4(0u, 0u, 0u, 1u);
-      int nq2 = 0;
-      if (leader) {
-        if (nq < ntasks) {
-          n0 = tk.task[2 * (int64_t)nq];
-          n1 = tk.task[2 * (int64_t)nq + 1];
-        }
-        nq2 = (int)(atomicAdd(tk.ctr + kCtrFwd, 1u) + gridDim.x);
-      }
-      const uint2 *L = list + (int64_t)(((uint64_t)t0.y << 32) | t0.x);
-      const int n = (int)t0.z, bt = (int)t0.w;
-      const Rec *rb = rec + (int64_t)(bt / T) * M;
-      if (leader) {
-        W.n = n;
-        W.bt = bt;
-        W.seg = t1.x;
-        W.nseg = t1.y;
-        W.part = t1.z;
-        W.next_block = 0;
-        W.done = 0;
-      }
-      // this warp's pairs of 32-entry chunks, all their entries in flight together
-      constexpr int kPairs = kFwdWin / 64 / kProd;
-      uint2 ent[2 * kPairs];
-#pragma unroll
-      for (int u = 0; u < 2 * kPairs; ++u) {
-        const int slot = 64 * ((u >> 1) * kProd + pw) + 32 * (u & 1) + lane;
-        ent[u] = slot < n ? L[slot] : make_uint2(0xffffffffu, 0u);
-      }
-      // records in batches of kB chunks in flight
-      constexpr int kB = kPairs >= 2 ? 4 : 2;
-#pragma unroll
-      for (int u0 = 0; u0 < 2 * kPairs; u0 += kB) {
-        if (64 * ((u0 >> 1) * kProd + pw) >= n) break;
-        Rec r[kB];
-#pragma unroll
-        for (int u = 0; u < kB; ++u) {
-          // an entry whose Gaussian index is out of range counts as empty
-          if (ent[u0 + u].x < (uint64_t)M)
-            r[u] = load_rec(rb + ent[u0 + u].x);
-          else
-            ent[u0 + u].y = 0u;
-        }
-        // lane k < 16: block k of the first chunk of a pair, lane 16 + k: of the second
-#pragma unroll
-        for (int u = 0; u < kB; u += 2)
-          W.bal[lane & 15][2 * (((u0 + u) >> 1) * kProd + pw) + (lane >> 4)] =
-              warp_transpose32((ent[u0 + u].y & 0xffffu) | (ent[u0 + u + 1].y << 16), lane);
-#pragma unroll
-        for (int u = 0; u < kB; ++u) {
-          const int slot = 64 * (((u0 + u) >> 1) * kProd + pw) + 32 * (u & 1) + lane;
-          W.sa[slot] = r[u].a;
-          W.sb[slot] = make_float2(r[u].b.x, r[u].b.y);
-        }
-      }
-      if (leader) {
-        S.desc[(it + 1) & 1][0] = n0;
-        S.desc[(it + 1) & 1][1] = n1;
-        nq = nq2;
-      }
-      __syncwarp();
-      mbar_arrive(&S.full[it & 1]);
+    if (e1.x < (uint64_t)M) {
+      m |= e1.y << 16;
+      r1 = load_rec(rb + e1.x);
     }
+    return m;
+  };
+  // this thread's pixels when it sums: half a row of block ob
+  const int id = threadIdx.x, ob = id >> 3, row = (id >> 1) & 3;
+  int cd = 0;  // descriptor in use
+  unsigned masks = 0;
+  {
+    const uint4 a = W.desc[0][0];
+    masks = fetch(a, entry(a, 0, 0), entry(a, 0, 1));
   }
-  // ---- consumers ----
-  const float nl2tau = -l2tau;  // kept: -e < -log2(tau)
-  unsigned short *slots = S.slots[warp];
-  unsigned nkept = 0, neval = 0;
-  for (int it = 0;; ++it) {
-    FwdWindow &W = S.win[it & 1];
-    if (!mbar_wait(&S.full[it & 1], (it >> 1) & 1)) {
-      if (lane == 0) atomicOr(tk.status, kStatusTimeout);
-      return;
-    }
-    const int n = W.n;
-    if (n < 0) break;
-    const int bt = W.bt;
+  while (W.desc[cd][0].z != 0u) {
+    const uint4 t0 = W.desc[cd][0];
+    const uint4 t1 = W.desc[cd][1];
+    const int ntask = (int)t0.z, bt = (int)t0.w;
+    const unsigned nseg = t1.y;
     const int b = bt / T, t = bt - b * T;
     const int tx = t % nt, ty = t / nt;
     const int x0 = tx * kTile, y0 = ty * kTile;
-    const int nw = ((n + 63) >> 6) << 1;  // words staged
-    for (;;) {
-      int k = 0;
-      if (lane == 0) k = atomicAdd(&W.next_block, 1);
-      k = __shfl_sync(0xffffffffu, k, 0);
-      if (k >= 16) break;
-      unsigned bits = lane < nw ? W.bal[k][lane] : 0u;
-      const int c = __popc(bits);
-      int incl = c;
+    float *o = proj + ((int64_t)b * d + y0) * d + x0;
+    float2 *part = reinterpret_cast<float2 *>(tk.part + (int64_t)t1.z * 256);
+    float2 run0 = make_float2(0.f, 0.f), run1 = run0;  // Kahan sums over the windows
+    for (int w0 = 0; w0 < ntask; w0 += kWin) {
+      const bool lastw = w0 + kWin >= ntask;
+      // the next window's entries (this task's or the next one's)
+      const uint4 na = lastw ? W.desc[cd ^ 1][0] : t0;
+      const int nw0 = lastw ? 0 : w0 + kWin;
+      const uint2 e0 = entry(na, nw0, 0), e1 = entry(na, nw0, 1);
+      // lane (k, h) = k + 16 h: word 2 hw + h of block k (bit l: slot 32 word + l)
+      const int h = lane >> 4;
+      const unsigned w = warp_transpose32(masks, lane);
+      const int c = __popc(w), o2 = __shfl_xor_sync(0xffffffffu, c, 16);
+      if (lane < 16) W.cnt[hw][lane] = (unsigned short)(c + o2);
+      W.sa[slot0] = r0.a;
+      W.sb[slot0] = make_float2(r0.b.x, r0.b.y);
+      W.sa[slot0 + 32] = r1.a;
+      W.sb[slot0 + 32] = make_float2(r1.b.x, r1.b.y);
+      __syncthreads();
+      // the blocks' items and threads (every warp, the same numbers)
+      int len = 0, before = 0;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
+      for (int q = 0; q < 4; ++q) {
+        if (q == hw) before = len;
+        len += W.cnt[q][lane & 15];
       }
-      const int nk = __shfl_sync(0xffffffffu, incl, 31);
+      int incl = len, ne = len > 0 ? 1 : 0;
+#pragma unroll
+      for (int s = 1; s < 16; s <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, s, 16);
+        const int x = __shfl_up_sync(0xffffffffu, ne, s, 16);
+        if ((lane & 15) >= s) {
+          incl += v;
+          ne += x;
+        }
+      }
+      const int N = __shfl_sync(0xffffffffu, incl, 15), nne = __shfl_sync(0xffffffffu, ne, 15);
+      const int st = incl - len;
+      // floor(a / N) for a = (128 - nne) st < 2^19, N <= 16 kWin: a / N is a
+      // multiple of 1 / N, so (a + 1/2) / N sits at least 1 / (2 N) from
+      // an integer, far more than the few-ulp error of the fast division
+      const float a = (float)((kThreads - nne) * st) + 0.5f;
+      if (hw == 0 && lane < 16) {
+        W.pstart[lane] = (unsigned short)st;
+        W.tfirst[lane] = (unsigned short)(ne - (len > 0 ? 1 : 0) + (N > 0 ? (int)__fdividef(a, (float)N) : 0));
+      }
+      if (hw == 0 && lane == 15) {
+        W.pstart[16] = (unsigned short)N;
+        W.tfirst[16] = kThreads;
+      }
+      // the records of this lane's word
       {
-        unsigned short *w = slots + (incl - c);
-        for (; bits; bits &= bits - 1) *w++ = (unsigned short)(32 * lane + __ffs(bits) - 1);
+        unsigned char *f = W.flat + st + before + (h ? o2 : 0);
+        const int first = 32 * (2 * hw + h);
+        for (unsigned m = w; m; m &= m - 1) *f++ = (unsigned char)(first + __ffs(m) - 1);
       }
-      __syncwarp();
-      // acc[4 h + x]: column x, rows 2 h and 2 h + 1
-      float2 acc[8];
+      __syncthreads();
+      masks = fetch(na, e0, e1);
+      {
+        // this thread's block is the last one whose range starts at or before
+        // it (an empty block's range is empty)
+        const int vt = threadIdx.x;
+        int k = 0;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] = make_float2(0.f, 0.f);
-      const float X0 = (float)(x0 + 4 * (k & 3)), Y0 = (float)(y0 + 4 * (k >> 2));
-      const float2 ys0 = make_float2(Y0, Y0 + 1.f), ys1 = make_float2(Y0 + 2.f, Y0 + 3.f);
-      for (int i = lane; i < nk; i += 32) {
-        const int slot = slots[i];
-        const float4 A = W.sa[slot];
-        const float2 Bv = W.sb[slot];
-        // -e = z1^2 + (z2^2 - l2A), z1 = u11 dx + u12 dy (u11 dx fused into
-        // the sum), z2 = u22 dy, two rows of a column in one packed operation
-        float2 dx[4];
+        for (int s = 8; s >= 1; s >>= 1)
+          if (W.tfirst[k + s] <= vt) k += s;
+        const int th0 = W.tfirst[k], nth = W.tfirst[k + 1] - th0, end = W.pstart[k + 1];
+        // acc[4 h + x]: column x, rows 2 h and 2 h + 1
+        float2 acc[8];
 #pragma unroll
-        for (int x = 0; x < 4; ++x) dx[x] = f2(__fsub_rn(X0 + (float)x, A.x));
+        for (int j = 0; j < 8; ++j) acc[j] = make_float2(0.f, 0.f);
+        const float X0 = (float)(x0 + 4 * (k & 3)), Y0 = (float)(y0 + 4 * (k >> 2));
+        const float2 ys0 = make_float2(Y0, Y0 + 1.f), ys1 = make_float2(Y0 + 2.f, Y0 + 3.f);
+        for (int i = W.pstart[k] + vt - th0; i < end; i += nth) {
+          const int slot = W.flat[i];
+          const float4 A = W.sa[slot];
+          const float2 Bv = W.sb[slot];
+          // -e = z1^2 + (z2^2 - l2A), z1 = u11 dx + u12 dy (u11 dx fused into
+          // the sum), z2 = u22 dy, two rows of a column in one packed operation
+          float2 dx[4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float2 dy = add2(h ? ys1 : ys0, f2(-A.y));
-          const float2 uy = mul2(f2(A.w), dy);
-          const float2 z2 = mul2(f2(Bv.x), dy);
-          const float2 nc = fma2(z2, z2, f2(-Bv.y));
+          for (int x = 0; x < 4; ++x) dx[x] = f2(__fsub_rn(X0 + (float)x, A.x));
 #pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            const float2 z = fma2(f2(A.z), dx[x], uy);
-            const float2 f = fma2(z, z, nc);
-            if (kCount)
-              nkept += (f.x < nl2tau) + (f.y < nl2tau);
-            else  // value on kept pairs (value > tau), zero elsewhere
-              acc[4 * h + x] = fma2(make_float2(ex2_approx(-f.x), ex2_approx(-f.y)),
-                                    make_float2(set_lt(f.x, nl2tau), set_lt(f.y, nl2tau)),
-                                    acc[4 * h + x]);
+          for (int g = 0; g < 2; ++g) {
+            const float2 dy = add2(g ? ys1 : ys0, f2(-A.y));
+            const float2 uy = mul2(f2(A.w), dy);
+            const float2 z2 = mul2(f2(Bv.x), dy);
+            const float2 nc = fma2(z2, z2, f2(-Bv.y));
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+              const float2 z = fma2(f2(A.z), dx[x], uy);
+              const float2 f = fma2(z, z, nc);
+              if (kCount)
+                nkept += (f.x < nl2tau) + (f.y < nl2tau);
+              else  // value on kept pairs (value > tau), zero elsewhere
+                acc[4 * g + x] = fma2(make_float2(ex2_approx(-f.x), ex2_approx(-f.y)),
+                                      make_float2(set_lt(f.x, nl2tau), set_lt(f.y, nl2tau)),
+                                      acc[4 * g + x]);
+            }
+          }
+          if (kCount) neval += 16;
+        }
+        const int sw = part_swizzle(vt);
+#pragma unroll
+        for (int g = 0; g < 2; ++g) {
+          W.part[vt][(2 * g) ^ sw] = make_float4(acc[4 * g].x, acc[4 * g + 1].x, acc[4 * g + 2].x, acc[4 * g + 3].x);
+          W.part[vt][(2 * g + 1) ^ sw] = make_float4(acc[4 * g].y, acc[4 * g + 1].y, acc[4 * g + 2].y, acc[4 * g + 3].y);
+        }
+      }
+      if (lastw && threadIdx.x == 0) {  // every thread has read this task's descriptor
+        task_at(nq, W.desc[cd][0], W.desc[cd][1]);
+        nq = claim();
+      }
+      __syncthreads();
+      if (kCount) continue;
+      // a pixel's partials in thread order
+      float2 sum = make_float2(0.f, 0.f);
+      const bool own = W.pstart[ob + 1] > W.pstart[ob];
+      if (own) {
+        const int v1 = W.tfirst[ob + 1];
+        for (int v = W.tfirst[ob]; v < v1; ++v) {
+          const float2 x = reinterpret_cast<const float2 *>(&W.part[v][row ^ part_swizzle(v)])[id & 1];
+          sum.x += x.x;
+          sum.y += x.y;
+        }
+        if (nseg == 1) {
+          run0 = kahan_add(run0, sum.x);
+          run1 = kahan_add(run1, sum.y);
+        }
+      } else {
+        sum.x = sum.y = __uint_as_float(kNoSum);
+      }
+      if (nseg > 1) __stcg(part + (int64_t)(t1.x + w0 / kWin) * 128 + id, sum);
+    }
+    if (!kCount) {
+      float2 *out = reinterpret_cast<float2 *>(o + (4 * (ob >> 2) + row) * d + 4 * (ob & 3)) + (id & 1);
+      bool write = nseg == 1;
+      if (!write) {
+        // the tile's last CTA adds its windows
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) W.last = atomicAdd(tk.done + bt, 1u) == nseg - 1;
+        __syncthreads();
+        write = W.last;
+        if (write) {
+          __threadfence();
+          if (threadIdx.x == 0) tk.done[bt] = 0u;  // as the next call expects it
+#pragma unroll 4
+          for (unsigned g = 0; g < t1.w; ++g) {
+            const float2 x = __ldcg(part + (int64_t)g * 128 + id);
+            if (__float_as_uint(x.x) != kNoSum) {
+              run0 = kahan_add(run0, x.x);
+              run1 = kahan_add(run1, x.y);
+            }
           }
         }
-        if (kCount) neval += 16;
       }
-      __syncwarp();  // the slots are read before the next block's replace them
-      if (kCount) continue;
-      // 16 pixels x 32 lanes -> the pixel of lane pair (2 p, 2 p + 1)
-      float v8[8], v4[4], v2[2];
-      const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        // lanes with bit 4 clear keep rows 0 and 1, the others rows 2 and 3
-        const float2 keep = b4 ? acc[4 + x] : acc[x], give = b4 ? acc[x] : acc[4 + x];
-        v8[x] = keep.x + __shfl_xor_sync(0xffffffffu, give.x, 16);
-        v8[4 + x] = keep.y + __shfl_xor_sync(0xffffffffu, give.y, 16);
-      }
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-        v4[x] = (b3 ? v8[4 + x] : v8[x]) + __shfl_xor_sync(0xffffffffu, b3 ? v8[x] : v8[4 + x], 8);
-#pragma unroll
-      for (int x = 0; x < 2; ++x)
-        v2[x] = (b2 ? v4[2 + x] : v4[x]) + __shfl_xor_sync(0xffffffffu, b2 ? v4[x] : v4[2 + x], 4);
-      float v1 = (b1 ? v2[1] : v2[0]) + __shfl_xor_sync(0xffffffffu, b1 ? v2[0] : v2[1], 2);
-      v1 += __shfl_xor_sync(0xffffffffu, v1, 1);
-      if (!(lane & 1)) W.out[k][lane >> 1] = v1;
-      // the warp that finishes the window's last block writes its pixels
-      __threadfence_block();
-      __syncwarp();
-      int dn = 0;
-      if (lane == 0) dn = atomicAdd(&W.done, 1);
-      dn = __shfl_sync(0xffffffffu, dn, 0);
-      if (dn != 15) continue;
-      __threadfence_block();
-      // lane: half a pixel row of the tile, two blocks' rows of four
-      const int row = lane >> 1, k0 = 4 * (row >> 2) + 2 * (lane & 1), p0 = 4 * (row & 3);
-      float4 v[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) v[h] = *reinterpret_cast<const float4 *>(&W.out[k0 + h][p0]);
-      const unsigned nseg = W.nseg;
-      float4 *o = reinterpret_cast<float4 *>(proj + ((int64_t)b * d + y0 + row) * d + x0 + 8 * (lane & 1));
-      if (nseg > 1) {
-        float4 *part = reinterpret_cast<float4 *>(tk.part + (int64_t)W.part * 256) + 2 * lane;
-        __stcg(part + (int64_t)W.seg * 64, v[0]);
-        __stcg(part + (int64_t)W.seg * 64 + 1, v[1]);
-        __threadfence();
-        __syncwarp();
-        unsigned prev = 0;
-        if (lane == 0) prev = atomicAdd(tk.done + bt, 1u);
-        if (__shfl_sync(0xffffffffu, prev, 0) != nseg - 1) continue;
-        __threadfence();
-        float2 s[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) s[j] = make_float2(0.f, 0.f);
-        for (unsigned g = 0; g < nseg; ++g) {
-          const float4 a = __ldcg(part + (int64_t)g * 64), c4 = __ldcg(part + (int64_t)g * 64 + 1);
-          const float x[8] = {a.x, a.y, a.z, a.w, c4.x, c4.y, c4.z, c4.w};
-#pragma unroll
-          for (int j = 0; j < 8; ++j) s[j] = kahan_add(s[j], x[j]);
-        }
-        if (lane == 0) tk.done[bt] = 0u;  // as the next call expects it
-        v[0] = make_float4(s[0].x - s[0].y, s[1].x - s[1].y, s[2].x - s[2].y, s[3].x - s[3].y);
-        v[1] = make_float4(s[4].x - s[4].y, s[5].x - s[5].y, s[6].x - s[6].y, s[7].x - s[7].y);
-      }
-      o[0] = v[0];
-      o[1] = v[1];
+      if (write) *out = make_float2(run0.x - run0.y, run1.x - run1.y);
     }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&S.empty[it & 1]);
+    cd ^= 1;
   }
   if (kCount) {
     for (int o = 16; o > 0; o >>= 1) {
@@ -504,14 +460,8 @@ __global__ void __launch_bounds__(32 * (kCons + kProd), kMinB) raster_fwd_kernel
 
 // The forward's kernel configurations (the autotuner's search space).
 static const FwdCfg kFwdCfgs[] = {
-    {6, 2, 3, "6 consumer and 2 producer warps, 3 CTAs/SM"},
-    {8, 2, 3, "8 consumer and 2 producer warps, 3 CTAs/SM"},
-    {8, 4, 2, "8 consumer and 4 producer warps, 2 CTAs/SM"},
-    {12, 4, 2, "12 consumer and 4 producer warps, 2 CTAs/SM"},
-    {10, 2, 2, "10 consumer and 2 producer warps, 2 CTAs/SM"},
-    {6, 2, 2, "6 consumer and 2 producer warps, 2 CTAs/SM"},
-    {8, 2, 2, "8 consumer and 2 producer warps, 2 CTAs/SM"},
-    {12, 4, 1, "12 consumer and 4 producer warps, 1 CTA/SM"},
+    {8, "8 CTAs/SM"}, {7, "7 CTAs/SM"}, {6, "6 CTAs/SM"}, {5, "5 CTAs/SM"},
+    {4, "4 CTAs/SM"}, {3, "3 CTAs/SM"}, {2, "2 CTAs/SM"}, {1, "1 CTA/SM"},
 };
 int fwd_config_count() { return (int)(sizeof(kFwdCfgs) / sizeof(kFwdCfgs[0])); }
 const FwdCfg &fwd_config(int i) { return kFwdCfgs[i]; }
@@ -523,40 +473,9 @@ static int sm_count() {
   return sms;
 }
 
-// Partial images that any lists of up to cap entries can need: a tile of
-// more than S entries has fewer than 2 len / S segments, and S is at least
-// total / (2 slots) (at most 4 slots of them) or 1024.
-constexpr int kFwdSlots = 3 * 256;  // CTAs that fit up to 256 SMs
-size_t raster_part_count(int64_t cap) {
-  return (size_t)(4 * kFwdSlots + 2 * (cap / kFwdWin + 1));
-}
-
-template <int kCons, int kProd, int kMinB, bool kCount>
-static cudaError_t launch_fwd_one(int grid, const Rec *rec, const uint2 *list, int64_t M, int d,
-                                  float l2tau, const RasterTasks &tk, float *proj,
-                                  unsigned long long *kept, cudaStream_t st) {
-  raster_fwd_kernel<kCons, kProd, kMinB, kCount>
-      <<<grid, 32 * (kCons + kProd), sizeof(FwdShared<kCons>), st>>>(rec, list, M, d, l2tau, tk, proj, kept);
-  return cudaGetLastError();
-}
-
-template <int kCons, int kProd, int kMinB>
-static cudaError_t configure_fwd_one() {
-  const int smem = (int)sizeof(FwdShared<kCons>);
-  const cudaError_t e = cudaFuncSetAttribute(raster_fwd_kernel<kCons, kProd, kMinB, false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(raster_fwd_kernel<kCons, kProd, kMinB, true>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-}
-
-cudaError_t raster_configure() {
-  cudaError_t e;
-  if ((e = configure_fwd_one<6, 2, 3>()) != cudaSuccess || (e = configure_fwd_one<8, 2, 3>()) != cudaSuccess ||
-      (e = configure_fwd_one<8, 4, 2>()) != cudaSuccess || (e = configure_fwd_one<12, 4, 2>()) != cudaSuccess ||
-      (e = configure_fwd_one<10, 2, 2>()) != cudaSuccess)
-    return e;
-  return cudaSuccess;
+size_t raster_task_count(int64_t cap, int64_t ntiles) {
+  // one per tile, and one more per full segment
+  return (size_t)(ntiles + cap / kWin + 1);
 }
 
 template <bool kCount>
@@ -565,20 +484,19 @@ static cudaError_t launch_fwd_any(int cfg, const Rec *rec, const uint2 *list,
                                   float l2tau, float *proj, unsigned long long *kept,
                                   const RasterTasks &tk, bool fresh, cudaStream_t st) {
   if (cfg < 0 || cfg >= fwd_config_count()) return cudaErrorInvalidValue;
-  const FwdCfg &c = kFwdCfgs[cfg];
   const int nt = d / kTile, ntiles = nt * nt * B, sms = sm_count();
   if (!fresh) {
     const cudaError_t e = cudaMemsetAsync(tk.ctr, 0, kCtrCount * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
   }
   raster_tasks_kernel<<<(ntiles + 255) / 256, 256, 0, st>>>(tile_start, ntiles, cap, d,
-                                                            min(sms * 3, kFwdSlots), tk, proj);
-  const int grid = sms * c.ctas;
-  if (c.cons == 6) return launch_fwd_one<6, 2, 3, kCount>(grid, rec, list, M, d, l2tau, tk, proj, kept, st);
-  if (c.cons == 10) return launch_fwd_one<10, 2, 2, kCount>(grid, rec, list, M, d, l2tau, tk, proj, kept, st);
-  if (c.cons == 12) return launch_fwd_one<12, 4, 2, kCount>(grid, rec, list, M, d, l2tau, tk, proj, kept, st);
-  if (c.prod == 4) return launch_fwd_one<8, 4, 2, kCount>(grid, rec, list, M, d, l2tau, tk, proj, kept, st);
-  return launch_fwd_one<8, 2, 3, kCount>(grid, rec, list, M, d, l2tau, tk, proj, kept, st);
+                                                            sms * 8, tk, proj);
+  const int grid = sms * kFwdCfgs[cfg].ctas;
+  if (kFwdCfgs[cfg].ctas > 7)
+    raster_fwd_kernel<8, kCount><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tk, proj, kept);
+  else
+    raster_fwd_kernel<7, kCount><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tk, proj, kept);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_raster_fwd(int cfg, const Rec *rec, const uint2 *list,

@@ -1,6 +1,6 @@
 """Tile lists at the lengths where the rasterisers cut them: one tile (d = 16)
 that holds every Gaussian, so a list's length is the Gaussian count; the
-segments are 256 entries in small calls and 1024 in large ones, chunks of 32
+segments are 256 entries in small calls and 512 in large ones, chunks of 32
 and 64 entries inside them.  Held to the contract's tolerances (gemtest.py)."""
 import numpy as np
 import pytest
@@ -45,6 +45,6 @@ def test_list_lengths_in_a_small_call(M):
 
 @pytest.mark.parametrize("M", [1023, 1024, 1025, 2049])
 def test_list_lengths_in_a_large_call(M):
-    """About a million entries: segments of 1024.  tau = 0, so that no pair
+    """About a million entries: the longest segments.  tau = 0, so that no pair
     is near the threshold."""
     _check(M, 1 + 1000000 // M, seed=M, tau=0.0)
