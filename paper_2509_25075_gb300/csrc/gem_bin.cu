@@ -214,6 +214,115 @@ __global__ void __launch_bounds__(kDThreads) digit_scatter_kernel(
   }
 }
 
+// Both passes of one row in one CTA, the row's elements in shared memory
+// between them (index, high byte): one launch instead of six, for rows of up
+// to 24576 keys.  Warp w owns the w-th of 32 equal stretches of the row and
+// visits it in order, 32 elements at a time, as the chunked form does; the
+// per-warp digit counts are 16-bit (a stretch has at most 768 elements, an
+// offset is below 24576).
+constexpr int kRowThreads = 1024;
+constexpr int64_t kRowMax = 24576;
+constexpr int kRowWarps = kRowThreads / 32;
+static size_t row_smem(int64_t M) {
+  const size_t m = (size_t)((M + 15) / 16 * 16);
+  return (size_t)kRowWarps * 256 * sizeof(uint16_t) + m * (sizeof(uint16_t) + 1);
+}
+
+__global__ void __launch_bounds__(kRowThreads) sort16_row_kernel(const uint16_t *__restrict__ key,
+                                                                 int M, uint32_t *__restrict__ perm) {
+  extern __shared__ __align__(16) unsigned char row_sm[];
+  __shared__ uint32_t part[4][256];
+  __shared__ uint32_t wsum[8];
+  uint16_t(*wc)[256] = reinterpret_cast<uint16_t(*)[256]>(row_sm);
+  uint16_t *idx = reinterpret_cast<uint16_t *>(row_sm + kRowWarps * 256 * sizeof(uint16_t));
+  unsigned char *high = reinterpret_cast<unsigned char *>(idx + (M + 15) / 16 * 16);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
+  const uint16_t *kr = key + (int64_t)blockIdx.x * M;
+  uint32_t *pr = perm + (int64_t)blockIdx.x * M;
+  const int seg = (M + kRowThreads - 1) / kRowThreads * 32;
+  const int s0 = min(M, warp * seg), s1 = min(M, s0 + seg);
+  uint32_t *wcw = reinterpret_cast<uint32_t *>(wc[warp]);
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int i = lane; i < 128; i += 32) wcw[i] = 0u;
+    __syncwarp();
+    // two 16-bit counts per word: no count reaches 65536
+#pragma unroll 4
+    for (int e = s0 + lane; e < s1; e += 32) {
+      const unsigned dg = pass == 0 ? kr[e] & 255u : high[e];
+      atomicAdd(&wcw[dg >> 1], 1u << (16 * (dg & 1)));
+    }
+    __syncthreads();
+    // thread (g, bin): the bin's counts of warps 8 g .. 8 g + 7
+    {
+      const int bin = threadIdx.x & 255, g = threadIdx.x >> 8;
+      uint32_t v[8], sum = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        v[k] = wc[8 * g + k][bin];
+        sum += v[k];
+      }
+      part[g][bin] = sum;
+      __syncthreads();
+      uint32_t before = 0, tot = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t x = part[q][bin];
+        if (q < g) before += x;
+        tot += x;
+      }
+      uint32_t incl = tot;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+      }
+      if (g == 0 && lane == 31) wsum[bin >> 5] = incl;
+      __syncthreads();
+      uint32_t run = incl - tot + before;
+      for (int w = 0; w < (bin >> 5); ++w) run += wsum[w];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        wc[8 * g + k][bin] = (uint16_t)run;
+        run += v[k];
+      }
+    }
+    __syncthreads();
+    for (int e0 = s0; e0 < s1; e0 += 32) {
+      const int e = e0 + lane;
+      const bool act = e < s1;
+      int dg = 256 + lane;  // tail lanes: a value no digit has
+      unsigned hi = 0, j = (unsigned)e;
+      if (act) {
+        if (pass == 0) {
+          const unsigned k = kr[e];
+          dg = (int)(k & 255u);
+          hi = k >> 8;
+        } else {
+          dg = high[e];
+          j = idx[e];
+        }
+      }
+      const unsigned peers = e0 + 32 <= s1 ? same_value_lanes<8>(dg) : same_value_lanes<9>(dg);
+      unsigned pos = 0;
+      if (act) pos = wc[warp][dg] + __popc(peers & lt);
+      __syncwarp();
+      if (act && lane == __ffs(peers) - 1) wc[warp][dg] = (uint16_t)(pos + __popc(peers));
+      __syncwarp();
+      if (act) {
+        if (pass == 0) {
+          idx[pos] = (uint16_t)j;
+          high[pos] = (unsigned char)hi;
+        } else {
+          pr[pos] = j;
+        }
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // ------------------------------------------------------ tile binning ----
 
 // Geometry of the region e > log2(tau) - margin of one record, in pixel
@@ -843,12 +952,23 @@ static cudaError_t bin_configure_one(int d) {
                               (d / kTile) * (d / kTile) * (int)sizeof(uint32_t));
 }
 cudaError_t bin_configure(int d) {
-  const cudaError_t e = bin_configure_one<false>(d);
+  cudaError_t e = cudaFuncSetAttribute(sort16_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)row_smem(kRowMax));
+  if (e == cudaSuccess) e = bin_configure_one<false>(d);
   return e != cudaSuccess ? e : bin_configure_one<true>(d);
 }
 
 cudaError_t launch_sort16(const uint16_t *key, int64_t M, int B, uint32_t *dcnt,
                           uint32_t *packed, uint32_t *perm, cudaStream_t st) {
+  // A row in one CTA takes about 1.5 us per 1000 keys, in as many rounds as
+  // the rows need; the chunked form spreads a row over the SMs, at 18 us per
+  // million keys of all rows plus six launches.  us, row and chunked form:
+  // M 2000, B 32: 9, 27; M 20000, B 256: 60, 90; M 50000, B 64: 77, 60.  A few
+  // long rows would leave most SMs idle.
+  if (M <= 8192 || (M <= kRowMax && B >= 32)) {
+    sort16_row_kernel<<<B, kRowThreads, row_smem(M), st>>>(key, (int)M, perm);
+    return cudaGetLastError();
+  }
   int nch = (int)bin_chunks_depth(M);
   dim3 g(nch, B);
   // low byte, then high byte (LSD); ties keep index order
