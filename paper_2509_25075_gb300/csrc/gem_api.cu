@@ -42,9 +42,8 @@ struct gem_ctx {
   int nbg = 1;
   float *proj = nullptr;   // internal projection of gem_forward
   float *dproj = nullptr;  // internal adjoint of gem_forward
-  float2 *Z = nullptr;
   float2 *tw = nullptr;
-  double *lossp = nullptr;
+  CtfScratch ctf{};
   int *status = nullptr;
   unsigned long long *kept = nullptr;
   KnnScratch knn{};
@@ -279,8 +278,10 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
             alloc(c, &c->part, (size_t)c->nbg * g.max_M * kNpar) &&
             alloc(c, &c->proj, (size_t)g.max_B * d * d) &&
             alloc(c, &c->dproj, (size_t)g.max_B * d * d) &&
-            alloc(c, &c->Z, (size_t)g.max_B * d * d) && alloc(c, &c->tw, (size_t)d) &&
-            alloc(c, &c->lossp, (size_t)g.max_B * (ctf_partials(d) + 1)) && alloc(c, &c->status, 1) &&
+            alloc(c, &c->ctf.Z, (size_t)g.max_B * d * d) && alloc(c, &c->tw, (size_t)d) &&
+            alloc(c, &c->ctf.lossp, (size_t)g.max_B * (ctf_partials(d) + 1)) &&
+            alloc(c, &c->ctf.consts, (size_t)g.max_B * kCtfConstFloats) &&
+            alloc(c, &c->ctf.done, (size_t)g.max_B + 1) && alloc(c, &c->status, 1) &&
             alloc(c, &c->kept, 2);
   ok = ok && alloc(c, &c->tasks.task, 2 * raster_task_count(c->cfg.max_pairs, (int64_t)g.max_B * c->T)) &&
        alloc(c, &c->tasks.done, (size_t)g.max_B * c->T) &&
@@ -326,6 +327,7 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
           cudaSuccess ||
       (e = cudaMemset(c->status, 0, sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(c->knn.ticket, 0, sizeof(int))) != cudaSuccess ||
+      (e = cudaMemset(c->ctf.done, 0, ((size_t)g.max_B + 1) * sizeof(unsigned))) != cudaSuccess ||
       (e = cudaMemset(c->tasks.done, 0, (size_t)g.max_B * c->T * sizeof(unsigned))) != cudaSuccess ||
       (e = bin_configure(d)) != cudaSuccess || (e = ctf_configure(d)) != cudaSuccess) {
     snprintf(g_create_err, sizeof(g_create_err), "set-up: %s", cudaGetErrorString(e));
@@ -473,9 +475,9 @@ int gem_ctf_loss(gem_ctx *c, int32_t B, const float *proj, const float *ctf,
     return fail(c, GEM_EINVAL, "pass exactly one of ctf and ctf_params");
   if (B < 1 || B > c->cfg.max_B)
     return fail(c, GEM_EINVAL, "B=%d outside 1..max_B=%d", B, c->cfg.max_B);
-  StageScope sc(c, GEM_STAGE_CTF, 3 + (loss_img || loss ? 1 : 0) + (loss ? 1 : 0));
+  StageScope sc(c, GEM_STAGE_CTF, 3);
   cudaError_t e = launch_ctf_loss(c->cfg.d, B, c->cfg.apix, c->tw, proj, ctf,
-                                  ctf_params, images, c->Z, c->lossp, pred, dproj, loss_img,
+                                  ctf_params, images, c->ctf, pred, dproj, loss_img,
                                   loss, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "ctf_loss");
   return GEM_OK;

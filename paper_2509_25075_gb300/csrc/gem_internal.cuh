@@ -388,9 +388,16 @@ cudaError_t launch_fsc(int d, float apix, float thr, const float2 *tw, const flo
                        const float *X2, float2 *P, float2 *Q, double *part, double *fsc,
                        double *sums, double *resolution, cudaStream_t st);
 
+constexpr int kCtfConstFloats = 16;  // room for an image's CTF constants
+struct CtfScratch {
+  float2 *Z;       // [B][d][d] spectrum
+  double *lossp;   // [B * (partials + 1)]
+  float *consts;   // [B][kCtfConstFloats]
+  unsigned *done;  // [B + 1] counters, zero between calls
+};
 cudaError_t launch_ctf_loss(int d, int B, float apix, const float2 *tw,
                             const float *proj, const float *ctf, const float *ctf_params,
-                            const float *images, float2 *Z, double *lossp, float *pred,
+                            const float *images, const CtfScratch &s, float *pred,
                             float *dproj, double *loss_img, double *loss, cudaStream_t st);
 
 }  // namespace gem

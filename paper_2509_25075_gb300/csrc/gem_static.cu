@@ -24,16 +24,18 @@ namespace {
 constexpr int64_t kStaticSpectrum = 1 << 20;  // float2 elements
 constexpr int64_t kStaticLoss = 1 << 16;      // doubles
 constexpr int kStaticMaxD = 768;
+constexpr int kStaticMaxB = kStaticSpectrum / (16 * 16);  // the smallest side is 16
 
 // The arrays' names are host-side stand-ins in host code: their device
 // addresses come from cudaGetSymbolAddress, once per device.
 __device__ __align__(256) float2 g_spectrum[kStaticSpectrum];
 __device__ __align__(256) double g_lossp[kStaticLoss];
 __device__ __align__(256) float2 g_twiddle[kStaticMaxD];
+__device__ __align__(256) float g_consts[kStaticMaxB * kCtfConstFloats];
+__device__ __align__(256) unsigned g_done[kStaticMaxB + 1];  // zero when the module loads
 
 struct StaticScratch {
-  float2 *spectrum = nullptr;
-  double *lossp = nullptr;
+  CtfScratch ctf{};
   float2 *twiddle = nullptr;
   bool ready = false;
 };
@@ -52,8 +54,10 @@ cudaError_t static_scratch(int dev, StaticScratch &out) {
   StaticScratch &s = g_scratch[dev];
   if (!s.ready) {
     cudaError_t e;
-    if ((e = cudaGetSymbolAddress((void **)&s.spectrum, g_spectrum)) != cudaSuccess) return e;
-    if ((e = cudaGetSymbolAddress((void **)&s.lossp, g_lossp)) != cudaSuccess) return e;
+    if ((e = cudaGetSymbolAddress((void **)&s.ctf.Z, g_spectrum)) != cudaSuccess) return e;
+    if ((e = cudaGetSymbolAddress((void **)&s.ctf.lossp, g_lossp)) != cudaSuccess) return e;
+    if ((e = cudaGetSymbolAddress((void **)&s.ctf.consts, g_consts)) != cudaSuccess) return e;
+    if ((e = cudaGetSymbolAddress((void **)&s.ctf.done, g_done)) != cudaSuccess) return e;
     if ((e = cudaGetSymbolAddress((void **)&s.twiddle, g_twiddle)) != cudaSuccess) return e;
     s.ready = true;
   }
@@ -107,8 +111,11 @@ extern "C" int gem_ctf_loss_static(int32_t d, float apix, int32_t B, const float
   cudaStream_t st = (cudaStream_t)cuda_stream;
   static_twiddle_kernel<<<(d + 255) / 256, 256, 0, st>>>(s.twiddle, d);
   if (cudaGetLastError() != cudaSuccess) return GEM_ECUDA;
-  if (launch_ctf_loss(d, B, apix, s.twiddle, proj, ctf, ctf_params, images, s.spectrum,
-                      s.lossp, pred, dproj, loss_img, loss, st) != cudaSuccess)
+  // the counters are shared by every caller: whatever a call that overlapped
+  // with another one left in them goes
+  if (cudaMemsetAsync(s.ctf.done, 0, (size_t)(B + 1) * sizeof(unsigned), st) != cudaSuccess)
+    return GEM_ECUDA;
+  if (launch_ctf_loss(d, B, apix, s.twiddle, proj, ctf, ctf_params, images, s.ctf, pred, dproj, loss_img, loss, st) != cudaSuccess)
     return GEM_ECUDA;
   return GEM_OK;
 }
