@@ -13,7 +13,7 @@
 //   [z][y][x] -> [kx][z][y] -> [ky][kx][z] -> [kz][ky][kx].
 // Each pass reads and writes the volume once; its stages meet shared memory
 // once or twice (gem_fft.cuh).  Same bits as a round trip per stage: two
-// 256^3 maps 664 -> 292 us.
+// 256^3 maps 664 -> 293 us, the shell sums as they were.
 #include <math.h>
 
 #include "gem_fft.cuh"
@@ -22,7 +22,7 @@
 namespace gem {
 
 constexpr int kFThreads = 256;
-constexpr int kShellBlocks = 608;  // 4 per SM on 152 SMs
+constexpr int kShellBlocks = 1216;  // 8 per SM on 152 SMs
 // Lines per CTA of the transform passes: 16 (their transposed stores then
 // fill 128-byte lines) up to sides whose 16 lines leave room for four CTAs
 // per SM, else 8.
@@ -74,81 +74,143 @@ __global__ void __launch_bounds__(kFThreads) fsc_pass_cplx_kernel(const float2 *
 }
 
 // Shell of a frequency with squared norm k2: the integer s with
-// (s - 1/2)^2 <= k2 < (s + 1/2)^2, i.e. 4 s^2 - 4 s + 1 <= 4 k2 < 4 s^2 + 4 s + 1.
+// (s - 1/2)^2 <= k2 < (s + 1/2)^2.  No k2 comes closer to a boundary than
+// s^2 - s, whose root lies 1 / (8 s) below it: far more than the rounding of
+// the root and of the sum for every s <= 1024.
 __device__ __forceinline__ int shell_of(int k2) {
-  int s = (int)floorf(sqrtf((float)k2) + 0.5f);
-  while (s > 0 && 4 * k2 < 4 * s * s - 4 * s + 1) --s;
-  while (4 * k2 >= 4 * s * s + 4 * s + 1) ++s;
-  return s;
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"((float)k2));
+  return (int)(r + 0.5f);
 }
 
-// Inclusive sum of v over the run of equal keys ending at each lane (runs
-// are maximal sequences of consecutive lanes with the same key; bit l of
-// run_mask is set when lane l continues the run of lane l - 1).
-__device__ __forceinline__ float seg_scan(float v, int lane, unsigned run_mask) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const float u = __shfl_up_sync(0xffffffffu, v, o);
-    // lane - o lies in the same run iff every lane in (lane - o, lane] does
-    const unsigned need = ((1u << o) - 1u) << (lane - o + 1);
-    if (lane >= o && (run_mask & need) == need) v += u;
-  }
-  return v;
+// One step of an inclusive sum over the run of equal keys ending at each lane:
+// add the value o lanes below where that lane belongs to the run.
+__device__ __forceinline__ float seg_add(float v, int o, bool take) {
+  const float u = __shfl_up_sync(0xffffffffu, v, o);
+  return take ? v + u : v;
 }
 
 // Per-block sums over the shells 0 .. nsh-1 of Re(F1 F2^*), |F1|^2, |F2|^2,
 // written to part[blk][3][nsh].  A warp takes 32 consecutive frequencies;
 // neighbouring frequencies mostly share a shell, so each run of equal shells
 // (at most 32 terms) is summed in float32 by a segmented warp scan and added
-// to the block's float64 accumulators once.  Voxel indices fit in 32 bits
-// (d <= 768).
-__global__ void __launch_bounds__(kFThreads) fsc_shell_kernel(const float2 *__restrict__ F,
-                                                              int d, int nsh,
+// once to the warp's own sums in shared memory.  Within half a row the shell
+// is monotone, so the runs of one step have different shells and the sums
+// need no atomics.
+//
+// A sum is a pair of floats, its value and the rounding errors of that value
+// (exact, by Knuth's two-sum), converted to float64 when the block is done:
+// this GPU's float64 adds run at a 64th of its float32 adds, and three of
+// them and their conversions per step were the kernel's bound.  The pair's
+// error is 2^-48 of the sum per addition, against the 2^-24 of the runs.
+// Runs of 1e30 and more, infinities and NaN go to float64 sums of their own.
+//
+// Then the instructions bound it, and after them the load: the part of the
+// volume inside the last shell (half of it), once.  A unit is the least whole
+// number q of rows that 32 divides (two rows on sides like 48 or 432, else
+// one), so a warp works out row numbers once per unit, and steps beyond the
+// last shell load and sum nothing.  The warp follows a unit with its mirror
+// image, which then finds both its operands in L1.  Against one pass over all
+// frequencies with divisions, two loads each and float64 atomics: side 256,
+// the whole call 293 -> 219 us (287 with float64 sums).
+template <int N>
+__global__ void __launch_bounds__(kFThreads) fsc_shell_kernel(const float2 *__restrict__ F, int nsh,
                                                               double *__restrict__ part) {
-  extern __shared__ double acc[];  // [3][nsh]
-  for (int i = threadIdx.x; i < 3 * nsh; i += blockDim.x) acc[i] = 0.0;
+  constexpr int q = N % 32 ? 2 : 1, h = N / 2, kUnits = N / q;  // units per plane
+  static_assert(q * N % 32 == 0, "a unit is whole warps");
+  constexpr int kWarps = kFThreads / 32;
+  extern __shared__ double big[];  // [3][nsh], then the warps' pairs [kWarps][3][nsh]
+  float2 *acc = reinterpret_cast<float2 *>(big + 3 * nsh);
+  for (int i = threadIdx.x; i < 3 * nsh; i += kFThreads) big[i] = 0.0;
+  for (int i = threadIdx.x; i < kWarps * 3 * nsh; i += kFThreads) acc[i] = make_float2(0.f, 0.f);
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const unsigned n = (unsigned)d * d * d, ud = (unsigned)d;
-  const int h = d / 2;
-  const unsigned stride = gridDim.x * blockDim.x;
-  for (unsigned base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < n; base += stride) {
-    const unsigned i = base + lane;
-    int s = nsh;  // out of range: contributes nothing
-    float num = 0.f, p1 = 0.f, p2 = 0.f;
-    if (i < n) {
-      const unsigned row = i / ud;
-      const int kx = (int)(i - row * ud), ky = (int)(row % ud), kz = (int)(row / ud);
-      const int sx = kx < h ? kx : kx - d, sy = ky < h ? ky : ky - d, sz = kz < h ? kz : kz - d;
-      s = shell_of(sx * sx + sy * sy + sz * sz);
-      if (s < nsh) {
-        const int mx = kx ? d - kx : 0, my = ky ? d - ky : 0, mz = kz ? d - kz : 0;
-        const float2 Z = F[i];
-        const float2 Zm = F[((unsigned)mz * ud + (unsigned)my) * ud + (unsigned)mx];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float2 *mine = acc + warp * 3 * nsh;
+  auto add = [&](int k, float v) {
+    if (fabsf(v) < 1e30f) {
+      const float2 a = mine[k];
+      const float t = a.x + v, w = t - a.x;
+      mine[k] = make_float2(t, a.y + ((a.x - (t - w)) + (v - w)));
+    } else {
+      atomicAdd(&big[k], (double)v);
+    }
+  };
+  const int lim = nsh * nsh - nsh + 1;  // the last shell is nsh - 1: k2 < lim
+  const int nunit = (h + 1) * kUnits, step = gridDim.x * kWarps;
+  for (int u2 = 2 * (blockIdx.x * kWarps + warp); u2 < 2 * nunit; u2 += (u2 & 1) ? 2 * step - 1 : 1) {
+    int kz = (u2 >> 1) / kUnits, j = (u2 >> 1) - kz * kUnits;
+    if (u2 & 1) {  // the mirror image; a plane that is its own is done already
+      if (kz == 0 || kz == h) continue;
+      kz = N - kz;
+      j = j ? kUnits - j : 0;
+    }
+    const int sz = kz < h ? kz : kz - N, z2 = sz * sz;
+    const int mz = kz ? N - kz : 0;
+    const int ky0 = j * q;
+#pragma unroll 2
+    for (int i0 = 0; i0 < q * N; i0 += 32) {
+      const int e = i0 + lane, r = q > 1 && e >= N ? 1 : 0;
+      const int kx = e - r * N, ky = ky0 + r;
+      const int sx = kx < h ? kx : kx - N, sy = ky < h ? ky : ky - N;
+      const int k2 = sx * sx + sy * sy + z2;
+      const bool in = k2 < lim;
+      if (!__any_sync(0xffffffffu, in)) continue;
+      int s = nsh;  // out of range: contributes nothing
+      float num = 0.f, p1 = 0.f, p2 = 0.f;
+      if (in) {
+        s = shell_of(k2);
+        const int mx = kx ? N - kx : 0, my = ky ? N - ky : 0;
+        const float2 Z = F[(kz * N + ky) * N + kx];
+        const float2 Zm = F[(mz * N + my) * N + mx];
         const float f1r = 0.5f * (Z.x + Zm.x), f1i = 0.5f * (Z.y - Zm.y);
         const float f2r = 0.5f * (Z.y + Zm.y), f2i = -0.5f * (Z.x - Zm.x);
         num = fmaf(f1r, f2r, f1i * f2i);
         p1 = fmaf(f1r, f1r, f1i * f1i);
         p2 = fmaf(f2r, f2r, f2i * f2i);
-      } else {
-        s = nsh;
       }
-    }
-    const int prev = __shfl_up_sync(0xffffffffu, s, 1);
-    const unsigned run_mask = __ballot_sync(0xffffffffu, lane > 0 && prev == s);
-    num = seg_scan(num, lane, run_mask);
-    p1 = seg_scan(p1, lane, run_mask);
-    p2 = seg_scan(p2, lane, run_mask);
-    const int next = __shfl_down_sync(0xffffffffu, s, 1);
-    if ((lane == 31 || next != s) && s < nsh) {
-      atomicAdd(&acc[s], (double)num);
-      atomicAdd(&acc[nsh + s], (double)p1);
-      atomicAdd(&acc[2 * nsh + s], (double)p2);
+      const int prev = __shfl_up_sync(0xffffffffu, s, 1);
+      // bit l of m: lanes l - o .. l share a run
+      unsigned m = __ballot_sync(0xffffffffu, lane > 0 && prev == s);
+      const bool last = lane == 31 || !(m >> (lane + 1) & 1u);
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        if (!m) break;
+        const bool take = m >> lane & 1u;
+        num = seg_add(num, o, take);
+        p1 = seg_add(p1, o, take);
+        p2 = seg_add(p2, o, take);
+        m &= m << o;
+      }
+      const bool write = last && s < nsh;
+      if (i0 / h == (i0 + 31) / h) {
+        if (write) {
+          add(s, num);
+          add(nsh + s, p1);
+          add(2 * nsh + s, p2);
+        }
+      } else {  // rows' halves meet here: one run at a time
+        for (unsigned w = __ballot_sync(0xffffffffu, write); w; w &= w - 1) {
+          if (lane == __ffs(w) - 1) {
+            add(s, num);
+            add(nsh + s, p1);
+            add(2 * nsh + s, p2);
+          }
+          __syncwarp();
+        }
+      }
+      __syncwarp();
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 3 * nsh; i += blockDim.x)
-    part[(size_t)blockIdx.x * 3 * nsh + i] = acc[i];
+  for (int i = threadIdx.x; i < 3 * nsh; i += kFThreads) {
+    double t = big[i];
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+      const float2 a = acc[w * 3 * nsh + i];
+      t += (double)a.x + (double)a.y;
+    }
+    part[(size_t)blockIdx.x * 3 * nsh + i] = t;
+  }
 }
 
 // One block per shell: the block sums in a fixed order.
@@ -185,6 +247,8 @@ __global__ void __launch_bounds__(512) fsc_final_kernel(const double *__restrict
                                                         double *__restrict__ sums,
                                                         double *__restrict__ resolution) {
   extern __shared__ double f[];  // [nsh]
+  __shared__ int first;          // the first shell below the threshold
+  if (threadIdx.x == 0) first = nsh;
   for (int s = threadIdx.x; s < nsh; s += blockDim.x) {
     const double a = tot[s], b = tot[nsh + s], c = tot[2 * nsh + s];
     const double den = sqrt(b * c);
@@ -197,25 +261,31 @@ __global__ void __launch_bounds__(512) fsc_final_kernel(const double *__restrict
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0 && resolution) {
+  if (!resolution) return;
+  for (int s = 1 + threadIdx.x; s < nsh; s += blockDim.x)
+    if (f[s] < thr) atomicMin(&first, s);
+  __syncthreads();
+  if (threadIdx.x == 0) {
     double kstar = (double)(nsh - 1);
-    for (int s = 1; s < nsh; ++s) {
-      if (f[s] < thr) {
-        const double a = f[s - 1], b = f[s];
-        const double frac = a > b ? (a - thr) / (a - b) : 0.0;
-        kstar = (s - 1) + fmin(fmax(frac, 0.0), 1.0);
-        break;
-      }
+    if (first < nsh) {
+      const double a = f[first - 1], b = f[first];
+      const double frac = a > b ? (a - thr) / (a - b) : 0.0;
+      kstar = (first - 1) + fmin(fmax(frac, 0.0), 1.0);
     }
     resolution[0] = kstar > 0.0 ? (double)d * apix / kstar : INFINITY;
   }
 }
 
+static int shell_smem(int nsh) { return (kFThreads / 32 + 1) * 3 * nsh * (int)sizeof(double); }
+
 template <int N>
 static cudaError_t fsc_configure_side() {
   const int smem = (int)sizeof(FscSmem<N>);
-  const cudaError_t e = cudaFuncSetAttribute(fsc_pass_real_kernel<N>,
+  cudaError_t e = cudaFuncSetAttribute(fsc_pass_real_kernel<N>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fsc_shell_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             shell_smem(N / 2 + 1));
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(fsc_pass_cplx_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               smem);
@@ -234,12 +304,14 @@ cudaError_t fsc_configure(int d) {
 
 template <int N>
 static void launch_fsc_passes(const float2 *tw, const float *X1, const float *X2, float2 *P, float2 *Q,
-                              cudaStream_t st) {
+                              double *part, cudaStream_t st) {
   const size_t smem = sizeof(FscSmem<N>);
   const dim3 g(N / fsc_lines(N), N);
   fsc_pass_real_kernel<N><<<g, kFThreads, smem, st>>>(X1, X2, tw, P);
   fsc_pass_cplx_kernel<N><<<g, kFThreads, smem, st>>>(P, tw, Q);
   fsc_pass_cplx_kernel<N><<<g, kFThreads, smem, st>>>(Q, tw, P);
+  const int nsh = N / 2 + 1;
+  fsc_shell_kernel<N><<<kShellBlocks, kFThreads, shell_smem(nsh), st>>>(P, nsh, part);
 }
 
 // block partials, then the folded sums
@@ -249,9 +321,9 @@ cudaError_t launch_fsc(int d, float apix, float thr, const float2 *tw, const flo
                        const float *X2, float2 *P, float2 *Q, double *part, double *fsc,
                        double *sums, double *resolution, cudaStream_t st) {
   switch (d) {
-#define X(N)                                     \
-  case N:                                        \
-    launch_fsc_passes<N>(tw, X1, X2, P, Q, st);  \
+#define X(N)                                          \
+  case N:                                             \
+    launch_fsc_passes<N>(tw, X1, X2, P, Q, part, st); \
     break;
     GEM_FFT_SIDES(X)
 #undef X
@@ -259,7 +331,6 @@ cudaError_t launch_fsc(int d, float apix, float thr, const float2 *tw, const flo
       return cudaErrorInvalidValue;
   }
   const int nsh = d / 2 + 1;
-  fsc_shell_kernel<<<kShellBlocks, kFThreads, 3 * nsh * sizeof(double), st>>>(P, d, nsh, part);
   double *tot = part + (size_t)kShellBlocks * 3 * nsh;
   fsc_fold_kernel<<<nsh, 256, 0, st>>>(part, kShellBlocks, nsh, tot);
   fsc_final_kernel<<<1, 512, nsh * sizeof(double), st>>>(tot, nsh, d, apix, thr, fsc, sums,
