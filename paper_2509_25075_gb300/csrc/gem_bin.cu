@@ -339,15 +339,16 @@ struct RowGeo {
   float px, py;  // centre
   float k4a, D;  // 4 al kap (infinite when tau = 0), 4 al ga - be^2
   float i2a, sl; // 1 / (2 al), -be / (2 al)
-  float dyL;
-  float xext, yext;
+  float dyL, yext;
 };
 
 // The approximate square roots and divisions (a few ulp) are absorbed by the
-// margin already in kap, so the ranges stay supersets of the exact ones.
+// margin already in kap, so the ranges stay supersets of the exact ones.  (A
+// rounding of the root's argument is one of kap.)
 __device__ __forceinline__ float sqrt_approx(float x) {
-  x = fmaxf(x, 0.f);
-  return x * rsqrtf(fmaxf(x, 1e-30f));
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 0.f)));
+  return r;
 }
 
 __device__ __forceinline__ RowGeo make_row_geo(const Rec &r, float l2tau) {
@@ -365,44 +366,56 @@ __device__ __forceinline__ RowGeo make_row_geo(const Rec &r, float l2tau) {
   G.D = t * t;
   G.k4a = 4.f * al * kap;
   const float iD = __fdividef(1.f, G.D);
-  G.xext = sqrt_approx(4.f * ga * kap * iD);
+  const float xext = sqrt_approx(4.f * ga * kap * iD);
   G.yext = sqrt_approx(G.k4a * iD);
-  G.dyL = be * G.xext * __fdividef(0.5f, ga);
+  G.dyL = be * xext * __fdividef(0.5f, ga);
+  if (!(fabsf(G.dyL) < INFINITY && fabsf(G.sl) < INFINITY)) {
+    // tau = 0, or a region too wide or thin for float32: whole rows
+    G.k4a = G.yext = INFINITY;
+    G.D = G.sl = G.dyL = 0.f;
+    G.i2a = 1.f;
+  }
   return G;
 }
 
-// Block columns (4-pixel columns of the whole image, 0 .. nb-1) that the
-// region meets in block row by (pixel rows 4 by .. 4 by + 3), packed as
-// lo | hi << 8, or kNoRow.  Inside the strip the region's x-range is
-// [c - h, c + h] at the strip's two ends, widened to the region's own
-// x-extreme where the strip contains the row that reaches it.  Every
-// rounding step is explicit (no contraction the compiler could choose per
-// call site), so each inlined copy returns the same bits for the same input.
-constexpr unsigned kNoRow = 0x00ffu;  // lo = 255 > hi = 0
-// sqrt_approx with its product rounded on its own (never fused into a
-// neighbouring add)
-__device__ __forceinline__ float sqrt_rn_approx(float x) {
-  x = fmaxf(x, 0.f);
-  return __fmul_rn(x, rsqrtf(fmaxf(x, 1e-30f)));
-}
-__device__ __forceinline__ unsigned block_row_range(const RowGeo &G, int by, int nb) {
-  if (!(G.k4a < INFINITY)) return (unsigned)(nb - 1) << 8;  // tau = 0: every pixel counts
-  float a = __fsub_rn((float)(4 * by), G.py), b = __fadd_rn(a, 3.f);
+// The region's pixel columns [xl, xr] in the four pixel rows y0 .. y0 + 3;
+// false when it does not reach them.  Its left edge c - h is convex in dy with
+// its minimum at dyL, and its right edge is the left one's image in the
+// centre, so the strip's extremes are the edges at dyL and -dyL clamped to the
+// strip: two square roots and no comparison of candidates.  No product feeds
+// a plain sum, so there is nothing to contract and each inlined copy returns
+// the same bits.  (The counting pass is bound by issue, 78% of its slots, and
+// the integer pipe, 69%: against four candidate edges, two of them chosen by
+// comparison, and masks built per tile and row, a gradient step takes 1514 ->
+// 1488 us at d 128, M 20000, B 256 and 1674 -> 1654 us at d 128, M 50000,
+// B 64, scales 0.3-12 px.)
+__device__ __forceinline__ bool row_span(const RowGeo &G, float y0, float &xl, float &xr) {
+  float a = y0 - G.py, b = a + 3.f;
   a = fmaxf(a, -G.yext);
   b = fminf(b, G.yext);
-  if (!(a <= b)) return kNoRow;
-  const float ha = __fmul_rn(sqrt_rn_approx(__fmaf_rn(__fmul_rn(-G.D, a), a, G.k4a)), G.i2a);
-  const float hb = __fmul_rn(sqrt_rn_approx(__fmaf_rn(__fmul_rn(-G.D, b), b, G.k4a)), G.i2a);
-  const float ca = __fmul_rn(G.sl, a), cb = __fmul_rn(G.sl, b);
-  float xmin = fminf(__fsub_rn(ca, ha), __fsub_rn(cb, hb));
-  float xmax = fmaxf(__fadd_rn(ca, ha), __fadd_rn(cb, hb));
-  if (G.dyL >= a && G.dyL <= b) xmin = -G.xext;
-  if (-G.dyL >= a && -G.dyL <= b) xmax = G.xext;
-  // columns bx whose pixel centres [4 bx, 4 bx + 3] meet [px + xmin, px + xmax]
-  const float lo = fmaxf(ceilf(__fmul_rn(__fsub_rn(__fadd_rn(G.px, xmin), 3.f), 0.25f)), 0.f);
-  const float hi = fminf(floorf(__fmul_rn(__fadd_rn(G.px, xmax), 0.25f)), (float)(nb - 1));
-  if (!(lo <= hi)) return kNoRow;
-  return (unsigned)lo | ((unsigned)hi << 8);
+  const float ql = fminf(fmaxf(G.dyL, a), b), qr = fminf(fmaxf(-G.dyL, a), b);
+  xl = G.px + fmaf(-sqrt_approx(fmaf(-G.D * ql, ql, G.k4a)), G.i2a, G.sl * ql);
+  xr = G.px + fmaf(sqrt_approx(fmaf(-G.D * qr, qr, G.k4a)), G.i2a, G.sl * qr);
+  return a <= b;
+}
+
+// Block columns (4-pixel columns) lo .. hi within [first, last] whose pixels
+// meet [xl, xr]: 4 hi <= xr and 4 lo + 3 >= xl.  A NaN edge takes all of them.
+__device__ __forceinline__ int first_column(float xl, float first) {
+  return __float2int_ru(fmaxf(fmaf(xl, 0.25f, -0.75f), first));
+}
+__device__ __forceinline__ int last_column(float xr, float last) {
+  return __float2int_rd(fminf(xr * 0.25f, last));
+}
+
+// Block columns (0 .. nb-1 of the whole image) that the region meets in block
+// row by (pixel rows 4 by .. 4 by + 3), packed as lo | hi << 8, or kNoRow.
+constexpr unsigned kNoRow = 0x00ffu;  // lo = 255 > hi = 0
+__device__ __forceinline__ unsigned block_row_range(const RowGeo &G, int by, int nb) {
+  float xl, xr;
+  if (!row_span(G, (float)(4 * by), xl, xr)) return kNoRow;
+  const int lo = first_column(xl, 0.f), hi = last_column(xr, (float)(nb - 1));
+  return lo <= hi ? (unsigned)lo | ((unsigned)hi << 8) : kNoRow;
 }
 
 // Shared staging of one chunk of 256 Gaussians (depth order): each
@@ -611,31 +624,36 @@ __global__ void __launch_bounds__(kChunkT, 6) tile_count_kernel(
     }
   }
   // this thread's own Gaussian when it meets at most 2 x 2 tiles (after its
-  // share of the candidates, so that one barrier waits for both): the masks
-  // of tiles (ty0 + a, tx0 + q) in sm[2 a + q], each row's range clipped to
-  // each tile column as candidate_mask clips it
+  // share of the candidates, so that one barrier waits for both): each block
+  // row's eight columns are a byte of the upper or the lower tiles' word, and
+  // the masks of tiles (ty0 + a, tx0 + q) in sm[2 a + q] are its nibbles
   unsigned sm0 = 0, sm1 = 0, sm2 = 0, sm3 = 0;
   int nhs = 0;
   if (sbx.w > 0) {
     const RowGeo myg = S.geo[threadIdx.x];
-    for (int by = sbx.by0; by <= sbx.by1; ++by) {
-      const unsigned v = block_row_range(myg, by, nb);
-      const int lo = (int)(v & 255u), hi = (int)(v >> 8), sh = 4 * (by & 3);
-      const int bx0 = 4 * sbx.tx0;
-      unsigned c0 = 0, c1 = 0;
-      int l = max(lo, bx0), h = min(hi, bx0 + 3);
-      if (l <= h) c0 = ((1u << (h - l + 1)) - 1u) << (sh + l - bx0);
-      l = max(lo, bx0 + 4);
-      h = min(hi, bx0 + 7);
-      if (sbx.w > 1 && l <= h) c1 = ((1u << (h - l + 1)) - 1u) << (sh + l - bx0 - 4);
-      if ((by >> 2) == sbx.ty0) {
-        sm0 |= c0;
-        sm1 |= c1;
-      } else {
-        sm2 |= c0;
-        sm3 |= c1;
+    const int bx0 = 4 * sbx.tx0;
+    const float first = (float)bx0, last = (float)(bx0 + 4 * sbx.w - 1);
+    unsigned upper = 0, lower = 0;
+    float y0 = (float)(4 * sbx.by0);
+    for (int by = sbx.by0; by <= sbx.by1; ++by, y0 += 4.f) {
+      float xl, xr;
+      const bool some = row_span(myg, y0, xl, xr);
+      const int l = first_column(xl, first) - bx0, h = last_column(xr, last) - bx0;
+      if (some && l <= h) {  // 0 <= l, h <= 7
+        const unsigned v = ((2u << h) - (1u << l)) << (8 * (by & 3));
+        if ((by >> 2) == sbx.ty0) upper |= v;
+        else lower |= v;
       }
     }
+    auto nibbles = [](unsigned v) {
+      v &= 0x0f0f0f0fu;
+      v = (v | (v >> 4)) & 0x00ff00ffu;
+      return (v | (v >> 8)) & 0xffffu;
+    };
+    sm0 = nibbles(upper);
+    sm1 = nibbles(upper >> 4);
+    sm2 = nibbles(lower);
+    sm3 = nibbles(lower >> 4);
     const int t0 = sbx.ty0 * nt + sbx.tx0;
     if (sm0) atomicAdd(&tc[t0], 1u), ++nhs;
     if (sm1) atomicAdd(&tc[t0 + 1], 1u), ++nhs;
