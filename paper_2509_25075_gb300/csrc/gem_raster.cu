@@ -515,70 +515,89 @@ cudaError_t launch_count_kept(int cfg, const Rec *rec, const uint2 *list,
                               false, st);
 }
 
+// Sum of two packed pairs, rounded on its own: no product that goes into it is
+// contracted with it.
+__device__ __forceinline__ float2 add2_apart(float2 a, float2 b) {
+  float2 r;
+  asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
+      "add.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+      : "=f"(r.x), "=f"(r.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return r;
+}
+
 // The six moments of w = g * value over the 16 pixels of block k of the tile
 // at (x0, y0) for one record (centre A.x, A.y, first row of U in A.z, A.w;
 // u22, l2A), in the record's whitened coordinates z1 = u11 dx + u12 dy,
-// z2 = u22 dy, added to the running totals n[0..5], each a pair (upper rows
-// of the row pairs, lower rows):
+// z2 = u22 dy, added to the running totals (n0, n1), (n2, n3), (n4, n5):
 //   n0 = sum w, n1 = sum w z1, n2 = sum w z2,
 //   n3 = sum w (z1^2 - c^2), n4 = sum w z1 z2, n5 = sum w (z2^2 - c^2).
 // Rows are taken two at a time, one per half of a packed pair, so the row
 // terms (z2, and what is weighted by it) pack as naturally as the pixels'
-// (a fifth fewer instructions than pairs of columns, whose row terms are
-// scalars).  The second moments are taken about c^2 I, the whitened S^, per
-// block.  sg is the g tile: [row pair, column pair][block] = rows 2 h and
-// 2 h + 1 of column 2 c, then of column 2 c + 1.
+// (a sixth fewer instructions than pairs of columns, whose row terms are
+// scalars).  A row's sums are (pixel 0 + pixel 2) + (pixel 1 + pixel 3), and
+// the rows are added in order: the gradient's bits do not depend on how the
+// pixels are packed.  The second moments are taken about c^2 I, the whitened
+// S^, per block.  sg is the g tile: [row pair, column][block] = rows 2 h and
+// 2 h + 1 of column c, then of column c + 2.
 __device__ __forceinline__ void block_moments(const float4 (*__restrict__ sg)[16], int k, int x0,
                                               int y0, const float4 &A, float u22, float l2A,
-                                              float nl2tau, float2 (&n)[6]) {
+                                              float nl2tau, float2 (&n)[3]) {
   // the exponent rounded exactly as the forward rounds it, so that both
   // decide Eq. accu alike
   const float X0 = (float)(x0 + 4 * (k & 3)), Y0 = (float)(y0 + 4 * (k >> 2));
   float2 dx[4];
 #pragma unroll
   for (int x = 0; x < 4; ++x) dx[x] = f2(__fsub_rn(X0 + (float)x, A.x));
-  float2 m[6];
+  float m0, m1, m2, m3, m4, m5;
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const float2 dy = add2(make_float2(Y0 + (float)(2 * h), Y0 + (float)(2 * h + 1)), f2(-A.y));
     const float2 uy = mul2(f2(A.w), dy);
     const float2 z2 = mul2(f2(u22), dy);
     const float2 nc = fma2(z2, z2, f2(-l2A));
-    float2 s0, s1, s2;
+    float2 s0, s1, s2;  // the rows' sums of w, w z1 and w z1^2
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const float4 g4 = sg[2 * h + c][k];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        // -e = z1^2 + (z2^2 - l2A), as in the forward's terms
-        const float2 z = fma2(f2(A.z), dx[2 * c + q], uy);
-        const float2 f = fma2(z, z, nc);
-        // w = g * value on kept pairs (value > tau), zero elsewhere: g is
-        // masked to +0 on the integer pipe, which leaves the FMA pipe (this
-        // loop's busiest) the multiply
-        const float2 gm = make_float2(keep_or_zero(q ? g4.z : g4.x, f.x, nl2tau),
-                                      keep_or_zero(q ? g4.w : g4.y, f.y, nl2tau));
-        const float2 w = mul2(gm, make_float2(ex2_approx(-f.x), ex2_approx(-f.y)));
-        const float2 wz = mul2(w, z);
-        s0 = c + q ? add2(s0, w) : w;
-        s1 = c + q ? add2(s1, wz) : wz;
-        s2 = c + q ? fma2(wz, z, s2) : mul2(wz, z);
-      }
+      // -e = z1^2 + (z2^2 - l2A), as in the forward's terms
+      const float2 za = fma2(f2(A.z), dx[c], uy), zb = fma2(f2(A.z), dx[c + 2], uy);
+      const float2 fa = fma2(za, za, nc), fb = fma2(zb, zb, nc);
+      // w = g * value on kept pairs (value > tau), zero elsewhere: g is
+      // masked to +0 on the integer pipe, which leaves the FMA pipe (this
+      // loop's busiest) the multiply
+      const float2 ga = make_float2(keep_or_zero(g4.x, fa.x, nl2tau), keep_or_zero(g4.y, fa.y, nl2tau));
+      const float2 gb = make_float2(keep_or_zero(g4.z, fb.x, nl2tau), keep_or_zero(g4.w, fb.y, nl2tau));
+      const float2 wa = mul2(ga, make_float2(ex2_approx(-fa.x), ex2_approx(-fa.y)));
+      const float2 wb = mul2(gb, make_float2(ex2_approx(-fb.x), ex2_approx(-fb.y)));
+      const float2 wza = mul2(wa, za), wzb = mul2(wb, zb);
+      const float2 p0 = add2_apart(wa, wb), p1 = add2_apart(wza, wzb);
+      const float2 p2 = fma2(wzb, zb, mul2(wza, za));
+      s0 = c ? add2(s0, p0) : p0;
+      s1 = c ? add2(s1, p1) : p1;
+      s2 = c ? add2(s2, p2) : p2;
     }
-    // the rows' sums of w, w z1 and w z1^2, weighted by z2
+    // weighted by z2, row after row
     const float2 t = mul2(s0, z2);
-    m[0] = h ? add2(m[0], s0) : s0;
-    m[1] = h ? add2(m[1], s1) : s1;
-    m[2] = h ? add2(m[2], t) : t;
-    m[3] = h ? add2(m[3], s2) : s2;
-    m[4] = h ? fma2(s1, z2, m[4]) : mul2(s1, z2);
-    m[5] = h ? fma2(t, z2, m[5]) : mul2(t, z2);
+    m0 = h ? m0 + s0.x : s0.x;
+    m1 = h ? m1 + s1.x : s1.x;
+    m3 = h ? m3 + s2.x : s2.x;
+    m2 = h ? fmaf(s0.x, z2.x, m2) : t.x;
+    m4 = h ? fmaf(s1.x, z2.x, m4) : s1.x * z2.x;
+    m5 = h ? fmaf(t.x, z2.x, m5) : t.x * z2.x;
+    m0 += s0.y;
+    m1 += s1.y;
+    m3 += s2.y;
+    m2 = fmaf(s0.y, z2.y, m2);
+    m4 = fmaf(s1.y, z2.y, m4);
+    m5 = fmaf(t.y, z2.y, m5);
   }
   // second moments about c^2 I, then into the totals
-  m[3] = fma2(f2(-kC2), m[0], m[3]);
-  m[5] = fma2(f2(-kC2), m[0], m[5]);
-#pragma unroll
-  for (int i = 0; i < 6; ++i) n[i] = add2(n[i], m[i]);
+  m3 = fmaf(-kC2, m0, m3);
+  m5 = fmaf(-kC2, m0, m5);
+  n[0] = add2(n[0], make_float2(m0, m1));
+  n[1] = add2(n[1], make_float2(m2, m3));
+  n[2] = add2(n[2], make_float2(m4, m5));
 }
 
 // Entries of a backward unit: 256, less (down to 64) where that would leave
@@ -617,7 +636,7 @@ __global__ void __launch_bounds__(kThreads, kMinB) raster_bwd_kernel(
   constexpr int kWarps = kThreads / 32;
   constexpr int kWW = 32 * kPer;  // records per window
   constexpr int kBins = 256;      // (16 - blocks) * 16 + first block
-  __shared__ float4 sg_[kWarps][4][16];  // g by row pair and column pair of a block, and block
+  __shared__ float4 sg_[kWarps][4][16];  // g by row pair and column of a block, and block
   __shared__ float4 sa_[kWarps][kWW];    // px, py, u11, u12
   __shared__ float2 sb_[kWarps][kWW];    // u22, log2 A
   __shared__ uint32_t sj_[kWarps][kWW];
@@ -672,8 +691,8 @@ __global__ void __launch_bounds__(kThreads, kMinB) raster_bwd_kernel(
         float *u0 = reinterpret_cast<float *>(&sg[hp][k]) + lo;
         float *u1 = reinterpret_cast<float *>(&sg[hp + 1][k]) + lo;
         u0[0] = g[h].x;
-        u0[2] = g[h].y;
-        u1[0] = g[h].z;
+        u0[2] = g[h].z;
+        u1[0] = g[h].y;
         u1[2] = g[h].w;
       }
     }
@@ -755,18 +774,18 @@ __global__ void __launch_bounds__(kThreads, kMinB) raster_bwd_kernel(
         if (slot < nv) {
           const float4 A = sa[slot];
           const float2 Bv = sb[slot];
-          float2 tot[6];
+          float2 tot[3];
 #pragma unroll
-          for (int i = 0; i < 6; ++i) tot[i] = make_float2(0.f, 0.f);
+          for (int i = 0; i < 3; ++i) tot[i] = make_float2(0.f, 0.f);
           for (unsigned mm = smask[slot]; mm; mm &= mm - 1)
             block_moments(sg, __ffs(mm) - 1, x0, y0, A, Bv.x, Bv.y, nl2tau, tot);
           if (spread) {
             double *mo = mb + 6ull * sj[slot];
 #pragma unroll
-            for (int i = 0; i < 6; ++i) atomicAdd(mo + i, (double)(tot[i].x + tot[i].y));
+            for (int i = 0; i < 6; ++i) atomicAdd(mo + i, (double)(i & 1 ? tot[i / 2].y : tot[i / 2].x));
           } else {
 #pragma unroll
-            for (int i = 0; i < 6; ++i) red[7 * lane + i] = tot[i].x + tot[i].y;
+            for (int i = 0; i < 6; ++i) red[7 * lane + i] = i & 1 ? tot[i / 2].y : tot[i / 2].x;
           }
         }
         if (spread) continue;
