@@ -171,6 +171,40 @@ __global__ void __launch_bounds__(kChunkT) slice_write_kernel(
   }
 }
 
+// Few Gaussians: a CTA per slice goes over all their ranges, 1024 at a time,
+// and writes the slice's records and list itself; one launch where the form
+// above takes four.  The counts of a step's warps are double-buffered, so a
+// step has one barrier.
+constexpr int kSelThreads = 1024;
+__global__ void __launch_bounds__(kSelThreads) slice_select_kernel(
+    const QueryPrep *__restrict__ qp, const uint32_t *__restrict__ range, int64_t M, int k0, float apix,
+    int d, float l2tau, Rec *__restrict__ rec, uint32_t *__restrict__ sel, uint32_t *__restrict__ nsel) {
+  __shared__ uint32_t wn[2][kSelThreads / 32];
+  const int64_t k = blockIdx.x;
+  const unsigned z = (unsigned)(k0 + k);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t before = 0;  // of the earlier steps
+  int buf = 0;
+  unsigned next = threadIdx.x < M ? range[threadIdx.x] : 1u;  // 1: no slice
+  for (int64_t j0 = 0; j0 < M; j0 += kSelThreads, buf ^= 1) {
+    const int64_t j = j0 + threadIdx.x;
+    const unsigned r = next;
+    next = j + kSelThreads < M ? range[j + kSelThreads] : 1u;
+    const bool in = (r & 0xffffu) <= z && z <= (r >> 16);
+    const unsigned bits = __ballot_sync(0xffffffffu, in);
+    if (lane == 0) wn[buf][warp] = __popc(bits);
+    __syncthreads();
+    const uint32_t mine = wn[buf][lane];
+    const uint32_t lower = __reduce_add_sync(0xffffffffu, lane < warp ? mine : 0u);
+    if (in) {
+      sel[k * M + before + lower + __popc(bits & ((1u << lane) - 1u))] = (uint32_t)j;
+      rec[k * M + j] = slice_record(qp[j], (int)z, apix, d, l2tau);
+    }
+    before += __reduce_add_sync(0xffffffffu, mine);
+  }
+  if (threadIdx.x == 0) nsel[k] = before;
+}
+
 cudaError_t launch_query_prep(const float *params, int64_t M, int norm_mode, int shape, float apix,
                               int d, float l2tau, QueryPrep *qp, uint32_t *range, cudaStream_t st) {
   query_prep_kernel<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(params, M, norm_mode, shape, apix, d,
@@ -181,6 +215,14 @@ cudaError_t launch_query_prep(const float *params, int64_t M, int norm_mode, int
 cudaError_t launch_slices(const QueryPrep *qp, const uint32_t *range, int64_t M, int k0, int nslice,
                           float apix, int d, float l2tau, uint32_t *cnt, Rec *rec, uint32_t *sel,
                           uint32_t *nsel, cudaStream_t st) {
+  // Where the two forms meet: us per query of 16384 and 16385 Gaussians, 319
+  // and 327 at d 256 and 64 slices per batch, 289 and 299 at d 192 and 50, 258
+  // and 255 at d 64 and 16 (launches are most of it); at 4351 Gaussians, d
+  // 192, 50 slices, one launch 228 and four 279.
+  if (M <= 16384) {
+    slice_select_kernel<<<nslice, kSelThreads, 0, st>>>(qp, range, M, k0, apix, d, l2tau, rec, sel, nsel);
+    return cudaGetLastError();
+  }
   const int nch = (int)bin_chunks_tiles(M);
   const size_t smem = (size_t)nslice * 8 * sizeof(uint32_t);  // at most 24 KB (768 slices)
   slice_count_kernel<<<nch, kChunkT, smem, st>>>(range, M, k0, nslice, cnt);
