@@ -46,9 +46,11 @@ __device__ __forceinline__ void adam_entry(const AdamArgs &a, int m, unsigned j,
 
 // Bound by HBM: eight arrays of [M][11] floats read or written once.  A
 // thread takes kVec consecutive entries (four 16-byte loads in flight, four
-// stores) when all five arrays are 16-byte aligned, else one; M <= 2^24, so
-// entry numbers fit 32 bits.  M = 500000: 35 us with one entry per thread and
-// 64-bit remainders (5.0 TB/s), 25 us (6.9 TB/s) with four.
+// stores) when all five arrays are 16-byte aligned and that leaves the GPU two
+// CTAs per SM (at M = 6941 a call takes 2% longer with four entries per thread
+// than with one), else one; M <= 2^24, so entry numbers fit 32 bits.
+// M = 500000: 35 us with one entry per thread and 64-bit remainders (5.0
+// TB/s), 25 us (6.9 TB/s) with four.
 template <int kVec>
 __global__ void __launch_bounds__(256) adam_step_kernel(AdamArgs a, unsigned n,
                                                         float *__restrict__ raw,
@@ -100,7 +102,7 @@ cudaError_t launch_adam(const AdamArgs &a, int64_t M, float *raw, float *m, floa
                         const float *grad, float *params, const float *iso, cudaStream_t st) {
   const unsigned n = (unsigned)(M * kNpar);
   const uintptr_t all = (uintptr_t)raw | (uintptr_t)m | (uintptr_t)v | (uintptr_t)grad | (uintptr_t)params;
-  if ((all & 15u) == 0)
+  if ((all & 15u) == 0 && n >= 2 * 152 * 1024)
     adam_step_kernel<4><<<(n + 1023) / 1024, 256, 0, st>>>(a, n, raw, m, v, grad, params, iso);
   else
     adam_step_kernel<1><<<(n + 255) / 256, 256, 0, st>>>(a, n, raw, m, v, grad, params, iso);

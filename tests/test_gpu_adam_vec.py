@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("iso", [False, True])
-@pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 93, 94, 1000, 1024])
+@pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 93, 94, 1000, 28299, 28300, 28301, 28303])
 def test_aligned_and_unaligned_arrays_give_the_same_step(M, iso):
     ctx = gt.context(syn.Workload("av", d=16, M=M, B=1, seed=1))
     g = torch.Generator(device="cuda").manual_seed(M)
