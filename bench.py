@@ -783,7 +783,7 @@ def main():
         q_ms = sum(a.elapsed_time(b) for a, b in qe) / nq
         nbatch = -(-w.d // w.B)
         query = {"ms": q_ms, "voxels_per_s": w.d ** 3 / (q_ms / 1e3), "grid": w.d, "M": w.M, "tau": tq,
-                 "slice_batches": nbatch, "gpu_launches_per_call": 1 + 6 * nbatch,
+                 "slice_batches": nbatch, "gpu_launches_per_call": 1 + (7 if w.M <= 16384 else 9) * nbatch,
                  "l2": "flushed before each call (256 MB write)"}
         # Fourier shell correlation of the map against the map of perturbed
         # Gaussians (the two half-maps of Eq. fsc)
@@ -805,7 +805,7 @@ def main():
         f_ms = sum(a.elapsed_time(b) for a, b in fe) / nq
         f_bytes = 64 * w.d ** 3  # 3 FFT passes (read + write d^3 complex) and the shell pass (2 reads)
         f_gbs = f_bytes / (f_ms / 1e3) / 1e9
-        query["fsc"] = {"ms": f_ms, "resolution_A": float(fsc_out[2].item()), "gpu_launches_per_call": 5,
+        query["fsc"] = {"ms": f_ms, "resolution_A": float(fsc_out[2].item()), "gpu_launches_per_call": 6,
                         "roofline": {"bound": "hbm", "achieved": f_gbs, "peak": HBM_PEAK_GBS, "unit": "GB/s",
                                      "frac": f_gbs / HBM_PEAK_GBS, "algorithmic_bytes": f_bytes,
                                      "peak_note": HBM_PEAK_NOTE}}

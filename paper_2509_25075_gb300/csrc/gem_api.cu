@@ -389,7 +389,7 @@ static int check_project_args(gem_ctx *c, const float *params, int64_t M, int32_
 
 static int prep(gem_ctx *c, const float *params, int64_t M, int32_t B, const float *R,
                 const float *t) {
-  StageScope sc(c, GEM_STAGE_PREP, 9);
+  StageScope sc(c, GEM_STAGE_PREP, 3 + sort16_launches(M, 1));
   cudaError_t e;
   const gem_config &g = c->cfg;
   // slot order: a stable sort of the Gaussians by the 3D Morton key of their
@@ -425,7 +425,7 @@ int gem_project(gem_ctx *c, const float *params, int64_t M, int32_t B, const flo
   const gem_config &g = c->cfg;
   const uint32_t *perm = nullptr;
   {
-    StageScope sc(c, GEM_STAGE_BIN, g.zsort ? 10 : 4);
+    StageScope sc(c, GEM_STAGE_BIN, 4 + (g.zsort ? sort16_launches(M, B) : 0));
     c->have_bins = false;
     if ((e = launch_bin(c->rec, c->bin.key, M, B, g.d, c->l2tau, g.zsort, c->bin, &perm,
                         c->stream)) != cudaSuccess)

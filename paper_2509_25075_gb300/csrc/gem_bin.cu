@@ -976,14 +976,19 @@ cudaError_t bin_configure(int d) {
   return e != cudaSuccess ? e : bin_configure_one<true>(d);
 }
 
-cudaError_t launch_sort16(const uint16_t *key, int64_t M, int B, uint32_t *dcnt,
-                          uint32_t *packed, uint32_t *perm, cudaStream_t st) {
+static bool sort_by_row(int64_t M, int B) {
   // A row in one CTA takes about 1.5 us per 1000 keys, in as many rounds as
   // the rows need; the chunked form spreads a row over the SMs, at 18 us per
   // million keys of all rows plus six launches.  us, row and chunked form:
   // M 2000, B 32: 9, 27; M 20000, B 256: 60, 90; M 50000, B 64: 77, 60.  A few
   // long rows would leave most SMs idle.
-  if (M <= 8192 || (M <= kRowMax && B >= 32)) {
+  return M <= 8192 || (M <= kRowMax && B >= 32);
+}
+int sort16_launches(int64_t M, int B) { return sort_by_row(M, B) ? 1 : 6; }
+
+cudaError_t launch_sort16(const uint16_t *key, int64_t M, int B, uint32_t *dcnt,
+                          uint32_t *packed, uint32_t *perm, cudaStream_t st) {
+  if (sort_by_row(M, B)) {
     sort16_row_kernel<<<B, kRowThreads, row_smem(M), st>>>(key, (int)M, perm);
     return cudaGetLastError();
   }
