@@ -308,6 +308,7 @@ struct BinScratch {
 // scratch of the binning's sizes.
 cudaError_t launch_sort16(const uint16_t *key, int64_t M, int B, uint32_t *dcnt,
                           uint32_t *packed, uint32_t *perm, cudaStream_t st);
+int sort16_launches(int64_t M, int B);  // its kernels
 // Gaussian of each list entry: out[i] = slot_gauss[list[i].x] (the entries
 // hold slots), or list[i].x when slot_gauss is NULL.
 cudaError_t launch_map_slots(const uint2 *list, const uint32_t *slot_gauss, int64_t n,
