@@ -72,15 +72,11 @@ ALL_FP32_OPS_PER_KEPT_PAIR = {"raster_fwd": 10, "raster_bwd": 30}
 # (dram__bytes_read.sum + dram__bytes_write.sum, one pass each), valid while
 # the sources they depend on hash to the value they had then (null otherwise).
 CAPTURED_TRAFFIC = {
-    "source_sha256_16": "f60b6aff05b83873",
+    "source_sha256_16": "14fbb96e5e613126",
     "per_workload": {  # workload -> {configuration name: bytes per launch}
         "A5": {
-            "aligned, 256-record windows, 7 CTAs/SM, persistent longest-first": 623250688.0,
-            "aligned, 256-record windows, 6 CTAs/SM, persistent longest-first": 620255232.0,
-            "aligned, 256-record windows, 5 CTAs/SM, persistent longest-first": 611992064.0,
-            "1 lane per record, 256-record warp windows, persistent longest-first": 2406793216.0,
-            "1 lane per record, 256-record warp windows, persistent longest-first, 6 CTAs/SM": 2377032704.0,
-            "1 lane per record, 256-record warp windows, persistent longest-first, 5 CTAs/SM": 2201309952.0,
+            "8 CTAs/SM": 518239744.0,
+            "256-record warp windows, 5 CTAs/SM": 1214098688.0,
         },
     },
 }
