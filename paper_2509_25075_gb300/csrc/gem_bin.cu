@@ -412,6 +412,7 @@ __device__ __forceinline__ int last_column(float xr, float last) {
 // row by (pixel rows 4 by .. 4 by + 3), packed as lo | hi << 8, or kNoRow.
 constexpr unsigned kNoRow = 0x00ffu;  // lo = 255 > hi = 0
 __device__ __forceinline__ unsigned block_row_range(const RowGeo &G, int by, int nb) {
+  if (!(G.k4a < INFINITY)) return (unsigned)(nb - 1) << 8;  // tau = 0: every pixel counts
   float xl, xr;
   if (!row_span(G, (float)(4 * by), xl, xr)) return kNoRow;
   const int lo = first_column(xl, 0.f), hi = last_column(xr, (float)(nb - 1));
