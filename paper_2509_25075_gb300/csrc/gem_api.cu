@@ -37,7 +37,7 @@ struct gem_ctx {
 
   BinScratch bin{};
   double *mom = nullptr;   // [max_B][max_M][6] moments of the raster backward
-  bool mom_clean = false;  // every moment is zero (prep_bwd leaves them so)
+  bool mom_clean = false;  // every moment and the backward's counter are zero (prep_bwd leaves them so)
   float *part = nullptr;
   int nbg = 1;
   float *proj = nullptr;   // internal projection of gem_forward
@@ -90,7 +90,6 @@ struct gem_ctx {
   // batch of gem_query, binned for M = bins_M Gaussians, B = bins_B images
   // with threshold bins_l2tau
   bool have_bins = false;
-  bool bwd_fresh = false;  // no backward has taken the tasks of these bins yet
   bool bins_of_proj = false;
   int64_t bins_M = 0;
   int bins_B = 0;
@@ -442,7 +441,6 @@ int gem_project(gem_ctx *c, const float *params, int64_t M, int32_t B, const flo
     if ((e = launch_raster_fwd(fc, c->rec, c->bin.list, c->bin.tile_start, c->bin.cap, M, B, g.d,
                                c->l2tau, proj, c->tasks, true, c->stream)) != cudaSuccess)
       return cuda_fail(c, e, "raster_fwd");
-    c->bwd_fresh = true;
   }
   c->have_proj = true;
   return GEM_OK;
@@ -492,11 +490,14 @@ static int backward_common(gem_ctx *c, const float *dproj, float *grad, bool den
     return fail(c, GEM_ESTATE, "the last projection was dense: no tile lists to differentiate");
   const gem_config &g = c->cfg;
   cudaError_t e;
-  // the whole buffer, should an earlier pass have stopped before clearing it
+  // the whole buffer and the raster backward's counter, should an earlier pass
+  // have stopped before the chain rule cleared them
   size_t mbytes = (size_t)g.max_B * g.max_M * 6 * sizeof(double);
   {
     StageScope sc(c, GEM_STAGE_RASTER_BWD, 1);
-    if (!dense && !c->mom_clean && (e = cudaMemsetAsync(c->mom, 0, mbytes, c->stream)) != cudaSuccess)
+    if (!dense && !c->mom_clean &&
+        ((e = cudaMemsetAsync(c->mom, 0, mbytes, c->stream)) != cudaSuccess ||
+         (e = cudaMemsetAsync(c->tasks.ctr + kCtrBwd, 0, sizeof(unsigned), c->stream)) != cudaSuccess))
       return cuda_fail(c, e, "moment clear");
     c->mom_clean = false;
     if (dense)
@@ -504,13 +505,12 @@ static int backward_common(gem_ctx *c, const float *dproj, float *grad, bool den
     else
       e = launch_raster_bwd(active_bwd(c, c->B, c->M), c->rec, c->bin.list,
                             c->bin.tile_start, c->bin.cap, c->M, c->B, g.d, c->l2tau, dproj, c->mom,
-                            c->tasks, c->bwd_fresh, c->stream);
+                            c->tasks, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "raster_bwd");
-    if (!dense) c->bwd_fresh = false;
   }
   StageScope sc(c, GEM_STAGE_PREP_BWD, 2);
   if ((e = launch_prep_bwd(c->psort, c->gauss_slot, c->gp, c->M, c->B, c->R, c->t, g.apix, g.d, g.norm_mode, shape_flags(g),
-                           c->mom, c->part, c->nbg, grad, c->stream)) != cudaSuccess)
+                           c->mom, c->part, c->nbg, grad, c->tasks.ctr + kCtrBwd, c->stream)) != cudaSuccess)
     return cuda_fail(c, e, "prep_bwd");
   c->mom_clean = true;
   return GEM_OK;

@@ -193,13 +193,14 @@ cudaError_t launch_view_prep(const GaussPrep *gp, int64_t M, int B, const float 
                              Rec *rec, uint16_t *key, float *kept_R, float *kept_t,
                              cudaStream_t st);
 // Reads the float64 moments [B][M][6] and leaves them zero (the next
-// backward pass accumulates into them).
+// backward pass accumulates into them), and likewise the raster backward's
+// work counter bwd_ctr.
 // params (the slot-ordered copy), gp and the moments are by slot; grad
 // comes out by Gaussian through gauss_slot (NULL: slot i is Gaussian i).
 cudaError_t launch_prep_bwd(const float *params, const uint32_t *gauss_slot, const GaussPrep *gp,
                             int64_t M, int B, const float *R, const float *t, float apix, int d,
                             int norm_mode, int shape, double *mom, float *part, int nbg,
-                            float *grad, cudaStream_t st);
+                            float *grad, unsigned *bwd_ctr, cudaStream_t st);
 cudaError_t launch_inspect_records(const Rec *rec, const GaussPrep *gp,
                                    const uint32_t *slot_gauss, int64_t M, int B, const float *R,
                                    const float *t, float apix, int d, float *out,
@@ -341,7 +342,7 @@ struct RasterTasks {
                    // (first window, windows of the tile, the tile's first partial image, 0)
   float *part;     // [parts][256] partial images of tiles with several windows
   unsigned *done;  // [B * T] windows finished, zero between calls
-  unsigned *ctr;   // [kCtrCount], reset by the binning
+  unsigned *ctr;   // [kCtrCount], reset by the binning (kCtrBwd by the chain rule too)
 };
 size_t raster_task_count(int64_t cap, int64_t ntiles);
 // A configuration of the forward rasteriser: CTAs per SM.
@@ -364,12 +365,14 @@ struct BwdCfg {
 };
 int bwd_config_count();
 const BwdCfg &bwd_config(int i);
-// Runs the tasks that the last forward made of these bins.  fresh: no
-// backward has taken them yet.
+// Runs the tasks that the last forward made of these bins.  tk.ctr[kCtrBwd]
+// is zero when it starts: the binning clears it, and so does the chain rule
+// after every backward (on the device, so that a backward captured alone in a
+// graph finds it zero on each replay).
 cudaError_t launch_raster_bwd(int cfg, const Rec *rec, const uint2 *list,
                               const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
                               float l2tau, const float *dproj, double *mom, const RasterTasks &tk,
-                              bool fresh, cudaStream_t st);
+                              cudaStream_t st);
 cudaError_t launch_count_kept(int cfg, const Rec *rec, const uint2 *list,
                               const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
                               float l2tau, unsigned long long *kept, const RasterTasks &tk,

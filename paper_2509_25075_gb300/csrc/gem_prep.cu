@@ -285,8 +285,10 @@ struct Kahan {
 __global__ void __launch_bounds__(128) prep_bwd_kernel(
     const float *__restrict__ params, const GaussPrep *__restrict__ gp, int64_t M, int B,
     const float *__restrict__ R, const float *__restrict__ t, float apix, int d, int norm_mode,
-    int shape, double *__restrict__ mom, int per_group, float *__restrict__ part) {
+    int shape, double *__restrict__ mom, int per_group, float *__restrict__ part,
+    unsigned *__restrict__ bwd_ctr) {
   const int64_t sl = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (sl == 0 && blockIdx.y == 0) *bwd_ctr = 0u;  // as the next raster backward expects it
   int bg = blockIdx.y;
   if (sl >= M) return;
   GaussPrep g = gp[sl];
@@ -449,7 +451,7 @@ __global__ void __launch_bounds__(256) grad_sum_kernel(const float *__restrict__
 cudaError_t launch_prep_bwd(const float *params, const uint32_t *gauss_slot, const GaussPrep *gp,
                             int64_t M, int B, const float *R, const float *t, float apix, int d,
                             int norm_mode, int shape, double *mom, float *part, int nbg,
-                            float *grad, cudaStream_t st) {
+                            float *grad, unsigned *bwd_ctr, cudaStream_t st) {
   // views per thread: enough (Gaussian, view-group) threads to fill the GPU
   // (about 2^20), and no more, so that the per-Gaussian reads, the
   // view-independent chain rule and the partial sums are shared by as many
@@ -460,7 +462,7 @@ cudaError_t launch_prep_bwd(const float *params, const uint32_t *gauss_slot, con
   int groups = (B + per - 1) / per;
   dim3 grid((unsigned)((M + 127) / 128), (unsigned)groups);
   prep_bwd_kernel<<<grid, 128, 0, st>>>(params, gp, M, B, R, t, apix, d, norm_mode, shape, mom,
-                                        per, part);
+                                        per, part, bwd_ctr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   int64_t n = M * kNpar;

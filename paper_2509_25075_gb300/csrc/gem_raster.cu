@@ -825,13 +825,9 @@ const BwdCfg &bwd_config(int i) { return kBwdCfgs[i]; }
 cudaError_t launch_raster_bwd(int cfg, const Rec *rec, const uint2 *list,
                               const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
                               float l2tau, const float *dproj, double *mom, const RasterTasks &tk,
-                              bool fresh, cudaStream_t st) {
+                              cudaStream_t st) {
   if (cfg < 0 || cfg >= bwd_config_count()) return cudaErrorInvalidValue;
   const BwdCfg &c = kBwdCfgs[cfg];
-  if (!fresh) {  // the tasks stand; only the backward's counter starts again
-    const cudaError_t e = cudaMemsetAsync(tk.ctr + kCtrBwd, 0, sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
-  }
   const int grid = sm_count() * c.ctas, nt = d / kTile, ntiles = nt * nt * B;
   if (c.per == 8 && c.ctas == 6)
     raster_bwd_kernel<8, 6><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tile_start, ntiles, dproj, mom, tk);

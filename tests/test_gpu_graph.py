@@ -62,3 +62,53 @@ def test_step_replays_from_a_cuda_graph():
         ctx.close()
     finally:
         torch.cuda.set_stream(torch.cuda.default_stream())
+
+
+def test_backward_alone_replays_from_a_cuda_graph():
+    """A graph that holds only the backward of an earlier forward gives the
+    whole gradient on every replay, before and after eager backwards of the
+    same lists.  The lists hold more than 152 x 8 x 4 warps' units of at most
+    256 entries, so most units come from the backward's work counter."""
+    w = syn.Workload("graphb", d=64, M=8000, B=96, apix=1.2, seed=32)
+    s = torch.cuda.Stream()
+    torch.cuda.set_stream(s)
+    try:
+        inp = gt.inputs(w)
+        args = [gt.to_dev(inp[k]) for k in ("params", "R", "t")]
+        ctx, eager = (binding.Context(w.d, w.apix, w.B, w.M, tau=w.tau, stream=s) for _ in range(2))
+        proj = torch.empty(w.B, w.d, w.d, device=gt.DEV)
+        grad, ref = torch.zeros(w.M, 11, device=gt.DEV), torch.zeros(w.M, 11, device=gt.DEV)
+        fields = [gt.to_dev(syn.smooth_field(syn.Workload("f", d=w.d, M=1, B=w.B, seed=k))) * 1e-3
+                  for k in range(4)]
+        dproj = fields[0].clone()
+        for c in (ctx, eager):
+            c.gem_project(*args, proj)
+        assert ctx.gem_pair_count() > 152 * 8 * 4 * 256
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            ctx.gem_project_backward(dproj, grad)
+
+        def check(k, run):
+            dproj.copy_(fields[k])
+            grad.zero_()
+            run()
+            eager.gem_project_backward(fields[k], ref)
+            s.synchronize()
+            assert float((grad - ref).norm()) <= 1e-6 * float(ref.norm())
+
+        for k in range(3):
+            check(k, g.replay)
+        check(3, lambda: ctx.gem_project_backward(dproj, grad))
+        check(0, g.replay)
+        ctx.gem_pair_stats()  # makes the tasks of the lists again
+        check(1, g.replay)
+        check(2, g.replay)
+        ctx.gem_project(*args, proj)  # a new forward of the same sizes
+        check(0, g.replay)
+        check(1, lambda: ctx.gem_project_backward(dproj, grad))
+        assert ctx.gem_status() == binding.GEM_OK
+        ctx.close()
+        eager.close()
+    finally:
+        torch.cuda.set_stream(torch.cuda.default_stream())
