@@ -328,6 +328,9 @@ int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream) {
       (e = cudaMemset(c->knn.ticket, 0, sizeof(int))) != cudaSuccess ||
       (e = cudaMemset(c->ctf.done, 0, ((size_t)g.max_B + 1) * sizeof(unsigned))) != cudaSuccess ||
       (e = cudaMemset(c->tasks.done, 0, (size_t)g.max_B * c->T * sizeof(unsigned))) != cudaSuccess ||
+      // the copy and the clears are on the default stream, behind whatever is
+      // queued there; a non-blocking stream would not wait for them
+      (e = cudaStreamSynchronize(nullptr)) != cudaSuccess ||
       (e = bin_configure(d)) != cudaSuccess || (e = ctf_configure(d)) != cudaSuccess) {
     snprintf(g_create_err, sizeof(g_create_err), "set-up: %s", cudaGetErrorString(e));
     gem_destroy(c);
@@ -365,7 +368,7 @@ int gem_status(gem_ctx *c) {
   int st = 0;
   if ((e = cudaMemcpy(&st, c->status, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess)
     return cuda_fail(c, e, "status read");
-  if ((e = cudaMemset(c->status, 0, sizeof(int))) != cudaSuccess)
+  if ((e = cudaMemsetAsync(c->status, 0, sizeof(int), c->stream)) != cudaSuccess)
     return cuda_fail(c, e, "status clear");
   if (st & GEM_STATUS_CAPACITY)
     return fail(c, GEM_ECAPACITY, "pair list exceeded max_pairs=%lld",
