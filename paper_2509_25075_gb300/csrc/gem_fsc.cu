@@ -18,6 +18,7 @@
 
 #include "gem_fft.cuh"
 #include "gem_internal.cuh"
+#include "gem_pairsum.cuh"
 
 namespace gem {
 
@@ -98,12 +99,14 @@ __device__ __forceinline__ float seg_add(float v, int o, bool take) {
 // is monotone, so the runs of one step have different shells and the sums
 // need no atomics.
 //
-// A sum is a pair of floats, its value and the rounding errors of that value
-// (exact, by Knuth's two-sum), converted to float64 when the block is done:
-// this GPU's float64 adds run at a 64th of its float32 adds, and three of
-// them and their conversions per step were the kernel's bound.  The pair's
-// error is 2^-48 of the sum per addition, against the 2^-24 of the runs.
-// Runs of 1e30 and more, infinities and NaN go to float64 sums of their own.
+// A sum is a pair of floats, its value and the sum of that value's rounding
+// errors, added to without loss (gem_pairsum.cuh) and converted to float64
+// when the block is done: this GPU's float64 adds run at a 64th of its float32
+// adds, and three of them and their conversions per step were the kernel's
+// bound.  What the pair cannot hold (terms more than 48 bits apart, which is
+// rare), and runs of 1e30 and more, infinities and NaN, go to float64 sums of
+// their own, so nothing is rounded but the float64 additions there and at the
+// block's end: fewer than with float64 sums throughout.
 //
 // Then the instructions bound it, and after them the load: the part of the
 // volume inside the last shell (half of it), once.  A unit is the least whole
@@ -112,7 +115,7 @@ __device__ __forceinline__ float seg_add(float v, int o, bool take) {
 // last shell load and sum nothing.  The warp follows a unit with its mirror
 // image, which then finds both its operands in L1.  Against one pass over all
 // frequencies with divisions, two loads each and float64 atomics: side 256,
-// the whole call 293 -> 219 us (287 with float64 sums).
+// the whole call 293 -> 226 us (287 with float64 sums).
 template <int N>
 __global__ void __launch_bounds__(kFThreads) fsc_shell_kernel(const float2 *__restrict__ F, int nsh,
                                                               double *__restrict__ part) {
@@ -126,14 +129,20 @@ __global__ void __launch_bounds__(kFThreads) fsc_shell_kernel(const float2 *__re
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   float2 *mine = acc + warp * 3 * nsh;
-  auto add = [&](int k, float v) {
-    if (fabsf(v) < 1e30f) {
-      const float2 a = mine[k];
-      const float t = a.x + v, w = t - a.x;
-      mine[k] = make_float2(t, a.y + ((a.x - (t - w)) + (v - w)));
-    } else {
-      atomicAdd(&big[k], (double)v);
+  auto add = [&](int s, float num, float p1, float p2) {
+    if (p1 < 1e30f && p2 < 1e30f) {  // then |num| is as well
+      float2 a = mine[s], b = mine[nsh + s], c = mine[2 * nsh + s];
+      num = pair_add(a.x, a.y, num);
+      p1 = pair_add(b.x, b.y, p1);
+      p2 = pair_add(c.x, c.y, p2);
+      mine[s] = a;
+      mine[nsh + s] = b;
+      mine[2 * nsh + s] = c;
+      if (num == 0.f && p1 == 0.f && p2 == 0.f) return;
     }
+    atomicAdd(&big[s], (double)num);
+    atomicAdd(&big[nsh + s], (double)p1);
+    atomicAdd(&big[2 * nsh + s], (double)p2);
   };
   const int lim = nsh * nsh - nsh + 1;  // the last shell is nsh - 1: k2 < lim
   const int nunit = (h + 1) * kUnits, step = gridDim.x * kWarps;
@@ -182,19 +191,11 @@ __global__ void __launch_bounds__(kFThreads) fsc_shell_kernel(const float2 *__re
         m &= m << o;
       }
       const bool write = last && s < nsh;
-      if (i0 / h == (i0 + 31) / h) {
-        if (write) {
-          add(s, num);
-          add(nsh + s, p1);
-          add(2 * nsh + s, p2);
-        }
+      if (h % 32 == 0 || i0 / h == (i0 + 31) / h) {
+        if (write) add(s, num, p1, p2);
       } else {  // rows' halves meet here: one run at a time
         for (unsigned w = __ballot_sync(0xffffffffu, write); w; w &= w - 1) {
-          if (lane == __ffs(w) - 1) {
-            add(s, num);
-            add(nsh + s, p1);
-            add(2 * nsh + s, p2);
-          }
+          if (lane == __ffs(w) - 1) add(s, num, p1, p2);
           __syncwarp();
         }
       }

@@ -4,6 +4,11 @@ the claim beside the code, and these tests restate the computation in numpy
 with IEEE single-precision rounding and compare it with exact integer
 arithmetic.  (The compiled kernels are checked end to end by the GPU parity
 tests; these pin the arithmetic arguments themselves.)"""
+import ctypes
+import math
+import os
+import subprocess
+
 import numpy as np
 
 f32 = np.float32
@@ -119,3 +124,56 @@ def test_warp_bit_transpose():
     for k in range(16):
         assert int(out[k]) == sum(1 << l for l in range(32) if (int(m0[l]) >> k) & 1)
         assert int(out[16 + k]) == sum(1 << l for l in range(32) if (int(m1[l]) >> k) & 1)
+
+
+def _pair_sum(tmp_path):
+    """The FSC's running sum (csrc/gem_pairsum.cuh), compiled for the host and
+    used as the shell kernel uses it: pairs of floats, what does not fit them
+    in a float64 sum, all of it added in float64 at the end."""
+    csrc = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                        "paper_2509_25075_gb300", "csrc")
+    src = tmp_path / "s.cpp"
+    src.write_text("""#include "gem_pairsum.cuh"
+extern "C" double sum(const float *v, long n) {
+  float x = 0.f, e = 0.f;
+  double big = 0.0;
+  for (long i = 0; i < n; ++i) big += (double)gem::pair_add(x, e, v[i]);
+  return big + ((double)x + (double)e);
+}
+""")
+    so = str(tmp_path / "s.so")
+    subprocess.run(["g++", "-O2", "-ffp-contract=off", "-shared", "-fPIC", "-I", csrc, str(src), "-o", so],
+                   check=True)
+    lib = ctypes.CDLL(so)
+    lib.sum.restype = ctypes.c_double
+    lib.sum.argtypes = [ctypes.c_void_p, ctypes.c_long]
+    return lambda v: lib.sum(v.ctypes.data, len(v))
+
+
+def test_fsc_running_sum_is_no_worse_than_float64(tmp_path):
+    """Pairs and rest hold the sum exactly, so the result is off by the three
+    roundings of the float64 additions at the end: at most 2^-53 (|big| + 2
+    |sum|) for terms of one sign.  A float64 running sum rounds at every term.
+    Terms: magnitudes over 2^-60 .. 2^60 in random order (the pair alone spans
+    48 bits), shell-like powers, and sums that cancel."""
+    s = _pair_sum(tmp_path)
+    rng = np.random.default_rng(7)
+    for n in (1, 2, 7, 400):
+        for k in range(200):
+            kind = k % 3
+            if kind == 0:
+                v = (1 + rng.random(n)) * 2.0 ** rng.integers(-60, 60, n)
+            elif kind == 1:
+                v = rng.chisquare(2, n) * 10.0 ** rng.integers(0, 9)
+            else:
+                v = rng.normal(size=n) * 2.0 ** rng.integers(-20, 20, n)
+            v = np.ascontiguousarray(v.astype(f32))
+            exact = math.fsum(v.astype(np.float64))
+            run = 0.0
+            for x in v:
+                run += float(x)
+            off = abs(s(v) - exact)
+            scale = abs(exact) if kind < 2 else float(np.abs(v.astype(np.float64)).max())
+            assert off <= 3 * 2.0 ** -53 * scale, (n, k, off / scale)
+            if kind < 2 and n == 400:
+                assert off <= max(abs(run - exact), 2.0 ** -53 * scale * 2)
