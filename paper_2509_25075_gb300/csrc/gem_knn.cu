@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kKnnBlk) knn_bbox_kernel(const float *__restri
   if (!(h > 0.0)) h = 1.0;
   int n[3] = {1, 1, 1};
   bool fits = false;
-  for (int it = 0; it < 1024 && !fits; ++it, h *= 1.1) {
+  for (int it = 0; it < 1024 && !fits; ++it) {
     double cells = 1.0;
     for (int a = 0; a < 3; ++a) {
       double na = floor(ext[a] / h) + 1.0;
@@ -108,7 +108,9 @@ __global__ void __launch_bounds__(kKnnBlk) knn_bbox_kernel(const float *__restri
       cells *= n[a];
     }
     fits = cells <= (double)cap;
-    if (fits) break;
+    // no set of centres needs more than the cube root of the excess; flat and
+    // linear ones come closer step by step
+    if (!fits) h *= fmax(1.1, cbrt(cells / (double)cap));
   }
   if (!fits || !(h > 0.0) || !isfinite(h)) {  // absurd coordinates: one cell holds all
     n[0] = n[1] = n[2] = 1;
@@ -264,11 +266,11 @@ template <int K>
 struct KBest {
   float d[K];
   int i[K];
-  __device__ __forceinline__ void clear() {
+  __device__ __forceinline__ void fill(float dist, int index) {
 #pragma unroll
     for (int m = 0; m < K; ++m) {
-      d[m] = INFINITY;
-      i[m] = -1;
+      d[m] = dist;
+      i[m] = index;
     }
   }
   // A non-finite candidate's squared distance is infinite or not a number:
@@ -296,26 +298,19 @@ struct KBest {
       i[0] = j;
     }
   }
-  // The best k over the lanes' lists, which hold no index twice, left in
-  // every lane.
+  // The best k over the lanes' lists, which hold no index twice (but for the
+  // placeholders, which come last), left in every lane.  Distances are not
+  // negative, so their bits order as they do.
   __device__ __forceinline__ void merge_warp() {
     KBest<K> all;
 #pragma unroll
     for (int m = 0; m < K; ++m) {
-      float bd = d[0];
-      int bi = i[0];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float od = __shfl_xor_sync(0xffffffffu, bd, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (od < bd || (od == bd && (unsigned)oi < (unsigned)bi)) {
-          bd = od;
-          bi = oi;
-        }
-      }
-      all.d[m] = bd;
-      all.i[m] = bi;
-      if (i[0] == bi && bi >= 0) {  // this lane's head was the best: drop it
+      const unsigned mine = __float_as_uint(d[0]);
+      const unsigned bd = __reduce_min_sync(0xffffffffu, mine);
+      const unsigned bi = __reduce_min_sync(0xffffffffu, mine == bd ? (unsigned)i[0] : 0xffffffffu);
+      all.d[m] = __uint_as_float(bd);
+      all.i[m] = (int)bi;
+      if (mine == bd && (unsigned)i[0] == bi) {  // this lane's head was the best: drop it
 #pragma unroll
         for (int q = 0; q + 1 < K; ++q) {
           d[q] = d[q + 1];
@@ -343,18 +338,29 @@ __device__ __forceinline__ void knn_visit(KBest<K> &best, const float4 *__restri
 
 // One thread per centre, in cell order, for its cell and the 26 around it:
 // neighbouring threads read the same cells, and the cells of a row along x
-// are one run of the sorted centres, so the nine rows' bounds are loaded
-// together and the runs follow.  The centres that need further rings (those
-// in the thin outskirts of the clusters, whose rings hold hundreds of mostly
-// empty rows) are finished by the whole warp, one after the other, a row per
-// lane: a thread walking them alone is a chain of dependent loads.
+// are one run of the sorted centres.  A centre that needs further rings of
+// cells walks them in its thread as long as enough of its warp's lanes do; the
+// last ones (those in the thin outskirts of the clusters, whose rings hold
+// hundreds of mostly empty rows) are finished by the whole warp, one after the
+// other, a row per lane: a thread walking them alone is a chain of dependent
+// loads.
 //
-// Bound by the latency of those loads.  M = 500000, k = 1 (64 clusters):
-// 436 us with a gather of the parameter row per candidate and two bounds per
-// cell on M / 2 cells, 233 with sorted centres, rows and 3/2 M cells,
-// about 105 with the warp's part.
+// The line between the two: a ring costs a thread its rows, and the warp about
+// 2 + K / 4 + rows / 32 rows' time (the merge of the lanes' lists grows with K)
+// for each centre.  With the warp from the second ring on, sets whose centres
+// mostly need it (several neighbours, flat sets) waited for 32 searches in a
+// row; with constants half and twice these, times are the same within 10% but
+// for a few sets.
+//
+// Bound by the latency of the loads at k = 1, by insertions at k = 16 (hence
+// three CTAs per SM there: 80 registers).  Calls of M = 300000, us, with one
+// thread per centre, a gather of the parameter row per candidate and two bounds
+// per cell; with sorted centres, rows, 3/2 M cells and the warp from the
+// second ring on; now:  64 clusters, k = 1: 402, 145, 129; k = 4: 626, 486,
+// 243; k = 8: 918, 1034, 434; k = 16: 1743, 5889, 1076.  A plane, k = 1: 138,
+// 109, 74; k = 16: 533, 4787, 444.  Uniform, k = 8: 559, 854, 236.
 template <int K>
-__global__ void __launch_bounds__(kKnnBlk) knn_query_kernel(
+__global__ void __launch_bounds__(kKnnBlk, K > 8 ? 3 : 1) knn_query_kernel(
     const float4 *__restrict__ sorted, int64_t M, const KnnGrid *__restrict__ g,
     const int *__restrict__ start, float *__restrict__ dist, int32_t *__restrict__ idx) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -366,7 +372,7 @@ __global__ void __launch_bounds__(kKnnBlk) knn_query_kernel(
   if (t < M) me = sorted[t];
   const int i = __float_as_int(me.w);
   KBest<K> best;
-  best.clear();
+  best.fill(INFINITY, -1);
   const bool fin = t < M && isfinite(me.x) && isfinite(me.y) && isfinite(me.z);
   bool done = !fin;
   // everything in rings beyond r lies farther than r * h from the point
@@ -379,22 +385,85 @@ __global__ void __launch_bounds__(kKnnBlk) knn_query_kernel(
     const int cy = knn_axis_cell(me.y, G.lo[1], G.ih, n1);
     const int cz = knn_axis_cell(me.z, G.lo[2], G.ih, n2);
     const int x0 = max(cx - 1, 0), x1 = min(cx + 1, n0 - 1) + 1;
-    int qs[9], qe[9];
+    if constexpr (K == 1) {
+      int qs[9], qe[9];
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      const int z = cz + q / 3 - 1, y = cy + q % 3 - 1;
-      qs[q] = qe[q] = 0;
-      if (z >= 0 && z < n2 && y >= 0 && y < n1) {
-        const int *row = start + ((int64_t)z * n1 + y) * n0;
-        qs[q] = row[x0];
-        qe[q] = row[x1];
+      for (int q = 0; q < 9; ++q) {
+        const int z = cz + q / 3 - 1, y = cy + q % 3 - 1;
+        qs[q] = qe[q] = 0;
+        if (z >= 0 && z < n2 && y >= 0 && y < n1) {
+          const int *row = start + ((int64_t)z * n1 + y) * n0;
+          qs[q] = row[x0];
+          qe[q] = row[x1];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 9; ++q) knn_visit(best, sorted, qs[q], qe[q], me, i);
+    } else {
+      // many neighbours: the runs in a loop, whose body is the insertion of K
+      // compares (nine copies of it do not fit the instruction cache), the own
+      // cell first, whose centres are the likeliest to stay in the list; the
+      // next run's bounds are loaded meanwhile
+      auto bounds = [&](int h, int &qs, int &qe) {
+        const int q = h < 3 ? 4 : h < 7 ? h - 3 : h - 2;  // the own row is in three runs
+        const int z = cz + q / 3 - 1, y = cy + q % 3 - 1;
+        qs = qe = 0;
+        if (z >= 0 && z < n2 && y >= 0 && y < n1) {
+          const int *row = start + ((int64_t)z * n1 + y) * n0;
+          qs = row[h == 0 ? cx : h == 2 ? cx + 1 : x0];
+          qe = row[h == 0 ? cx + 1 : h == 1 ? cx : x1];
+        }
+      };
+      int ns, ne;
+      bounds(0, ns, ne);
+#pragma unroll 1
+      for (int h = 0; h < 11; ++h) {
+        const int qs = ns, qe = ne;
+        if (h < 10) bounds(h + 1, ns, ne);
+        knn_visit(best, sorted, qs, qe, me, i);
       }
     }
-#pragma unroll
-    for (int q = 0; q < 9; ++q) knn_visit(best, sorted, qs[q], qe[q], me, i);
     done = enough(best, 1) || rmax <= 1;
   }
-  for (unsigned todo = __ballot_sync(0xffffffffu, !done); todo; todo &= todo - 1) {
+  // row (z, y) of ring r about cell (cx, cy, cz), cut off at the grid's faces;
+  // the inner rows of a ring hold only its two end cells
+  auto visit_row = [&](KBest<K> &b, const float4 &p, int pi, int cx, int cy, int cz, int r, int z, int y) {
+    const int *row = start + ((int64_t)z * n1 + y) * n0;
+    const bool face = z == cz - r || z == cz + r || y == cy - r || y == cy + r;
+    const int a = cx - r, c = cx + r;  // the run a .. c, or the cells a and c
+    int qs = 0, qe = 0, rs = 0, re = 0;
+    if (face || a >= 0) {
+      qs = row[max(a, 0)];
+      qe = row[face ? min(c, n0 - 1) + 1 : a + 1];
+    }
+    if (!face && c < n0) {
+      rs = row[c];
+      re = row[c + 1];
+    }
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+      knn_visit(b, sorted, qs, qe, p, pi);
+      qs = rs;
+      qe = re;
+    }
+  };
+  int r0 = 2;
+  unsigned todo;
+  for (; (todo = __ballot_sync(0xffffffffu, !done)) != 0u; ++r0) {
+    const int cx = knn_axis_cell(me.x, G.lo[0], G.ih, n0);
+    const int cy = knn_axis_cell(me.y, G.lo[1], G.ih, n1);
+    const int cz = knn_axis_cell(me.z, G.lo[2], G.ih, n2);
+    const int z0 = max(cz - r0, 0), z1 = min(cz + r0, n2 - 1);
+    const int y0 = max(cy - r0, 0), y1 = min(cy + r0, n1 - 1);
+    const int rows = __reduce_max_sync(0xffffffffu, done ? 0 : (z1 - z0 + 1) * (y1 - y0 + 1));
+    if (__popc(todo) * (2 + K / 4 + rows / 32) < rows) break;
+    if (!done) {
+      for (int z = z0; z <= z1; ++z)
+        for (int y = y0; y <= y1; ++y) visit_row(best, me, i, cx, cy, cz, r0, z, y);
+      done = enough(best, r0) || r0 >= rmax;
+    }
+  }
+  for (; todo; todo &= todo - 1) {
     const int src = __ffs(todo) - 1;
     float4 p;
     p.x = __shfl_sync(0xffffffffu, me.x, src);
@@ -404,29 +473,23 @@ __global__ void __launch_bounds__(kKnnBlk) knn_query_kernel(
     const int cx = knn_axis_cell(p.x, G.lo[0], G.ih, n0);
     const int cy = knn_axis_cell(p.y, G.lo[1], G.ih, n1);
     const int cz = knn_axis_cell(p.z, G.lo[2], G.ih, n2);
-    // lane src starts from what it has, the others from nothing
+    // lane src starts from what it has, the others from placeholders at its
+    // k-th distance, which sort behind every centre that close
     KBest<K> b = best;
-    if (lane != src) b.clear();
-    for (int r = 2; r <= rmax; ++r) {
+    for (int r = r0; r <= rmax; ++r) {
+      const float kth = __shfl_sync(0xffffffffu, b.d[K - 1], src);
+      const int none = kth < INFINITY ? 0x7fffffff : -1;
+      if (lane != src) b.fill(kth, none);
       const int z0 = max(cz - r, 0), z1 = min(cz + r, n2 - 1);
       const int y0 = max(cy - r, 0), y1 = min(cy + r, n1 - 1);
-      const int x0 = max(cx - r, 0), x1 = min(cx + r, n0 - 1);
       const int ny = y1 - y0 + 1, rows = (z1 - z0 + 1) * ny;
       for (int q = lane; q < rows; q += 32) {
-        const int dz = q / ny, z = z0 + dz, y = y0 + (q - dz * ny);
-        const int *row = start + ((int64_t)z * n1 + y) * n0;
-        // inner rows of a ring hold only its two end cells
-        if (z == cz - r || z == cz + r || y == cy - r || y == cy + r) {
-          knn_visit(b, sorted, row[x0], row[x1 + 1], p, pi);
-        } else {
-          if (cx - r >= 0) knn_visit(b, sorted, row[cx - r], row[cx - r + 1], p, pi);
-          if (cx + r < n0) knn_visit(b, sorted, row[cx + r], row[cx + r + 1], p, pi);
-        }
+        const int dz = q / ny;
+        visit_row(b, p, pi, cx, cy, cz, r, z0 + dz, y0 + (q - dz * ny));
       }
       __syncwarp();
-      b.merge_warp();
-      if (enough(b, r)) break;
-      if (lane != src) b.clear();
+      if (__any_sync(0xffffffffu, lane != src && b.i[0] != none)) b.merge_warp();
+      if (__any_sync(0xffffffffu, lane == src && enough(b, r))) break;
     }
     if (lane == src) best = b;
   }
