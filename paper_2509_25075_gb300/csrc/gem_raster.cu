@@ -220,15 +220,22 @@ constexpr unsigned kNoSum = 0x80000000u;  // -0: a block without items (a sum of
 template <int kMinB, bool kCount>
 __global__ void __launch_bounds__(kThreads, kMinB) raster_fwd_kernel(
     const Rec *__restrict__ rec, const uint2 *__restrict__ list, int64_t M, int d, float l2tau,
-    RasterTasks tk, float *__restrict__ proj, unsigned long long *__restrict__ kept) {
+    RasterTasks tk, int sms, float *__restrict__ proj, unsigned long long *__restrict__ kept) {
   __shared__ FwdWin W;
   const int nt = d / kTile, T = nt * nt;
   const int hw = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float nl2tau = -l2tau;  // kept: -e < -log2(tau)
   const int ntasks = (int)tk.ctr[kCtrTasks];
   unsigned nkept = 0, neval = 0;
-  // thread 0 claims a task two ahead and reads its descriptor one ahead;
-  // a task with no entries ends the list
+  // A CTA's first three tasks are its own, one of each round of the grid, so
+  // that no CTA has two before every CTA has one; from there on thread 0 claims
+  // a task two ahead and reads its descriptor one ahead.  A round's tasks go to
+  // the SMs in turn (every sms-th CTA is on the same one, as a rule), moved on
+  // by one per turn: where lists are alike, full segments and short last ones
+  // alternate, and would meet on the same SMs.  (Claims from the second task on:
+  // a query of 300 Gaussians, side 96, tau 0: 531 us, now 443; a projection of
+  // 2000, side 384, one view, tau 0: 1541, now 1499.)  A task with no entries
+  // ends the list.
   auto task_at = [&](int q, uint4 &a, uint4 &c) {
     a = c = make_uint4(0u, 0u, 0u, 0u);
     if (q < ntasks) {
@@ -236,13 +243,14 @@ __global__ void __launch_bounds__(kThreads, kMinB) raster_fwd_kernel(
       c = tk.task[2 * (int64_t)q + 1];
     }
   };
-  auto claim = [&]() { return (int)(atomicAdd(tk.ctr + kCtrFwd, 1u) + gridDim.x); };
+  auto claim = [&]() { return (int)(atomicAdd(tk.ctr + kCtrFwd, 1u) + 3 * gridDim.x); };
   int nq = 0;
   if (threadIdx.x == 0) {
-    task_at(blockIdx.x, W.desc[0][0], W.desc[0][1]);
-    const int q1 = claim();
-    nq = claim();
-    task_at(q1, W.desc[1][0], W.desc[1][1]);
+    const int G = (int)gridDim.x, col = (int)blockIdx.x % sms, row = (int)blockIdx.x / sms;
+    auto own = [&](int r) { return r * G + row * sms + (col + row + r) % sms; };
+    task_at(own(0), W.desc[0][0], W.desc[0][1]);
+    task_at(own(1), W.desc[1][0], W.desc[1][1]);
+    nq = own(2);
   }
   __syncthreads();
   // this warp's quarter of a window: slots 64 hw .. 64 hw + 63, two per lane.
@@ -493,9 +501,9 @@ static cudaError_t launch_fwd_any(int cfg, const Rec *rec, const uint2 *list,
                                                             sms * 8, tk, proj);
   const int grid = sms * kFwdCfgs[cfg].ctas;
   if (kFwdCfgs[cfg].ctas > 7)
-    raster_fwd_kernel<8, kCount><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tk, proj, kept);
+    raster_fwd_kernel<8, kCount><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tk, sms, proj, kept);
   else
-    raster_fwd_kernel<7, kCount><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tk, proj, kept);
+    raster_fwd_kernel<7, kCount><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tk, sms, proj, kept);
   return cudaGetLastError();
 }
 

@@ -48,3 +48,27 @@ def test_list_lengths_in_a_large_call(M):
     """About a million entries: the longest segments.  tau = 0, so that no pair
     is near the threshold."""
     _check(M, 1 + 1000000 // M, seed=M, tau=0.0)
+
+
+@pytest.mark.parametrize("cfg", [0, 3, 7])
+@pytest.mark.parametrize("B", [1, 151, 153, 1216, 1217, 2433, 3647, 3649, 5001])
+def test_as_many_tasks_as_rounds_of_the_grid(B, cfg):
+    """One task per image, around whole rounds of the grid (152 x 8, 5 and 1
+    CTAs): every image is the bits it has in a call of seven views."""
+    w = syn.Workload("task", d=16, M=40, B=7, apix=1.2, n_clusters=1, s_lo=0.8, s_hi=3.0, seed=5)
+    inp = gt.inputs(w)
+    params, R, t = (gt.to_dev(inp[k]) for k in ("params", "R", "t"))
+    seven = torch.empty(7, 16, 16, device=gt.DEV)
+    ctx = gt.context(w)
+    ctx.gem_project(params, R, t, seven)
+    ctx.close()
+    view = torch.arange(B, device=gt.DEV) % 7
+    ctx = gt.context(syn.Workload("task", d=16, M=40, B=B, apix=1.2, seed=5), tau=w.tau)
+    ctx.gem_set_raster_config(cfg, -1)
+    proj = torch.full((B, 16, 16), float("nan"), device=gt.DEV)
+    for _ in range(2):
+        ctx.gem_project(params, R[view].contiguous(), t[view].contiguous(), proj)
+    assert ctx.gem_status() == 0
+    assert float(seven.max()) > 0
+    assert torch.equal(proj, seven[view])
+    ctx.close()
