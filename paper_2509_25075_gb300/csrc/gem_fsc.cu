@@ -16,6 +16,8 @@
 // 256^3 maps 664 -> 293 us, the shell sums as they were.
 #include <math.h>
 
+#include <algorithm>
+
 #include "gem_fft.cuh"
 #include "gem_internal.cuh"
 #include "gem_pairsum.cuh"
@@ -23,7 +25,7 @@
 namespace gem {
 
 constexpr int kFThreads = 256;
-constexpr int kShellBlocks = 1216;  // 8 per SM on 152 SMs
+constexpr int kShellBlocks = 1216;  // most blocks of the shell sums: 8 per SM on 152 SMs
 // Lines per CTA of the transform passes: 16 (their transposed stores then
 // fill 128-byte lines) up to sides whose 16 lines leave room for four CTAs
 // per SM, else 8.
@@ -91,6 +93,14 @@ __device__ __forceinline__ float seg_add(float v, int o, bool take) {
   return take ? v + u : v;
 }
 
+// CTAs of the shell sums that an SM's shared memory holds, at most 8.
+__host__ __device__ constexpr int shell_ctas(int n) {
+  const int fit = 228 * 1024 / (9 * 3 * (n / 2 + 1) * (int)sizeof(double) + 1024);
+  return fit < 8 ? fit : 8;
+}
+// Rows of a unit of the shell sums.
+__host__ __device__ constexpr int shell_rows(int n) { return n % 32 ? 2 : 1; }
+
 // Per-block sums over the shells 0 .. nsh-1 of Re(F1 F2^*), |F1|^2, |F2|^2,
 // written to part[blk][3][nsh].  A warp takes 32 consecutive frequencies;
 // neighbouring frequencies mostly share a shell, so each run of equal shells
@@ -115,11 +125,13 @@ __device__ __forceinline__ float seg_add(float v, int o, bool take) {
 // last shell load and sum nothing.  The warp follows a unit with its mirror
 // image, which then finds both its operands in L1.  Against one pass over all
 // frequencies with divisions, two loads each and float64 atomics: side 256,
-// the whole call 293 -> 226 us (287 with float64 sums).
+// the whole call 293 -> 220 us (287 with float64 sums).  Where a step lies in
+// one half of a row (sides that 64 divides), as few registers as leave room
+// for the CTAs that the shared memory holds: side 256, 226 -> 220 us.
 template <int N>
-__global__ void __launch_bounds__(kFThreads) fsc_shell_kernel(const float2 *__restrict__ F, int nsh,
-                                                              double *__restrict__ part) {
-  constexpr int q = N % 32 ? 2 : 1, h = N / 2, kUnits = N / q;  // units per plane
+__global__ void __launch_bounds__(kFThreads, N % 64 == 0 ? shell_ctas(N) : 1)
+    fsc_shell_kernel(const float2 *__restrict__ F, int nsh, double *__restrict__ part) {
+  constexpr int q = shell_rows(N), h = N / 2, kUnits = N / q;  // units per plane
   static_assert(q * N % 32 == 0, "a unit is whole warps");
   constexpr int kWarps = kFThreads / 32;
   extern __shared__ double big[];  // [3][nsh], then the warps' pairs [kWarps][3][nsh]
@@ -193,9 +205,10 @@ __global__ void __launch_bounds__(kFThreads) fsc_shell_kernel(const float2 *__re
       const bool write = last && s < nsh;
       if (h % 32 == 0 || i0 / h == (i0 + 31) / h) {
         if (write) add(s, num, p1, p2);
-      } else {  // rows' halves meet here: one run at a time
-        for (unsigned w = __ballot_sync(0xffffffffu, write); w; w &= w - 1) {
-          if (lane == __ffs(w) - 1) add(s, num, p1, p2);
+      } else {  // rows' halves meet here: one half's runs at a time
+#pragma unroll
+        for (int g = 0; g <= 31 / h + 1; ++g) {
+          if (write && e / h == i0 / h + g) add(s, num, p1, p2);
           __syncwarp();
         }
       }
@@ -303,6 +316,13 @@ cudaError_t fsc_configure(int d) {
   return cudaErrorInvalidValue;
 }
 
+// A block for every eight units of the half volume: beyond that (sides up to
+// 128) blocks would only clear, write and fold empty sums.
+static int shell_blocks(int d) {
+  constexpr int kWarps = kFThreads / 32;
+  return std::min(kShellBlocks, ((d / 2 + 1) * (d / shell_rows(d)) + kWarps - 1) / kWarps);
+}
+
 template <int N>
 static void launch_fsc_passes(const float2 *tw, const float *X1, const float *X2, float2 *P, float2 *Q,
                               double *part, cudaStream_t st) {
@@ -312,7 +332,7 @@ static void launch_fsc_passes(const float2 *tw, const float *X1, const float *X2
   fsc_pass_cplx_kernel<N><<<g, kFThreads, smem, st>>>(P, tw, Q);
   fsc_pass_cplx_kernel<N><<<g, kFThreads, smem, st>>>(Q, tw, P);
   const int nsh = N / 2 + 1;
-  fsc_shell_kernel<N><<<kShellBlocks, kFThreads, shell_smem(nsh), st>>>(P, nsh, part);
+  fsc_shell_kernel<N><<<shell_blocks(N), kFThreads, shell_smem(nsh), st>>>(P, nsh, part);
 }
 
 // block partials, then the folded sums
@@ -333,7 +353,7 @@ cudaError_t launch_fsc(int d, float apix, float thr, const float2 *tw, const flo
   }
   const int nsh = d / 2 + 1;
   double *tot = part + (size_t)kShellBlocks * 3 * nsh;
-  fsc_fold_kernel<<<nsh, 256, 0, st>>>(part, kShellBlocks, nsh, tot);
+  fsc_fold_kernel<<<nsh, 256, 0, st>>>(part, shell_blocks(d), nsh, tot);
   fsc_final_kernel<<<1, 512, nsh * sizeof(double), st>>>(tot, nsh, d, apix, thr, fsc, sums,
                                                          resolution);
   return cudaGetLastError();
