@@ -80,3 +80,34 @@ def test_fsc_rejects_bad_threshold():
     with pytest.raises(binding.GemError) as ei:
         ctx.gem_fsc(X, X, 1.5)
     assert ei.value.code == binding.GEM_EINVAL
+
+
+@pytest.mark.parametrize("d", [384, 432, 512, 576, 768])
+def test_fsc_large_sides(d):
+    """The shell sums at the sides whose transforms take 8 lines per block and
+    whose shell sums need more than 48 KB, against torch.fft in float64.  A
+    float32 transform of n values is off by at most about 2^-24 log2 n of
+    their rms (both maps share one complex transform), and a run of 32
+    products by 2^-19 of their absolute sum."""
+    g = torch.Generator(device="cuda").manual_seed(d)
+    a = torch.randn(d, d, d, device=gt.DEV, generator=g)
+    b = a + torch.randn(d, d, d, device=gt.DEV, generator=g)
+    ctx = _ctx(d)
+    _, sums, _ = ctx.gem_fsc(a, b)
+    assert ctx.gem_status() == 0
+    k = torch.fft.fftfreq(d, 1.0 / d, device=gt.DEV, dtype=torch.float64).round()
+    k2 = k[:, None, None] ** 2 + k[None, :, None] ** 2 + k[None, None, :] ** 2
+    shell = torch.floor(k2.sqrt() + 0.5).long()
+    n = d // 2 + 1
+    at = shell < n
+    shell = shell[at]
+    F1, F2 = (torch.fft.fftn(x.double())[at] for x in (a, b))
+    total = lambda x: torch.bincount(shell, x, n)  # noqa: E731
+    A1, A2 = F1.abs(), F2.abs()
+    delta = 2.0 ** -24 * np.log2(float(d) ** 3) * float((A1 ** 2 + A2 ** 2).mean().sqrt())
+    s1, s2 = total(A1), total(A2)
+    for i, (ref, terms) in enumerate([((F1 * F2.conj()).real, delta * (s1 + s2)),
+                                      (A1 ** 2, 2 * delta * s1), (A2 ** 2, 2 * delta * s2)]):
+        allow = terms + 2.0 ** -19 * total(ref.abs())
+        assert ((sums[i] - total(ref)).abs() <= allow).all()
+    ctx.close()
