@@ -779,7 +779,8 @@ def main():
         q_ms = sum(a.elapsed_time(b) for a, b in qe) / nq
         nbatch = -(-w.d // w.B)
         query = {"ms": q_ms, "voxels_per_s": w.d ** 3 / (q_ms / 1e3), "grid": w.d, "M": w.M, "tau": tq,
-                 "slice_batches": nbatch, "gpu_launches_per_call": 1 + (7 if w.M <= 16384 else 9) * nbatch,
+                 "slice_batches": nbatch, "gpu_launches_per_call": 1 + sum(7 if w.M <= 16384 or w.M * min(w.B, w.d - k) <= 400000 else 9
+                                                          for k in range(0, w.d, w.B)),
                  "l2": "flushed before each call (256 MB write)"}
         # Fourier shell correlation of the map against the map of perturbed
         # Gaussians (the two half-maps of Eq. fsc)

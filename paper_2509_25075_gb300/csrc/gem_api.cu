@@ -726,10 +726,18 @@ int gem_query(gem_ctx *c, const float *params, int64_t M, float tau, float *vol)
   const size_t slice = (size_t)g.d * g.d;
   for (int k0 = 0; k0 < g.d; k0 += g.max_B) {
     const int ns = g.d - k0 < g.max_B ? g.d - k0 : g.max_B;
-    if ((e = launch_slices(c->qp, c->slice_range, M, k0, ns, g.apix, g.d, l2tau, c->bin.tcnt, c->rec,
-                           c->bin.perm, c->nsel, c->stream)) != cudaSuccess ||
-        (e = launch_bin_selected(c->rec, c->bin.perm, c->nsel, M, ns, g.d, l2tau, c->bin,
-                                 c->stream)) != cudaSuccess ||
+    if (slices_all(M, ns)) {
+      const uint32_t *perm = nullptr;
+      e = launch_slices_all(c->qp, M, k0, ns, g.apix, g.d, l2tau, c->rec, c->stream);
+      if (e == cudaSuccess)
+        e = launch_bin(c->rec, c->bin.key, M, ns, g.d, l2tau, 0, c->bin, &perm, c->stream);
+    } else {
+      e = launch_slices(c->qp, c->slice_range, M, k0, ns, g.apix, g.d, l2tau, c->bin.tcnt, c->rec,
+                        c->bin.perm, c->nsel, c->stream);
+      if (e == cudaSuccess)
+        e = launch_bin_selected(c->rec, c->bin.perm, c->nsel, M, ns, g.d, l2tau, c->bin, c->stream);
+    }
+    if (e != cudaSuccess ||
         (e = launch_raster_fwd(active_fwd(c, ns, M), c->rec, c->bin.list,
                                c->bin.tile_start, c->bin.cap, M, ns, g.d, l2tau,
                                vol + (size_t)k0 * slice, c->tasks, true, c->stream)) !=

@@ -222,6 +222,12 @@ struct __align__(16) QueryPrep {
 // (first > last: none).
 cudaError_t launch_query_prep(const float *params, int64_t M, int norm_mode, int shape, float apix,
                               int d, float l2tau, QueryPrep *qp, uint32_t *range, cudaStream_t st);
+// Whether a batch of slices gives every Gaussian a record in every slice, or
+// lists the Gaussians that can matter in each.
+bool slices_all(int64_t M, int nslice);
+// Records of the slices k0 .. k0 + nslice - 1 for every Gaussian: rec[b][j].
+cudaError_t launch_slices_all(const QueryPrep *qp, int64_t M, int k0, int nslice, float apix, int d,
+                              float l2tau, Rec *rec, cudaStream_t st);
 // Records of the slices k0 .. k0 + nslice - 1 for the Gaussians that can
 // exceed tau there: rec[b][j], their indices in ascending order sel[b][..],
 // their number nsel[b].  cnt [chunks][nslice] is scratch.

@@ -119,6 +119,14 @@ __device__ __forceinline__ Rec slice_record(const QueryPrep &g, int k, float api
   return r;
 }
 
+// Few (slice, Gaussian) pairs: a record of every Gaussian in every slice.
+__global__ void __launch_bounds__(256) slice_all_kernel(const QueryPrep *__restrict__ qp, int64_t M,
+                                                        int k0, float apix, int d, float l2tau,
+                                                        Rec *__restrict__ rec) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < M) rec[(int64_t)blockIdx.y * M + j] = slice_record(qp[j], k0 + (int)blockIdx.y, apix, d, l2tau);
+}
+
 // Which Gaussians of chunk blockIdx.x (256 of them) meet which slices of the
 // batch: one bit per Gaussian, bm[slice][8].
 __device__ __forceinline__ void slice_bits(uint32_t *bm, const uint32_t *__restrict__ range, int64_t M,
@@ -209,6 +217,20 @@ cudaError_t launch_query_prep(const float *params, int64_t M, int norm_mode, int
                               int d, float l2tau, QueryPrep *qp, uint32_t *range, cudaStream_t st) {
   query_prep_kernel<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(params, M, norm_mode, shape, apix, d,
                                                                  l2tau, qp, range);
+  return cudaGetLastError();
+}
+
+// Where a record of every Gaussian in every slice and the lists of those that
+// can matter meet: us per batch, all and lists, of M Gaussians and n slices.
+// d 256: M 16000, n 8: 40, 50; M 20000, n 16: 49, 56; M 50000, n 4: 45, 50, n 8:
+// 52, 51; M 100000, n 4: 52, 51, n 8: 66, 58; M 300000, n 1: 54, 59, n 2: 66, 62.
+// d 64: M 20000, n 16: 51, 62; M 50000, n 8: 54, 58; M 100000, n 8: 78, 72.
+bool slices_all(int64_t M, int nslice) { return M * nslice <= 400000; }
+
+cudaError_t launch_slices_all(const QueryPrep *qp, int64_t M, int k0, int nslice, float apix, int d,
+                              float l2tau, Rec *rec, cudaStream_t st) {
+  const dim3 grid((unsigned)((M + 255) / 256), (unsigned)nslice);
+  slice_all_kernel<<<grid, 256, 0, st>>>(qp, M, k0, apix, d, l2tau, rec);
   return cudaGetLastError();
 }
 
