@@ -89,12 +89,15 @@ __device__ __forceinline__ int64_t segment_length(int64_t total, int slots) {
   return (max((int64_t)1, min((int64_t)kSegMax, S)) + kWin - 1) / kWin * kWin;
 }
 
+// A CTA takes kPer tiles, one per thread, and its eight warps share the zeros of
+// the empty ones.
+template <int kPer>
 __global__ void __launch_bounds__(256) raster_tasks_kernel(const int64_t *__restrict__ tile_start,
                                                            int ntiles, int64_t cap, int d, int slots,
                                                            RasterTasks tk, float *__restrict__ proj) {
-  __shared__ unsigned wsum[2][8], base_sh[2];
+  __shared__ unsigned wsum[2][8], base_sh[2], empty[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * 256 + threadIdx.x;
+  const int i0 = blockIdx.x * kPer, i = (int)threadIdx.x < kPer ? i0 + (int)threadIdx.x : ntiles;
   const int64_t total = tile_start[ntiles];
   // lists that overflowed their capacity are incomplete: every list counts
   // as empty (the status word reports it)
@@ -119,9 +122,11 @@ __global__ void __launch_bounds__(256) raster_tasks_kernel(const int64_t *__rest
       incp += v;
     }
   }
+  const unsigned none = __ballot_sync(0xffffffffu, i < ntiles && nseg == 0);
   if (lane == 31) {
     wsum[0][warp] = inc;
     wsum[1][warp] = incp;
+    empty[warp] = none;
   }
   __syncthreads();
   unsigned at = inc - nseg, part = incp - mine, all = 0, allp = 0;
@@ -134,7 +139,7 @@ __global__ void __launch_bounds__(256) raster_tasks_kernel(const int64_t *__rest
     all += wsum[0][w];
     allp += wsum[1][w];
   }
-  if (i == 0) tk.ctr[kCtrSegment] = (unsigned)S;
+  if (i0 + threadIdx.x == 0) tk.ctr[kCtrSegment] = (unsigned)S;
   if (threadIdx.x == 0) {
     base_sh[0] = atomicAdd(tk.ctr + kCtrTasks, all);
     base_sh[1] = atomicAdd(tk.ctr + kCtrParts, allp);
@@ -152,8 +157,9 @@ __global__ void __launch_bounds__(256) raster_tasks_kernel(const int64_t *__rest
   }
   if (proj) {
     const int nt = d / kTile, T = nt * nt;
-    for (unsigned e = __ballot_sync(0xffffffffu, i < ntiles && nseg == 0); e; e &= e - 1) {
-      const int bt = blockIdx.x * 256 + warp * 32 + __ffs(e) - 1;
+    for (int k = warp; k < kPer; k += 8) {
+      if (!(empty[k >> 5] >> (k & 31) & 1u)) continue;
+      const int bt = i0 + k;
       const int b = bt / T, t = bt - b * T;
       float *o = proj + ((int64_t)b * d + (t / nt) * kTile) * d + (t % nt) * kTile;
 #pragma unroll
@@ -497,8 +503,11 @@ static cudaError_t launch_fwd_any(int cfg, const Rec *rec, const uint2 *list,
     const cudaError_t e = cudaMemsetAsync(tk.ctr, 0, kCtrCount * sizeof(unsigned), st);
     if (e != cudaSuccess) return e;
   }
-  raster_tasks_kernel<<<(ntiles + 255) / 256, 256, 0, st>>>(tile_start, ntiles, cap, d,
-                                                            sms * 8, tk, proj);
+  // small calls: fewer tiles per CTA, so that more CTAs share the zeros
+  if (ntiles <= 32 * sms)
+    raster_tasks_kernel<32><<<(ntiles + 31) / 32, 256, 0, st>>>(tile_start, ntiles, cap, d, sms * 8, tk, proj);
+  else
+    raster_tasks_kernel<256><<<(ntiles + 255) / 256, 256, 0, st>>>(tile_start, ntiles, cap, d, sms * 8, tk, proj);
   const int grid = sms * kFwdCfgs[cfg].ctas;
   if (kFwdCfgs[cfg].ctas > 7)
     raster_fwd_kernel<8, kCount><<<grid, kThreads, 0, st>>>(rec, list, M, d, l2tau, tk, sms, proj, kept);
