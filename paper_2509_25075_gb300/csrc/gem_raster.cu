@@ -617,11 +617,13 @@ __device__ __forceinline__ void block_moments(const float4 (*__restrict__ sg)[16
   n[2] = add2(n[2], make_float2(m4, m5));
 }
 
-// Entries of a backward unit: 256, less (down to 64) where that would leave
-// warps of the grid without one.
+// Entries of a backward unit: 256, or 128 where the lists hold no more than one
+// and a half times 256 for every warp of the grid, so that the last units take
+// less of the time.  us per backward with units of 64, 128, 256, by entries per
+// warp / 256 (d 128, M 20000): 0.8: 71, 72, 90; 1.26: 98, 91, 101; 1.5: 110, 104,
+// 107; 2: 141, 128, 127; 4: 279, 218, 202.
 __device__ __forceinline__ int unit_length(int64_t total, int nwarps) {
-  const int64_t U = (total / nwarps + 31) / 32 * 32;
-  return (int)max((int64_t)64, min((int64_t)256, U));
+  return total <= 384 * (int64_t)nwarps ? 128 : 256;
 }
 
 // a5.  Every warp works on its own: a unit is up to 256 consecutive entries of
@@ -631,52 +633,62 @@ __device__ __forceinline__ int unit_length(int64_t total, int nwarps) {
 // sorts each window of its unit by (number of blocks, first block) and runs
 // it in rounds of 32 records, one lane per record: the lanes of a round have
 // loops of one length, and mostly read the same blocks of g at the same time
-// (a broadcast instead of bank conflicts).  The moments of a round are added
-// to memory six lanes per record, which costs the L1 a sixth of the tag
-// lookups of one lane per record and about a tenth more instructions: the
-// better of the two at 2.5 list entries per (view, Gaussian) and four blocks
-// each (d 128, M 20000, B 256: 0.53 against 0.59 ms), the worse at 4.2 and
-// 5.5 (d 128, M 50000, B 64, scales 0.3-12 px: 0.66 against 0.62 ms), where
-// a record's evaluation takes longer; the line lies at 3 entries.
+// (a broadcast instead of bank conflicts).
+//
+// The moments of a round are added to memory one lane per record, or six lanes
+// per record, which costs the L1 a sixth of the tag lookups and about a tenth
+// more instructions.  Six lanes are the better where records have few blocks
+// to evaluate between their additions.  us per backward, one lane and six, by
+// list entries per (view, Gaussian): 1.24 (d 128, M 20000, B 128): 229, 218;
+// 1.75 (d 384, M 300000, B 8): 283, 262; 1.88 (d 128, M 20000) B 32: 93, 97,
+// B 96: 221, 206; 2.08, B 32: 101, 106, B 96: 232, 224; 2.45, B 32: 119, 126,
+// B 256: 626, 639; 4.2 (scales 0.3-12 px, M 50000, B 64): 723, 758.  The line
+// lies at 2.  Each form is an instance of its own: one loop with both took 1 to
+// 3% longer.
 //
 // What bounds it: the FMA pipe (57% of its cycles) and issue (66%).  Against
 // CTAs of four warps that walked a whole tile's list, the longest lists first
-// (us per launch, the default configuration then, the one the autotuner
-// picked, now): d 384, M 500000, B 16: 1033, 901, 792; d 128, M 20000, B 256:
-// 568, 568, 540; d 128, M 50000, B 64, scales 0.3-12 px: 1150, 846, 637;
-// d 64, M 2000, B 32: 44, 42, 26.
-template <int kPer, int kMinB>
-__global__ void __launch_bounds__(kThreads, kMinB) raster_bwd_kernel(
-    const Rec *__restrict__ rec, const uint2 *__restrict__ list, int64_t M, int d, float l2tau,
-    const int64_t *__restrict__ tile_start, int ntiles, const float *__restrict__ dproj,
-    double *__restrict__ mom, RasterTasks tk) {
-  constexpr int kWarps = kThreads / 32;
-  constexpr int kWW = 32 * kPer;  // records per window
-  constexpr int kBins = 256;      // (16 - blocks) * 16 + first block
-  __shared__ float4 sg_[kWarps][4][16];  // g by row pair and column of a block, and block
-  __shared__ float4 sa_[kWarps][kWW];    // px, py, u11, u12
-  __shared__ float2 sb_[kWarps][kWW];    // u22, log2 A
-  __shared__ uint32_t sj_[kWarps][kWW];
-  __shared__ unsigned short smask_[kWarps][kWW];
-  __shared__ float red_[kWarps][32 * 7];  // a round's moments, one word of padding per record
-  static_assert(sizeof(sa_[0]) >= kBins * sizeof(int), "the bins lie where the records go");
+// (us per backward, the default configuration then and now): d 384, M 500000,
+// B 3: 699, 271; d 128, M 20000, B 256: 677, 623; d 128, M 50000, B 64, scales
+// 0.3-12 px: 1084, 715; d 64, M 2000, B 32: 57, 35, but B 320: 115, 121 (the
+// step of these: 406, 354).
+// One warp's shared memory.
+template <int kPer>
+struct BwdWarp {
+  static constexpr int kWW = 32 * kPer;  // records per window
+  static constexpr int kBins = 256;      // (16 - blocks) * 16 + first block
+  float4 sg[4][16];                      // g by row pair and column of a block, and block
+  float4 sa[kWW];                        // px, py, u11, u12
+  float2 sb[kWW];                        // u22, log2 A
+  uint32_t sj[kWW];
+  unsigned short smask[kWW];
+  float red[32 * 7];  // a round's moments, one word of padding per record
+  static_assert(sizeof(float4) * kWW >= kBins * sizeof(int), "the bins lie where the records go");
+};
+
+// The walk of one warp; spread: the moments of a round are added one lane per
+// record, else six.
+template <bool spread, int kPer>
+__device__ __forceinline__ void bwd_walk(
+    BwdWarp<kPer> &S, const Rec *__restrict__ rec, const uint2 *__restrict__ list, int64_t M, int d,
+    float l2tau, int64_t total, const float *__restrict__ dproj, double *__restrict__ mom,
+    const RasterTasks &tk) {
+  constexpr int kWarps = kThreads / 32, kWW = 32 * kPer;
   const int nt = d / kTile, T = nt * nt;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float nl2tau = -l2tau;  // kept: -e < -log2(tau)
-  float4(*sg)[16] = sg_[warp];
-  float4 *sa = sa_[warp];
-  float2 *sb = sb_[warp];
-  uint32_t *sj = sj_[warp];
-  unsigned short *smask = smask_[warp];
-  float *red = red_[warp];
+  float4(*sg)[16] = S.sg;
+  float4 *sa = S.sa;
+  float2 *sb = S.sb;
+  uint32_t *sj = S.sj;
+  unsigned short *smask = S.smask;
+  float *red = S.red;
   const int lr = lane < 30 ? lane / 6 : 64, lc = lane % 6;  // record and moment a lane adds
   int *bins = reinterpret_cast<int *>(sa);
   const int nwarps = (int)gridDim.x * kWarps;
-  const int64_t total = tile_start[ntiles];
   const int unit = unit_length(total, nwarps);
   const int per_task = ((int)tk.ctr[kCtrSegment] + unit - 1) / unit;  // units of a task
   const int64_t nunits = (int64_t)tk.ctr[kCtrTasks] * per_task;
-  const bool spread = total > 3 * (int64_t)(ntiles / T) * M;
   int64_t u = blockIdx.x * kWarps + warp;
   uint4 t0 = make_uint4(0u, 0u, 0u, 0u);
   if (u < nunits) t0 = tk.task[2 * (u / per_task)];
@@ -825,6 +837,20 @@ __global__ void __launch_bounds__(kThreads, kMinB) raster_bwd_kernel(
     u = nu;
     t0 = tn;
   }
+}
+
+template <int kPer, int kMinB>
+__global__ void __launch_bounds__(kThreads, kMinB) raster_bwd_kernel(
+    const Rec *__restrict__ rec, const uint2 *__restrict__ list, int64_t M, int d, float l2tau,
+    const int64_t *__restrict__ tile_start, int ntiles, const float *__restrict__ dproj,
+    double *__restrict__ mom, RasterTasks tk) {
+  __shared__ BwdWarp<kPer> S[kThreads / 32];
+  const int nt = d / kTile;
+  const int64_t total = tile_start[ntiles];
+  if (total > 2 * (int64_t)(ntiles / (nt * nt)) * M)
+    bwd_walk<true, kPer>(S[threadIdx.x >> 5], rec, list, M, d, l2tau, total, dproj, mom, tk);
+  else
+    bwd_walk<false, kPer>(S[threadIdx.x >> 5], rec, list, M, d, l2tau, total, dproj, mom, tk);
 }
 
 // The backward's kernel configurations (the autotuner's search space):

@@ -72,3 +72,35 @@ def test_as_many_tasks_as_rounds_of_the_grid(B, cfg):
     assert float(seven.max()) > 0
     assert torch.equal(proj, seven[view])
     ctx.close()
+
+
+@pytest.mark.parametrize("d,M,copies", [(16, 1500, 110), (16, 1500, 111), (16, 1500, 112), (64, 100, 103),
+                                        (64, 100, 104), (64, 100, 105), (64, 100, 1)])
+def test_backward_of_repeated_views(d, M, copies):
+    """Calls on either side of the line between units of 128 and 256 entries
+    (384 x 3040 entries), with few and with many entries per Gaussian and view
+    (the two ways to add the moments): seven views over and over give the
+    gradient of the seven, as often."""
+    w = syn.Workload("rep", d=d, M=M, B=7, apix=1.2, n_clusters=1, s_lo=0.8, s_hi=3.0, seed=6)
+    inp = gt.inputs(w)
+    params, R, t = (gt.to_dev(inp[k]) for k in ("params", "R", "t"))
+    g = gt.to_dev(syn.smooth_field(w) * 1e-3)
+    grads = []
+    for k in (1, copies):
+        view = torch.arange(7 * k, device=gt.DEV) % 7
+        ctx = gt.context(syn.Workload("rep", d=d, M=M, B=7 * k, apix=1.2, seed=6), tau=0.0,
+                         max_pairs=7 * k * M * (d // 16) ** 2)
+        proj = torch.empty(7 * k, d, d, device=gt.DEV)
+        Rk, tk = R[view].contiguous(), t[view].contiguous()
+        ctx.gem_project(params, Rk, tk, proj)
+        grad = torch.empty(M, 11, device=gt.DEV)
+        ctx.gem_project_backward(g[view].contiguous(), grad)
+        assert ctx.gem_status() == 0
+        assert ctx.gem_pair_count() == 7 * k * M * (d // 16) ** 2
+        grads.append(grad.double())
+        ctx.close()
+    if copies == 1:  # the seven views themselves, against the oracle
+        ref = oracle.grad(inp["params"], inp["R"], inp["t"], d, w.apix, 0.0, g.cpu().numpy())
+        assert np.linalg.norm(grads[0].cpu().numpy() - ref) <= 1e-4 * np.linalg.norm(ref)
+    err = float((grads[1] / copies - grads[0]).norm())
+    assert err <= 1e-6 * float(grads[0].norm())
