@@ -652,8 +652,10 @@ __device__ __forceinline__ int unit_length(int64_t total, int nwarps) {
 // B 3: 699, 271; d 128, M 20000, B 256: 677, 623; d 128, M 50000, B 64, scales
 // 0.3-12 px: 1084, 715; d 64, M 2000, B 32: 57, 35, but B 320: 115, 121 (the
 // step of these: 406, 354).
-// One warp's shared memory.
-template <int kPer>
+
+// One warp's shared memory.  A round's moments have kRed words per record: one
+// of padding where that does not cost a CTA.
+template <int kPer, int kRed>
 struct BwdWarp {
   static constexpr int kWW = 32 * kPer;  // records per window
   static constexpr int kBins = 256;      // (16 - blocks) * 16 + first block
@@ -662,15 +664,15 @@ struct BwdWarp {
   float2 sb[kWW];                        // u22, log2 A
   uint32_t sj[kWW];
   unsigned short smask[kWW];
-  float red[32 * 7];  // a round's moments, one word of padding per record
+  float red[32 * kRed];                  // a round's moments
   static_assert(sizeof(float4) * kWW >= kBins * sizeof(int), "the bins lie where the records go");
 };
 
 // The walk of one warp; spread: the moments of a round are added one lane per
 // record, else six.
-template <bool spread, int kPer>
+template <bool spread, int kPer, int kRed>
 __device__ __forceinline__ void bwd_walk(
-    BwdWarp<kPer> &S, const Rec *__restrict__ rec, const uint2 *__restrict__ list, int64_t M, int d,
+    BwdWarp<kPer, kRed> &S, const Rec *__restrict__ rec, const uint2 *__restrict__ list, int64_t M, int d,
     float l2tau, int64_t total, const float *__restrict__ dproj, double *__restrict__ mom,
     const RasterTasks &tk) {
   constexpr int kWarps = kThreads / 32, kWW = 32 * kPer;
@@ -814,7 +816,7 @@ __device__ __forceinline__ void bwd_walk(
             for (int i = 0; i < 6; ++i) atomicAdd(mo + i, (double)(i & 1 ? tot[i / 2].y : tot[i / 2].x));
           } else {
 #pragma unroll
-            for (int i = 0; i < 6; ++i) red[7 * lane + i] = i & 1 ? tot[i / 2].y : tot[i / 2].x;
+            for (int i = 0; i < 6; ++i) red[kRed * lane + i] = i & 1 ? tot[i / 2].y : tot[i / 2].x;
           }
         }
         if (spread) continue;
@@ -822,11 +824,11 @@ __device__ __forceinline__ void bwd_walk(
         // six lanes add one record's six moments, five records at a time: the
         // warp's addresses then lie in five or so lines, not in 32
         const int left = min(32, nv - r0);
-        const float *rp = red + 7 * lr + lc;
+        const float *rp = red + kRed * lr + lc;
         const uint32_t *jp = sj + r0 + lr;
 #pragma unroll
         for (int i = 0; i < 7; ++i)
-          if (5 * i + lr < left) atomicAdd(mbl + 6ull * jp[5 * i], (double)rp[35 * i]);
+          if (5 * i + lr < left) atomicAdd(mbl + 6ull * jp[5 * i], (double)rp[5 * kRed * i]);
         __syncwarp();  // read before the next round's replace them
       }
     }
@@ -844,13 +846,16 @@ __global__ void __launch_bounds__(kThreads, kMinB) raster_bwd_kernel(
     const Rec *__restrict__ rec, const uint2 *__restrict__ list, int64_t M, int d, float l2tau,
     const int64_t *__restrict__ tile_start, int ntiles, const float *__restrict__ dproj,
     double *__restrict__ mom, RasterTasks tk) {
-  __shared__ BwdWarp<kPer> S[kThreads / 32];
+  // six CTAs of 256-record windows fit an SM's shared memory to the byte
+  constexpr int kRed = kPer == 8 && kMinB == 6 ? 6 : 7;
+  __shared__ BwdWarp<kPer, kRed> S[kThreads / 32];
+  static_assert(kMinB * (sizeof(S) + 1024) <= 228 * 1024, "kMinB CTAs fit an SM's shared memory");
   const int nt = d / kTile;
   const int64_t total = tile_start[ntiles];
   if (total > 2 * (int64_t)(ntiles / (nt * nt)) * M)
-    bwd_walk<true, kPer>(S[threadIdx.x >> 5], rec, list, M, d, l2tau, total, dproj, mom, tk);
+    bwd_walk<true, kPer, kRed>(S[threadIdx.x >> 5], rec, list, M, d, l2tau, total, dproj, mom, tk);
   else
-    bwd_walk<false, kPer>(S[threadIdx.x >> 5], rec, list, M, d, l2tau, total, dproj, mom, tk);
+    bwd_walk<false, kPer, kRed>(S[threadIdx.x >> 5], rec, list, M, d, l2tau, total, dproj, mom, tk);
 }
 
 // The backward's kernel configurations (the autotuner's search space):
