@@ -163,3 +163,50 @@ def test_persistent_backward_matches_the_per_tile_backward():
             lanes = name.split(" per record")[0]
             base = out[lanes + " per record, 128-record warp windows"]
             assert np.linalg.norm(gr - base) <= 1e-6 * np.linalg.norm(base), name
+
+
+def _config_results(w, tau, backward):
+    """Projection (or gradient) of w under every configuration of its kind."""
+    inp = gt.inputs(w)
+    args = [gt.to_dev(inp[k]) for k in ("params", "R", "t")]
+    g = gt.to_dev(syn.smooth_field(w) * 1e-3)
+    ctx = gt.context(w, tau=tau)
+    out = []
+    for i in range(len(_n_configs()[backward])):
+        ctx.gem_set_raster_config(*((-1, i) if backward else (i, -1)))
+        proj = torch.empty(w.B, w.d, w.d, device=gt.DEV)
+        ctx.gem_project(*args, proj)
+        if backward:
+            proj = torch.empty(w.M, 11, device=gt.DEV)
+            ctx.gem_project_backward(g, proj)
+        out.append(proj)
+    assert ctx.gem_status() == 0
+    n = ctx.gem_pair_count()
+    ctx.close()
+    return out, n
+
+
+# lists of several segments in few tiles; more segments and units than any
+# configuration has warps at once (units of both lengths)
+AGREE = [
+    (syn.Workload("agree16", d=16, M=1500, B=3, apix=1.2, n_clusters=1, s_lo=0.8, s_hi=3.0, seed=21), 0.0, 4000),
+    (syn.Workload("agree64", d=64, M=8000, B=96, apix=1.2, seed=22), None, 152 * 8 * 4 * 256),
+]
+
+
+@pytest.mark.parametrize("w,tau,least", AGREE, ids=lambda x: getattr(x, "name", None))
+def test_forward_configurations_agree_bitwise(w, tau, least):
+    out, n = _config_results(w, w.tau if tau is None else tau, 0)
+    assert n > least and len(out) == 8
+    for img in out[1:]:
+        assert torch.equal(img, out[0])
+
+
+@pytest.mark.parametrize("w,tau,least", AGREE, ids=lambda x: getattr(x, "name", None))
+def test_backward_configurations_agree(w, tau, least):
+    """The windows only regroup the records into rounds: the moments are
+    float64 sums of the same partials in another order."""
+    out, n = _config_results(w, w.tau if tau is None else tau, 1)
+    assert n > least and len(out) == 10
+    for grad in out[1:]:
+        assert float((grad - out[0]).norm()) <= 1e-6 * float(out[0].norm())
