@@ -800,7 +800,8 @@ def main():
             fe[i][1].record(stream)
         torch.cuda.synchronize()
         f_ms = sum(a.elapsed_time(b) for a, b in fe) / nq
-        f_bytes = 64 * w.d ** 3  # 3 FFT passes (read + write d^3 complex) and the shell pass (2 reads)
+        # 3 FFT passes (read + write d^3 complex) and the shell pass (one read of the ball inside the last shell)
+        f_bytes = int((48 + 8 * math.pi / 6) * w.d ** 3)
         f_gbs = f_bytes / (f_ms / 1e3) / 1e9
         query["fsc"] = {"ms": f_ms, "resolution_A": float(fsc_out[2].item()), "gpu_launches_per_call": 6,
                         "roofline": {"bound": "hbm", "achieved": f_gbs, "peak": HBM_PEAK_GBS, "unit": "GB/s",

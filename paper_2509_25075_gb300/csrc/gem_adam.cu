@@ -49,8 +49,9 @@ __device__ __forceinline__ void adam_entry(const AdamArgs &a, int m, unsigned j,
 // stores) when all five arrays are 16-byte aligned and that leaves the GPU two
 // CTAs per SM (at M = 6941 a call takes 2% longer with four entries per thread
 // than with one), else one; M <= 2^24, so entry numbers fit 32 bits.
-// M = 500000: 35 us with one entry per thread and 64-bit remainders (5.0
-// TB/s), 25 us (6.9 TB/s) with four.
+// M = 500000 (176 MB): 35 us with one entry per thread and 64-bit remainders,
+// 25 us with four, where a copy of as many bytes takes 26 (a repeated step
+// finds part of them in the 129 MB L2).
 template <int kVec>
 __global__ void __launch_bounds__(256) adam_step_kernel(AdamArgs a, unsigned n,
                                                         float *__restrict__ raw,

@@ -507,8 +507,8 @@ static int backward_common(gem_ctx *c, const float *dproj, float *grad, bool den
       e = launch_dense_bwd(c->rec, c->M, c->B, g.d, c->l2tau, dproj, c->mom, c->stream);
     else
       e = launch_raster_bwd(active_bwd(c, c->B, c->M), c->rec, c->bin.list,
-                            c->bin.tile_start, c->bin.cap, c->M, c->B, g.d, c->l2tau, dproj, c->mom,
-                            c->tasks, c->stream);
+                            c->bin.tile_start, c->M, c->B, g.d, c->l2tau, dproj, c->mom, c->tasks,
+                            c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "raster_bwd");
   }
   StageScope sc(c, GEM_STAGE_PREP_BWD, 2);

@@ -39,9 +39,11 @@
 
 namespace gem {
 
-// Lines per CTA in every pass: 16 where two line buffers of 16 lines would
-// leave room for four CTAs per SM (sides up to 208), else 8 (large images:
-// more, smaller CTAs, so the last wave is short).
+// Lines per CTA in every pass: 16 up to side 208, else 8 (large images: more,
+// smaller CTAs, so the last wave is short).  The line was drawn when a CTA held
+// two line buffers (d 384, B 16: 16 lines 0.168 ms, 8 lines 0.125; d 128, B 256:
+// 0.151 and 0.167); the second pass's line count is also the order in which an
+// image's loss is summed, so it stays.
 constexpr int kCtfThreads = 256;
 __host__ __device__ constexpr int ctf_lines(int d) { return d <= 208 ? 16 : 8; }
 

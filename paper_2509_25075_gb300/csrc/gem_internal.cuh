@@ -376,8 +376,8 @@ const BwdCfg &bwd_config(int i);
 // after every backward (on the device, so that a backward captured alone in a
 // graph finds it zero on each replay).
 cudaError_t launch_raster_bwd(int cfg, const Rec *rec, const uint2 *list,
-                              const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
-                              float l2tau, const float *dproj, double *mom, const RasterTasks &tk,
+                              const int64_t *tile_start, int64_t M, int B, int d, float l2tau,
+                              const float *dproj, double *mom, const RasterTasks &tk,
                               cudaStream_t st);
 cudaError_t launch_count_kept(int cfg, const Rec *rec, const uint2 *list,
                               const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,

@@ -16,7 +16,7 @@
 // the threshold is), and only those get a record and enter the binning.  With
 // a record of every Gaussian in every slice, the records and the count pass
 // over them were 60% of a query (d 256, M 100000, batches of 64 slices:
-// 1.27 ms; 0.49 ms now).
+// 1.27 ms; 0.43 ms now).
 #include "gem_internal.cuh"
 
 namespace gem {
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(kChunkT) slice_write_kernel(
 
 // Few Gaussians: a CTA per slice goes over all their ranges, 1024 at a time,
 // and writes the slice's records and list itself; one launch where the form
-// above takes four.  The counts of a step's warps are double-buffered, so a
+// above takes three.  The counts of a step's warps are double-buffered, so a
 // step has one barrier.
 constexpr int kSelThreads = 1024;
 __global__ void __launch_bounds__(kSelThreads) slice_select_kernel(
@@ -240,7 +240,7 @@ cudaError_t launch_slices(const QueryPrep *qp, const uint32_t *range, int64_t M,
   // Where the two forms meet: us per query of 16384 and 16385 Gaussians, 319
   // and 327 at d 256 and 64 slices per batch, 289 and 299 at d 192 and 50, 258
   // and 255 at d 64 and 16 (launches are most of it); at 4351 Gaussians, d
-  // 192, 50 slices, one launch 228 and four 279.
+  // 192, 50 slices, one launch 228 and three 279.
   if (M <= 16384) {
     slice_select_kernel<<<nslice, kSelThreads, 0, st>>>(qp, range, M, k0, apix, d, l2tau, rec, sel, nsel);
     return cudaGetLastError();

@@ -79,8 +79,8 @@ constexpr int kSegMax = 512;    // entries of the longest segment
 // (the last one shorter); a task is one segment, and the warps that take it
 // work on pieces of it, so that nobody walks a long list alone (the longest
 // list of a workload holds five to twenty times the mean) and a call with few
-// tiles still fills the SMs.  S is a multiple of the forward's window: 1024,
-// less where that would leave resident warps without a segment.  Tasks follow
+// tiles still fills the SMs.  S is a multiple of the forward's window: 512,
+// or 256 where that would leave resident CTAs without a segment.  Tasks follow
 // the tiles' index order up to the order in which the CTAs here claim their
 // ranges, so neighbouring tiles, which share records, are in flight together.
 // Empty tiles get their zeros here and no task.
@@ -871,8 +871,8 @@ int bwd_config_count() { return (int)(sizeof(kBwdCfgs) / sizeof(kBwdCfgs[0])); }
 const BwdCfg &bwd_config(int i) { return kBwdCfgs[i]; }
 
 cudaError_t launch_raster_bwd(int cfg, const Rec *rec, const uint2 *list,
-                              const int64_t *tile_start, int64_t cap, int64_t M, int B, int d,
-                              float l2tau, const float *dproj, double *mom, const RasterTasks &tk,
+                              const int64_t *tile_start, int64_t M, int B, int d, float l2tau,
+                              const float *dproj, double *mom, const RasterTasks &tk,
                               cudaStream_t st) {
   if (cfg < 0 || cfg >= bwd_config_count()) return cudaErrorInvalidValue;
   const BwdCfg &c = kBwdCfgs[cfg];
@@ -905,7 +905,9 @@ __global__ void __launch_bounds__(256) dense_fwd_kernel(const Rec *__restrict__ 
   for (int64_t j = 0; j < M; ++j) {
     Rec r = rb[j];
     float dx = (float)u - r.a.x, dy = (float)v - r.a.y;
-    // -e = z1^2 + (z2^2 - l2A), rounded as the tiled forms round it
+    // -e = z1^2 + (z2^2 - l2A), every product rounded (the tiled forms fuse
+    // u11 dx into z1's sum, so a pair within that rounding of tau can be kept
+    // by one and not by the other)
     float z1 = __fadd_rn(__fmul_rn(r.a.z, dx), __fmul_rn(r.a.w, dy));
     float z2 = __fmul_rn(r.b.x, dy);
     float ff = __fmaf_rn(z1, z1, __fmaf_rn(z2, z2, -r.b.y));
