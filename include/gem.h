@@ -96,7 +96,9 @@ int gem_config_default(gem_config *cfg, int32_t d, float apix, int32_t max_B, in
  * 32 B x max_B x max_M (projected records) + 48 B x max_B x max_M (moments)
  * + 16 B x max_pairs (list entries with their block masks, and the
  * binning's hit records) + 20 B x max_B x d^2 (images, spectra) and
- * a few small tables.  Errors: GEM_EINVAL, GEM_ENOMEM, GEM_ECUDA. */
+ * a few small tables.  Waits for what is queued on the legacy default stream,
+ * its own clears among it, so the context can be used on any stream at once.
+ * Errors: GEM_EINVAL, GEM_ENOMEM, GEM_ECUDA. */
 int gem_create(gem_ctx **out, const gem_config *cfg, void *cuda_stream);
 
 /* Message of the last gem_create that failed on this thread ("" after a success). */

@@ -384,7 +384,7 @@ __device__ __forceinline__ RowGeo make_row_geo(const Rec &r, float l2tau) {
 // centre, so the strip's extremes are the edges at dyL and -dyL clamped to the
 // strip: two square roots and no comparison of candidates.  No product feeds
 // a plain sum, so there is nothing to contract and each inlined copy returns
-// the same bits.  (The counting pass is bound by issue, 77% of its slots, and
+// the same bits.  (The counting pass is bound by issue, 78% of its slots, and
 // the integer pipe, 63%: against four candidate edges, two of them chosen by
 // comparison, and masks built per tile and row, a gradient step takes 1514 ->
 // 1488 us at d 128, M 20000, B 256 and 1674 -> 1654 us at d 128, M 50000,

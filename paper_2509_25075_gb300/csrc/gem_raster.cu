@@ -646,7 +646,8 @@ __device__ __forceinline__ int unit_length(int64_t total, int nwarps) {
 // lies at 2.  Each form is an instance of its own: one loop with both took 1 to
 // 3% longer.
 //
-// What bounds it: the FMA pipe (57% of its cycles) and issue (66%).  Against
+// What bounds it: the L1 (72%: the scattered additions), issue (65% of the
+// slots) and the FMA pipe (57% of its cycles), at d 384, M 500000.  Against
 // CTAs of four warps that walked a whole tile's list, the longest lists first
 // (us per backward, the default configuration then and now): d 384, M 500000,
 // B 3: 699, 271; d 128, M 20000, B 256: 677, 623; d 128, M 50000, B 64, scales
