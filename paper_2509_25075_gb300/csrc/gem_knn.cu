@@ -352,15 +352,17 @@ __device__ __forceinline__ void knn_visit(KBest<K> &best, const float4 *__restri
 // row; with constants half and twice these, times are the same within 10% but
 // for a few sets.
 //
-// Bound by the latency of the loads at k = 1, by insertions at k = 16 (hence
-// three CTAs per SM there: 80 registers).  Calls of M = 300000, us, with one
-// thread per centre, a gather of the parameter row per candidate and two bounds
-// per cell; with sorted centres, rows, 3/2 M cells and the warp from the
-// second ring on; now:  64 clusters, k = 1: 402, 145, 129; k = 4: 626, 486,
-// 243; k = 8: 918, 1034, 434; k = 16: 1743, 5889, 1076.  A plane, k = 1: 138,
-// 109, 74; k = 16: 533, 4787, 444.  Uniform, k = 8: 559, 854, 236.
+// Bound by the latency of the loads at k = 1, by insertions at k = 16, which
+// wait for each other: as many CTAs per SM as the lists leave registers for
+// (left to the compiler, three instead of four at k = 8: 583 us, not 426, below).
+// Calls of M = 300000, us, with one thread per centre, a gather of the
+// parameter row per candidate and two bounds per cell; with sorted centres,
+// rows, 3/2 M cells and the warp from the second ring on; now:  64 clusters,
+// k = 1: 402, 145, 129; k = 4: 626, 486, 245; k = 8: 918, 1034, 426; k = 16: 1743,
+// 5889, 1075.  A plane, k = 1: 138, 109, 74; k = 16: 533, 4787, 443.  Uniform,
+// k = 8: 559, 854, 233.
 template <int K>
-__global__ void __launch_bounds__(kKnnBlk, K > 8 ? 3 : 1) knn_query_kernel(
+__global__ void __launch_bounds__(kKnnBlk, K > 8 ? 3 : K > 4 ? 4 : 5) knn_query_kernel(
     const float4 *__restrict__ sorted, int64_t M, const KnnGrid *__restrict__ g,
     const int *__restrict__ start, float *__restrict__ dist, int32_t *__restrict__ idx) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
