@@ -619,11 +619,13 @@ __device__ __forceinline__ void block_moments(const float4 (*__restrict__ sg)[16
 
 // Entries of a backward unit: 256, or 128 where the lists hold no more than one
 // and a half times 256 for every warp of the grid, so that the last units take
-// less of the time.  us per backward with units of 64, 128, 256, by entries per
-// warp / 256 (d 128, M 20000): 0.8: 71, 72, 90; 1.26: 98, 91, 101; 1.5: 110, 104,
-// 107; 2: 141, 128, 127; 4: 279, 218, 202.
+// less of the time, or 64 where they hold no more than 32 and most warps would
+// have none.  us per backward with units of 64, 128, 256, by entries per
+// warp / 256: 0.01 (d 64, M 2000): 20, 21, -; 0.125: 29, 31, -; 0.2: 40, 34, -;
+// 0.8 (d 128, M 20000): 71, 72, 90; 1.26: 98, 91, 101; 1.5: 110, 104, 107; 2: 141,
+// 128, 127; 4: 279, 218, 202.
 __device__ __forceinline__ int unit_length(int64_t total, int nwarps) {
-  return total <= 384 * (int64_t)nwarps ? 128 : 256;
+  return total <= 32 * (int64_t)nwarps ? 64 : total <= 384 * (int64_t)nwarps ? 128 : 256;
 }
 
 // a5.  Every warp works on its own: a unit is up to 256 consecutive entries of
