@@ -354,7 +354,7 @@ __device__ __forceinline__ void knn_visit(KBest<K> &best, const float4 *__restri
 //
 // Bound by the latency of the loads at k = 1, by insertions at k = 16, which
 // wait for each other: as many CTAs per SM as the lists leave registers for
-// (left to the compiler, three instead of four at k = 8: 583 us, not 426, below).
+// (three instead of four at k = 8: 583 us, not 426, below).
 // Calls of M = 300000, us, with one thread per centre, a gather of the
 // parameter row per candidate and two bounds per cell; with sorted centres,
 // rows, 3/2 M cells and the warp from the second ring on; now:  64 clusters,
